@@ -197,10 +197,20 @@ uint32_t rollout_mlp_tiled_eb(int shape, uint32_t episodes);
 int launch_rollout_mlp_tiled(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 bool rollout_tl_tc_supported(const RolloutMlpArgs& a);
 int launch_rollout_tl_tc(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
+uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
+int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
 static bool use_tiled(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice)
 {
     return choice != EVO_ROLLOUT_GENERIC && rollout_mlp_tiled_shape(task, n_layers, sizes) >= 0;
+}
+
+// Any other number of layers, or wider ones: the tensor-core kernel with the weights in shared memory, as long as
+// they fit it (0 otherwise; the runtime-shape kernel then reads them through the caches).
+static uint32_t mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t episodes)
+{
+    if (choice != EVO_ROLLOUT_AUTO || use_tiled(task, n_layers, sizes, choice)) return 0;
+    return rollout_mlp_mma_eb(task, n_layers, sizes, episodes);
 }
 
 void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
@@ -210,10 +220,13 @@ void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
         *n_eb = (cfg.episodes + *EB - 1u) / *EB;
         return;
     }
-    uint32_t eb = cfg.episodes < 32u ? cfg.episodes : 32u;
-    // few members: split the episodes of a member over more blocks to fill the SMs
-    while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * 148u)
-        eb = (eb + 1u) / 2u;
+    uint32_t eb = mma_eb(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.episodes);
+    if (eb == 0u) {
+        eb = cfg.episodes < 32u ? cfg.episodes : 32u;
+        // few members: split the episodes of a member over more blocks to fill the SMs
+        while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * 148u)
+            eb = (eb + 1u) / 2u;
+    }
     *EB = eb;
     *n_eb = (cfg.episodes + eb - 1u) / eb;
 }
@@ -242,6 +255,10 @@ int launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a_in, uint32_t ker
         launches += r;
     } else if (tiled_ok && kernel_choice != EVO_ROLLOUT_GENERIC) {
         const int r = launch_rollout_mlp_tiled(st, a, status);
+        if (r < 0) return r;
+        launches += r;
+    } else if (mma_eb(a.task, a.n_layers, a.sizes, kernel_choice, a.E) != 0u) {
+        const int r = launch_rollout_mlp_mma(st, a, status);
         if (r < 0) return r;
         launches += r;
     } else {

@@ -1,0 +1,361 @@
+// Control roll-out for any multi-layer policy whose weights fit one SM's shared memory, on warp-level
+// tensor-core products (mma_split.cuh).
+//
+// Block = (member, EB episodes).  The member's weights are split into fp16 pairs once and kept in shared
+// memory in operand order: a 16x16 tile is one 128-bit load per lane and part.  A warp takes 16 units of a
+// layer (several if the layer has more than the block's warps), applies bias and tanh to its accumulators in
+// registers, and writes the two fp16 parts of the result as the next layer's B operand.  A layer so costs one
+// barrier, and the serial chain of a step is about 230 clocks per layer.  The dynamics of the tanh-linear task
+// are one more layer ([A | B] on the state with the action behind it); the cart-pole's five inputs are taken
+// in fp32, and a warp of its own steps the task, which works on the coming step while the layers run.
+//
+// Bounds: shared-memory reads of the weight operands (1 KB per tile and step) at many members per SM, the chain
+// of a step at few.
+//
+// Paper: Section 2 (roll-out loop, central seeds), Section 4 (get_actions over the population with parameters as
+// data; stateless task step; identical initial observations).
+#include "internal.h"
+#include "async.cuh"
+#include "mma_split.cuh"
+#include "noise.cuh"
+#include "tasks.cuh"
+
+namespace evo {
+namespace {
+
+using namespace ms;
+
+constexpr uint32_t kXPitch = 48 * 2 + 16;           // bytes per column of the [x 28 | 0 4 | a 8 | 0 8] operand
+constexpr size_t kMaxSmem = 220u * 1024u;
+
+struct Plan {
+    uint32_t mt[EVO_MAX_LAYERS + 1], kt[EVO_MAX_LAYERS + 1];   // 16-unit and 16-input tiles of a layer; last entry: dynamics
+    uint32_t tile0[EVO_MAX_LAYERS + 1];             // first tile of a layer in the operand area
+    uint32_t bias0[EVO_MAX_LAYERS + 1];             // first float of a layer's biases
+    uint32_t tiles, biases, pitch;                  // pitch: bytes per column of the hidden operands
+    uint32_t warps;                                 // layer warps
+    size_t   smem;
+};
+
+// EB episodes as MMA columns: 4 in pairs (hi and lo side by side), 8 in planes (hi rows, then lo rows)
+template <int EB> struct Cols;
+template <> struct Cols<4> { static constexpr int rows = 8, values = 2; };
+template <> struct Cols<8> { static constexpr int rows = 16, values = 4; };
+
+__device__ __forceinline__ void stsm_x4_t(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
+                 :: "r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+
+// values of this lane (EB = 4: units g, g + 8 of episode t; EB = 8: unit g of episodes 2t, 2t + 1, then unit g + 8)
+// as 16 units from `unit0` on of an operand
+template <int EB>
+__device__ __forceinline__ void store_units(uint32_t base, uint32_t pitch, uint32_t unit0, int lane, const float* v)
+{
+    if constexpr (EB == 4) {
+        const uint32_t addr = base + (lane & 7) * pitch + (unit0 + 8u * ((lane >> 3) & 1)) * 2u;
+        stsm_x2_t(addr, split_pair(v[0]), split_pair(v[1]));
+    } else {
+        const uint32_t addr = base + ((lane & 7) + 8 * (lane >> 4)) * pitch + (unit0 + 8u * ((lane >> 3) & 1)) * 2u;
+        const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
+        const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
+        const __half2 l0 = __floats2half2_rn(v[0] - f0.x, v[1] - f0.y), l1 = __floats2half2_rn(v[2] - f1.x, v[3] - f1.y);
+        stsm_x4_t(addr, *reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1),
+                  *reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+    }
+}
+
+// pre-activations of 16 units: tiles = the units' weight tiles in operand order, b0/b1 their biases (units g, g + 8)
+template <int EB>
+__device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint32_t in, uint32_t pitch, int lane, float b0,
+                                          float b1, float* v)
+{
+    const uint32_t addr = EB == 4 ? in + (lane & 7) * pitch + 16u * ((lane >> 3) & 1)
+                                  : in + ((lane & 7) + 8 * (lane >> 4)) * pitch + 16u * ((lane >> 3) & 1);
+    if constexpr (EB == 4) {
+        float h[4] = { b0, 0.f, b1, 0.f }, l[4] = { 0.f, 0.f, 0.f, 0.f };
+#pragma unroll 4
+        for (uint32_t k = 0; k < kt; ++k) {
+            const uint4 wh = tiles[k * 64u + lane], wl = tiles[k * 64u + 32u + lane];
+            uint32_t x0, x1;
+            ldsm_x2(addr + 32u * k, x0, x1);
+            mma_k16(h, wh, x0, x1);
+            mma_k16(l, wl, x0, x1);
+        }
+        v[0] = (h[0] + h[1]) + (l[0] + l[1]);
+        v[1] = (h[2] + h[3]) + (l[2] + l[3]);
+    } else {
+        float hh[4] = { b0, b0, b1, b1 }, hl[4] = { 0.f, 0.f, 0.f, 0.f }, lh[4] = { 0.f, 0.f, 0.f, 0.f };
+#pragma unroll 4
+        for (uint32_t k = 0; k < kt; ++k) {
+            const uint4 wh = tiles[k * 64u + lane], wl = tiles[k * 64u + 32u + lane];
+            uint32_t x0, x1, y0, y1;
+            ldsm_x4(addr + 32u * k, x0, x1, y0, y1);
+            mma_k16(hh, wh, x0, x1);
+            mma_k16(hl, wh, y0, y1);
+            mma_k16(lh, wl, x0, x1);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = hh[i] + (hl[i] + lh[i]);
+    }
+}
+
+template <int EB> __device__ __forceinline__ void tanh_values(float* v)
+{
+    if constexpr (EB == 4) tanh2(v[0], v[1]);
+    else tanh4(v[0], v[1], v[2], v[3]);
+}
+
+template <int EB, bool CART>
+__global__ void __launch_bounds__(288)
+k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
+{
+    constexpr int NV = Cols<EB>::values;
+    extern __shared__ __align__(16) unsigned char mma_smem[];
+    __shared__ float obs[5][EB], act[EB], x0s[kTlNx][EB], rets[9][EB];
+    uint4* tiles = reinterpret_cast<uint4*>(mma_smem);
+    float* bias = reinterpret_cast<float*>(mma_smem + static_cast<size_t>(p.tiles) * 1024u);
+    float* w_in = bias + p.biases;                                   // cart-pole: [unit][8] = five weights, bias
+    const uint32_t buf0 = smem_u32(w_in + (CART ? p.mt[0] * 128u : 0u));
+    const uint32_t buf_bytes = Cols<EB>::rows * p.pitch;
+    const uint32_t xbuf = buf0 + 2u * buf_bytes;                     // tanh-linear: two state operands
+    constexpr uint32_t xbuf_bytes = Cols<EB>::rows * kXPitch;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const uint32_t member = blockIdx.x, eb = blockIdx.y, e0 = eb * EB;
+    const int nE = min(static_cast<uint32_t>(EB), a.E - e0);
+    const uint32_t layers = a.n_layers, nw = p.warps;
+    const bool layer_warp = warp < static_cast<int>(nw);
+    const PhiloxKey key = philox_key(a.k0, a.k1);
+    dep_wait();
+    const uint32_t generation = status->generation;
+    const float* th = a.theta + static_cast<size_t>(member) * a.ldD;
+
+    // ---- weights: rows of theta -> operand tiles (whole warps, one tile at a time) --------------------
+    {
+        uint32_t off = 0;
+        for (uint32_t l = 0; l < layers; ++l) {
+            const int ni = static_cast<int>(a.sizes[l]), no = static_cast<int>(a.sizes[l + 1]);
+            const float* W = th + off;
+            const float* B = W + ni * no;
+            off += static_cast<uint32_t>(ni * no + no);
+            if (CART && l == 0) {
+                for (uint32_t i = tid; i < p.mt[0] * 128u; i += blockDim.x) {
+                    const int u = static_cast<int>(i >> 3), k = static_cast<int>(i & 7u);
+                    w_in[i] = (u < no && k < 6) ? (k < 5 ? __ldg(W + u * 5 + k) : __ldg(B + u)) : 0.f;
+                }
+                continue;
+            }
+            for (uint32_t i = warp; i < p.mt[l] * p.kt[l]; i += blockDim.x >> 5) {
+                uint4 hi, lo;
+                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, hi, lo);
+                tiles[(p.tile0[l] + i) * 64u + lane] = hi;
+                tiles[(p.tile0[l] + i) * 64u + 32u + lane] = lo;
+            }
+            for (uint32_t i = tid; i < p.mt[l] * 16u; i += blockDim.x) bias[p.bias0[l] + i] = static_cast<int>(i) < no ? __ldg(B + i) : 0.f;
+        }
+        if (!CART) {                                                 // x' = tanh([A | 0 | B] [x | 0 | a])
+            const float* A = a.task_const;
+            const float* Bm = a.task_const + kTlNx * kTlNx;
+            for (uint32_t i = warp; i < 6u; i += blockDim.x >> 5) {
+                uint4 hi, lo;
+                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, hi, lo);
+                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, hi, lo);
+                tiles[(p.tile0[layers] + i) * 64u + lane] = hi;
+                tiles[(p.tile0[layers] + i) * 64u + 32u + lane] = lo;
+            }
+            for (uint32_t i = tid; i < 2u * xbuf_bytes / 4u; i += blockDim.x)
+                reinterpret_cast<uint32_t*>(mma_smem + (xbuf - smem_u32(mma_smem)))[i] = 0u;
+        }
+    }
+
+    // ---- reset: seeded start states, the same for every member -----------------------------------------
+    CartpoleFast cpc{};
+    CpState cps{};
+    float snc = 0.f, csc = 1.f, ret = 0.f, ret2 = 0.f;
+    const int te = lane % EB;                                        // task warp: its lane's episode (others mirror)
+    if (CART) {
+        if (!layer_warp) {
+            cpc = cartpole_fast_const(a.tp);
+            cps = cartpole_reset(key, generation, e0 + min(te, nE - 1), a.tp[EVO_CP_INIT_RANGE]);
+            sincos_fast(cps.th, snc, csc);
+            if (lane < EB) { obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd; }
+        }
+        __syncthreads();
+    } else {
+        for (int i = tid; i < (static_cast<int>(kTlNx) / 4) * EB; i += blockDim.x) {
+            const int q = i / EB, e = i % EB;
+            const float4 z = stream_normal4(key, 1u, generation, e0 + min(e, nE - 1), q);
+            x0s[4 * q][e] = z.x; x0s[4 * q + 1][e] = z.y; x0s[4 * q + 2][e] = z.z; x0s[4 * q + 3][e] = z.w;
+        }
+        __syncthreads();
+        for (uint32_t m = warp; m < 2u; m += nw) {
+            float v[NV];
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
+                const int e = EB == 4 ? t : 2 * t + (i & 1);
+                v[i] = row < kTlNx ? x0s[row][e] : 0.f;
+                if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
+            }
+            store_units<EB>(xbuf, kXPitch, 16u * m, lane, v);
+        }
+        __syncthreads();
+    }
+
+    // ---- time loop -----------------------------------------------------------------------------------------
+    for (uint32_t step = 0; step < a.T; ++step) {
+        const uint32_t xin = xbuf + (step & 1u) * xbuf_bytes, xout = xbuf + ((step + 1u) & 1u) * xbuf_bytes;
+        CpAhead ahead{};
+        if (CART && !layer_warp) ahead = cartpole_ahead(cpc, cps, snc, csc);
+        for (uint32_t l = 0; l < layers; ++l) {
+            const bool last = l + 1u == layers;
+            const uint32_t in = l == 0u ? xin : buf0 + ((l + 1u) & 1u) * buf_bytes, out = buf0 + (l & 1u) * buf_bytes;
+            const uint32_t in_pitch = l == 0u ? kXPitch : p.pitch;
+            if (layer_warp) {
+                for (uint32_t m = warp; m < p.mt[l]; m += nw) {
+                    float v[NV];
+                    if (CART && l == 0u) {
+                        const float* wa = w_in + (16u * m + g) * 8u;
+                        const float4 w0 = *reinterpret_cast<const float4*>(wa), w1 = *reinterpret_cast<const float4*>(wa + 64);
+                        const float2 q0 = *reinterpret_cast<const float2*>(wa + 4), q1 = *reinterpret_cast<const float2*>(wa + 68);
+#pragma unroll
+                        for (int i = 0; i < NV; ++i) {
+                            const int e = EB == 4 ? t : 2 * t + (i & 1);
+                            const bool up = i >= NV / 2;
+                            float s = fmaf(up ? w1.x : w0.x, obs[0][e], up ? q1.y : q0.y);
+                            s = fmaf(up ? w1.y : w0.y, obs[1][e], s);
+                            s = fmaf(up ? w1.z : w0.z, obs[2][e], s);
+                            s = fmaf(up ? w1.w : w0.w, obs[3][e], s);
+                            v[i] = fmaf(up ? q1.x : q0.x, obs[4][e], s);
+                        }
+                    } else {
+                        const float* bb = bias + p.bias0[l] + 16u * m + g;
+                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], v);
+                    }
+                    tanh_values<EB>(v);
+                    if (!last) {
+                        store_units<EB>(out, p.pitch, 16u * m, lane, v);
+                    } else if (CART) {
+                        if (g == 0) {
+                            if (EB == 4) act[t] = v[0];
+                            else { act[2 * t] = v[0]; act[2 * t + 1] = v[1]; }
+                        }
+                    } else {                                         // units 8..15 are padding: zeros
+#pragma unroll
+                        for (int i = 0; i < NV; ++i) {
+                            v[i] *= a.action_scale;
+                            if (i < NV / 2) { if (EB == 4 || !(i & 1)) ret = fmaf(-0.01f * v[i], v[i], ret); else ret2 = fmaf(-0.01f * v[i], v[i], ret2); }
+                        }
+                        store_units<EB>(xin, kXPitch, 32u, lane, v);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        if (CART) {
+            if (!layer_warp) {
+                cartpole_finish(cpc, ahead, a.action_scale * act[te], cps, snc, csc);
+                ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
+                if (lane < EB) {
+                    obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
+                    if (a.trace && step < a.trace_T && te < nE)
+                        *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
+                            make_float4(cps.x, cps.xd, cps.th, cps.thd);
+                }
+            }
+        } else {
+            for (uint32_t m = warp; m < 2u; m += nw) {
+                float v[NV];
+                unit_sums<EB>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane, 0.f, 0.f, v);
+                tanh_values<EB>(v);
+                store_units<EB>(xout, kXPitch, 16u * m, lane, v);
+#pragma unroll
+                for (int i = 0; i < NV; ++i) {
+                    const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
+                    const int e = EB == 4 ? t : 2 * t + (i & 1);
+                    if (step + 1u < a.T) {                           // reward of the next step: its pre-step state (padding rows are 0)
+                        if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
+                    }
+                    if (a.trace && step < a.trace_T && e < nE && row < kTlNx)
+                        a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + row] = v[i];
+                }
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- block return: fixed order --------------------------------------------------------------------------
+    if (CART) {
+        if (!layer_warp && lane < EB) rets[0][te] = ret;
+    } else {
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+            ret += __shfl_xor_sync(0xffffffffu, ret, off);
+            ret2 += __shfl_xor_sync(0xffffffffu, ret2, off);
+        }
+        if (g == 0) {
+            if (EB == 4) rets[warp][t] = ret;
+            else { rets[warp][2 * t] = ret; rets[warp][2 * t + 1] = ret2; }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        float s = 0.f;
+        for (int e = 0; e < nE; ++e)
+            for (uint32_t w = 0; w < (CART ? 1u : nw); ++w) s += rets[w][e];
+        if (EVO_IN_BOUNDS(status, EVO_SITE_FIT_PARTIAL, static_cast<size_t>(member) * a.n_eb + eb, static_cast<size_t>(a.P) * a.n_eb))
+            a.fit_partial[static_cast<size_t>(member) * a.n_eb + eb] = s;
+    }
+}
+
+Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB)
+{
+    Plan p = {};
+    const bool cart = task == EVO_TASK_CARTPOLE;
+    uint32_t widest = 0;
+    for (uint32_t l = 0; l < n_layers; ++l) {
+        p.mt[l] = (sizes[l + 1] + 15u) / 16u;
+        p.kt[l] = l == 0u ? 2u : (sizes[l] + 15u) / 16u;
+        p.bias0[l] = p.biases;
+        p.tile0[l] = p.tiles;
+        if (!(cart && l == 0u)) { p.tiles += p.mt[l] * p.kt[l]; p.biases += p.mt[l] * 16u; }
+        if (p.mt[l] > widest) widest = p.mt[l];
+    }
+    p.tile0[n_layers] = p.tiles;
+    p.mt[n_layers] = 2; p.kt[n_layers] = 3;
+    if (!cart) { p.tiles += 6u; if (widest < 2u) widest = 2u; }
+    p.pitch = widest * 32u + 16u;
+    p.warps = widest < 8u ? widest : 8u;
+    const uint32_t rows = EB == 4u ? 8u : 16u;
+    p.smem = static_cast<size_t>(p.tiles) * 1024u + p.biases * 4u + (cart ? p.mt[0] * 512u : 0u) + 2u * rows * p.pitch +
+             (cart ? 0u : 2u * rows * kXPitch);
+    return p;
+}
+
+}  // namespace
+
+// Episodes per block: 4, or 8 if a member has more (three MMAs then serve twice the episodes that two do).  0: the
+// weights do not fit.
+uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes)
+{
+    const uint32_t eb = episodes > 4u ? 8u : 4u;
+    return make_plan(task, n_layers, sizes, eb).smem <= kMaxSmem ? eb : 0u;
+}
+
+int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status)
+{
+    const Plan p = make_plan(a.task, a.n_layers, a.sizes, a.EB);
+    if (p.smem > kMaxSmem) return -2;
+    const bool cart = a.task == EVO_TASK_CARTPOLE;
+    auto kernel = a.EB == 4u ? (cart ? k_rollout_mlp_mma<4, true> : k_rollout_mlp_mma<4, false>)
+                             : (cart ? k_rollout_mlp_mma<8, true> : k_rollout_mlp_mma<8, false>);
+    if (!a.attr_done &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) != cudaSuccess)
+        return -1;
+    const uint32_t threads = 32u * (p.warps + (cart ? 1u : 0u));
+    return launch_dependent(kernel, dim3(a.P, a.n_eb), dim3(threads), p.smem, st, a, p, status) == cudaSuccess ? 1 : -1;
+}
+
+}  // namespace evo

@@ -162,4 +162,112 @@ __device__ __forceinline__ CpState cartpole_step_fast(const CartpoleConst& c, co
     return cartpole_step_fast_sc(c, s, force, sn, cs);
 }
 
+
+// ---- the same step split around the force -----------------------------------------------------------
+// The policy's force is the last thing a step waits for, and the step is a serial chain per episode, so
+// whatever does not need the force is done before it arrives.  At a fixed angle the angular acceleration is
+//     w' = A - B F - C w^2      A = g s / den, B = c / (M den), C = m l s c / (M den), den = l (4/3 - m c^2 / M)
+// and the angles of the first two Runge-Kutta stages are known without F (the second is half a step of the present
+// angular velocity on).  After F there remain four short multiply-add chains; the sin/cos rotations of
+// the third and fourth stage run side by side, because an angle needs only the velocity of the stage before.
+struct CartpoleFast { float g, inv_m, ml, ml_m, l43, lm, h, h2, w6; };
+struct CpAhead { float k1, b1, ww, a2, b2, c2, s2, cs2; };       // what the coming step knows without the force
+
+__device__ __forceinline__ CartpoleFast cartpole_fast_const(const float* tp)
+{
+    CartpoleFast c;
+    c.g = tp[EVO_CP_GRAVITY];
+    c.inv_m = 1.0f / (tp[EVO_CP_CART_MASS] + tp[EVO_CP_POLE_MASS]);
+    c.ml = tp[EVO_CP_POLE_MASS] * tp[EVO_CP_POLE_HALF_LENGTH];
+    c.ml_m = c.ml * c.inv_m;
+    c.l43 = tp[EVO_CP_POLE_HALF_LENGTH] * (4.0f / 3.0f);
+    c.lm = tp[EVO_CP_POLE_HALF_LENGTH] * tp[EVO_CP_POLE_MASS] * c.inv_m;
+    c.h = tp[EVO_CP_DT]; c.h2 = 0.5f * c.h; c.w6 = c.h * (1.0f / 6.0f);
+    return c;
+}
+
+// (sn, cs) turned through the small angle d (Taylor to d^7 / d^8: error < 3e-6 even at |d| = 1)
+__device__ __forceinline__ void turn_by(float d, float sn, float cs, float& s2, float& c2)
+{
+    const float z = d * d;
+    float sd = fmaf(z, -1.98412698e-4f, 8.33333333e-3f);
+    float cd = fmaf(z, 2.48015873e-5f, -1.38888889e-3f);
+    sd = fmaf(sd, z, -1.66666667e-1f);
+    cd = fmaf(cd, z, 4.16666667e-2f);
+    sd = fmaf(sd * z, d, d);
+    cd = fmaf(cd, z, -0.5f);
+    cd = fmaf(cd, z, 1.0f);
+    s2 = fmaf(sn, cd, cs * sd);
+    c2 = fmaf(cs, cd, -sn * sd);
+}
+
+__device__ __forceinline__ void cartpole_terms(const CartpoleFast& c, float sn, float cs, float& a, float& b, float& k)
+{
+    const float inv_den = __fdividef(1.0f, fmaf(-c.lm * cs, cs, c.l43));
+    a = c.g * sn * inv_den;
+    b = cs * c.inv_m * inv_den;
+    k = b * (c.ml * sn);
+}
+
+__device__ __forceinline__ CpAhead cartpole_ahead(const CartpoleFast& c, const CpState& s, float sn, float cs)
+{
+    CpAhead p;
+    float a1, c1;
+    cartpole_terms(c, sn, cs, a1, p.b1, c1);
+    p.ww = s.thd * s.thd;
+    p.k1 = fmaf(-c1, p.ww, a1);
+    turn_by(c.h2 * s.thd, sn, cs, p.s2, p.cs2);
+    cartpole_terms(c, p.s2, p.cs2, p.a2, p.b2, p.c2);
+    return p;
+}
+
+// The rest of the step: new state, and sin/cos of its angle (quarter turn taken from the last stage's angle, which is
+// within the step's error of the new one; polynomials as in sincos_fast).
+__device__ __forceinline__ void cartpole_finish(const CartpoleFast& c, const CpAhead& p, float force, CpState& s, float& sn,
+                                                float& cs)
+{
+    const float w1 = fmaf(-p.b1, force, p.k1);
+    const float o2 = fmaf(c.h2, w1, s.thd);
+    const float w2 = fmaf(-p.c2, o2 * o2, fmaf(-p.b2, force, p.a2));
+    const float o3 = fmaf(c.h2, w2, s.thd);
+    float s3, c3, s4, c4, a, b, k;
+    turn_by(c.h2 * o2, sn, cs, s3, c3);
+    turn_by(c.h * o3, sn, cs, s4, c4);
+    const float kf = rintf(fmaf(c.h, o3, s.th) * 0.636619772f);
+    cartpole_terms(c, s3, c3, a, b, k);
+    const float o33 = o3 * o3;
+    const float w3 = fmaf(-k, o33, fmaf(-b, force, a));
+    const float o4 = fmaf(c.h, w3, s.thd);
+    cartpole_terms(c, s4, c4, a, b, k);
+    const float o44 = o4 * o4;
+    const float w4 = fmaf(-k, o44, fmaf(-b, force, a));
+    const float fm = force * c.inv_m;
+    const float x1 = fmaf(c.ml_m, fmaf(p.ww, sn, -w1 * cs), fm);
+    const float x2 = fmaf(c.ml_m, fmaf(o2 * o2, p.s2, -w2 * p.cs2), fm);
+    const float x3 = fmaf(c.ml_m, fmaf(o33, s3, -w3 * c3), fm);
+    const float x4 = fmaf(c.ml_m, fmaf(o44, s4, -w4 * c4), fm);
+    const float v2 = fmaf(c.h2, x1, s.xd), v3 = fmaf(c.h2, x2, s.xd), v4 = fmaf(c.h, x3, s.xd);
+    const float th = fmaf(c.w6, (s.thd + o4) + 2.0f * (o2 + o3), s.th);
+    s.x = fmaf(c.w6, (s.xd + v4) + 2.0f * (v2 + v3), s.x);
+    s.xd = fmaf(c.w6, (x1 + x4) + 2.0f * (x2 + x3), s.xd);
+    s.thd = fmaf(c.w6, (w1 + w4) + 2.0f * (w2 + w3), s.thd);
+    s.th = th;
+    float r = fmaf(kf, -1.57079637f, th);
+    r = fmaf(kf, 4.37113883e-8f, r);
+    const float z = r * r;
+    float sp = fmaf(z, 2.75573192e-6f, -1.98412698e-4f);
+    float cp = fmaf(z, 2.48015873e-5f, -1.38888889e-3f);
+    sp = fmaf(sp, z, 8.33333333e-3f);
+    cp = fmaf(cp, z, 4.16666667e-2f);
+    sp = fmaf(sp, z, -1.66666667e-1f);
+    cp = fmaf(cp, z, -0.5f);
+    const float s0 = fmaf(sp * z, r, r);
+    const float c0 = fmaf(cp, z, 1.0f);
+    const int q = __float2int_rn(kf) & 3;
+    const float u = (q & 1) ? s0 : c0;
+    const float v = (q & 1) ? c0 : s0;
+    cs = (q == 1 || q == 2) ? -u : u;
+    sn = (q >= 2) ? -v : v;
+}
+
 }  // namespace evo

@@ -1,0 +1,65 @@
+"""Control roll-outs on warp-level tensor-core products against the oracle, at the shapes where the tiling can go
+wrong: widths at and around multiples of 16, one layer to five, layers of fewer and of more units than a
+block has warps for, episode counts around the 4 and 8 that a block takes."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import rel_err, oracle_fitness, cartpole_features
+from paper_2202_05008_b200 import Solver, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# the bounds of the control roll-outs: state 1e-4 of a component's RMS, fitness 1e-3
+STATE_TOL, FIT_TOL = 1e-4, 1e-3
+
+
+def check(sizes, episodes, T, pop=4, scale=0.25, theta=None, generation=0):
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=pop, episodes=episodes, horizon=T, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
+    s = Solver(w, trace_steps=T)
+    if theta is None:
+        theta = W.random_parameters(sum(sizes), pop, w.param_dim, scale=scale)
+    if generation:
+        s.set_state(generation=generation)
+    arg = s.padded_rows(pop)
+    arg[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    trace = torch.zeros(pop, episodes, T, 4 if sizes[0] == 5 else 28, device="cuda")
+    fit = s.rollout(arg, trace=trace)
+    again = s.rollout(arg).clone()
+    assert s.sync_status() == 0
+    assert torch.equal(fit, again)
+    fit_o, traces_o = oracle_fitness(w, theta, generation, T, want_trace=True)
+    assert rel_err(fit.cpu().numpy(), fit_o, floor=1.0) < FIT_TOL
+    for m in range(pop):
+        got, want = trace[m].cpu().numpy().astype(np.float64), traces_o[m]
+        if sizes[0] == 5:
+            got, want = cartpole_features(got), cartpole_features(want)
+        for i in range(got.shape[-1]):
+            assert rel_err(got[..., i], want[..., i]) < STATE_TOL, (m, i)
+    s.close()
+
+
+@pytest.mark.parametrize("sizes", [(28, 8), (28, 17, 8), (28, 16, 15, 8), (28, 64, 64, 64, 8), (28, 130, 5, 33, 16, 8),
+                                   (28, 200, 8), (28, 129, 129, 8)])
+@pytest.mark.parametrize("episodes", [1, 4, 5, 9])
+def test_tanh_linear_shapes(sizes, episodes):
+    check(sizes, episodes, 40, scale=0.05)
+
+
+@pytest.mark.parametrize("sizes", [(5, 1), (5, 33, 1), (5, 16, 16, 16, 1), (5, 200, 12, 1), (5, 129, 7, 3, 31, 1)])
+@pytest.mark.parametrize("episodes", [1, 4, 5, 17])
+def test_cartpole_shapes(sizes, episodes):
+    check(sizes, episodes, 60)
+
+
+def test_a_nan_parameter_reaches_the_fitness():
+    sizes = (28, 24, 24, 24, 8)
+    w = W.CFG4.with_(pop_size=4, episodes=4, horizon=5, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
+    s = Solver(w)
+    arg = s.padded_rows(4)
+    arg[1, 3] = float("nan")                               # a first-layer weight
+    arg[2, 24 * 28 + 24 + 24 * 24] = float("nan")          # a second-layer bias
+    fit = s.rollout(arg)
+    assert torch.isnan(fit).tolist() == [False, True, True, False] and s.sync_status() == 0
+    s.close()
