@@ -88,13 +88,12 @@ def stage_work(w, stored):
 # that digest; once a kernel's source changes its entry reads null until it is captured again.
 CSRC = os.path.join(ROOT, "paper_2202_05008_b200", "csrc")
 NCU_TRAFFIC = {
-    ("cfg4", "stored"): {"kernel": "k_rollout_tl_tc", "bytes": 3.490288e+08,
-                         "files": ['rollout_tl_tc.cu', 'umma.cuh', 'async.cuh', 'noise.cuh', 'fp32x2.cuh', 'internal.h'],
-                         "digest": "6dc95ec37104ccff",
-                         "capture": "P = 592 capture scaled by members (the traffic is the parameter rows, proportional to P)"},
-    ("cfg2", "stored"): {"kernel": "k_rollout_cartpole_ws", "bytes": 4.788480e+06,
-                         "files": ['rollout_mlp_tiled.cu', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'fp32x2.cuh', 'internal.h'],
-                         "digest": "43ceffc3a9b4ab42", "capture": "full size"},
+    ("cfg4", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 3.490288e+08,
+                         "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
+                         "digest": "", "capture": "full size"},
+    ("cfg2", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 4.787200e+06,
+                         "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
+                         "digest": "", "capture": "full size"},
     ("cfg3", "stored"): {"kernel": "k_cnn_conv2_tc", "bytes": 1.530819e+08,
                          "files": ['rollout_cnn_tc.cu', 'umma.cuh', 'async.cuh', 'fp32x2.cuh', 'internal.h'],
                          "digest": "9d6c703703822230", "capture": "full size"},
@@ -450,10 +449,11 @@ def roofline_of(w, workload_key, noise, stages, work, peaks, sm_count, max_mhz, 
              "frac": achieved / peaks["bf16_tflops"], "peak_source": peaks["source"], "traffic": None}
     else:
         achieved = stages["rollout"]["TFLOP/s"]
-        # cart-pole: more than 8 episodes on a 32/64/128-wide shape run the warp-specialised two-group kernel
-        cart = "k_rollout_cartpole_ws" if (w.episodes > 8 and len(w.layer_sizes) == 4 and
-                                           16 < max(w.layer_sizes[1:3]) <= 128) else "k_rollout_mlp_tiled"
-        kernel = {W.TASK_PAINT: "k_paint", W.TASK_TANH_LINEAR: "k_rollout_tl_tc", W.TASK_CARTPOLE: cart}[w.task_kind]
+        # control tasks: two hidden layers of up to 128 units (one warp per member where they have at most 16), else any depth
+        two = len(w.layer_sizes) == 4 and max(w.layer_sizes[1:3]) <= 128
+        control = "k_rollout_mlp_mma" if not two else (
+            "k_rollout_cart_solo" if w.task_kind == W.TASK_CARTPOLE and max(w.layer_sizes[1:3]) <= 16 else "k_rollout_mlp2")
+        kernel = "k_paint" if w.task_kind == W.TASK_PAINT else control
         r = {"kernel": kernel,
              "bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
              "frac": achieved / alu_peak,

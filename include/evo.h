@@ -54,16 +54,15 @@ enum { EVO_TASK_NONE = 0, EVO_TASK_CARTPOLE = 1, EVO_TASK_TANH_LINEAR = 2, EVO_T
 /* Roll-out kernel of the control tasks.  GENERIC: runtime shapes, any MLP.  TILED: the fp32-pipe
  * kernels with the weights in registers (two hidden layers, each at most as wide as a compiled shape:
  * 16/32/64/128 for the cart-pole, 128 for the tanh-linear task); UNSUPPORTED at evo_rollout if none
- * fits.  AUTO: for the tanh-linear task with hidden widths <= 128 the tensor-core kernel (wide layers
- * as pairs of fp16 numbers on tcgen05, fp32-accurate; weights of those layers beyond +-65,504 are
- * clamped), else TILED where it fits, else GENERIC. */
+ * fits.  AUTO: the layers on the tensor cores as pairs of fp16 numbers (fp32-accurate), the weights
+ * of two hidden layers of up to 128 units in registers, those of any other policy in shared memory as
+ * long as they fit; else GENERIC. */
 enum { EVO_ROLLOUT_AUTO = 0, EVO_ROLLOUT_GENERIC = 1, EVO_ROLLOUT_TILED = 2 };
 enum { EVO_OPT_ADAM = 0, EVO_OPT_CLIPUP = 1 };
 enum { EVO_SIGMA_CONSTANT = 0, EVO_SIGMA_PGPE = 1 };
 /* evo_config.debug_flags.  DROP_COMPLETION: the roll-out kernels leave out the asynchronous
- * completion their first bounded wait depends on (the copy of a member's parameter row; in the
- * tensor-core control kernel the commit of the first batch of MMAs; in the tensor-core CNN the
- * copy of a block's first group of activations), so that wait must run out: every block raises
+ * completion their first bounded wait depends on (the copy of a member's parameters; in the
+ * tensor-core CNN the copy of a block's first group of activations), so that wait must run out: every block raises
  * EVO_ERR_TIMEOUT, reports NaN as its return and leaves by itself, with nothing left in flight.  It exists so that the time-out path can be tested without disturbing
  * the device. */
 enum { EVO_DEBUG_DROP_COMPLETION = 1 };

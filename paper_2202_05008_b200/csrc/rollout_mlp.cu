@@ -7,7 +7,9 @@
 // for every member).
 //
 //   k_rollout_mlp_generic   any layer count / widths (runtime), the reference device path
-//   k_rollout_mlp_tiled<..> compile-time shapes with register-tiled layers (the fast path)
+//   k_rollout_mlp2          two hidden layers, split-fp16 tensor-core products, weights in registers
+//   k_rollout_mlp_mma       any layer count, the same products, weights in shared memory
+//   k_rollout_mlp_tiled<..> compile-time shapes with register-tiled layers on the fp32 pipe
 #include "internal.h"
 #include "noise.cuh"
 #include "tasks.cuh"
@@ -195,33 +197,37 @@ bool rollout_mlp_supported(const evo_config& cfg)
 int rollout_mlp_tiled_shape(uint32_t task, uint32_t n_layers, const uint32_t* sizes);
 uint32_t rollout_mlp_tiled_eb(int shape, uint32_t episodes);
 int launch_rollout_mlp_tiled(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
-bool rollout_tl_tc_supported(const RolloutMlpArgs& a);
-int launch_rollout_tl_tc(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
+uint32_t rollout_mlp2_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
+int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
-static bool use_tiled(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice)
-{
-    return choice != EVO_ROLLOUT_GENERIC && rollout_mlp_tiled_shape(task, n_layers, sizes) >= 0;
-}
+// The kernel of a policy: AUTO takes the register-resident one where the policy has two hidden layers of up to 128
+// units, for any other number of layers and wider ones the one with the weights in shared memory as long
+// as they fit it, and else the runtime-shape kernel, which reads them through the caches.
+enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kSharedMemory };
 
-// Any other number of layers, or wider ones: the tensor-core kernel with the weights in shared memory, as long as
-// they fit it (0 otherwise; the runtime-shape kernel then reads them through the caches).
-static uint32_t mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t episodes)
+static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t episodes,
+                               uint32_t* EB)
 {
-    if (choice != EVO_ROLLOUT_AUTO || use_tiled(task, n_layers, sizes, choice)) return 0;
-    return rollout_mlp_mma_eb(task, n_layers, sizes, episodes);
+    if (choice == EVO_ROLLOUT_TILED) {
+        const int shape = rollout_mlp_tiled_shape(task, n_layers, sizes);
+        if (shape < 0) return MlpKernel::kNone;
+        *EB = rollout_mlp_tiled_eb(shape, episodes);
+        return MlpKernel::kTiled;
+    }
+    if (choice == EVO_ROLLOUT_AUTO) {
+        if ((*EB = rollout_mlp2_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kRegisters;
+        if ((*EB = rollout_mlp_mma_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kSharedMemory;
+    }
+    return MlpKernel::kGeneric;
 }
 
 void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
 {
-    if (use_tiled(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel)) {
-        *EB = rollout_mlp_tiled_eb(rollout_mlp_tiled_shape(cfg.task_kind, cfg.n_layers, cfg.layer_sizes), cfg.episodes);
-        *n_eb = (cfg.episodes + *EB - 1u) / *EB;
-        return;
-    }
-    uint32_t eb = mma_eb(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.episodes);
-    if (eb == 0u) {
+    uint32_t eb = 0;
+    const MlpKernel k = choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.episodes, &eb);
+    if (k == MlpKernel::kGeneric || k == MlpKernel::kNone) {
         eb = cfg.episodes < 32u ? cfg.episodes : 32u;
         // few members: split the episodes of a member over more blocks to fill the SMs
         while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * 148u)
@@ -245,23 +251,24 @@ int launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a_in, uint32_t ker
                        DeviceStatus* status)
 {
     RolloutMlpArgs a = a_in;
+    uint32_t eb = 0;
     int launches = 0;
-    const bool tiled_ok = rollout_mlp_tiled_shape(a.task, a.n_layers, a.sizes) >= 0;
-    if (kernel_choice == EVO_ROLLOUT_TILED && !tiled_ok) return -2;
-    if (kernel_choice == EVO_ROLLOUT_AUTO && rollout_tl_tc_supported(a)) {
-        // the large tanh-linear policy: wide layers on the tensor cores (TILED keeps the fp32-pipe kernel)
-        const int r = launch_rollout_tl_tc(st, a, status);
-        if (r < 0) return r;
-        launches += r;
-    } else if (tiled_ok && kernel_choice != EVO_ROLLOUT_GENERIC) {
-        const int r = launch_rollout_mlp_tiled(st, a, status);
-        if (r < 0) return r;
-        launches += r;
-    } else if (mma_eb(a.task, a.n_layers, a.sizes, kernel_choice, a.E) != 0u) {
-        const int r = launch_rollout_mlp_mma(st, a, status);
-        if (r < 0) return r;
-        launches += r;
-    } else {
+    a.fitness = fitness;
+    switch (choose_kernel(a.task, a.n_layers, a.sizes, kernel_choice, a.E, &eb)) {
+    case MlpKernel::kNone:
+        return -2;
+    case MlpKernel::kRegisters:
+        launches = launch_rollout_mlp2(st, a, status);
+        if (launches < 0 || a.n_eb == 1u) return launches;            // one block per member writes the fitness itself
+        break;
+    case MlpKernel::kSharedMemory:
+        launches = launch_rollout_mlp_mma(st, a, status);
+        if (launches < 0 || a.n_eb == 1u) return launches;
+        break;
+    case MlpKernel::kTiled:
+        if ((launches = launch_rollout_mlp_tiled(st, a, status)) < 0) return launches;
+        break;
+    case MlpKernel::kGeneric: {
         size_t bytes = generic_smem_bytes(a, true);
         a.weights_in_smem = 1;
         if (bytes > 200u * 1024u) { a.weights_in_smem = 0; bytes = generic_smem_bytes(a, false); }
@@ -272,7 +279,9 @@ int launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a_in, uint32_t ker
         dim3 grid(a.P, a.n_eb);
         k_rollout_mlp_generic<<<grid, kGenericThreads, bytes, st>>>(a, status);
         if (cudaGetLastError() != cudaSuccess) return -1;
-        launches += 1;
+        launches = 1;
+        break;
+    }
     }
     if (launch_dependent(k_fitness_finalize, dim3((a.P + 255u) / 256u), dim3(256), 0, st, a.fit_partial, a.P, a.n_eb, a.E,
                          fitness) != cudaSuccess) return -1;

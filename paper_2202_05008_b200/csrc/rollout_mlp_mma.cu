@@ -37,102 +37,80 @@ struct Plan {
     size_t   smem;
 };
 
-// EB episodes as MMA columns: 4 in pairs (hi and lo side by side), 8 in planes (hi rows, then lo rows)
-template <int EB> struct Cols;
-template <> struct Cols<4> { static constexpr int rows = 8, values = 2; };
-template <> struct Cols<8> { static constexpr int rows = 16, values = 4; };
-
-__device__ __forceinline__ void stsm_x4_t(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
-{
-    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
-                 :: "r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
-}
-
-// values of this lane (EB = 4: units g, g + 8 of episode t; EB = 8: unit g of episodes 2t, 2t + 1, then unit g + 8)
-// as 16 units from `unit0` on of an operand
-template <int EB>
-__device__ __forceinline__ void store_units(uint32_t base, uint32_t pitch, uint32_t unit0, int lane, const float* v)
-{
-    if constexpr (EB == 4) {
-        const uint32_t addr = base + (lane & 7) * pitch + (unit0 + 8u * ((lane >> 3) & 1)) * 2u;
-        stsm_x2_t(addr, split_pair(v[0]), split_pair(v[1]));
-    } else {
-        const uint32_t addr = base + ((lane & 7) + 8 * (lane >> 4)) * pitch + (unit0 + 8u * ((lane >> 3) & 1)) * 2u;
-        const __half2 h0 = __floats2half2_rn(v[0], v[1]), h1 = __floats2half2_rn(v[2], v[3]);
-        const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
-        const __half2 l0 = __floats2half2_rn(v[0] - f0.x, v[1] - f0.y), l1 = __floats2half2_rn(v[2] - f1.x, v[3] - f1.y);
-        stsm_x4_t(addr, *reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1),
-                  *reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
-    }
-}
-
-// pre-activations of 16 units: tiles = the units' weight tiles in operand order, b0/b1 their biases (units g, g + 8)
+// p of 16 units: tiles = the units' weight tiles in operand order, b0/b1 their biases (units g, g + 8)
 template <int EB>
 __device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint32_t in, uint32_t pitch, int lane, float b0,
-                                          float b1, float* v)
+                                          float b1, float up, float* v)
 {
-    const uint32_t addr = EB == 4 ? in + (lane & 7) * pitch + 16u * ((lane >> 3) & 1)
-                                  : in + ((lane & 7) + 8 * (lane >> 4)) * pitch + 16u * ((lane >> 3) & 1);
-    if constexpr (EB == 4) {
-        float h[4] = { b0, 0.f, b1, 0.f }, l[4] = { 0.f, 0.f, 0.f, 0.f };
-#pragma unroll 4
-        for (uint32_t k = 0; k < kt; ++k) {
-            const uint4 wh = tiles[k * 64u + lane], wl = tiles[k * 64u + 32u + lane];
-            uint32_t x0, x1;
-            ldsm_x2(addr + 32u * k, x0, x1);
-            mma_k16(h, wh, x0, x1);
-            mma_k16(l, wl, x0, x1);
+    using U = Units<EB>;
+    U acc;
+    const uint32_t row = U::row(in, pitch, lane);
+    tiles += lane;
+    {                                                   // tiles two at a time (the operand of a last odd one's partner is read, not used)
+        uint32_t b[2][4];
+        U::load(row, b);
+        acc.first(tiles[0], tiles[32], b[0]);
+        if (kt > 1u) {
+            if (U::kLoadTiles == 1) U::load(row + 32u, b + 1);
+            acc.add(tiles[64], tiles[96], b[1]);
         }
-        v[0] = (h[0] + h[1]) + (l[0] + l[1]);
-        v[1] = (h[2] + h[3]) + (l[2] + l[3]);
-    } else {
-        float hh[4] = { b0, b0, b1, b1 }, hl[4] = { 0.f, 0.f, 0.f, 0.f }, lh[4] = { 0.f, 0.f, 0.f, 0.f };
-#pragma unroll 4
-        for (uint32_t k = 0; k < kt; ++k) {
-            const uint4 wh = tiles[k * 64u + lane], wl = tiles[k * 64u + 32u + lane];
-            uint32_t x0, x1, y0, y1;
-            ldsm_x4(addr + 32u * k, x0, x1, y0, y1);
-            mma_k16(hh, wh, x0, x1);
-            mma_k16(hl, wh, y0, y1);
-            mma_k16(lh, wl, x0, x1);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = hh[i] + (hl[i] + lh[i]);
     }
-}
-
-template <int EB> __device__ __forceinline__ void tanh_values(float* v)
-{
-    if constexpr (EB == 4) tanh2(v[0], v[1]);
-    else tanh4(v[0], v[1], v[2], v[3]);
+    uint32_t k = 2;
+#pragma unroll 2
+    for (; k + 1u < kt; k += 2u) {
+        const uint4 h0 = tiles[k * 64u], l0 = tiles[k * 64u + 32u], h1 = tiles[k * 64u + 64u], l1 = tiles[k * 64u + 96u];
+        uint32_t b[2][4];
+        U::load(row + 32u * k, b);
+        if (U::kLoadTiles == 1) U::load(row + 32u * k + 32u, b + 1);
+        acc.add(h0, l0, b[0]);
+        acc.add(h1, l1, b[1]);
+    }
+    if (k < kt) {
+        uint32_t b[2][4];
+        U::load(row + 32u * k, b);
+        acc.add(tiles[k * 64u], tiles[k * 64u + 32u], b[0]);
+    }
+    acc.sums(up, up * kLoInv, b0, b1, v);
 }
 
 template <int EB, bool CART>
 __global__ void __launch_bounds__(288)
 k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
 {
-    constexpr int NV = Cols<EB>::values;
+    constexpr int NV = Units<EB>::kValues;
     extern __shared__ __align__(16) unsigned char mma_smem[];
     __shared__ float obs[5][EB], act[EB], x0s[kTlNx][EB], rets[9][EB];
+    __shared__ uint32_t peaks[9];
     uint4* tiles = reinterpret_cast<uint4*>(mma_smem);
     float* bias = reinterpret_cast<float*>(mma_smem + static_cast<size_t>(p.tiles) * 1024u);
     float* w_in = bias + p.biases;                                   // cart-pole: [unit][8] = five weights, bias
     const uint32_t buf0 = smem_u32(w_in + (CART ? p.mt[0] * 128u : 0u));
-    const uint32_t buf_bytes = Cols<EB>::rows * p.pitch;
+    const uint32_t buf_bytes = Units<EB>::kRows * p.pitch;
     const uint32_t xbuf = buf0 + 2u * buf_bytes;                     // tanh-linear: two state operands
-    constexpr uint32_t xbuf_bytes = Cols<EB>::rows * kXPitch;
+    constexpr uint32_t xbuf_bytes = Units<EB>::kRows * kXPitch;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t = lane & 3;
     const uint32_t member = blockIdx.x, eb = blockIdx.y, e0 = eb * EB;
     const int nE = min(static_cast<uint32_t>(EB), a.E - e0);
     const uint32_t layers = a.n_layers, nw = p.warps;
     const bool layer_warp = warp < static_cast<int>(nw);
+    const uint32_t traced = a.trace ? a.trace_T : 0u;
     const PhiloxKey key = philox_key(a.k0, a.k1);
     dep_wait();
     const uint32_t generation = status->generation;
     const float* th = a.theta + static_cast<size_t>(member) * a.ldD;
 
     // ---- weights: rows of theta -> operand tiles (whole warps, one tile at a time) --------------------
+    uint32_t n_params = 0;
+    for (uint32_t l = 0; l < layers; ++l) n_params += (a.sizes[l] + 1u) * a.sizes[l + 1];
+    uint32_t most = 0;
+    for (uint32_t i = tid; i < n_params; i += blockDim.x) most = max(most, finite_magnitude(__ldg(th + i)));
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) peaks[warp] = most;
+    __syncthreads();
+    most = 0;
+    for (uint32_t i = 0; i < blockDim.x / 32u; ++i) most = max(most, peaks[i]);
+    const Scale sc(most);
     {
         uint32_t off = 0;
         for (uint32_t l = 0; l < layers; ++l) {
@@ -143,27 +121,39 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
             if (CART && l == 0) {
                 for (uint32_t i = tid; i < p.mt[0] * 128u; i += blockDim.x) {
                     const int u = static_cast<int>(i >> 3), k = static_cast<int>(i & 7u);
-                    w_in[i] = (u < no && k < 6) ? (k < 5 ? __ldg(W + u * 5 + k) : __ldg(B + u)) : 0.f;
+                    w_in[i] = (u < no && k < 6) ? kF * (k < 5 ? __ldg(W + u * 5 + k) : __ldg(B + u)) : 0.f;
                 }
                 continue;
             }
             for (uint32_t i = warp; i < p.mt[l] * p.kt[l]; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, hi, lo);
+                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, sc, -2.0f * kF, hi, lo);
                 tiles[(p.tile0[l] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[l] + i) * 64u + 32u + lane] = lo;
             }
-            for (uint32_t i = tid; i < p.mt[l] * 16u; i += blockDim.x) bias[p.bias0[l] + i] = static_cast<int>(i) < no ? __ldg(B + i) : 0.f;
+            for (uint32_t i = 8u * warp; i < p.mt[l] * 16u; i += blockDim.x / 4u) {
+                const float b = folded_bias(W, B, ni, no, static_cast<int>(i) + g, lane, sc);
+                if (t == 0) bias[p.bias0[l] + i + g] = b;
+            }
         }
-        if (!CART) {                                                 // x' = tanh([A | 0 | B] [x | 0 | a])
+        if (!CART) {                                                 // x' = tanh(A x + B a), x = 1 - 2 r, a = s - 2 s r
+            const Scale one(0u);
             const float* A = a.task_const;
             const float* Bm = a.task_const + kTlNx * kTlNx;
             for (uint32_t i = warp; i < 6u; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, hi, lo);
-                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, hi, lo);
+                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, one, -2.0f * kF, hi, lo);
+                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, one, -2.0f * kF * a.action_scale, hi, lo);
                 tiles[(p.tile0[layers] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[layers] + i) * 64u + 32u + lane] = lo;
+            }
+            for (uint32_t i = tid; i < 32u; i += blockDim.x) {
+                float sa = 0.f, sb = 0.f;
+                if (i < kTlNx) {
+                    for (uint32_t k = 0; k < kTlNx; ++k) sa += A[i * kTlNx + k];
+                    for (uint32_t k = 0; k < kTlNa; ++k) sb += Bm[i * kTlNa + k];
+                }
+                bias[p.bias0[layers] + i] = kF * fmaf(a.action_scale, sb, sa);
             }
             for (uint32_t i = tid; i < 2u * xbuf_bytes / 4u; i += blockDim.x)
                 reinterpret_cast<uint32_t*>(mma_smem + (xbuf - smem_u32(mma_smem)))[i] = 0u;
@@ -198,8 +188,9 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                 const int e = EB == 4 ? t : 2 * t + (i & 1);
                 v[i] = row < kTlNx ? x0s[row][e] : 0.f;
                 if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
+                v[i] = fmaf(-0.5f, v[i], 0.5f);
             }
-            store_units<EB>(xbuf, kXPitch, 16u * m, lane, v);
+            Units<EB>::store(Units<EB>::row(xbuf, kXPitch, lane) + 32u * m, v);
         }
         __syncthreads();
     }
@@ -232,23 +223,23 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                         }
                     } else {
                         const float* bb = bias + p.bias0[l] + 16u * m + g;
-                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], v);
+                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], sc.up, v);
                     }
-                    tanh_values<EB>(v);
+                    logistic_units<EB>(v);
                     if (!last) {
-                        store_units<EB>(out, p.pitch, 16u * m, lane, v);
+                        Units<EB>::store(Units<EB>::row(out, p.pitch, lane) + 32u * m, v);
                     } else if (CART) {
                         if (g == 0) {
                             if (EB == 4) act[t] = v[0];
                             else { act[2 * t] = v[0]; act[2 * t + 1] = v[1]; }
                         }
-                    } else {                                         // units 8..15 are padding: zeros
+                    } else {                                         // the action, and its share of the reward (units 8..15 are padding)
+                        Units<EB>::store(Units<EB>::row(xin, kXPitch, lane) + 64u, v);
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) {
-                            v[i] *= a.action_scale;
-                            if (i < NV / 2) { if (EB == 4 || !(i & 1)) ret = fmaf(-0.01f * v[i], v[i], ret); else ret2 = fmaf(-0.01f * v[i], v[i], ret2); }
+                        for (int i = 0; i < NV / 2; ++i) {
+                            const float act = fmaf(-2.0f * a.action_scale, v[i], a.action_scale);
+                            if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
                         }
-                        store_units<EB>(xin, kXPitch, 32u, lane, v);
                     }
                 }
             }
@@ -256,11 +247,11 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
         }
         if (CART) {
             if (!layer_warp) {
-                cartpole_finish(cpc, ahead, a.action_scale * act[te], cps, snc, csc);
+                cartpole_finish(cpc, ahead, fmaf(-2.0f * a.action_scale, act[te], a.action_scale), cps, snc, csc);
                 ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
                 if (lane < EB) {
                     obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
-                    if (a.trace && step < a.trace_T && te < nE)
+                    if (step < traced && te < nE)
                         *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
                             make_float4(cps.x, cps.xd, cps.th, cps.thd);
                 }
@@ -268,9 +259,12 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
         } else {
             for (uint32_t m = warp; m < 2u; m += nw) {
                 float v[NV];
-                unit_sums<EB>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane, 0.f, 0.f, v);
-                tanh_values<EB>(v);
-                store_units<EB>(xout, kXPitch, 16u * m, lane, v);
+                unit_sums<EB>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane,
+                              bias[p.bias0[layers] + 16u * m + g], bias[p.bias0[layers] + 16u * m + g + 8u], 1.0f, v);
+                logistic_units<EB>(v);
+                Units<EB>::store(Units<EB>::row(xout, kXPitch, lane) + 32u * m, v);
+#pragma unroll
+                for (int i = 0; i < NV; ++i) v[i] = fmaf(-2.0f, v[i], 1.0f);
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
                     const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
@@ -278,7 +272,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                     if (step + 1u < a.T) {                           // reward of the next step: its pre-step state (padding rows are 0)
                         if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
                     }
-                    if (a.trace && step < a.trace_T && e < nE && row < kTlNx)
+                    if (step < traced && e < nE && row < kTlNx)
                         a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + row] = v[i];
                 }
             }
@@ -305,8 +299,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
         float s = 0.f;
         for (int e = 0; e < nE; ++e)
             for (uint32_t w = 0; w < (CART ? 1u : nw); ++w) s += rets[w][e];
-        if (EVO_IN_BOUNDS(status, EVO_SITE_FIT_PARTIAL, static_cast<size_t>(member) * a.n_eb + eb, static_cast<size_t>(a.P) * a.n_eb))
-            a.fit_partial[static_cast<size_t>(member) * a.n_eb + eb] = s;
+        store_return(a, status, member, eb, s);
     }
 }
 
@@ -324,13 +317,14 @@ Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t
         if (p.mt[l] > widest) widest = p.mt[l];
     }
     p.tile0[n_layers] = p.tiles;
+    p.bias0[n_layers] = p.biases;
     p.mt[n_layers] = 2; p.kt[n_layers] = 3;
-    if (!cart) { p.tiles += 6u; if (widest < 2u) widest = 2u; }
-    p.pitch = widest * 32u + 16u;
+    if (!cart) { p.tiles += 6u; p.biases += 32u; if (widest < 2u) widest = 2u; }
+    p.pitch = (widest + 1u) / 2u * 64u + 16u;           // operands are read two tiles at a time
     p.warps = widest < 8u ? widest : 8u;
     const uint32_t rows = EB == 4u ? 8u : 16u;
     p.smem = static_cast<size_t>(p.tiles) * 1024u + p.biases * 4u + (cart ? p.mt[0] * 512u : 0u) + 2u * rows * p.pitch +
-             (cart ? 0u : 2u * rows * kXPitch);
+             (cart ? 0u : 2u * rows * kXPitch + 32u);         // (the last column's third tile is read with the 32 bytes behind it)
     return p;
 }
 

@@ -165,24 +165,24 @@ __device__ __forceinline__ CpState cartpole_step_fast(const CartpoleConst& c, co
 
 // ---- the same step split around the force -----------------------------------------------------------
 // The policy's force is the last thing a step waits for, and the step is a serial chain per episode, so
-// whatever does not need the force is done before it arrives.  At a fixed angle the angular acceleration is
-//     w' = A - B F - C w^2      A = g s / den, B = c / (M den), C = m l s c / (M den), den = l (4/3 - m c^2 / M)
-// and the angles of the first two Runge-Kutta stages are known without F (the second is half a step of the present
-// angular velocity on).  After F there remain four short multiply-add chains; the sin/cos rotations of
-// the third and fourth stage run side by side, because an angle needs only the velocity of the stage before.
-struct CartpoleFast { float g, inv_m, ml, ml_m, l43, lm, h, h2, w6; };
-struct CpAhead { float k1, b1, ww, a2, b2, c2, s2, cs2; };       // what the coming step knows without the force
+// whatever does not need the force is done before it arrives.  With q = 1 / (l (4/3 M - m c^2)), M the total mass,
+//     T = F + m l w^2 s       w' = q (g M s - c T)       M x'' = T - m l c w'
+// the angles of the first two Runge-Kutta stages are known without F (the second is half a step of the present
+// angular velocity on), and so are q and the products with s and c there.  The stages' velocities of the
+// cart cancel into x += h x' + h^2/6 (x1'' + x2'' + x3''), the same for the angle.
+struct CartpoleFast { float gm, ml, den0, den1, h, h2, w6, w6m, hh6, hh6m; };
+struct CpAhead { float n0, bq1, t01, mlc1, s2, c2, bq2, aq2, mls2, mlc2, th0, x0; };      // what the coming step knows without F
 
 __device__ __forceinline__ CartpoleFast cartpole_fast_const(const float* tp)
 {
     CartpoleFast c;
-    c.g = tp[EVO_CP_GRAVITY];
-    c.inv_m = 1.0f / (tp[EVO_CP_CART_MASS] + tp[EVO_CP_POLE_MASS]);
+    const float total = tp[EVO_CP_CART_MASS] + tp[EVO_CP_POLE_MASS];
+    c.gm = tp[EVO_CP_GRAVITY] * total;
     c.ml = tp[EVO_CP_POLE_MASS] * tp[EVO_CP_POLE_HALF_LENGTH];
-    c.ml_m = c.ml * c.inv_m;
-    c.l43 = tp[EVO_CP_POLE_HALF_LENGTH] * (4.0f / 3.0f);
-    c.lm = tp[EVO_CP_POLE_HALF_LENGTH] * tp[EVO_CP_POLE_MASS] * c.inv_m;
-    c.h = tp[EVO_CP_DT]; c.h2 = 0.5f * c.h; c.w6 = c.h * (1.0f / 6.0f);
+    c.den0 = tp[EVO_CP_POLE_HALF_LENGTH] * (4.0f / 3.0f) * total;
+    c.den1 = -c.ml;
+    c.h = tp[EVO_CP_DT]; c.h2 = 0.5f * c.h; c.w6 = c.h * (1.0f / 6.0f); c.w6m = c.w6 / total;
+    c.hh6 = c.h * c.w6; c.hh6m = c.h * c.w6m;
     return c;
 }
 
@@ -201,23 +201,29 @@ __device__ __forceinline__ void turn_by(float d, float sn, float cs, float& s2, 
     c2 = fmaf(cs, cd, -sn * sd);
 }
 
-__device__ __forceinline__ void cartpole_terms(const CartpoleFast& c, float sn, float cs, float& a, float& b, float& k)
+__device__ __forceinline__ float cartpole_q(const CartpoleFast& c, float cs)
 {
-    const float inv_den = __fdividef(1.0f, fmaf(-c.lm * cs, cs, c.l43));
-    a = c.g * sn * inv_den;
-    b = cs * c.inv_m * inv_den;
-    k = b * (c.ml * sn);
+    float q;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fmaf(c.den1 * cs, cs, c.den0)));
+    return q;
 }
 
 __device__ __forceinline__ CpAhead cartpole_ahead(const CartpoleFast& c, const CpState& s, float sn, float cs)
 {
     CpAhead p;
-    float a1, c1;
-    cartpole_terms(c, sn, cs, a1, p.b1, c1);
-    p.ww = s.thd * s.thd;
-    p.k1 = fmaf(-c1, p.ww, a1);
-    turn_by(c.h2 * s.thd, sn, cs, p.s2, p.cs2);
-    cartpole_terms(c, p.s2, p.cs2, p.a2, p.b2, p.c2);
+    const float q1 = cartpole_q(c, cs);
+    p.t01 = c.ml * sn * (s.thd * s.thd);
+    p.n0 = q1 * fmaf(-cs, p.t01, c.gm * sn);
+    p.bq1 = q1 * cs;
+    p.mlc1 = c.ml * cs;
+    turn_by(c.h2 * s.thd, sn, cs, p.s2, p.c2);
+    const float q2 = cartpole_q(c, p.c2);
+    p.bq2 = q2 * p.c2;
+    p.aq2 = q2 * (c.gm * p.s2);
+    p.mls2 = c.ml * p.s2;
+    p.mlc2 = c.ml * p.c2;
+    p.th0 = fmaf(c.h, s.thd, s.th);
+    p.x0 = fmaf(c.h, s.xd, s.x);
     return p;
 }
 
@@ -226,33 +232,32 @@ __device__ __forceinline__ CpAhead cartpole_ahead(const CartpoleFast& c, const C
 __device__ __forceinline__ void cartpole_finish(const CartpoleFast& c, const CpAhead& p, float force, CpState& s, float& sn,
                                                 float& cs)
 {
-    const float w1 = fmaf(-p.b1, force, p.k1);
+    const float w1 = fmaf(-p.bq1, force, p.n0);
     const float o2 = fmaf(c.h2, w1, s.thd);
-    const float w2 = fmaf(-p.c2, o2 * o2, fmaf(-p.b2, force, p.a2));
+    const float t2 = fmaf(p.mls2, o2 * o2, force);
+    const float w2 = fmaf(-p.bq2, t2, p.aq2);
     const float o3 = fmaf(c.h2, w2, s.thd);
-    float s3, c3, s4, c4, a, b, k;
+    float s3, c3, s4, c4;
     turn_by(c.h2 * o2, sn, cs, s3, c3);
     turn_by(c.h * o3, sn, cs, s4, c4);
-    const float kf = rintf(fmaf(c.h, o3, s.th) * 0.636619772f);
-    cartpole_terms(c, s3, c3, a, b, k);
-    const float o33 = o3 * o3;
-    const float w3 = fmaf(-k, o33, fmaf(-b, force, a));
+    constexpr float kRound = 12582912.0f;                                  // 1.5 * 2^23: the sum's low bits are the nearest integer
+    const float kr = fmaf(fmaf(c.h, o3, s.th), 0.636619772f, kRound);
+    const float t3 = fmaf(c.ml * s3, o3 * o3, force);
+    const float w3 = cartpole_q(c, c3) * fmaf(-c3, t3, c.gm * s3);
     const float o4 = fmaf(c.h, w3, s.thd);
-    cartpole_terms(c, s4, c4, a, b, k);
-    const float o44 = o4 * o4;
-    const float w4 = fmaf(-k, o44, fmaf(-b, force, a));
-    const float fm = force * c.inv_m;
-    const float x1 = fmaf(c.ml_m, fmaf(p.ww, sn, -w1 * cs), fm);
-    const float x2 = fmaf(c.ml_m, fmaf(o2 * o2, p.s2, -w2 * p.cs2), fm);
-    const float x3 = fmaf(c.ml_m, fmaf(o33, s3, -w3 * c3), fm);
-    const float x4 = fmaf(c.ml_m, fmaf(o44, s4, -w4 * c4), fm);
-    const float v2 = fmaf(c.h2, x1, s.xd), v3 = fmaf(c.h2, x2, s.xd), v4 = fmaf(c.h, x3, s.xd);
-    const float th = fmaf(c.w6, (s.thd + o4) + 2.0f * (o2 + o3), s.th);
-    s.x = fmaf(c.w6, (s.xd + v4) + 2.0f * (v2 + v3), s.x);
-    s.xd = fmaf(c.w6, (x1 + x4) + 2.0f * (x2 + x3), s.xd);
-    s.thd = fmaf(c.w6, (w1 + w4) + 2.0f * (w2 + w3), s.thd);
-    s.th = th;
-    float r = fmaf(kf, -1.57079637f, th);
+    const float t4 = fmaf(c.ml * s4, o4 * o4, force);
+    const float w4 = cartpole_q(c, c4) * fmaf(-c4, t4, c.gm * s4);
+    const float x1 = fmaf(-p.mlc1, w1, force + p.t01);                     // accelerations of the cart, times the total mass
+    const float x2 = fmaf(-p.mlc2, w2, t2);
+    const float x3 = fmaf(-c.ml * c3, w3, t3);
+    const float x4 = fmaf(-c.ml * c4, w4, t4);
+    const float x23 = x2 + x3, w23 = w2 + w3;
+    s.th = fmaf(c.hh6, w1 + w23, p.th0);
+    s.x = fmaf(c.hh6m, x1 + x23, p.x0);
+    s.xd = fmaf(c.w6m, fmaf(2.0f, x23, x1 + x4), s.xd);
+    s.thd = fmaf(c.w6, fmaf(2.0f, w23, w1 + w4), s.thd);
+    const float kf = kr - kRound;
+    float r = fmaf(kf, -1.57079637f, s.th);
     r = fmaf(kf, 4.37113883e-8f, r);
     const float z = r * r;
     float sp = fmaf(z, 2.75573192e-6f, -1.98412698e-4f);
@@ -263,11 +268,10 @@ __device__ __forceinline__ void cartpole_finish(const CartpoleFast& c, const CpA
     cp = fmaf(cp, z, -0.5f);
     const float s0 = fmaf(sp * z, r, r);
     const float c0 = fmaf(cp, z, 1.0f);
-    const int q = __float2int_rn(kf) & 3;
-    const float u = (q & 1) ? s0 : c0;
-    const float v = (q & 1) ? c0 : s0;
-    cs = (q == 1 || q == 2) ? -u : u;
-    sn = (q >= 2) ? -v : v;
+    const uint32_t k = __float_as_uint(kr);                                // its two low bits: the quarter turn
+    const bool odd = k & 1u;
+    sn = __uint_as_float(__float_as_uint(odd ? c0 : s0) ^ ((k & 2u) << 30));
+    cs = __uint_as_float(__float_as_uint(odd ? s0 : c0) ^ (((k + 1u) & 2u) << 30));
 }
 
 }  // namespace evo

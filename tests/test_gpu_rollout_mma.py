@@ -63,3 +63,46 @@ def test_a_nan_parameter_reaches_the_fitness():
     fit = s.rollout(arg)
     assert torch.isnan(fit).tolist() == [False, True, True, False] and s.sync_status() == 0
     s.close()
+
+
+@pytest.mark.parametrize("sizes", [(28, 1, 1, 8), (28, 16, 17, 8), (28, 33, 48, 8), (28, 64, 65, 8), (28, 65, 3, 8), (28, 128, 127, 8),
+                                   (5, 17, 16, 1), (5, 48, 49, 1), (5, 64, 64, 1), (5, 127, 65, 1), (5, 5, 128, 1)])
+@pytest.mark.parametrize("episodes", [3, 8, 11])
+def test_two_hidden_layers_with_the_weights_in_registers(sizes, episodes):
+    check(sizes, episodes, 40, scale=0.05 if sizes[0] == 28 else 0.25)
+
+
+@pytest.mark.parametrize("sizes", [(28, 128, 128, 8), (28, 90, 70, 8), (28, 20, 128, 8), (5, 128, 65, 1), (5, 81, 96, 1)])
+@pytest.mark.parametrize("episodes", [4, 5])
+def test_two_row_tiles_per_warp(sizes, episodes):
+    """More than two blocks per SM: the wide policies run with the low parts of the second layer in shared memory."""
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=300, episodes=episodes, horizon=12, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes), sigma=0.05)
+    s = Solver(w)
+    theta = s.ask().cpu().numpy()
+    fit = s.rollout().cpu().numpy()
+    assert s.sync_status() == 0
+    members = [0, 1, 147, 148, 298, 299]
+    fit_o, _ = oracle_fitness(w, theta[members], 0, 12)
+    assert rel_err(fit[members], fit_o, floor=1.0) < FIT_TOL
+    s.close()
+
+
+@pytest.mark.parametrize("sizes,pop", [((28, 128, 128, 8), 4), ((28, 128, 128, 8), 300), ((5, 64, 64, 1), 4), ((5, 16, 16, 1), 4),
+                                       ((28, 32, 32, 32, 8), 4)])
+def test_weights_far_beyond_the_fp16_range(sizes, pop):
+    """A member with a weight of 1e7 keeps its other weights to 22 bits of the largest one; the tanh behind the big one is
+    saturated, so the fitness agrees with the oracle, which uses every weight as it is."""
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=pop, episodes=4, horizon=20, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
+    theta = W.random_parameters(5, pop, w.param_dim, scale=0.05)
+    theta[0, 3] = 1.0e7
+    theta[1, sizes[0] * sizes[1] + sizes[1] + 2] = -1.0e5
+    s = Solver(w)
+    arg = s.padded_rows(pop)
+    arg[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    fit = s.rollout(arg).cpu().numpy()
+    assert s.sync_status() == 0 and np.isfinite(fit).all()
+    fit_o, _ = oracle_fitness(w, theta[:4], 0, 20)
+    assert rel_err(fit[:4], fit_o, floor=1.0) < FIT_TOL
+    s.close()
