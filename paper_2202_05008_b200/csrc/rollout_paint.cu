@@ -12,24 +12,34 @@
 // e = (bx - ax)(py - ay) - (by - ay)(px - ax) are all >= 0 or all <= 0; a triangle without area
 // paints nothing.
 //
-// k_paint: block = (member, 32 x 16 pixel tile), thread = 4 horizontally adjacent pixels with their
-// colours in registers.  The block first turns the member's parameters into triangle records in
-// shared memory and drops the triangles whose bounding box misses the tile; the pixel loop then
-// walks the surviving records (broadcast shared-memory loads).  Plain fp32 arithmetic.
+// k_paint: block = (member, a run of 16 x 8 pixel rectangles).  The block turns the member's parameters into
+// triangle records in shared memory; after that its four warps are independent.  A warp takes a rectangle at a
+// time, 4 adjacent pixels of a row per lane with their colours in registers.  Its lanes first classify 32
+// triangles at once against the rectangle: an edge function is linear, so its largest and smallest value over the
+// rectangle lie at corners, and a triangle is outside (an edge's largest value is below -kMargin), or an edge is
+// passed by the whole rectangle (its smallest value is above kMargin) or has to be tested per pixel.  The margin is several
+// times the rounding error of an edge value, so the classes are exact with respect to the fp32 coverage rule above.
+// Only the triangles that matter are then walked, in order, from the ballots, with the tests that cut the rectangle; the
+// covering ones without any.  Bound by instruction issue (84 %).  64 triangles on 128 x 128 pixels, 1,024 members in
+// mid-training: 357 us with tiles of 32 x 16 pixels, a list of the triangles whose bounding box meets the tile and
+// every test per pixel; 183 us with the classes; 151 us with the tests per edge.
 #include "internal.h"
 
 namespace evo {
 
 constexpr int kPaintThreads = 128;
-constexpr int kPaintTileW = 32, kPaintTileH = 16;
+constexpr uint32_t kRectW = 16, kRectH = 8;
 constexpr int kPaintMaxTriangles = 512;
+constexpr float kMargin = 4e-6f;          // an edge value of points in the unit square is off by less than 1e-6
+constexpr float kThin = 2e-5f;            // below this area the three edge values do not tell inside from outside by one sign
 
-struct PaintTri {                 // 16 floats
-    float x0, y0, x1, y1, x2, y2;
-    float r, g, b, a;
+// 20 floats: lanes that read consecutive records with 128-bit loads meet no bank conflict
+struct PaintTri {
+    float4 e[3];                  // x, y of a vertex; x, y of the edge from it, turned so that inside is positive (not if thin)
     float xmin, xmax, ymin, ymax;
-    float pad0, pad1;
+    float ar, ag, ab, rest;       // alpha times the colour, 1 - alpha
 };
+enum : uint8_t { kPaintsNothing = 0, kOrdinary = 1, kThinTriangle = 2 };
 
 __device__ __forceinline__ float paint_unit(float v)
 {
@@ -50,127 +60,171 @@ struct PaintArgs {
     uint32_t n_tri, W, H;
     float background;
     const float* target;          // [H][W][3]
-    float* partial;               // [P][tiles] sums of squared differences
+    float* partial;               // [P][blocks per member] sums of squared differences
     float* canvas;                // nullable: [P][H][W][3]
-    uint32_t tiles_x, tiles_y;
+    uint32_t rects_x, rects, rects_per_block;
 };
 
 __global__ void __launch_bounds__(kPaintThreads)
 k_paint(const PaintArgs a)
 {
-    // sized by the launch: n_tri records, then n_tri indices of the triangles that touch the tile, in order
+    // sized by the launch: n_tri records, then n_tri kinds
     extern __shared__ __align__(16) unsigned char paint_smem[];
     PaintTri* tri = reinterpret_cast<PaintTri*>(paint_smem);
-    uint16_t* keep = reinterpret_cast<uint16_t*>(paint_smem + sizeof(PaintTri) * a.n_tri);
-    __shared__ uint32_t n_keep;
-    __shared__ uint32_t warp_count[kPaintThreads / 32];
+    uint8_t* kind = paint_smem + sizeof(PaintTri) * a.n_tri;
     __shared__ float warp_sum[kPaintThreads / 32];
 
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t member = blockIdx.x, tile = blockIdx.y;
-    const uint32_t tx = tile % a.tiles_x, ty = tile / a.tiles_x;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const uint32_t member = blockIdx.x;
     const float inv_w = __fdiv_rn(1.0f, static_cast<float>(a.W)), inv_h = __fdiv_rn(1.0f, static_cast<float>(a.H));
-    const uint32_t i0 = tx * kPaintTileW, j0 = ty * kPaintTileH;
-    const uint32_t i1 = min(i0 + kPaintTileW, a.W) - 1u, j1 = min(j0 + kPaintTileH, a.H) - 1u;
-    // pixel centres covered by the tile
-    const float tile_x0 = __fmul_rn(__fadd_rn(static_cast<float>(i0), 0.5f), inv_w);
-    const float tile_x1 = __fmul_rn(__fadd_rn(static_cast<float>(i1), 0.5f), inv_w);
-    const float tile_y0 = __fmul_rn(__fadd_rn(static_cast<float>(j0), 0.5f), inv_h);
-    const float tile_y1 = __fmul_rn(__fadd_rn(static_cast<float>(j1), 0.5f), inv_h);
     const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
+    dep_wait();
+    dep_trigger();
 
-    // ---- triangle records; ordered list of those that can touch the tile ----------------------
-    if (tid == 0) n_keep = 0u;
-    __syncthreads();
-    for (uint32_t base = 0; base < a.n_tri; base += kPaintThreads) {
-        const uint32_t k = base + tid;
-        bool touches = false;
-        if (k < a.n_tri) {
-            const float2* src = reinterpret_cast<const float2*>(p + k * 10u);     // 40-byte records
-            const float2 v0 = __ldg(src), v1 = __ldg(src + 1), v2 = __ldg(src + 2), v3 = __ldg(src + 3), v4 = __ldg(src + 4);
-            PaintTri t;
-            t.x0 = paint_unit(v0.x); t.y0 = paint_unit(v0.y);
-            t.x1 = paint_unit(v1.x); t.y1 = paint_unit(v1.y);
-            t.x2 = paint_unit(v2.x); t.y2 = paint_unit(v2.y);
-            t.r = paint_unit(v3.x); t.g = paint_unit(v3.y); t.b = paint_unit(v4.x); t.a = paint_unit(v4.y);
-            t.xmin = fminf(t.x0, fminf(t.x1, t.x2)); t.xmax = fmaxf(t.x0, fmaxf(t.x1, t.x2));
-            t.ymin = fminf(t.y0, fminf(t.y1, t.y2)); t.ymax = fmaxf(t.y0, fmaxf(t.y1, t.y2));
-            t.pad0 = 0.f; t.pad1 = 0.f;
-            tri[k] = t;
-            const bool has_area = paint_edge(t.x0, t.y0, t.x1, t.y1, t.x2, t.y2) != 0.0f;
-            // a pixel centre of the tile inside the closed box exists only if the ranges overlap
-            touches = has_area && t.a > 0.0f && !(t.xmax < tile_x0 || t.xmin > tile_x1 || t.ymax < tile_y0 || t.ymin > tile_y1);
-        }
-        const uint32_t ballot = __ballot_sync(0xffffffffu, touches);
-        if (lane == 0) warp_count[warp] = __popc(ballot);
-        __syncthreads();
-        uint32_t offset = n_keep;
-        for (uint32_t w = 0; w < warp; ++w) offset += warp_count[w];
-        if (touches) keep[offset + __popc(ballot & ((1u << lane) - 1u))] = static_cast<uint16_t>(k);
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t total = 0;
-            for (uint32_t w = 0; w < kPaintThreads / 32; ++w) total += warp_count[w];
-            n_keep += total;
-        }
-        __syncthreads();
+    for (uint32_t k = tid; k < a.n_tri; k += kPaintThreads) {
+        const float2* src = reinterpret_cast<const float2*>(p + k * 10u);     // 40-byte records
+        const float2 v0 = __ldg(src), v1 = __ldg(src + 1), v2 = __ldg(src + 2), v3 = __ldg(src + 3), v4 = __ldg(src + 4);
+        const float x0 = paint_unit(v0.x), y0 = paint_unit(v0.y), x1 = paint_unit(v1.x), y1 = paint_unit(v1.y);
+        const float x2 = paint_unit(v2.x), y2 = paint_unit(v2.y), alpha = paint_unit(v4.y);
+        const float area = paint_edge(x0, y0, x1, y1, x2, y2);
+        // turning an edge negates its value exactly
+        const float s = area <= -kThin ? -1.0f : 1.0f;
+        PaintTri t;
+        t.e[0] = make_float4(x0, y0, s * __fsub_rn(x1, x0), s * __fsub_rn(y1, y0));
+        t.e[1] = make_float4(x1, y1, s * __fsub_rn(x2, x1), s * __fsub_rn(y2, y1));
+        t.e[2] = make_float4(x2, y2, s * __fsub_rn(x0, x2), s * __fsub_rn(y0, y2));
+        t.xmin = fminf(x0, fminf(x1, x2)); t.xmax = fmaxf(x0, fmaxf(x1, x2));
+        t.ymin = fminf(y0, fminf(y1, y2)); t.ymax = fmaxf(y0, fmaxf(y1, y2));
+        t.ar = alpha * paint_unit(v3.x); t.ag = alpha * paint_unit(v3.y); t.ab = alpha * paint_unit(v4.x); t.rest = 1.0f - alpha;
+        tri[k] = t;
+        kind[k] = area == 0.0f || alpha == 0.0f ? kPaintsNothing : fabsf(area) < kThin ? kThinTriangle : kOrdinary;
     }
-    const uint32_t n_list = n_keep;
+    __syncthreads();
 
-    // ---- pixel loop: 4 adjacent pixels of one row per thread -------------------------------------
-    const uint32_t row = j0 + tid / (kPaintTileW / 4), col = i0 + (tid % (kPaintTileW / 4)) * 4u;
-    const float py = __fmul_rn(__fadd_rn(static_cast<float>(row), 0.5f), inv_h);
-    float px[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) px[q] = __fmul_rn(__fadd_rn(static_cast<float>(col + q), 0.5f), inv_w);
-    float cr[4], cg[4], cb[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) { cr[q] = a.background; cg[q] = a.background; cb[q] = a.background; }
-
-    for (uint32_t n = 0; n < n_list; ++n) {
-        const float4* rec = reinterpret_cast<const float4*>(&tri[keep[n]]);
-        const float4 va = rec[0], vb = rec[1], vc = rec[2], vd = rec[3];
-        const float x0 = va.x, y0 = va.y, x1 = va.z, y1 = va.w, x2 = vb.x, y2 = vb.y;
-        const float r = vb.z, g = vb.w, b = vc.x, alpha = vc.y;
-        const float xmin = vc.z, xmax = vc.w, ymin = vd.x, ymax = vd.y;
-        if (py < ymin || py > ymax) continue;                        // whole thread outside the box
-        // the three edges: differences of the vertices once, of the point per pixel
-        const float dx0 = __fsub_rn(x1, x0), dy0 = __fsub_rn(y1, y0);
-        const float dx1 = __fsub_rn(x2, x1), dy1 = __fsub_rn(y2, y1);
-        const float dx2 = __fsub_rn(x0, x2), dy2 = __fsub_rn(y0, y2);
-        const float t10 = __fmul_rn(dx0, __fsub_rn(py, y0));
-        const float t11 = __fmul_rn(dx1, __fsub_rn(py, y1));
-        const float t12 = __fmul_rn(dx2, __fsub_rn(py, y2));
+    float sq = 0.f;
+    const uint32_t first = blockIdx.y * a.rects_per_block, last = min(first + a.rects_per_block, a.rects);
+    for (uint32_t rect = first + warp; rect < last; rect += kPaintThreads / 32) {
+        const uint32_t i0 = (rect % a.rects_x) * kRectW, j0 = (rect / a.rects_x) * kRectH;
+        const uint32_t i1 = min(i0 + kRectW, a.W) - 1u, j1 = min(j0 + kRectH, a.H) - 1u;
+        // pixel centres at the rectangle's corners
+        const float X0 = __fmul_rn(__fadd_rn(static_cast<float>(i0), 0.5f), inv_w), X1 = __fmul_rn(__fadd_rn(static_cast<float>(i1), 0.5f), inv_w);
+        const float Y0 = __fmul_rn(__fadd_rn(static_cast<float>(j0), 0.5f), inv_h), Y1 = __fmul_rn(__fadd_rn(static_cast<float>(j1), 0.5f), inv_h);
+        const uint32_t prow = j0 + (lane >> 2), col = i0 + (lane & 3u) * 4u;
+        const float py = __fmul_rn(__fadd_rn(static_cast<float>(prow), 0.5f), inv_h);
+        float px[4], cr[4], cg[4], cb[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const float e0 = __fsub_rn(t10, __fmul_rn(dy0, __fsub_rn(px[q], x0)));
-            const float e1 = __fsub_rn(t11, __fmul_rn(dy1, __fsub_rn(px[q], x1)));
-            const float e2 = __fsub_rn(t12, __fmul_rn(dy2, __fsub_rn(px[q], x2)));
-            const bool same_sign = (e0 >= 0.0f && e1 >= 0.0f && e2 >= 0.0f) || (e0 <= 0.0f && e1 <= 0.0f && e2 <= 0.0f);
-            if (same_sign && px[q] >= xmin && px[q] <= xmax) {
-                cr[q] = fmaf(alpha, r - cr[q], cr[q]);
-                cg[q] = fmaf(alpha, g - cg[q], cg[q]);
-                cb[q] = fmaf(alpha, b - cb[q], cb[q]);
+            px[q] = __fmul_rn(__fadd_rn(static_cast<float>(col + q), 0.5f), inv_w);
+            cr[q] = a.background; cg[q] = a.background; cb[q] = a.background;
+        }
+
+        for (uint32_t base = 0; base < a.n_tri; base += 32u) {
+            // what the walk has to look at per pixel: the box, each edge, or (thin triangles) the three edges with either sign
+            bool walk = false, box_cuts = false, cuts[3] = { false, false, false }, thin = false;
+            const uint32_t k = base + lane;
+            if (k < a.n_tri) {
+                const uint8_t what = kind[k];
+                const PaintTri& t = tri[k];
+                // a pixel centre of the rectangle inside the closed box exists only if the ranges overlap
+                walk = what != kPaintsNothing && !(t.xmax < X0 || t.xmin > X1 || t.ymax < Y0 || t.ymin > Y1);
+                thin = what == kThinTriangle;
+                box_cuts = t.xmin > X0 || t.xmax < X1 || t.ymin > Y0 || t.ymax < Y1;
+                if (walk && !thin) {
+                    float highest = 1.0f;                             // smallest of the edges' largest values
+                    bool any = false;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        const float4 e = t.e[i];
+                        const float ya = e.z * (Y0 - e.y), yb = e.z * (Y1 - e.y), xa = e.w * (X0 - e.x), xb = e.w * (X1 - e.x);
+                        highest = fminf(highest, fmaxf(ya, yb) - fminf(xa, xb));
+                        cuts[i] = fminf(ya, yb) - fmaxf(xa, xb) <= kMargin;
+                        any = any || cuts[i];
+                    }
+                    walk = highest >= -kMargin;
+                    box_cuts = box_cuts && any;                       // inside all edges by the margin is inside the box
+                }
+            }
+            uint32_t todo = __ballot_sync(0xffffffffu, walk);
+            const uint32_t boxes = __ballot_sync(0xffffffffu, box_cuts), thins = __ballot_sync(0xffffffffu, thin);
+            const uint32_t cut0 = __ballot_sync(0xffffffffu, cuts[0]), cut1 = __ballot_sync(0xffffffffu, cuts[1]),
+                           cut2 = __ballot_sync(0xffffffffu, cuts[2]);
+            const uint32_t tested = boxes | thins | cut0 | cut1 | cut2;
+            while (todo) {
+                const uint32_t n = __ffs(static_cast<int>(todo)) - 1u, bit = todo & (0u - todo);
+                todo ^= bit;
+                const PaintTri& t = tri[base + n];
+                const float4 c = *reinterpret_cast<const float4*>(&t.ar);
+                if (!(tested & bit)) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        cr[q] = fmaf(c.w, cr[q], c.x); cg[q] = fmaf(c.w, cg[q], c.y); cb[q] = fmaf(c.w, cb[q], c.z);
+                    }
+                    continue;
+                }
+                float lo[4] = { 0.f, 0.f, 0.f, 0.f };                 // inside: >= 0
+                auto edge = [&](const float4 e, float* f) {
+                    const float ty = __fmul_rn(e.z, __fsub_rn(py, e.y));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) f[q] = __fsub_rn(ty, __fmul_rn(e.w, __fsub_rn(px[q], e.x)));
+                };
+                if (thins & bit) {
+                    float f0[4], f1[4], f2[4];
+                    edge(t.e[0], f0); edge(t.e[1], f1); edge(t.e[2], f2);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float least = fminf(f0[q], fminf(f1[q], f2[q])), most = fmaxf(f0[q], fmaxf(f1[q], f2[q]));
+                        lo[q] = fmaxf(least, -most);
+                    }
+                } else {
+                    float f[4];
+                    if (cut0 & bit) {
+                        edge(t.e[0], f);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) lo[q] = f[q];
+                    }
+                    if (cut1 & bit) {
+                        edge(t.e[1], f);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) lo[q] = fminf(lo[q], f[q]);
+                    }
+                    if (cut2 & bit) {
+                        edge(t.e[2], f);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) lo[q] = fminf(lo[q], f[q]);
+                    }
+                }
+                if (boxes & bit) {
+                    const float4 box = *reinterpret_cast<const float4*>(&t.xmin);
+                    const bool in_rows = py >= box.z && py <= box.w;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (!(in_rows && px[q] >= box.x && px[q] <= box.y)) lo[q] = -1.0f;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (lo[q] >= 0.0f) {
+                        cr[q] = fmaf(c.w, cr[q], c.x); cg[q] = fmaf(c.w, cg[q], c.y); cb[q] = fmaf(c.w, cb[q], c.z);
+                    }
             }
         }
-    }
 
-    // ---- squared distance to the target, fixed-order block sum --------------------------------------
-    float sq = 0.f;
-    if (row < a.H) {
+        // squared distance to the target
+        if (prow < a.H) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (col + q < a.W) {
-                const size_t at = (static_cast<size_t>(row) * a.W + col + q) * 3u;
-                const float d0 = cr[q] - __ldg(a.target + at), d1 = cg[q] - __ldg(a.target + at + 1), d2 = cb[q] - __ldg(a.target + at + 2);
-                sq += d0 * d0 + d1 * d1 + d2 * d2;
-                if (a.canvas) {
-                    float* out = a.canvas + static_cast<size_t>(member) * a.W * a.H * 3u + at;
-                    out[0] = cr[q]; out[1] = cg[q]; out[2] = cb[q];
+            for (int q = 0; q < 4; ++q) {
+                if (col + q < a.W) {
+                    const size_t at = (static_cast<size_t>(prow) * a.W + col + q) * 3u;
+                    const float d0 = cr[q] - __ldg(a.target + at), d1 = cg[q] - __ldg(a.target + at + 1), d2 = cb[q] - __ldg(a.target + at + 2);
+                    sq += d0 * d0 + d1 * d1 + d2 * d2;
+                    if (a.canvas) {
+                        float* out = a.canvas + static_cast<size_t>(member) * a.W * a.H * 3u + at;
+                        out[0] = cr[q]; out[1] = cg[q]; out[2] = cb[q];
+                    }
                 }
             }
         }
     }
+    // fixed-order sum of the block
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
     if (lane == 0) warp_sum[warp] = sq;
@@ -178,13 +232,15 @@ k_paint(const PaintArgs a)
     if (tid == 0) {
         float total = 0.f;
         for (int w = 0; w < kPaintThreads / 32; ++w) total += warp_sum[w];
-        a.partial[static_cast<size_t>(member) * gridDim.y + tile] = total;
+        a.partial[static_cast<size_t>(member) * gridDim.y + blockIdx.y] = total;
     }
 }
 
 __global__ void k_paint_finalize(const float* __restrict__ partial, uint32_t P, uint32_t tiles, float inv_count,
                                  float* __restrict__ fitness)
 {
+    dep_wait();
+    dep_trigger();
     const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= P) return;
     float s = 0.f;
@@ -195,38 +251,46 @@ __global__ void k_paint_finalize(const float* __restrict__ partial, uint32_t P, 
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
-static uint32_t paint_tiles(uint32_t W, uint32_t H)
+struct PaintSplit { uint32_t rects_x, rects, per_block, blocks; };
+
+// A block builds the member's records, so it should have some rectangles to use them on; about 24 blocks per SM in all even
+// out what the rectangles of a painting differ by.
+static PaintSplit paint_split(uint32_t P, uint32_t W, uint32_t H)
 {
-    return ((W + kPaintTileW - 1) / kPaintTileW) * ((H + kPaintTileH - 1) / kPaintTileH);
+    PaintSplit s;
+    s.rects_x = (W + kRectW - 1u) / kRectW;
+    s.rects = s.rects_x * ((H + kRectH - 1u) / kRectH);
+    const uint64_t share = static_cast<uint64_t>(s.rects) * P / (148u * 24u);
+    s.per_block = share < 4u ? 4u : share > s.rects ? (s.rects + 3u) / 4u * 4u : static_cast<uint32_t>(share) / 4u * 4u;
+    s.blocks = (s.rects + s.per_block - 1u) / s.per_block;
+    return s;
 }
 
 bool paint_supported(uint32_t param_dim, uint32_t W, uint32_t H)
 {
     return param_dim % 10u == 0 && param_dim / 10u >= 1 && param_dim / 10u <= kPaintMaxTriangles &&
-           W >= 1 && H >= 1 && W <= 4096 && H <= 4096 && paint_tiles(W, H) <= 65535u;
+           W >= 1 && H >= 1 && W <= 4096 && H <= 4096;
 }
 
 size_t paint_scratch_bytes(uint32_t P, uint32_t W, uint32_t H)
 {
-    return static_cast<size_t>(P) * paint_tiles(W, H) * sizeof(float);
+    return static_cast<size_t>(P) * paint_split(P, W, H).blocks * sizeof(float);
 }
 
 int launch_rollout_paint(cudaStream_t st, const float* theta, uint32_t ldD, uint32_t P, uint32_t param_dim,
                          uint32_t W, uint32_t H, float background, const float* target, void* scratch,
                          float* fitness, float* canvas)
 {
+    const PaintSplit s = paint_split(P, W, H);
     PaintArgs a;
     a.theta = theta; a.ldD = ldD; a.P = P; a.n_tri = param_dim / 10u; a.W = W; a.H = H;
     a.background = background; a.target = target; a.partial = static_cast<float*>(scratch); a.canvas = canvas;
-    a.tiles_x = (W + kPaintTileW - 1) / kPaintTileW; a.tiles_y = (H + kPaintTileH - 1) / kPaintTileH;
-    const uint32_t tiles = a.tiles_x * a.tiles_y;
-    dim3 grid(P, tiles);
-    const size_t smem = (sizeof(PaintTri) + sizeof(uint16_t)) * a.n_tri;       // at most 33 KB
-    k_paint<<<grid, kPaintThreads, smem, st>>>(a);
-    if (cudaGetLastError() != cudaSuccess) return -1;
+    a.rects_x = s.rects_x; a.rects = s.rects; a.rects_per_block = s.per_block;
+    const size_t smem = (sizeof(PaintTri) + sizeof(uint8_t)) * a.n_tri;        // at most 41 KB
+    if (launch_dependent(k_paint, dim3(P, s.blocks), dim3(kPaintThreads), smem, st, a) != cudaSuccess) return -1;
     const float inv = 1.0f / (3.0f * static_cast<float>(W) * static_cast<float>(H));
-    k_paint_finalize<<<(P + 255u) / 256u, 256, 0, st>>>(a.partial, P, tiles, inv, fitness);
-    if (cudaGetLastError() != cudaSuccess) return -1;
+    if (launch_dependent(k_paint_finalize, dim3((P + 255u) / 256u), dim3(256), 0, st, a.partial, P, s.blocks, inv, fitness) != cudaSuccess)
+        return -1;
     return 2;
 }
 

@@ -100,3 +100,20 @@ def test_painting_gets_closer_to_the_target():
     target = torch.tensor(W.paint_target(w.seed, 64, 64), device="cuda")
     _, hist = run(w, 150, target=target)
     assert hist[-1][0] > hist[0][0] + 0.01 and hist[-1][0] > -0.06
+
+
+@pytest.mark.parametrize("n_tri,width,height", [(1, 1, 1), (31, 16, 8), (33, 17, 9), (64, 15, 7), (512, 40, 20), (40, 300, 3)])
+def test_rectangle_classes_at_ragged_canvases_and_triangle_counts(n_tri, width, height):
+    """Triangles of all sizes, also ones that cover whole rectangles, and thin ones, where the rectangles and the groups of
+    32 triangles are not full.  Colours: 2e-6 per 8 layers, as above."""
+    w = _workload(n_tri, width, height, P=4, bg=0.5)
+    rng = np.random.default_rng(n_tri)
+    theta = rng.uniform(-1.2, 1.2, (4, 10 * n_tri)).astype(np.float32)
+    tri = theta.reshape(4, n_tri, 10)
+    tri[:, ::5, :6] *= 30.0                                      # corners of the canvas: large triangles and degenerate ones
+    tri[:, 1::7, 4:6] = tri[:, 1::7, 0:2] + 1e-5                 # thin ones
+    theta, fit, canvas, target = _render(w, theta)
+    for m in range(4):
+        want = oracle.paint_render(theta[m].reshape(-1, 10), width, height, 0.5)
+        assert np.max(np.abs(canvas[m] - want)) < 2e-6 * max(1, n_tri // 8)
+        assert abs(fit[m] - oracle.paint_fitness(theta[m].reshape(-1, 10), width, height, target, 0.5)) < 1e-6
