@@ -9,7 +9,8 @@
 // contraction [Wh | Wx | b] . [h; onehot(token); 1] with bf16 operands and fp32 accumulation; the
 // read-out out.W . h likewise.
 //
-//   k_s2s_simple  CUDA cores, one block per (member, 16 queries): the plain version.
+//   k_s2s_simple  CUDA cores, one block per (member, 16 queries): the plain version, which also writes logits.
+//   k_s2s_mma     h = 32, 64, 96: warp-level tensor-core products, weights and cell state in registers.
 //   k_s2s_tc      tcgen05, one block per (member, 128 queries), one block per SM.  The member's
 //                 [4h = 512] x [K = 144] weight tile (bf16, 144 KB) stays in shared memory for a
 //                 whole phase (encoder, then decoder); the B operand is the hidden state of the 128
@@ -189,11 +190,238 @@ k_s2s_simple(const S2sArgs a)
 __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, uint32_t n_chunks, float inv_count,
                                float* __restrict__ fitness)
 {
+    dep_wait();
+    dep_trigger();
     const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= P) return;
     float s = 0.f;
     for (uint32_t t = 0; t < n_chunks; ++t) s += partial[static_cast<size_t>(m) * n_chunks + t];
     fitness[m] = -s * inv_count;
+}
+
+// ------------------------------------------------------------------------------------------
+// Narrow cells (h = 32, 64, 96) on warp-level tensor-core products.  Block = (member, up to 64 queries); a warp owns 8
+// hidden units with all four of their gates, rows (input | forget) and (cell | output) of two 16-row operand tiles that
+// it keeps in registers for a whole phase, so a lane's accumulators are the four pre-activations of its
+// (unit, two queries) and the cell state never leaves its registers.  The hidden state travels through shared memory
+// as the B operand [query][h; onehot(token); 1], two buffers, one barrier per step.
+//
+// The gates in fp32: sigma(x) = 1 / (1 + 2^(-x log2 e)), tanh(x) = 2 sigma(2 x) - 1.  The special-function unit, which takes 8
+// clocks per warp for an exponential and 16 for a reciprocal, bounds the kernel, so a cell's four gates share one
+// reciprocal and two cells share that of tanh(c): 64 clocks per cell and step.  The CUDA-core version took one
+// fp32 multiply-add per weight and query on top: h = 64, 2 digits, 300 members x 100 queries: 765 us, here 88 us.
+// ------------------------------------------------------------------------------------------
+constexpr int kMmaTiles = 8;                     // n-tiles of 8 queries per block
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_bf16_first(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// 2^(-x log2 e), held below 2^30 so that a product of four (1 + e) stays finite
+__device__ __forceinline__ float gate_exp(float x)
+{
+    float e;
+    asm("{\n\t.reg .f32 t;\n\tmul.f32 t, %1, 0fBFB8AA3B;\n\tmin.NaN.f32 t, t, 0f41F00000;\n\tex2.approx.ftz.f32 %0, t;\n\t}" : "=f"(e) : "f"(x));
+    return e;
+}
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// One LSTM cell's state from its pre-activations (that of the cell gate doubled); returns the output gate.
+__device__ __forceinline__ float lstm_cell(float pi, float pf, float pg2, float po, float& c)
+{
+    const float a = gate_exp(pi) + 1.0f, b = gate_exp(pf) + 1.0f, d = gate_exp(po) + 1.0f, e = gate_exp(pg2) + 1.0f;
+    const float ab = a * b, de = d * e, r = rcp_approx(ab * de);
+    const float rab = r * de, rde = r * ab;
+    c = fmaf(rab * a, c, rab * b * fmaf(2.0f, rde * d, -1.0f));
+    return rde * e;
+}
+// tanh of two cell states (|c| is at most the number of steps, so nothing overflows)
+__device__ __forceinline__ void tanh_two(float c0, float c1, float& t0, float& t1)
+{
+    float e0, e1;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(c0 * -2.885390082f));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(c1 * -2.885390082f));
+    const float a = e0 + 1.0f, b = e1 + 1.0f, r = rcp_approx(a * b);
+    t0 = fmaf(2.0f, r * b, -1.0f);
+    t1 = fmaf(2.0f, r * a, -1.0f);
+}
+
+template <int H>
+__global__ void __launch_bounds__(4 * H)
+k_s2s_mma(const S2sArgs a, uint32_t chunk_q)
+{
+    constexpr int KH = H / 16, KT = KH + 1, kWarps = H / 8, kQ = 8 * kMmaTiles;
+    constexpr uint32_t kPitch = (H + 16) * 2 + 16;               // bytes per query of the operand: rows of 8 queries fall in distinct banks
+    __shared__ __align__(16) unsigned char bop[2 * kQ * kPitch + 32];      // two buffers (the last row's last k-tile is read with the 16 bytes behind it)
+    __shared__ __align__(16) uint4 out_w[KH * 32];               // read-out weights in operand order
+    __shared__ float out_b[16];
+    __shared__ uint8_t enc[kQ][kS2sMaxTe], dec[kQ][kS2sMaxTd], tgt[kQ][kS2sMaxTd];
+    __shared__ float loss_w[kWarps];
+
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t4 = lane & 3;
+    const uint32_t member = blockIdx.x, q0 = blockIdx.y * chunk_q;
+    const uint32_t nq = min(chunk_q, a.B - q0), nt = (nq + 7u) / 8u;
+    const uint32_t Te = 2 * a.nd + 1, Td = a.nd + 1, T = Te + Td;
+    const PhiloxKey key = philox_key(a.k0, a.k1);
+    dep_wait();
+    dep_trigger();
+    const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
+    constexpr size_t cell = static_cast<size_t>(4) * H * kVocab + static_cast<size_t>(4) * H * H + 4u * H;
+
+    if (tid < kQ) s2s_query(key, a.status->generation, q0 + min(static_cast<uint32_t>(tid), nq - 1u), a.nd, enc[tid], dec[tid], tgt[tid]);
+    for (uint32_t i = tid; i < sizeof(bop) / 16u; i += 4 * H) reinterpret_cast<uint4*>(bop)[i] = make_uint4(0u, 0u, 0u, 0u);
+    {
+        const float* oW = p + 2 * cell;
+        for (int i = tid; i < KH * 32; i += 4 * H) {
+            const int k = (i >> 5) * 16 + 2 * (i & 3), r = (i & 31) >> 2;
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {                        // rows r, r + 8; inputs k, k + 1 and k + 8, k + 9
+                const int row = r + 8 * (j & 1), col = k + 8 * (j >> 1);
+                w[j] = row < kVocab ? pack_bf16(__ldg(oW + row * H + col), __ldg(oW + row * H + col + 1)) : 0u;
+            }
+            out_w[i] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        if (tid < 16) out_b[tid] = tid < kVocab ? __ldg(oW + kVocab * H + tid) : 0.f;
+    }
+    __syncthreads();
+    auto write_token = [&](uint32_t buf, uint32_t n, uint32_t tok) {
+        uint32_t w[8];
+        const uint32_t one = (tok & 1u) ? 0x3F800000u : 0x00003F80u;      // bf16 1.0 in the upper / lower half
+#pragma unroll
+        for (uint32_t i = 0; i < 8u; ++i) w[i] = (i == (tok >> 1)) ? one : 0u;
+        w[6] |= 0x00003F80u;                                      // input 12: the constant 1 of the bias
+        uint4* dst = reinterpret_cast<uint4*>(bop + buf * (kQ * kPitch) + n * kPitch + H * 2);
+        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    };
+    if (tid < kQ) write_token(0u, tid, enc[tid][0]);
+
+    float c[kMmaTiles][2];
+#pragma unroll
+    for (int j = 0; j < kMmaTiles; ++j) c[j][0] = c[j][1] = 0.f;
+    float loss = 0.f;
+    const uint32_t bop0 = smem_u32(bop), ld_row = (lane & 7) * kPitch + 16u * (lane >> 3), st_row = lane * kPitch + 16u * warp;
+    const int u = 8 * warp + g;                                   // this lane's hidden unit
+
+    for (uint32_t phase = 0; phase < 2u; ++phase) {
+        const float* Wx = p + (phase ? cell : 0);
+        const float* Wh = Wx + static_cast<size_t>(4) * H * kVocab;
+        const float* bb = Wh + static_cast<size_t>(4) * H * H;
+        uint4 w[2][KT];
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int k = 0; k < KT; ++k) {
+                uint32_t v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int gate = 2 * m + (j & 1), row = gate * H + u, col = 2 * t4 + 8 * (j >> 1);
+                    const float s = gate == 2 ? 2.0f : 1.0f;      // the cell gate is doubled (exact in bf16)
+                    if (k < KH) {
+                        const float2 x = __ldg(reinterpret_cast<const float2*>(Wh + static_cast<size_t>(row) * H + 16 * k + col));
+                        v[j] = pack_bf16(s * x.x, s * x.y);
+                    } else {
+                        const float x = col < kVocab ? __ldg(Wx + row * kVocab + col) : col == kVocab ? __ldg(bb + row) : 0.f;
+                        const float y = col < kVocab ? __ldg(Wx + row * kVocab + col + 1) : 0.f;
+                        v[j] = pack_bf16(s * x, s * y);
+                    }
+                }
+                w[m][k] = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        __syncthreads();
+        for (uint32_t t = phase ? Te : 0u; t < (phase ? T : Te); ++t) {
+            const uint32_t src = bop0 + (t & 1u) * (kQ * kPitch), dst = bop0 + ((t + 1u) & 1u) * (kQ * kPitch);
+#pragma unroll
+            for (int j4 = 0; j4 < kMmaTiles; j4 += 4) {
+                if (static_cast<uint32_t>(j4) < nt) {
+                    uint32_t hp[4];
+#pragma unroll
+                    for (int jj = 0; jj < 4; ++jj) {
+                        const int j = j4 + jj;
+                        hp[jj] = 0u;
+                        if (static_cast<uint32_t>(j) < nt) {
+                            float x[4], y[4];                     // (input, forget) and (cell, output) of two queries
+                            const uint32_t row = src + j * 8u * kPitch + ld_row;
+#pragma unroll
+                            for (int k = 0; k < KT; k += 2) {
+                                uint32_t b0, b1, b2, b3;
+                                asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                             : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
+                                if (k == 0) { mma_bf16_first(x, w[0][0], b0, b1); mma_bf16_first(y, w[1][0], b0, b1); }
+                                else { mma_bf16(x, w[0][k], b0, b1); mma_bf16(y, w[1][k], b0, b1); }
+                                if (k + 1 < KT) { mma_bf16(x, w[0][k + 1 < KT ? k + 1 : k], b2, b3); mma_bf16(y, w[1][k + 1 < KT ? k + 1 : k], b2, b3); }
+                            }
+                            const float o0 = lstm_cell(x[0], x[2], y[0], y[2], c[j][0]);
+                            const float o1 = lstm_cell(x[1], x[3], y[1], y[3], c[j][1]);
+                            float t0, t1;
+                            tanh_two(c[j][0], c[j][1], t0, t1);
+                            hp[jj] = pack_bf16(o0 * t0, o1 * t1);
+                        }
+                    }
+                    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
+                                 :: "r"(dst + j4 * 8u * kPitch + st_row), "r"(hp[0]), "r"(hp[1]), "r"(hp[2]), "r"(hp[3]) : "memory");
+                }
+            }
+            if (t + 1u < T && tid < kQ) write_token((t + 1u) & 1u, tid, t + 1u < Te ? enc[tid][t + 1u] : dec[tid][t + 1u - Te]);
+            __syncthreads();
+            if (t >= Te) {
+                // read-out and cross-entropy of this position, an n-tile per warp; the next step's products need the same buffer
+                for (uint32_t j = warp; j < nt; j += kWarps) {
+                    float l[4];
+                    const uint32_t row = dst + j * 8u * kPitch + ld_row;
+#pragma unroll
+                    for (int k = 0; k < KH; k += 2) {
+                        uint32_t b0, b1, b2, b3;
+                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                     : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
+                        if (k == 0) mma_bf16_first(l, out_w[lane], b0, b1);
+                        else mma_bf16(l, out_w[k * 32 + lane], b0, b1);
+                        mma_bf16(l, out_w[k * 32 + 32 + lane], b2, b3);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {                 // query 2 t4 + i: token g and, for g < 4, token g + 8
+                        const uint32_t n = j * 8u + 2u * t4 + i;
+                        const int target = tgt[n][t - Te];
+                        const float l0 = l[i] + out_b[g], l1 = g < kVocab - 8 ? l[2 + i] + out_b[g + 8] : -INFINITY;
+                        float mx = fmaxf(l0, l1), at = target == g ? l0 : target == g + 8 ? l1 : 0.f;
+#pragma unroll
+                        for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                        float se = expf(l0 - mx) + (g < kVocab - 8 ? expf(l1 - mx) : 0.f);
+#pragma unroll
+                        for (int off = 4; off < 32; off <<= 1) {
+                            se += __shfl_xor_sync(0xffffffffu, se, off);
+                            at += __shfl_xor_sync(0xffffffffu, at, off);
+                        }
+                        if (g == 0 && n < nq) loss += (mx + logf(se)) - at;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
+    if (lane == 0) loss_w[warp] = loss;
+    __syncthreads();
+    if (tid == 0) {
+        float total = 0.f;
+        for (int i = 0; i < kWarps; ++i) total += loss_w[i];
+        a.partial[static_cast<size_t>(member) * a.n_chunks + blockIdx.y] = total;
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -581,9 +809,19 @@ bool s2s_supported(uint32_t h, uint32_t nd, uint32_t B)
 
 static uint32_t s2s_chunks(uint32_t B, bool tc) { return tc ? (B + kTcQ - 1) / kTcQ : (B + kSimpleQ - 1) / kSimpleQ; }
 
+// Queries per block of the narrow kernel: up to 64, spread evenly over the fewest chunks, in whole n-tiles; a small population
+// takes smaller chunks (down to one tile of 8) until there are two blocks for every SM.
+static uint32_t s2s_mma_chunk(uint32_t P, uint32_t B)
+{
+    const uint32_t tiles = (B + 7u) / 8u;
+    uint32_t chunks = (tiles + kMmaTiles - 1u) / kMmaTiles;
+    while (chunks < tiles && static_cast<uint64_t>(P) * chunks < 2u * 148u) ++chunks;
+    return (tiles + chunks - 1u) / chunks * 8u;
+}
+
 size_t s2s_scratch_bytes(uint32_t P, uint32_t B)
 {
-    return static_cast<size_t>(P) * s2s_chunks(B, false) * sizeof(float);     // the finer split bounds both
+    return static_cast<size_t>(P) * ((B + 7u) / 8u) * sizeof(float);          // the finest split any kernel uses
 }
 
 int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32_t P, uint32_t h, uint32_t nd,
@@ -594,12 +832,13 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
     if (want_tc && (h != kTcH || logits)) {
         if (kernel_choice == EVO_ROLLOUT_TILED) return -2;       // asked for explicitly, not available
     }
-    const bool tc = want_tc && h == kTcH && !logits;
+    const bool tc = want_tc && h == kTcH && !logits, mma = want_tc && h != kTcH && !logits;
     S2sArgs a;
     a.theta = theta; a.ldD = ldD; a.P = P; a.h = h; a.nd = nd; a.B = B;
     a.k0 = k0; a.k1 = k1; a.status = status;
     a.partial = static_cast<float*>(scratch);
-    a.n_chunks = s2s_chunks(B, tc);
+    const uint32_t chunk_q = mma ? s2s_mma_chunk(P, B) : 0u;
+    a.n_chunks = mma ? (B + chunk_q - 1u) / chunk_q : s2s_chunks(B, tc);
     a.logits = logits;
     if (tc) {
         static int sm_count = 0;
@@ -613,14 +852,17 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
         const uint32_t items = P * a.n_chunks;
         const uint32_t grid = items < static_cast<uint32_t>(sm_count) ? items : static_cast<uint32_t>(sm_count);
         k_s2s_tc<<<grid, kTcThreads, sizeof(S2sSmem), st>>>(a, status);
+    } else if (mma) {
+        auto kernel = h == 32u ? k_s2s_mma<32> : h == 64u ? k_s2s_mma<64> : k_s2s_mma<96>;
+        if (launch_dependent(kernel, dim3(P, a.n_chunks), dim3(4u * h), 0, st, a, chunk_q) != cudaSuccess) return -1;
     } else {
         dim3 grid(P, a.n_chunks);
         k_s2s_simple<<<grid, 128, 0, st>>>(a);
     }
     if (cudaGetLastError() != cudaSuccess) return -1;
     const float inv = 1.0f / (static_cast<float>(B) * static_cast<float>(nd + 1));
-    k_s2s_finalize<<<(P + 255u) / 256u, 256, 0, st>>>(a.partial, P, a.n_chunks, inv, fitness);
-    if (cudaGetLastError() != cudaSuccess) return -1;
+    if (launch_dependent(k_s2s_finalize, dim3((P + 255u) / 256u), dim3(256), 0, st, a.partial, P, a.n_chunks, inv, fitness) != cudaSuccess)
+        return -1;
     return 2;
 }
 

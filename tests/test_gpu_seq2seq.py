@@ -144,3 +144,21 @@ def test_config_errors():
     s.ask()
     with pytest.raises(EvoError):
         s.rollout()                                               # the tensor-core kernel needs h = 128
+
+
+@pytest.mark.parametrize("h", [32, 64, 96])
+@pytest.mark.parametrize("nd,B,P", [(1, 1, 2), (3, 7, 6), (2, 64, 4), (2, 65, 300), (4, 129, 6)])
+def test_narrow_cells_on_tensor_cores_match_oracle(h, nd, B, P):
+    """n-tiles of 8 queries and blocks of up to 8 of them, full and not; against the bf16 oracle and the CUDA-core kernel
+    (both round the same operands; left are accumulation order and gates to about 3e-7)."""
+    w = _workload(h, nd, B, P=P, sigma=0.2)
+    a, b = Solver(w), Solver(w, rollout_kernel=ROLLOUT_GENERIC)
+    theta = a.ask().cpu().numpy(); b.ask()
+    fa = a.rollout().clone(); again = a.rollout(); fb = b.rollout()
+    assert a.sync_status() == 0 and b.sync_status() == 0
+    assert torch.equal(fa, again)
+    assert torch.max(torch.abs(fa - fb)) < FIT_TOL
+    members = [0, P - 1]
+    want = _oracle_fits(w, theta[members], 0)
+    for i, m in enumerate(members):
+        assert abs(float(fa[m]) - want[i][0]) < FIT_TOL
