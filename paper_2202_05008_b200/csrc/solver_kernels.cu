@@ -61,11 +61,10 @@ int launch_task_constants(cudaStream_t st, uint32_t task, uint32_t k0, uint32_t 
 // ask: one thread per (column quad, chunk of pairs).  Writes are 128-bit and coalesced along
 // the row; the centre quad is loaded once per thread and reused for all pairs of the chunk.
 // ------------------------------------------------------------------------------------------
-constexpr uint32_t kAskPairsPerThread = 8;
-
-__global__ void __launch_bounds__(256, 8)
+__global__ void __launch_bounds__(256, 4)
 k_ask(const float* __restrict__ center, const float* __restrict__ sigma_vec, PhiloxKey key,
-      const DeviceStatus* __restrict__ status, uint32_t pair0, uint32_t H, uint32_t D, uint32_t ldD, float* __restrict__ theta, float* __restrict__ eps)
+      const DeviceStatus* __restrict__ status, uint32_t pair0, uint32_t H, uint32_t D, uint32_t ldD, uint32_t pairs_per_thread,
+      float* __restrict__ theta, float* __restrict__ eps)
 {
     dep_wait();
     dep_trigger();                       // the roll-out that follows may be set up
@@ -76,8 +75,8 @@ k_ask(const float* __restrict__ center, const float* __restrict__ sigma_vec, Phi
     const float4 c = reinterpret_cast<const float4*>(center)[quad];
     const float4 sg = reinterpret_cast<const float4*>(sigma_vec)[quad];      // one sigma per dimension
     const bool full = d0 + 4u <= D;
-    for (uint32_t j = blockIdx.y * kAskPairsPerThread; j < H; j += gridDim.y * kAskPairsPerThread) {
-        const uint32_t jend = min(j + kAskPairsPerThread, H);
+    for (uint32_t j = blockIdx.y * pairs_per_thread; j < H; j += gridDim.y * pairs_per_thread) {
+        const uint32_t jend = min(j + pairs_per_thread, H);
         for (uint32_t jj = j; jj < jend; ++jj) {
             float4 z = stream_normal4(key, 0u, generation, pair0 + jj, quad);   // counters use the global pair
             if (!full) {                       // ragged tail and padding columns carry zeros
@@ -108,10 +107,14 @@ int launch_ask(cudaStream_t st, const float* center, const float* sigma_vec, uin
                float* eps)
 {
     const uint32_t quads = ldD / 4u;
-    dim3 grid((quads + 255u) / 256u, (H + kAskPairsPerThread - 1u) / kAskPairsPerThread);
+    // Eight pairs per thread reuse the centre; a small problem is one wave whose length is what a thread does, so it takes fewer.
+    const uint32_t bx = (quads + 255u) / 256u;
+    uint32_t ppt = 8u;
+    while (ppt > 1u && static_cast<uint64_t>(bx) * ((H + ppt - 1u) / ppt) < 148u * 6u) ppt /= 2u;
+    dim3 grid(bx, (H + ppt - 1u) / ppt);
     if (grid.y > 65535u) grid.y = 65535u;
     return launch_dependent(k_ask, grid, dim3(256), 0, st, center, sigma_vec, philox_key(k0, k1), status, pair0, H, D, ldD,
-                            theta, eps) == cudaSuccess ? 1 : -1;
+                            ppt, theta, eps) == cudaSuccess ? 1 : -1;
 }
 
 // ------------------------------------------------------------------------------------------
