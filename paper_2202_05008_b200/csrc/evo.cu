@@ -127,6 +127,7 @@ static evo_status make_layout(const evo_config& c, Layout* L)
     L->grad_sum = take(2 * row);                                // fp64, summed over shards by the caller
     L->sigma_sum = take(c.sigma_mode == EVO_SIGMA_PGPE ? row : 0);
     L->norms = take(clipup_norm_doubles(ldD) * sizeof(double));
+    L->counters = take(tell_counter_words(ldD) * sizeof(uint32_t));
     L->fit_partial = take(Pl * L->n_eb * sizeof(float));
     L->task_const = take(kTlNx * (kTlNx + kTlNa) * sizeof(float));
     size_t cnn = 0;
@@ -196,7 +197,7 @@ evo_status evo_create(const evo_config* cfg_in, void* d_workspace, size_t worksp
     s->k0 = static_cast<uint32_t>(s->cfg.seed & 0xFFFFFFFFull);
     s->k1 = static_cast<uint32_t>(s->cfg.seed >> 32);
     const Layout& L = s->lay;
-    int n = launch_init(s->stream, reinterpret_cast<float*>(s->ws + L.center),
+    int n = launch_init(s->stream, reinterpret_cast<uint32_t*>(s->ws + L.counters), reinterpret_cast<float*>(s->ws + L.center),
                         reinterpret_cast<float*>(s->ws + L.m), reinterpret_cast<float*>(s->ws + L.v),
                         reinterpret_cast<float*>(s->ws + L.g), reinterpret_cast<float*>(s->ws + L.sigma),
                         s->cfg.sigma, s->cfg.param_dim, L.ldD,
@@ -332,12 +333,15 @@ evo_status evo_rollout(evo_solver* s, const float* d_theta, float* d_fitness, fl
     return EVO_OK;
 }
 
-static TellArgs tell_args(evo_solver* s)
+static TellArgs tell_args(evo_solver* s, const float* d_fitness)
 {
     const evo_config& c = s->cfg;
     const Layout& L = s->lay;
     TellArgs t;
-    t.u = reinterpret_cast<const float*>(s->ws + L.u);
+    t.fitness = d_fitness;
+    t.rank = reinterpret_cast<int32_t*>(s->ws + L.rank);
+    t.u = reinterpret_cast<float*>(s->ws + L.u);
+    t.counters = reinterpret_cast<uint32_t*>(s->ws + L.counters);
     t.eps = c.noise_mode == EVO_NOISE_STORED ? reinterpret_cast<const float*>(s->ws + L.eps) : nullptr;
     t.k0 = s->k0; t.k1 = s->k1;
     t.H = s->local_pop / 2; t.D = c.param_dim; t.ldD = L.ldD; t.splits = L.grad_splits;
@@ -362,13 +366,7 @@ evo_status evo_tell(evo_solver* s, const float* d_fitness)
     if (!s || !d_fitness) return EVO_ERR_INVALID_ARG;
     if (s->cfg.shard_pairs) return EVO_ERR_UNSUPPORTED;        // a shard needs the exchange in between
     if (!s->asked || s->telling) return EVO_ERR_BAD_ORDER;
-    const Layout& L = s->lay;
-    const TellArgs t = tell_args(s);
-    int n = launch_rank(s->stream, d_fitness, s->cfg.pop_size, reinterpret_cast<int32_t*>(s->ws + L.rank),
-                        reinterpret_cast<float*>(s->ws + L.u), t.status);
-    if (n < 0) return EVO_ERR_CUDA;
-    s->launches += n;
-    n = launch_gradient_update(s->stream, t);
+    const int n = launch_gradient_update(s->stream, tell_args(s, d_fitness));
     if (n < 0) return EVO_ERR_CUDA;
     s->launches += n;
     s->asked = false;
@@ -381,13 +379,8 @@ evo_status evo_tell_begin(evo_solver* s, const float* d_fitness_all)
     if (!s || !d_fitness_all) return EVO_ERR_INVALID_ARG;
     if (!s->asked || s->telling) return EVO_ERR_BAD_ORDER;
     const Layout& L = s->lay;
-    const TellArgs t = tell_args(s);
-    int n = launch_rank(s->stream, d_fitness_all, s->cfg.pop_size, reinterpret_cast<int32_t*>(s->ws + L.rank),
-                        reinterpret_cast<float*>(s->ws + L.u), t.status);
-    if (n < 0) return EVO_ERR_CUDA;
-    s->launches += n;
-    n = launch_gradient_sums(s->stream, t, reinterpret_cast<double*>(s->ws + L.grad_sum),
-                             reinterpret_cast<float*>(s->ws + L.sigma_sum));
+    const int n = launch_gradient_sums(s->stream, tell_args(s, d_fitness_all), reinterpret_cast<double*>(s->ws + L.grad_sum),
+                                       reinterpret_cast<float*>(s->ws + L.sigma_sum));
     if (n < 0) return EVO_ERR_CUDA;
     s->launches += n;
     s->telling = true;
@@ -408,9 +401,8 @@ evo_status evo_tell_end(evo_solver* s)
     if (!s) return EVO_ERR_INVALID_ARG;
     if (!s->telling) return EVO_ERR_BAD_ORDER;
     const Layout& L = s->lay;
-    const TellArgs t = tell_args(s);
-    const int n = launch_update_from_sums(s->stream, t, reinterpret_cast<const double*>(s->ws + L.grad_sum),
-                                          reinterpret_cast<const float*>(s->ws + L.sigma_sum));
+    const int n = launch_update_from_sums(s->stream, tell_args(s, nullptr), reinterpret_cast<double*>(s->ws + L.grad_sum),
+                                          reinterpret_cast<float*>(s->ws + L.sigma_sum));
     if (n < 0) return EVO_ERR_CUDA;
     s->launches += n;
     s->telling = false;

@@ -41,6 +41,16 @@ static double* static_scratch_for_current_device(cudaError_t* err)
     return g_scratch_ptr[dev];
 }
 
+// as many splits as fill the SMs several times over, at least 16 pairs each
+static uint32_t static_splits(uint32_t H, uint32_t ldS)
+{
+    const uint32_t blocks_x = (ldS / 4u + 255u) / 256u;
+    uint32_t s = (148u * 32u + blocks_x - 1u) / blocks_x;
+    if (s > 64u) s = 64u;
+    const uint32_t most = (H + 15u) / 16u;
+    return s > most ? most : s;
+}
+
 // partial[s][d] = sum over the pairs of split s of (u[2j] - u[2j+1]) * eps[j][d]   (fp64)
 __global__ void __launch_bounds__(128)
 k_grad_partial_static(const float* __restrict__ u, const float* __restrict__ eps, uint32_t H,
@@ -95,7 +105,7 @@ extern "C" evo_status evo_es_gradient_static(const float* d_u, const float* d_ep
     if ((static_cast<size_t>(param_dim) + 31u) / 32u * 32u > kStaticScratchDoubles) return EVO_ERR_WORKSPACE;
     const uint32_t ldS = (param_dim + 31u) / 32u * 32u;             // row pitch inside the scratch
     // as many splits as the plan for this shape wants, but no more than the fixed array holds
-    uint32_t splits = gradient_splits(H, ldS);
+    uint32_t splits = static_splits(H, ldS);
     const size_t fit = kStaticScratchDoubles / ldS;
     if (splits > fit) splits = static_cast<uint32_t>(fit);
     const uint32_t pps = (H + splits - 1u) / splits;

@@ -74,7 +74,7 @@ struct RolloutMlpArgs {
 
 struct Layout {                  // byte offsets into the workspace
     size_t status, center, m, v, g, sigma, theta, eps, u, rank, grad_partial, sigma_partial, grad_sum,
-           sigma_sum, norms,
+           sigma_sum, norms, counters,
            fit_partial, task_const, cnn_scratch, total;
     uint32_t ldD, grad_splits, n_eb, EB;
     size_t canary[kMaxRegions];  // checked build: offset of the guard words behind each region, in layout order
@@ -82,17 +82,18 @@ struct Layout {                  // byte offsets into the workspace
 };
 
 // ---- launchers (each returns the number of kernels it launched, or -1 on a launch error) ----
-int launch_init(cudaStream_t st, float* center, float* m, float* v, float* g, float* sigma_vec,
+int launch_init(cudaStream_t st, uint32_t* counters, float* center, float* m, float* v, float* g, float* sigma_vec,
                 float sigma, uint32_t D, uint32_t ldD, DeviceStatus* status, uint32_t wait_cycles_log2,
                 uint32_t debug_flags);
 int launch_task_constants(cudaStream_t st, uint32_t task, uint32_t k0, uint32_t k1, float* task_const);
 int launch_ask(cudaStream_t st, const float* center, const float* sigma_vec, uint32_t k0, uint32_t k1,
                const DeviceStatus* status, uint32_t pair0, uint32_t H, uint32_t D, uint32_t ldD, float* theta,
                float* eps);
-int launch_rank(cudaStream_t st, const float* fitness, uint32_t P, int32_t* rank, float* u,
-                DeviceStatus* status);
 struct TellArgs {
-    const float* u;               // centred-rank weights [P]
+    const float* fitness;         // [P], of the whole population
+    int32_t* rank;                // [P]
+    float* u;                     // centred-rank weights [P]
+    uint32_t* counters;           // blocks that have arrived; zero between tells
     const float* eps;             // stored noise, or NULL = regenerate from the counters
     uint32_t k0, k1, H, D, ldD, splits;   // H = pairs summed here (the shard's)
     uint32_t pair0, P;            // first global pair of the shard; global population size
@@ -110,7 +111,8 @@ struct TellArgs {
 int launch_gradient_update(cudaStream_t st, const TellArgs& a);
 // the two halves of the sharded tell: partial sums -> reduce buffers; reduce buffers -> update
 int launch_gradient_sums(cudaStream_t st, const TellArgs& a, double* grad_sum, float* sigma_sum);
-int launch_update_from_sums(cudaStream_t st, const TellArgs& a, const double* grad_sum, const float* sigma_sum);
+int launch_update_from_sums(cudaStream_t st, const TellArgs& a, double* grad_sum, float* sigma_sum);
+size_t tell_counter_words(uint32_t ldD);
 size_t clipup_norm_doubles(uint32_t ldD);
 uint32_t gradient_splits(uint32_t H, uint32_t ldD);
 

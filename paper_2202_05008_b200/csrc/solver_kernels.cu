@@ -9,12 +9,13 @@ namespace evo {
 // ------------------------------------------------------------------------------------------
 // init / task constants
 // ------------------------------------------------------------------------------------------
-__global__ void k_init(float* center, float* m, float* v, float* g, float* sigma_vec, float sigma,
+__global__ void k_init(uint32_t* counters, uint32_t n_counters, float* center, float* m, float* v, float* g, float* sigma_vec, float sigma,
                        uint32_t D, uint32_t ldD, DeviceStatus* status, uint32_t wait_cycles_log2,
                        uint32_t debug_flags)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < ldD) { center[i] = 0.f; m[i] = 0.f; v[i] = 0.f; g[i] = 0.f; sigma_vec[i] = (i < D) ? sigma : 0.f; }
+    if (i < n_counters) counters[i] = 0u;
     if (i == 0) {
         status->sticky = 0; status->nonfinite = 0; status->adam_step = 0; status->generation = 0;
         status->wait_cycles_log2 = wait_cycles_log2; status->debug_flags = debug_flags;
@@ -22,11 +23,11 @@ __global__ void k_init(float* center, float* m, float* v, float* g, float* sigma
     }
 }
 
-int launch_init(cudaStream_t st, float* center, float* m, float* v, float* g, float* sigma_vec,
+int launch_init(cudaStream_t st, uint32_t* counters, float* center, float* m, float* v, float* g, float* sigma_vec,
                 float sigma, uint32_t D, uint32_t ldD, DeviceStatus* status, uint32_t wait_cycles_log2,
                 uint32_t debug_flags)
 {
-    k_init<<<(ldD + 255) / 256, 256, 0, st>>>(center, m, v, g, sigma_vec, sigma, D, ldD, status,
+    k_init<<<(ldD + 255) / 256, 256, 0, st>>>(counters, static_cast<uint32_t>(tell_counter_words(ldD)), center, m, v, g, sigma_vec, sigma, D, ldD, status,
                                               wait_cycles_log2, debug_flags);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
@@ -119,108 +120,123 @@ int launch_ask(cudaStream_t st, const float* center, const float* sigma_vec, uin
 
 // ------------------------------------------------------------------------------------------
 // centred rank by counting: rank_m = #{k : f_k < f_m or (f_k == f_m and k < m)}
+//
+// Fitness values become keys whose unsigned order is that of the floats (-0 taken as +0), so that against a run of
+// entries that lies wholly on one side of m the whole rule is one comparison, key_k < key_m + (run before m).  A warp
+// ranks M members at once: its lanes hold different entries, an entry is loaded once for all M.
 // ------------------------------------------------------------------------------------------
-constexpr uint32_t kRankTile = 2048;
+// Keys in shared memory at a time.  Few, because the tell kernel's first blocks come to an SM while ranking ends there and find
+// the split of shared memory and L1 as it is: with 8,192 keys too little L1 is left for their loads in flight
+// (131,072 columns x 16,384 members: tell 848 us instead of 733).
+constexpr uint32_t kRankTile = 4096;
+constexpr uint32_t kRankRun = 128;               // entries per warp step: four per lane
 
-__global__ void __launch_bounds__(256)
-k_rank(const float* __restrict__ fitness, uint32_t P, int32_t* __restrict__ rank,
-       float* __restrict__ u, DeviceStatus* status)
+__device__ __forceinline__ uint32_t rank_key(float f)
 {
-    __shared__ float tile[kRankTile];
-    dep_wait();
-    dep_trigger();
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    const float fm = (m < P) ? fitness[m] : 0.f;
-    if (m < P && fm != fm) atomicOr(&status->nonfinite, 1u);
-    uint32_t below = 0;
-    for (uint32_t base = 0; base < P; base += kRankTile) {
-        const uint32_t n = min(kRankTile, P - base);
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) tile[i] = fitness[base + i];
-        __syncthreads();
-        if (m < P) {
-            for (uint32_t i = 0; i < n; ++i) {
-                const float fk = tile[i];
-                below += (fk < fm || (fk == fm && base + i < m)) ? 1u : 0u;
+    const uint32_t b = __float_as_uint(__fadd_rn(f, 0.0f));
+    return b ^ (static_cast<uint32_t>(static_cast<int32_t>(b) >> 31) | 0x80000000u);
+}
+
+// adds the entries [first, first + n) of the population, whose keys lie at `keys` (padded to whole runs with ~0), to below[]
+template <int M>
+__device__ __forceinline__ void count_below(const uint32_t* keys, uint32_t first, uint32_t n, uint32_t m0, const uint32_t (&key)[M],
+                                            uint32_t (&below)[M], uint32_t lane)
+{
+    for (uint32_t i = 0; i < n; i += kRankRun) {
+        const uint4 k = *reinterpret_cast<const uint4*>(keys + i + 4u * lane);
+        const uint32_t at = first + i;
+        if (at + kRankRun <= m0 || at >= m0 + M) {
+            const uint32_t before = at < m0 ? 1u : 0u;
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                const uint32_t t = key[j] + before;
+                below[j] += (k.x < t ? 1u : 0u) + (k.y < t ? 1u : 0u) + (k.z < t ? 1u : 0u) + (k.w < t ? 1u : 0u);
             }
+        } else {
+            const uint32_t kk[4] = { k.x, k.y, k.z, k.w };
+#pragma unroll
+            for (int j = 0; j < M; ++j)
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    below[j] += (kk[c] < key[j] || (kk[c] == key[j] && at + 4u * lane + c < m0 + j)) ? 1u : 0u;
         }
     }
-    if (m < P && EVO_IN_BOUNDS(status, EVO_SITE_RANK, m, P)) {
-        rank[m] = static_cast<int32_t>(below);
-        u[m] = __fadd_rn(__fdiv_rn(__uint2float_rn(below), __uint2float_rn(P - 1u)), -0.5f);
-    }
 }
 
-// Larger populations: the comparisons of a member are split over blockIdx.y (one fitness tile of
-// `tile_n` <= kRankTile entries each) and summed with integer atomics (exact, order-independent); a
-// second kernel turns counts into centred ranks.
+__device__ __forceinline__ float centred_rank(uint32_t below, uint32_t P)
+{
+    return __fadd_rn(__fdiv_rn(__uint2float_rn(below), __uint2float_rn(P - 1u)), -0.5f);
+}
+
+template <int M>
 __global__ void __launch_bounds__(256)
-k_rank_count(const float* __restrict__ fitness, uint32_t P, uint32_t tile_n, int32_t* __restrict__ rank,
-             DeviceStatus* status)
+k_rank(const float* __restrict__ fitness, uint32_t P, int32_t* __restrict__ rank, float* __restrict__ u, DeviceStatus* status)
 {
-    __shared__ float tile[kRankTile];
+    __shared__ __align__(16) uint32_t keys[kRankTile];
     dep_wait();
     dep_trigger();
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t base = blockIdx.y * tile_n;
-    const uint32_t n = min(tile_n, P - base);
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) tile[i] = fitness[base + i];
-    __syncthreads();
-    if (m >= P) return;
-    const float fm = fitness[m];
-    if (blockIdx.y == 0 && fm != fm) atomicOr(&status->nonfinite, 1u);
-    uint32_t below = 0;
-#pragma unroll 8
-    for (uint32_t i = 0; i < n; ++i) {
-        const float fk = tile[i];
-        below += (fk < fm || (fk == fm && base + i < m)) ? 1u : 0u;
+    const uint32_t lane = threadIdx.x & 31u, m0 = (blockIdx.x * 8u + (threadIdx.x >> 5)) * M;
+    uint32_t key[M], below[M];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const float f = m0 + j < P ? fitness[m0 + j] : 0.f;
+        if (lane == 0 && f != f) atomicOr(&status->nonfinite, 1u);
+        key[j] = rank_key(f);
+        below[j] = 0u;
     }
-    atomicAdd(rank + m, static_cast<int32_t>(below));
-}
-
-__global__ void k_rank_zero(int32_t* __restrict__ rank, uint32_t P)
-{
-    dep_wait();
-    dep_trigger();
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < P) rank[m] = 0;
-}
-
-__global__ void k_rank_finish(const int32_t* __restrict__ rank, uint32_t P, float* __restrict__ u)
-{
-    dep_wait();
-    dep_trigger();
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < P)
-        u[m] = __fadd_rn(__fdiv_rn(__uint2float_rn(static_cast<uint32_t>(rank[m])), __uint2float_rn(P - 1u)), -0.5f);
+    for (uint32_t base = 0; base < P; base += kRankTile) {
+        const uint32_t n = min(kRankTile, P - base), padded = (n + kRankRun - 1u) / kRankRun * kRankRun;
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < padded; i += blockDim.x) keys[i] = i < n ? rank_key(fitness[base + i]) : 0xFFFFFFFFu;
+        __syncthreads();
+        if (m0 < P) count_below<M>(keys, base, n, m0, key, below, lane);
+    }
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const uint32_t r = __reduce_add_sync(0xffffffffu, below[j]);
+        if (lane == 0 && m0 + j < P && EVO_IN_BOUNDS(status, EVO_SITE_RANK, m0 + j, P)) {
+            rank[m0 + j] = static_cast<int32_t>(r);
+            u[m0 + j] = centred_rank(r, P);
+        }
+    }
 }
 
 int launch_rank(cudaStream_t st, const float* fitness, uint32_t P, int32_t* rank, float* u,
                 DeviceStatus* status)
 {
-    const uint32_t bx = (P + 255u) / 256u;
-    if (P <= 1024u) {      // a handful of blocks, each thread against the whole population: a few microseconds
-        return launch_dependent(k_rank, dim3(bx), dim3(256), 0, st, fitness, P, rank, u, status) == cudaSuccess ? 1 : -1;
-    }
-    // From there on one kernel of P / 256 blocks leaves most of the GPU idle (P = 4,096: 16 blocks, 63 us):
-    // tiles of 256 comparisons up to P = 8,192 (P = 4,096: 256 blocks), of 2,048 beyond.
-    const uint32_t tile_n = P <= 8192u ? 256u : kRankTile;
-    if (launch_dependent(k_rank_zero, dim3(bx), dim3(256), 0, st, rank, P) != cudaSuccess) return -1;
-    dim3 grid(bx, (P + tile_n - 1u) / tile_n);
-    if (launch_dependent(k_rank_count, grid, dim3(256), 0, st, fitness, P, tile_n, rank, status) != cudaSuccess) return -1;
-    return launch_dependent(k_rank_finish, dim3(bx), dim3(256), 0, st, rank, P, u) == cudaSuccess ? 3 : -1;
+    // About 128 blocks of eight warps up to P = 4,096, where the kernel is a matter of latency (P = 1,024: 5 us against 17 for
+    // one thread per member); from there on four members per warp, bound by the comparisons (P = 16,384: 64 us; one
+    // thread per member, split over blocks with atomics: 88; eight members per warp: 66).
+    const uint32_t m = P <= 1024u ? 1u : P <= 2048u ? 2u : 4u;
+    auto kernel = m == 1u ? k_rank<1> : m == 2u ? k_rank<2> : k_rank<4>;
+    return launch_dependent(kernel, dim3((P + 8u * m - 1u) / (8u * m)), dim3(256), 0, st, fitness, P, rank, u, status) == cudaSuccess
+               ? 1 : -1;
 }
 
 // ------------------------------------------------------------------------------------------
-// ES gradient.  partial[s][d] = sum over the pairs of split s of (u[2j]-u[2j+1]) * eps[j][d],
-// one thread per column quad.  Products and sums are fp64: the Adam step lr*g/(|g|+eps) is
-// ill-conditioned where |g| is near adam_eps, so the cancellation error of an fp32 sum
-// (~1e-7 of RMS(g)) would move those coordinates by far more than the 1e-5 parity bound.  The
-// stored-noise kernel is HBM-bound (4 bytes per term), so the fp64 arithmetic is hidden.
-// Summation order is fixed (two interleaved accumulators per column, splits added in order);
-// no floating-point atomics anywhere, so results are run-to-run identical.
-// REGEN recomputes eps from the Philox counters instead of reading it.
+// tell: ES gradient and optimiser step in one kernel.
+//
+// Block = (64 column quads) x (a split of the pairs); its 256 threads are 64 quads x 4 pair lanes, so even a few hundred
+// columns keep a few blocks' worth of loads in flight (256 quads x 1 lane where the columns are many: 643 us against 621 at
+// 131,072 columns, 8,192 pairs).  Stored noise wants five blocks per SM: 64 bytes per thread in flight (four blocks: 745
+// against 733 us with the ranking).  Products and sums are fp64: the Adam step lr*g/(|g|+eps) is
+// ill-conditioned where |g| is near adam_eps, so the cancellation error of an fp32 sum (~1e-7 of RMS(g)) would
+// move those coordinates by far more than the 1e-5 parity bound.  The stored-noise form is HBM-bound (4 bytes
+// per term; 4.3 GB in 621 us), so the fp64 arithmetic is hidden.  REGEN recomputes eps from the Philox counters instead of
+// reading it.  SIGMA also accumulates the PGPE sigma gradient sum_j ((u[2j]+u[2j+1])/2) (eps^2 - 1) in fp32 (a plain step on
+// sigma follows, which is not ill-conditioned like Adam's normalised step).
+//
+// The block that finds itself the last of its columns (a counter, no waiting) adds the splits' partial sums and takes the step
+// for them; the last of those closes the tell.  RANK: each block also ranks the members of its own pairs.  A tell of a
+// small problem is then one launch where it was four (rank, gradient, update, close): a matter of launches
+// and of memory round trips between them (generation of the CNN, 64 members: 106 -> 98 us).
+// All summation orders are fixed; no floating-point atomics anywhere, so results are run-to-run identical.
 // ------------------------------------------------------------------------------------------
+constexpr uint32_t kTellQuads = 64, kTellLanes = 4;
+constexpr int kGradRows = 4;           // noise rows in flight per thread
+constexpr uint32_t kRankInTell = 2048; // largest population ranked inside k_tell
+constexpr uint32_t kTellPairs = 256;   // ... and most pairs of a split then
+
 struct Acc4 { double x, y, z, w; };
 
 __device__ __forceinline__ void acc_fma(Acc4& a, double wd, const float4& e)
@@ -230,12 +246,6 @@ __device__ __forceinline__ void acc_fma(Acc4& a, double wd, const float4& e)
     a.z = fma(wd, static_cast<double>(e.z), a.z);
     a.w = fma(wd, static_cast<double>(e.w), a.w);
 }
-
-constexpr int kGradThreads = 256;      // threads per block of the gradient kernel
-constexpr int kGradRows = 4;           // noise rows in flight per thread (multiple of 2)
-
-// SIGMA also accumulates the PGPE sigma gradient sum_j ((u[2j]+u[2j+1])/2) (eps^2 - 1) in fp32 (a plain
-// step on sigma follows, which is not ill-conditioned like Adam's normalised step).
 __device__ __forceinline__ void sig_fma(float4& a, float sj, const float4& e)
 {
     a.x = fmaf(sj, fmaf(e.x, e.x, -1.0f), a.x);
@@ -244,342 +254,468 @@ __device__ __forceinline__ void sig_fma(float4& a, float sj, const float4& e)
     a.w = fmaf(sj, fmaf(e.w, e.w, -1.0f), a.w);
 }
 
-template <bool REGEN, bool SIGMA>
-__global__ void __launch_bounds__(kGradThreads)
-k_grad_partial(const float* __restrict__ u, const float* __restrict__ eps, PhiloxKey key,
-               uint32_t pair0, uint32_t H, uint32_t D, uint32_t ldD,
-               uint32_t pairs_per_split, double* __restrict__ partial, float* __restrict__ sigma_partial,
-               const DeviceStatus* status)
+__device__ __forceinline__ double power(double b, uint32_t n)
 {
+    double r = 1.0;
+    for (; n; n >>= 1, b *= b)
+        if (n & 1u) r *= b;
+    return r;
+}
+
+enum : uint32_t { kStepAdam = 0, kStepClipup = 1, kStepSums = 2 };
+
+struct StepArgs {
+    uint32_t mode, ldD;
+    double inv_pop;
+    float lr, beta1, beta2, adam_eps, momentum, max_speed, sigma_lr, sigma_max_change, inv_pairs;
+    float *sigma_vec, *center, *m, *v, *g;
+    double* grad_sum; float* sigma_sum;      // kStepSums: where the sums go
+    double* norms;                           // ClipUp: per column block |v|^2, v.g, |g|^2; then the two factors of the step and whether to take it
+    DeviceStatus* status;
+};
+
+// One column quad's step from its summed gradient (fp64, unscaled) and sigma gradient.
+__device__ __forceinline__ void quad_step(const StepArgs& a, uint32_t quad, const double (&sum)[4], const float (&ss)[4], bool sigma,
+                                          float corr1, float corr2, double (&dots)[3])
+{
+    if (a.mode == kStepSums) {
+        double2* out = reinterpret_cast<double2*>(a.grad_sum) + 2u * quad;
+        out[0] = make_double2(sum[0], sum[1]);
+        out[1] = make_double2(sum[2], sum[3]);
+        if (sigma) reinterpret_cast<float4*>(a.sigma_sum)[quad] = make_float4(ss[0], ss[1], ss[2], ss[3]);
+        return;
+    }
+    const float4 s4 = reinterpret_cast<const float4*>(a.sigma_vec)[quad];
+    float sg[4] = { s4.x, s4.y, s4.z, s4.w }, gg[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) gg[i] = static_cast<float>(sum[i] * (static_cast<double>(sg[i]) * a.inv_pop));
+    reinterpret_cast<float4*>(a.g)[quad] = make_float4(gg[0], gg[1], gg[2], gg[3]);
+    const float4 m4 = reinterpret_cast<const float4*>(a.m)[quad];
+    float mm[4] = { m4.x, m4.y, m4.z, m4.w };
+    if (a.mode == kStepAdam) {
+        const float4 c4 = reinterpret_cast<const float4*>(a.center)[quad], v4 = reinterpret_cast<const float4*>(a.v)[quad];
+        float cc[4] = { c4.x, c4.y, c4.z, c4.w }, vv[4] = { v4.x, v4.y, v4.z, v4.w };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            mm[i] = a.beta1 * mm[i] + (1.f - a.beta1) * gg[i];
+            vv[i] = a.beta2 * vv[i] + (1.f - a.beta2) * gg[i] * gg[i];
+            const float mhat = mm[i] * corr1;
+            const float vhat = vv[i] * corr2;
+            cc[i] += a.lr * mhat / (sqrtf(vhat) + a.adam_eps);
+        }
+        reinterpret_cast<float4*>(a.m)[quad] = make_float4(mm[0], mm[1], mm[2], mm[3]);
+        reinterpret_cast<float4*>(a.v)[quad] = make_float4(vv[0], vv[1], vv[2], vv[3]);
+        if (EVO_IN_BOUNDS(a.status, EVO_SITE_UPDATE, 4u * quad + 3u, a.ldD))
+            reinterpret_cast<float4*>(a.center)[quad] = make_float4(cc[0], cc[1], cc[2], cc[3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            dots[0] += static_cast<double>(mm[i]) * mm[i];
+            dots[1] += static_cast<double>(mm[i]) * gg[i];
+            dots[2] += static_cast<double>(gg[i]) * gg[i];
+        }
+    }
+    if (sigma) {                             // PGPE sigma step with a relative-change limit
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float gs = sg[i] * a.inv_pairs * ss[i];
+            const float lo = sg[i] * (1.f - a.sigma_max_change), hi = sg[i] * (1.f + a.sigma_max_change);
+            sg[i] = fminf(fmaxf(sg[i] + a.sigma_lr * gs, lo), hi);
+        }
+        reinterpret_cast<float4*>(a.sigma_vec)[quad] = make_float4(sg[0], sg[1], sg[2], sg[3]);
+    }
+}
+
+// ClipUp: vel = momentum vel + (lr / |g|) g, scaled back if it is longer than max_speed; center += vel.  The length follows
+// from the three dot products, so one pass is enough.  factor = lr / |g|, scale = the clip.
+__device__ __forceinline__ void clipup_quad(const StepArgs& a, uint32_t quad, float factor, float scale)
+{
+    const float4 g4 = reinterpret_cast<const float4*>(a.g)[quad];
+    float4 v4 = reinterpret_cast<const float4*>(a.m)[quad], c4 = reinterpret_cast<const float4*>(a.center)[quad];
+    v4.x = scale * fmaf(a.momentum, v4.x, factor * g4.x); v4.y = scale * fmaf(a.momentum, v4.y, factor * g4.y);
+    v4.z = scale * fmaf(a.momentum, v4.z, factor * g4.z); v4.w = scale * fmaf(a.momentum, v4.w, factor * g4.w);
+    c4.x += v4.x; c4.y += v4.y; c4.z += v4.z; c4.w += v4.w;
+    reinterpret_cast<float4*>(a.m)[quad] = v4;
+    reinterpret_cast<float4*>(a.center)[quad] = c4;
+}
+
+// fixed-order sum over the block of three values per thread; every thread gets them
+__device__ __forceinline__ void block_dots(double (&d)[3], double (*red)[3])
+{
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) d[i] += __shfl_xor_sync(0xffffffffu, d[i], off);
+    if (lane == 0)
+        for (int i = 0; i < 3; ++i) red[warp][i] = d[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w][i];
+        d[i] = t;
+    }
+    __syncthreads();
+}
+
+// Closes a tell (256 threads of one block, after every column's step): ClipUp's factors, and its step where the columns are
+// few; the counters.
+constexpr uint32_t kClipupInClose = 8192;       // most column quads a single block moves; more take a kernel of their own
+
+__device__ __forceinline__ void close_tell(const StepArgs& a, uint32_t n_blocks, bool skip, double (*red)[3])
+{
+    if (a.mode == kStepClipup && !skip) {
+        double d[3] = { 0., 0., 0. };
+        for (uint32_t b = threadIdx.x; b < n_blocks; b += 256u)
+            for (int i = 0; i < 3; ++i) d[i] += __ldcg(a.norms + 3u * b + i);
+        block_dots(d, red);
+        const double k = d[2] > 0.0 ? static_cast<double>(a.lr) / sqrt(d[2]) : 0.0, mom = a.momentum;
+        const double vn = sqrt(fmax(mom * mom * d[0] + 2.0 * mom * k * d[1] + k * k * d[2], 0.0));
+        const float factor = static_cast<float>(k);
+        const float scale = vn > static_cast<double>(a.max_speed) ? static_cast<float>(static_cast<double>(a.max_speed) / vn) : 1.0f;
+        if (a.ldD / 4u <= kClipupInClose) {
+            for (uint32_t q = threadIdx.x; q < a.ldD / 4u; q += 256u) clipup_quad(a, q, factor, scale);
+        } else if (threadIdx.x == 0) {
+            a.norms[3u * n_blocks] = factor; a.norms[3u * n_blocks + 1u] = scale; a.norms[3u * n_blocks + 2u] = 1.0;
+        }
+    } else if (a.mode == kStepClipup && threadIdx.x == 0) {
+        a.norms[3u * n_blocks + 2u] = 0.0;                   // the step is left out
+    }
+    if (threadIdx.x == 0) {
+        if (skip) {
+            a.status->sticky |= (1u << EVO_ERR_NONFINITE);
+            a.status->nonfinite = 0;
+        } else {
+            a.status->adam_step += 1u;
+        }
+        a.status->generation += 1u;
+    }
+}
+
+// Whether this block is the last of n to arrive at a counter; the last one sets it back to zero.  What the others wrote
+// before they arrived is visible to it.
+__device__ __forceinline__ bool last_to_arrive(uint32_t* counter, uint32_t n, uint32_t* shared_flag)
+{
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const uint32_t before = atomicAdd(counter, 1u);
+        *shared_flag = before + 1u == n;
+        if (before + 1u == n) *counter = 0u;
+    }
+    __syncthreads();
+    if (*shared_flag) __threadfence();
+    return *shared_flag != 0u;
+}
+
+// counters: [0, column blocks) splits that have arrived, [column blocks] columns
+template <bool REGEN, bool SIGMA, bool RANK>
+__global__ void __launch_bounds__(256, SIGMA || RANK || REGEN ? 3 : 5)
+k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __restrict__ u, const float* __restrict__ eps,
+       PhiloxKey key, uint32_t pair0, uint32_t H, uint32_t P, uint32_t D, uint32_t pairs_per_split, double* __restrict__ partial,
+       float* __restrict__ sigma_partial, uint32_t* __restrict__ counters, const StepArgs a)
+{
+    __shared__ double sums[kTellLanes - 1][kTellQuads][4];
+    __shared__ float ssums[SIGMA ? kTellLanes - 1 : 1][SIGMA ? kTellQuads : 1][4];
+    __shared__ __align__(16) uint32_t keys[RANK ? kRankInTell : 4];
+    __shared__ float2 uu_s[RANK ? kTellPairs : 1];
+    __shared__ double red[8][3];
+    __shared__ float corr[2];
+    __shared__ uint32_t flag;
     dep_wait();
     dep_trigger();
-    if (status->nonfinite) return;
-    const uint32_t quad = blockIdx.x * blockDim.x + threadIdx.x;
-    if (quad * 4u >= ldD) return;
+    DeviceStatus* status = a.status;
+    const uint32_t ldD = a.ldD;
+    const uint32_t q = threadIdx.x % kTellQuads, lane = threadIdx.x / kTellQuads;
+    const uint32_t quad = blockIdx.x * kTellQuads + q;
+    const bool live = quad * 4u < ldD;
     const uint32_t generation = status->generation;
     const uint32_t j0 = blockIdx.y * pairs_per_split;
     const uint32_t j1 = min(H, j0 + pairs_per_split);
-    Acc4 acc[2] = { {0., 0., 0., 0.}, {0., 0., 0., 0.} };
-    float4 sacc[2] = { make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f) };
+    const uint32_t first = j0 + lane;
     const float2* up = reinterpret_cast<const float2*>(u) + pair0;    // u is global, eps rows are the shard's
-    uint32_t j = j0;
-    for (; j + kGradRows <= j1; j += kGradRows) {
-        float4 e[kGradRows];
-        double w[kGradRows];
-        float sj[kGradRows];
+    auto noise = [&](uint32_t j) -> float4 {
+        if (REGEN) return stream_normal4(key, 0u, generation, pair0 + j, quad);
+        return __ldcs(reinterpret_cast<const float4*>(eps + static_cast<size_t>(j) * ldD) + quad);
+    };
+    constexpr bool kPrefetch = RANK && !REGEN;             // the first rows of stored noise are on their way while the ranks are counted
+    float4 e[kGradRows];
+    if constexpr (kPrefetch) {
 #pragma unroll
-        for (int i = 0; i < kGradRows; ++i) {
-            if (REGEN) e[i] = stream_normal4(key, 0u, generation, pair0 + j + i, quad);
-            else e[i] = __ldcs(reinterpret_cast<const float4*>(eps + static_cast<size_t>(j + i) * ldD) + quad);
-            const float2 uu = __ldg(up + j + i);
-            w[i] = static_cast<double>(uu.x) - static_cast<double>(uu.y);   // exact
-            sj[i] = 0.5f * (uu.x + uu.y);
+        for (int i = 0; i < kGradRows; ++i) e[i] = live && first < j1 ? noise(min(first + i * kTellLanes, j1 - 1u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if constexpr (RANK) {
+        const uint32_t wl = threadIdx.x & 31u, padded = (P + kRankRun - 1u) / kRankRun * kRankRun;
+        for (uint32_t i = threadIdx.x; i < padded; i += 256u) {
+            const float f = i < P ? fitness[i] : 0.f;
+            if (f != f) atomicOr(&status->nonfinite, 1u);
+            keys[i] = i < P ? rank_key(f) : 0xFFFFFFFFu;
         }
-#pragma unroll
-        for (int i = 0; i < kGradRows; ++i) {
-            acc_fma(acc[i & 1], w[i], e[i]);
-            if (SIGMA) sig_fma(sacc[i & 1], sj[i], e[i]);
+        __syncthreads();
+        for (uint32_t j = j0 + (threadIdx.x >> 5); j < j1; j += 8u) {          // a warp ranks a pair
+            const uint32_t mk[2] = { keys[2u * j], keys[2u * j + 1u] };
+            uint32_t below[2] = { 0u, 0u };
+            count_below<2>(keys, 0u, P, 2u * j, mk, below, wl);
+            const uint32_t r0 = __reduce_add_sync(0xffffffffu, below[0]), r1 = __reduce_add_sync(0xffffffffu, below[1]);
+            if (wl == 0) {
+                const float2 uu = make_float2(centred_rank(r0, P), centred_rank(r1, P));
+                uu_s[j - j0] = uu;
+                if (blockIdx.x == 0 && EVO_IN_BOUNDS(status, EVO_SITE_RANK, 2u * j + 1u, P)) {
+                    reinterpret_cast<int2*>(rank)[j] = make_int2(static_cast<int>(r0), static_cast<int>(r1));
+                    reinterpret_cast<float2*>(u)[j] = uu;
+                }
+            }
         }
+        __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < kGradRows - 1; ++i) {      // tail keeps the accumulator assignment j % 2
-        if (j + i < j1) {
-            float4 e;
-            if (REGEN) e = stream_normal4(key, 0u, generation, pair0 + j + i, quad);
-            else e = __ldcs(reinterpret_cast<const float4*>(eps + static_cast<size_t>(j + i) * ldD) + quad);
-            const float2 uu = __ldg(up + j + i);
-            acc_fma(acc[i & 1], static_cast<double>(uu.x) - static_cast<double>(uu.y), e);
-            if (SIGMA) sig_fma(sacc[i & 1], 0.5f * (uu.x + uu.y), e);
-        }
-    }
-    double r[4] = { acc[0].x + acc[1].x, acc[0].y + acc[1].y, acc[0].z + acc[1].z, acc[0].w + acc[1].w };
-    if (REGEN && quad * 4u + 4u > D) {             // recomputed noise exists only for real columns
-#pragma unroll
-        for (uint32_t i = 0; i < 4u; ++i)
-            if (quad * 4u + i >= D) r[i] = 0.;
-    }
-    double2* out = reinterpret_cast<double2*>(partial + static_cast<size_t>(blockIdx.y) * ldD) + 2u * quad;
-    if (EVO_IN_BOUNDS(status, EVO_SITE_GRAD_PARTIAL, static_cast<size_t>(blockIdx.y) * ldD + 4u * quad + 3u,
-                      static_cast<size_t>((H + pairs_per_split - 1u) / pairs_per_split) * ldD)) {
-        out[0] = make_double2(r[0], r[1]);
-        out[1] = make_double2(r[2], r[3]);
-    }
-    if (SIGMA) {
-        float4 sr = make_float4(sacc[0].x + sacc[1].x, sacc[0].y + sacc[1].y, sacc[0].z + sacc[1].z, sacc[0].w + sacc[1].w);
-        if (quad * 4u + 4u > D) {                  // padding columns carry no sigma signal
-            if (quad * 4u + 0u >= D) sr.x = 0.f;
-            if (quad * 4u + 1u >= D) sr.y = 0.f;
-            if (quad * 4u + 2u >= D) sr.z = 0.f;
-            if (quad * 4u + 3u >= D) sr.w = 0.f;
-        }
-        reinterpret_cast<float4*>(sigma_partial + static_cast<size_t>(blockIdx.y) * ldD)[quad] = sr;
-    }
-}
 
-// Sum the splits in order, scale by sigma[d]/P, round the gradient to fp32; then either take the
-// Adam ascent step (ADAM) or leave the step to the ClipUp kernels and emit this block's share of
-// |g|^2; finally adapt sigma if a sigma gradient was accumulated.
-template <bool ADAM>
-__global__ void __launch_bounds__(256)
-k_update(const double* __restrict__ partial, const float* __restrict__ sigma_partial, uint32_t splits,
-         uint32_t ldD, double inv_pop, float lr, float beta1, float beta2, float adam_eps,
-         float sigma_lr, float sigma_max_change, float inv_pairs, float* __restrict__ sigma_vec,
-         float* __restrict__ center, float* __restrict__ m, float* __restrict__ v, float* __restrict__ g,
-         double* __restrict__ norm_partial, const DeviceStatus* status)
-{
-    dep_wait();
-    dep_trigger();
-    if (status->nonfinite) return;
-    __shared__ float corr[2];
-    __shared__ double red[256];
-    if (ADAM && threadIdx.x == 0) {
-        const double t = static_cast<double>(status->adam_step + 1u);
-        corr[0] = static_cast<float>(1.0 / (1.0 - pow(static_cast<double>(beta1), t)));
-        corr[1] = static_cast<float>(1.0 / (1.0 - pow(static_cast<double>(beta2), t)));
+    Acc4 acc = { 0., 0., 0., 0. }, acc2 = acc;             // two chains of sums
+    float4 sacc = make_float4(0.f, 0.f, 0.f, 0.f), sacc2 = sacc;
+    if (live) {
+        auto weight = [&](uint32_t j) { return RANK ? uu_s[j - j0] : __ldg(up + j); };
+        auto add = [&](int i, const float2& uu, const float4& z) {
+            acc_fma(i & 1 ? acc2 : acc, static_cast<double>(uu.x) - static_cast<double>(uu.y), z);            // (exact difference)
+            if (SIGMA) sig_fma(i & 1 ? sacc2 : sacc, 0.5f * (uu.x + uu.y), z);
+        };
+        uint32_t j = first;
+        if constexpr (kPrefetch) {
+            // rows beyond the split are its last row again, with weight 0
+#pragma unroll
+            for (int i = 0; i < kGradRows; ++i)
+                add(i, j + i * kTellLanes < j1 ? weight(j + i * kTellLanes) : make_float2(0.f, 0.f), e[i]);
+            j += kGradRows * kTellLanes;
+        }
+        if constexpr (REGEN) {
+            // (four rows sampled before the first is added: 1,440 us instead of 1,399 at 1,000,003 columns, 1,000 pairs)
+#pragma unroll 4
+            for (; j < j1; j += kTellLanes) add(0, weight(j), noise(j));
+        } else {
+            for (; j + (kGradRows - 1) * kTellLanes < j1; j += kGradRows * kTellLanes) {
+                float2 w[kGradRows];
+#pragma unroll
+                for (int i = 0; i < kGradRows; ++i) { e[i] = noise(j + i * kTellLanes); w[i] = weight(j + i * kTellLanes); }
+#pragma unroll
+                for (int i = 0; i < kGradRows; ++i) add(i, w[i], e[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < kGradRows - 1; ++i)
+                if (j + i * kTellLanes < j1) add(i, weight(j + i * kTellLanes), noise(j + i * kTellLanes));
+        }
+        acc.x += acc2.x; acc.y += acc2.y; acc.z += acc2.z; acc.w += acc2.w;
+        if (SIGMA) { sacc.x += sacc2.x; sacc.y += sacc2.y; sacc.z += sacc2.z; sacc.w += sacc2.w; }
+    }
+    // the pair lanes in order
+    if (lane > 0) {
+        sums[lane - 1u][q][0] = acc.x; sums[lane - 1u][q][1] = acc.y; sums[lane - 1u][q][2] = acc.z; sums[lane - 1u][q][3] = acc.w;
+        if (SIGMA) { ssums[lane - 1u][q][0] = sacc.x; ssums[lane - 1u][q][1] = sacc.y; ssums[lane - 1u][q][2] = sacc.z; ssums[lane - 1u][q][3] = sacc.w; }
     }
     __syncthreads();
-    const uint32_t quad = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = quad * 4u < ldD;
-    double gsq = 0.0;
-    if (live) {
-        double sum[4] = { 0., 0., 0., 0. };
-        for (uint32_t k = 0; k < splits; ++k) {
-            const double2* p = reinterpret_cast<const double2*>(partial + static_cast<size_t>(k) * ldD) + 2u * quad;
-            const double2 a = p[0], b = p[1];
-            sum[0] += a.x; sum[1] += a.y; sum[2] += b.x; sum[3] += b.y;
-        }
-        const float4 s4 = reinterpret_cast<const float4*>(sigma_vec)[quad];
-        float sg[4] = { s4.x, s4.y, s4.z, s4.w };
-        float gg[4];
+    double r[4] = { acc.x, acc.y, acc.z, acc.w };
+    float sr[4] = { sacc.x, sacc.y, sacc.z, sacc.w };
+    if (lane == 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            gg[i] = static_cast<float>(sum[i] * (static_cast<double>(sg[i]) * inv_pop));
-            gsq += static_cast<double>(gg[i]) * static_cast<double>(gg[i]);
+            const bool real = quad * 4u + i < D;           // padding columns carry nothing (recomputed noise exists there too)
+            r[i] = real ? ((r[i] + sums[0][q][i]) + (sums[1][q][i] + sums[2][q][i])) : 0.0;
+            if (SIGMA) sr[i] = real ? ((sr[i] + ssums[0][q][i]) + (ssums[1][q][i] + ssums[2][q][i])) : 0.0f;
         }
-        reinterpret_cast<float4*>(g)[quad] = make_float4(gg[0], gg[1], gg[2], gg[3]);
-        if (ADAM) {
-            float4 c4 = reinterpret_cast<float4*>(center)[quad];
-            float4 m4 = reinterpret_cast<float4*>(m)[quad];
-            float4 v4 = reinterpret_cast<float4*>(v)[quad];
-            float cc[4] = { c4.x, c4.y, c4.z, c4.w }, mm[4] = { m4.x, m4.y, m4.z, m4.w },
-                  vv[4] = { v4.x, v4.y, v4.z, v4.w };
+    }
+    if (gridDim.y > 1u) {
+        if (lane == 0 && live) {
+            double2* out = reinterpret_cast<double2*>(partial + static_cast<size_t>(blockIdx.y) * ldD) + 2u * quad;
+            if (EVO_IN_BOUNDS(status, EVO_SITE_GRAD_PARTIAL, static_cast<size_t>(blockIdx.y) * ldD + 4u * quad + 3u,
+                              static_cast<size_t>(gridDim.y) * ldD)) {
+                out[0] = make_double2(r[0], r[1]);
+                out[1] = make_double2(r[2], r[3]);
+            }
+            if (SIGMA) reinterpret_cast<float4*>(sigma_partial + static_cast<size_t>(blockIdx.y) * ldD)[quad] = make_float4(sr[0], sr[1], sr[2], sr[3]);
+        }
+        if (!last_to_arrive(counters + blockIdx.x, gridDim.y, &flag)) return;
+        // the last block of these columns: the splits, an equal part of them per pair lane, the parts in order
+        const uint32_t per = (gridDim.y + kTellLanes - 1u) / kTellLanes;
+        double t[4] = { 0., 0., 0., 0. };
+        float st[4] = { 0.f, 0.f, 0.f, 0.f };
+        if (live)
+#pragma unroll 4
+            for (uint32_t k = lane * per; k < min((lane + 1u) * per, gridDim.y); ++k) {
+                const double2* p = reinterpret_cast<const double2*>(partial + static_cast<size_t>(k) * ldD) + 2u * quad;
+                const double2 x = __ldcg(p), y = __ldcg(p + 1);
+                t[0] += x.x; t[1] += x.y; t[2] += y.x; t[3] += y.y;
+                if (SIGMA) {
+                    const float4 z = __ldcg(reinterpret_cast<const float4*>(sigma_partial + static_cast<size_t>(k) * ldD) + quad);
+                    st[0] += z.x; st[1] += z.y; st[2] += z.z; st[3] += z.w;
+                }
+            }
+        if (lane > 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { sums[lane - 1u][q][i] = t[i]; if (SIGMA) ssums[lane - 1u][q][i] = st[i]; }
+        }
+        __syncthreads();
+        if (lane == 0) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                mm[i] = beta1 * mm[i] + (1.f - beta1) * gg[i];
-                vv[i] = beta2 * vv[i] + (1.f - beta2) * gg[i] * gg[i];
-                const float mhat = mm[i] * corr[0];
-                const float vhat = vv[i] * corr[1];
-                cc[i] += lr * mhat / (sqrtf(vhat) + adam_eps);
+                r[i] = (t[i] + sums[0][q][i]) + (sums[1][q][i] + sums[2][q][i]);
+                if (SIGMA) sr[i] = (st[i] + ssums[0][q][i]) + (ssums[1][q][i] + ssums[2][q][i]);
             }
-            reinterpret_cast<float4*>(m)[quad] = make_float4(mm[0], mm[1], mm[2], mm[3]);
-            reinterpret_cast<float4*>(v)[quad] = make_float4(vv[0], vv[1], vv[2], vv[3]);
-            if (EVO_IN_BOUNDS(status, EVO_SITE_UPDATE, 4u * quad + 3u, ldD))
-                reinterpret_cast<float4*>(center)[quad] = make_float4(cc[0], cc[1], cc[2], cc[3]);
         }
-        if (sigma_partial) {                            // PGPE sigma step with a relative-change limit
-            float ss[4] = { 0.f, 0.f, 0.f, 0.f };
-            for (uint32_t k = 0; k < splits; ++k) {
-                const float4 p = reinterpret_cast<const float4*>(sigma_partial + static_cast<size_t>(k) * ldD)[quad];
-                ss[0] += p.x; ss[1] += p.y; ss[2] += p.z; ss[3] += p.w;
-            }
+    }
+
+    // this block has its columns' sums in lane 0's threads; a NaN fitness leaves everything as it is
+    const bool skip = *reinterpret_cast<volatile uint32_t*>(&status->nonfinite) != 0u;
+    if (a.mode == kStepAdam && threadIdx.x < 2u) {
+        const double beta = threadIdx.x ? a.beta2 : a.beta1;
+        corr[threadIdx.x] = static_cast<float>(1.0 / (1.0 - power(beta, status->adam_step + 1u)));
+    }
+    __syncthreads();
+    double dots[3] = { 0., 0., 0. };
+    if (lane == 0 && live) {
+        if (a.mode == kStepSums && skip) {                 // the all-reduce still runs on defined values
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float gs = sg[i] * inv_pairs * ss[i];
-                const float lo = sg[i] * (1.f - sigma_max_change), hi = sg[i] * (1.f + sigma_max_change);
-                sg[i] = fminf(fmaxf(sg[i] + sigma_lr * gs, lo), hi);
-            }
-            reinterpret_cast<float4*>(sigma_vec)[quad] = make_float4(sg[0], sg[1], sg[2], sg[3]);
+            for (int i = 0; i < 4; ++i) { r[i] = 0.0; sr[i] = 0.0f; }
         }
+        if (a.mode == kStepSums || !skip) quad_step(a, quad, r, sr, SIGMA, corr[0], corr[1], dots);
     }
-    if (!ADAM) {                                        // fixed-order block sum of |g|^2
-        red[threadIdx.x] = gsq;
-        __syncthreads();
-        for (uint32_t off = 128; off > 0; off >>= 1) {
-            if (threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
-            __syncthreads();
+    if (a.mode == kStepSums) return;
+    if (a.mode == kStepClipup) {
+        block_dots(dots, red);
+        if (threadIdx.x < 3u) a.norms[3u * blockIdx.x + threadIdx.x] = dots[threadIdx.x];
+    }
+    if (last_to_arrive(counters + gridDim.x, gridDim.x, &flag)) close_tell(a, gridDim.x, skip, red);
+}
+
+// The second half of a sharded tell: the step from the sums that the caller has added over the shards.
+__global__ void __launch_bounds__(256)
+k_step_from_sums(uint32_t* __restrict__ counters, bool sigma, const StepArgs a)
+{
+    __shared__ double red[8][3];
+    __shared__ float corr[2];
+    __shared__ uint32_t flag;
+    dep_wait();
+    dep_trigger();
+    const bool skip = a.status->nonfinite != 0u;
+    if (a.mode == kStepAdam && threadIdx.x < 2u) {
+        const double beta = threadIdx.x ? a.beta2 : a.beta1;
+        corr[threadIdx.x] = static_cast<float>(1.0 / (1.0 - power(beta, a.status->adam_step + 1u)));
+    }
+    __syncthreads();
+    const uint32_t quad = blockIdx.x * 256u + threadIdx.x;
+    double dots[3] = { 0., 0., 0. };
+    if (quad * 4u < a.ldD && !skip) {
+        const double2* p = reinterpret_cast<const double2*>(a.grad_sum) + 2u * quad;
+        const double2 x = p[0], y = p[1];
+        const double r[4] = { x.x, x.y, y.x, y.y };
+        float sr[4] = { 0.f, 0.f, 0.f, 0.f };
+        if (sigma) {
+            const float4 z = reinterpret_cast<const float4*>(a.sigma_sum)[quad];
+            sr[0] = z.x; sr[1] = z.y; sr[2] = z.z; sr[3] = z.w;
         }
-        if (threadIdx.x == 0) norm_partial[blockIdx.x] = red[0];
+        quad_step(a, quad, r, sr, sigma, corr[0], corr[1], dots);
     }
+    if (a.mode == kStepClipup) {
+        block_dots(dots, red);
+        if (threadIdx.x < 3u) a.norms[3u * blockIdx.x + threadIdx.x] = dots[threadIdx.x];
+    }
+    if (last_to_arrive(counters, gridDim.x, &flag)) close_tell(a, gridDim.x, skip, red);
 }
 
-// ClipUp, step 1: vel = momentum vel + lr g/|g| and this block's share of |vel|^2.
-// norm_partial: [0, nb) block sums of |g|^2 (in), [nb, 2nb) block sums of |vel|^2 (out).
+// ClipUp's step for many columns (a single block took 39 us for 1,000,003 of them, and as long again for the length)
 __global__ void __launch_bounds__(256)
-k_clipup_velocity(const float* __restrict__ g, float* __restrict__ vel, uint32_t ldD, float lr, float momentum,
-                  double* __restrict__ norm_partial, uint32_t nb, const DeviceStatus* status)
-{
-    if (status->nonfinite) return;
-    __shared__ double red[256];
-    __shared__ float inv_gnorm;
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (uint32_t b = 0; b < nb; ++b) s += norm_partial[b];           // same order in every block
-        inv_gnorm = s > 0.0 ? static_cast<float>(1.0 / sqrt(s)) : 0.f;
-    }
-    __syncthreads();
-    const uint32_t quad = blockIdx.x * blockDim.x + threadIdx.x;
-    double vsq = 0.0;
-    if (quad * 4u < ldD) {
-        const float4 g4 = reinterpret_cast<const float4*>(g)[quad];
-        float4 v4 = reinterpret_cast<float4*>(vel)[quad];
-        const float k = lr * inv_gnorm;
-        v4.x = fmaf(momentum, v4.x, k * g4.x); v4.y = fmaf(momentum, v4.y, k * g4.y);
-        v4.z = fmaf(momentum, v4.z, k * g4.z); v4.w = fmaf(momentum, v4.w, k * g4.w);
-        reinterpret_cast<float4*>(vel)[quad] = v4;
-        vsq = static_cast<double>(v4.x) * v4.x + static_cast<double>(v4.y) * v4.y +
-              static_cast<double>(v4.z) * v4.z + static_cast<double>(v4.w) * v4.w;
-    }
-    red[threadIdx.x] = vsq;
-    __syncthreads();
-    for (uint32_t off = 128; off > 0; off >>= 1) {
-        if (threadIdx.x < off) red[threadIdx.x] += red[threadIdx.x + off];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) norm_partial[nb + blockIdx.x] = red[0];
-}
-
-// ClipUp, step 2: clip |vel| to max_speed and move the centre.
-__global__ void __launch_bounds__(256)
-k_clipup_apply(float* __restrict__ vel, float* __restrict__ center, uint32_t ldD, float max_speed,
-               const double* __restrict__ norm_partial, uint32_t nb, const DeviceStatus* status)
-{
-    if (status->nonfinite) return;
-    __shared__ float scale;
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (uint32_t b = 0; b < nb; ++b) s += norm_partial[nb + b];
-        const double vn = sqrt(s);
-        scale = vn > static_cast<double>(max_speed) ? static_cast<float>(static_cast<double>(max_speed) / vn) : 1.0f;
-    }
-    __syncthreads();
-    const uint32_t quad = blockIdx.x * blockDim.x + threadIdx.x;
-    if (quad * 4u >= ldD) return;
-    float4 v4 = reinterpret_cast<float4*>(vel)[quad];
-    float4 c4 = reinterpret_cast<float4*>(center)[quad];
-    v4.x *= scale; v4.y *= scale; v4.z *= scale; v4.w *= scale;
-    c4.x += v4.x; c4.y += v4.y; c4.z += v4.z; c4.w += v4.w;
-    reinterpret_cast<float4*>(vel)[quad] = v4;
-    reinterpret_cast<float4*>(center)[quad] = c4;
-}
-
-// Closes a tell: the Adam step counter advances only if the update was applied; the generation
-// counter (the random streams of the next ask and roll-out) always does.
-__global__ void k_tell_finish(DeviceStatus* status)
+k_clipup_apply(uint32_t n_blocks, const StepArgs a)
 {
     dep_wait();
     dep_trigger();
-    if (status->nonfinite) {
-        status->sticky |= (1u << EVO_ERR_NONFINITE);
-        status->nonfinite = 0;
-    } else {
-        status->adam_step += 1u;
-    }
-    status->generation += 1u;
+    if (a.norms[3u * n_blocks + 2u] == 0.0) return;
+    const float factor = static_cast<float>(a.norms[3u * n_blocks]), scale = static_cast<float>(a.norms[3u * n_blocks + 1u]);
+    const uint32_t quad = blockIdx.x * 256u + threadIdx.x;
+    if (quad * 4u < a.ldD) clipup_quad(a, quad, factor, scale);
 }
+
+static uint32_t tell_blocks(uint32_t ldD) { return (ldD / 4u + kTellQuads - 1u) / kTellQuads; }
 
 uint32_t gradient_splits(uint32_t H, uint32_t ldD)
 {
-    // enough thread blocks to fill 148 SMs several times over, a pure function of the shape
-    const uint32_t blocks_x = (ldD / 4u + kGradThreads - 1u) / kGradThreads;
-    uint32_t s = (148u * 32u + blocks_x - 1u) / blocks_x;
+    // Four waves of eight blocks per SM (with two the last one shows: 131,072 columns, 8,192 pairs 745 us against 660), as long
+    // as every pair lane keeps two rounds of loads; a pure function of the shape.
+    const uint32_t bx = tell_blocks(ldD);
+    uint32_t s = (148u * 32u + bx - 1u) / bx;
     if (s > 64u) s = 64u;
-    const uint32_t max_s = (H + 15u) / 16u;            // at least 16 pairs per split
-    if (s > max_s) s = max_s;
-    if (s < 1u) s = 1u;
+    const uint32_t most = (H + 2u * kGradRows * kTellLanes - 1u) / (2u * kGradRows * kTellLanes);
+    if (s > most) s = most;
+    return s < 1u ? 1u : s;
+}
+
+size_t clipup_norm_doubles(uint32_t ldD) { return 3u * (tell_blocks(ldD) + 1u); }
+size_t tell_counter_words(uint32_t ldD) { return tell_blocks(ldD) + 1u; }
+
+static StepArgs step_args(const TellArgs& a, uint32_t mode, double* grad_sum, float* sigma_sum)
+{
+    StepArgs s;
+    s.mode = mode; s.ldD = a.ldD;
+    s.inv_pop = 1.0 / static_cast<double>(a.P);
+    s.lr = a.lr; s.beta1 = a.beta1; s.beta2 = a.beta2; s.adam_eps = a.adam_eps; s.momentum = a.clipup_momentum;
+    s.max_speed = a.clipup_max_speed; s.sigma_lr = a.sigma_lr; s.sigma_max_change = a.sigma_max_change;
+    s.inv_pairs = 2.0f / static_cast<float>(a.P);
+    s.sigma_vec = a.sigma_vec; s.center = a.center; s.m = a.m; s.v = a.v; s.g = a.g;
+    s.grad_sum = grad_sum; s.sigma_sum = sigma_sum; s.norms = a.norms; s.status = a.status;
     return s;
 }
 
-size_t clipup_norm_doubles(uint32_t ldD) { return 2u * ((ldD / 4u + 255u) / 256u); }
-
 template <bool REGEN, bool SIGMA>
-static void launch_grad(dim3 grid, cudaStream_t st, const TellArgs& a, uint32_t pps)
+static cudaError_t launch_tell_kernel(cudaStream_t st, const TellArgs& a, const StepArgs& s, bool ranks, dim3 grid, uint32_t pps)
 {
-    launch_dependent(k_grad_partial<REGEN, SIGMA>, grid, dim3(kGradThreads), 0, st, a.u, a.eps, philox_key(a.k0, a.k1),
-                     a.pair0, a.H, a.D, a.ldD, pps, a.partial, a.sigma_partial, a.status);
+    auto kernel = ranks ? k_tell<REGEN, SIGMA, true> : k_tell<REGEN, SIGMA, false>;
+    return launch_dependent(kernel, grid, dim3(256), 0, st, a.fitness, a.rank, a.u, a.eps, philox_key(a.k0, a.k1), a.pair0, a.H, a.P,
+                            a.D, pps, a.partial, a.sigma_partial, a.counters, s);
 }
 
-static int launch_partials(cudaStream_t st, const TellArgs& a, uint32_t* used_out)
+// ranks + gradient sums (+ the step, unless mode is kStepSums)
+static int launch_tell(cudaStream_t st, const TellArgs& a, uint32_t mode, double* grad_sum, float* sigma_sum)
 {
-    const uint32_t quads = a.ldD / 4u;
     const uint32_t pps = (a.H + a.splits - 1u) / a.splits;
-    const uint32_t used = (a.H + pps - 1u) / pps;      // splits that own at least one pair
-    dim3 grid((quads + kGradThreads - 1u) / kGradThreads, used);
-    const bool sig = a.sigma_partial != nullptr;
-    if (a.eps) { if (sig) launch_grad<false, true>(grid, st, a, pps); else launch_grad<false, false>(grid, st, a, pps); }
-    else       { if (sig) launch_grad<true, true>(grid, st, a, pps);  else launch_grad<true, false>(grid, st, a, pps); }
-    *used_out = used;
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
-}
-
-// optimiser step (and sigma step) from `splits` rows of partial sums
-static int launch_step(cudaStream_t st, const TellArgs& a, const double* partial, const float* sigma_partial,
-                       uint32_t splits)
-{
-    const uint32_t quads = a.ldD / 4u;
-    const double inv_pop = 1.0 / static_cast<double>(a.P);
-    const float inv_pairs = 2.0f / static_cast<float>(a.P);
-    const uint32_t nb = (quads + 255u) / 256u;
-    int launches = 0;
-    if (a.optimizer == EVO_OPT_ADAM) {
-        if (launch_dependent(k_update<true>, dim3(nb), dim3(256), 0, st, partial, sigma_partial, splits, a.ldD, inv_pop, a.lr,
-                             a.beta1, a.beta2, a.adam_eps, a.sigma_lr, a.sigma_max_change, inv_pairs, a.sigma_vec,
-                             a.center, a.m, a.v, a.g, a.norms, a.status) != cudaSuccess) return -1;
-        launches += 1;
-    } else {
-        if (launch_dependent(k_update<false>, dim3(nb), dim3(256), 0, st, partial, sigma_partial, splits, a.ldD, inv_pop, a.lr,
-                             a.beta1, a.beta2, a.adam_eps, a.sigma_lr, a.sigma_max_change, inv_pairs, a.sigma_vec,
-                             a.center, a.m, a.v, a.g, a.norms, a.status) != cudaSuccess) return -1;
-        k_clipup_velocity<<<nb, 256, 0, st>>>(a.g, a.m, a.ldD, a.lr, a.clipup_momentum, a.norms, nb, a.status);
-        if (cudaGetLastError() != cudaSuccess) return -1;
-        k_clipup_apply<<<nb, 256, 0, st>>>(a.m, a.center, a.ldD, a.clipup_max_speed, a.norms, nb, a.status);
-        if (cudaGetLastError() != cudaSuccess) return -1;
-        launches += 3;
+    const dim3 grid(tell_blocks(a.ldD), (a.H + pps - 1u) / pps);       // splits that own at least one pair
+    // Every column block repeats the ranking of its split's members, P comparisons each: worth it while the repetition costs
+    // less than a launch (a few microseconds; 570 column blocks x 1,024 members would add about 10).
+    const bool whole = 2u * a.H == a.P && a.pair0 == 0u;
+    const bool ranks = whole && a.P <= kRankInTell && pps <= kTellPairs && static_cast<uint64_t>(grid.x) * a.P <= 65536u;
+    int launches = 1;
+    if (!ranks) {
+        if (launch_rank(st, a.fitness, a.P, a.rank, a.u, a.status) < 0) return -1;
+        ++launches;
     }
-    if (launch_dependent(k_tell_finish, dim3(1), dim3(1), 0, st, a.status) != cudaSuccess) return -1;
-    return launches + 1;
+    const StepArgs s = step_args(a, mode, grad_sum, sigma_sum);
+    const bool sig = a.sigma_partial != nullptr;
+    const cudaError_t e = a.eps ? (sig ? launch_tell_kernel<false, true>(st, a, s, ranks, grid, pps) : launch_tell_kernel<false, false>(st, a, s, ranks, grid, pps))
+                                : (sig ? launch_tell_kernel<true, true>(st, a, s, ranks, grid, pps) : launch_tell_kernel<true, false>(st, a, s, ranks, grid, pps));
+    if (e != cudaSuccess) return -1;
+    if (mode == kStepClipup && a.ldD / 4u > kClipupInClose) {
+        if (launch_dependent(k_clipup_apply, dim3((a.ldD / 4u + 255u) / 256u), dim3(256), 0, st, grid.x, s) != cudaSuccess) return -1;
+        ++launches;
+    }
+    return launches;
 }
 
 int launch_gradient_update(cudaStream_t st, const TellArgs& a)
 {
-    uint32_t used = 0;
-    const int n1 = launch_partials(st, a, &used);
-    if (n1 < 0) return -1;
-    const int n2 = launch_step(st, a, a.partial, a.sigma_partial, used);
-    return n2 < 0 ? -1 : n1 + n2;
-}
-
-// splits -> one row each, in split order (the buffers the caller sums across shards); a skipped
-// update (NaN fitness) leaves zeros so that the all-reduce still runs on defined values
-__global__ void __launch_bounds__(256)
-k_sum_splits(const double* __restrict__ partial, const float* __restrict__ sigma_partial, uint32_t splits,
-             uint32_t ldD, double* __restrict__ grad_sum, float* __restrict__ sigma_sum, const DeviceStatus* status)
-{
-    const uint32_t d = blockIdx.x * blockDim.x + threadIdx.x;
-    if (d >= ldD) return;
-    const bool skip = status->nonfinite != 0;
-    double s = 0.0;
-    float t = 0.f;
-    if (!skip) {
-        for (uint32_t k = 0; k < splits; ++k) s += partial[static_cast<size_t>(k) * ldD + d];
-        if (sigma_partial)
-            for (uint32_t k = 0; k < splits; ++k) t += sigma_partial[static_cast<size_t>(k) * ldD + d];
-    }
-    grad_sum[d] = s;
-    if (sigma_sum) sigma_sum[d] = t;
+    return launch_tell(st, a, a.optimizer == EVO_OPT_ADAM ? kStepAdam : kStepClipup, nullptr, nullptr);
 }
 
 int launch_gradient_sums(cudaStream_t st, const TellArgs& a, double* grad_sum, float* sigma_sum)
 {
-    uint32_t used = 0;
-    if (launch_partials(st, a, &used) < 0) return -1;
-    k_sum_splits<<<(a.ldD + 255u) / 256u, 256, 0, st>>>(a.partial, a.sigma_partial, used, a.ldD, grad_sum,
-                                                        a.sigma_partial ? sigma_sum : nullptr, a.status);
-    return cudaGetLastError() == cudaSuccess ? 2 : -1;
+    return launch_tell(st, a, kStepSums, grad_sum, sigma_sum);
 }
 
-int launch_update_from_sums(cudaStream_t st, const TellArgs& a, const double* grad_sum, const float* sigma_sum)
+int launch_update_from_sums(cudaStream_t st, const TellArgs& a, double* grad_sum, float* sigma_sum)
 {
-    return launch_step(st, a, grad_sum, a.sigma_partial ? sigma_sum : nullptr, 1u);
+    const uint32_t mode = a.optimizer == EVO_OPT_ADAM ? kStepAdam : kStepClipup;
+    const StepArgs s = step_args(a, mode, grad_sum, sigma_sum);
+    const uint32_t nb = (a.ldD / 4u + 255u) / 256u;
+    if (launch_dependent(k_step_from_sums, dim3(nb), dim3(256), 0, st, a.counters, a.sigma_partial != nullptr, s) != cudaSuccess) return -1;
+    if (mode == kStepClipup && a.ldD / 4u > kClipupInClose) {
+        if (launch_dependent(k_clipup_apply, dim3(nb), dim3(256), 0, st, nb, s) != cudaSuccess) return -1;
+        return 2;
+    }
+    return 1;
 }
 
 }  // namespace evo

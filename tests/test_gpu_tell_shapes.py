@@ -1,0 +1,51 @@
+"""tell where its kernel's tiles and splits are not full: columns around 256 (64 quads), pairs around the 32 of a split, populations
+ranked inside the gradient kernel and by a kernel of their own (more than 2,048 members, or many columns), ties across the
+128 entries that a warp compares at a time.  Ranks exact; centre, moments and gradient to 1e-5 of their RMS, as
+everywhere (fp64 sums)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import rel_err
+from paper_2202_05008_b200 import Solver, workloads as W
+
+pytestmark = pytest.mark.gpu
+F32 = lambda x: float(np.float32(x))
+
+
+@pytest.mark.parametrize("P,D", [(2, 1), (64, 255), (66, 256), (62, 257), (130, 1025), (2046, 300), (2048, 33), (2050, 33), (4098, 70),
+                                 (8200, 40), (16386, 9), (1024, 70000)])
+@pytest.mark.parametrize("noise_mode", [W.NOISE_STORED, W.NOISE_REGENERATED])
+@pytest.mark.parametrize("clipup", [False, True])
+def test_tell_shapes(P, D, noise_mode, clipup):
+    w = W.Workload("tell", P, D, seed=P + D, sigma=0.1, optimizer=W.OPT_CLIPUP if clipup else W.OPT_ADAM)
+    s = Solver(w, noise_mode=noise_mode)
+    rng = np.random.default_rng(P)
+    for gen in range(2):
+        c0 = s.center().cpu().numpy()
+        m0, v0 = (x.cpu().numpy().astype(np.float64) for x in s.moments())
+        s.ask()
+        f = np.round(rng.standard_normal(P) * 20).astype(np.float32)          # plenty of ties
+        f[rng.integers(0, P, 3)] = [np.inf, -np.inf, -0.0]
+        s.tell(torch.tensor(f, device="cuda"))
+        assert s.sync_status() == 0
+        rank, u = (x.cpu().numpy() for x in s.ranks())
+        rank_o, u_o, _ = oracle.centered_rank(f)
+        assert (rank == rank_o).all() and (u == u_o).all()
+        _, eps_o = oracle.ask(w.seed, gen, P, D, c0, w.sigma)
+        g_o = oracle.gradient(u_o, eps_o, F32(w.sigma))
+        assert rel_err(s.gradient().cpu().numpy(), g_o) < 1e-5
+        if not clipup:
+            c_o, m_o, v_o = oracle.adam(c0.astype(np.float64), m0, v0, g_o, gen + 1, F32(w.lr), F32(0.9), F32(0.999), F32(1e-8))
+            keep = np.abs(g_o) >= 1e-6 * np.sqrt(np.mean(g_o ** 2))
+            assert rel_err(s.center().cpu().numpy()[keep], c_o[keep]) < 1e-5
+            assert rel_err(s.moments()[0].cpu().numpy(), m_o) < 1e-5 and rel_err(s.moments()[1].cpu().numpy(), v_o) < 1e-5
+        else:
+            vel = 0.9 * m0 + F32(w.lr) * g_o / np.sqrt(np.sum(g_o ** 2))
+            n, most = np.sqrt(np.sum(vel ** 2)), 2 * F32(w.lr)
+            vel = vel * (most / n if n > most else 1.0)
+            assert rel_err(s.moments()[0].cpu().numpy(), vel) < 1e-5
+            assert rel_err(s.center().cpu().numpy(), c0 + vel) < 1e-5
+    assert s.counters() == (2, 2)
+    s.close()
