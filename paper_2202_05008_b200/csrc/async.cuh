@@ -35,26 +35,38 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst_smem, const void* src
                  :: "r"(dst_smem), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// Bounded wait.  try_wait is given a suspend-time hint, so a waiting warp sleeps in hardware
-// instead of taking issue slots from the warps that work; the loop re-arms it until the phase
-// completes or ~2^(*max_cycles_log2) SM clocks have passed (the limit lives in the device status
-// block, so a test can make it short).
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, const uint32_t* max_cycles_log2)
+__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t done;
     asm volatile("{\n\t.reg .pred p;\n\t"
                  "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                  "selp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
+    return done != 0u;
+}
+// as above, but the warp may sleep up to 20 us for the phase
+__device__ __forceinline__ bool mbar_sleep_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
+    return done != 0u;
+}
+
+// Bounded wait.  try_wait is given a suspend-time hint, so a waiting warp sleeps in hardware
+// instead of taking issue slots from the warps that work; the loop re-arms it until the phase
+// completes or ~2^(*max_cycles_log2) SM clocks have passed (the limit lives in the device status
+// block, so a test can make it short).  The clock and the limit are read only after a first sleep that did not
+// see the phase complete: a wait is on the path from one role to the next.
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, const uint32_t* max_cycles_log2)
+{
+    if (mbar_try_wait(bar, parity) || mbar_sleep_wait(bar, parity)) return true;
     const long long t0 = clock64();
-    const long long limit = 1ll << *max_cycles_log2;      // read only once the wait has to sleep
+    const long long limit = 1ll << *max_cycles_log2;
     for (;;) {
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(bar), "r"(parity), "r"(20000u) : "memory");     // hint: 20 us
-        if (done) return true;
+        if (mbar_sleep_wait(bar, parity)) return true;
         if (clock64() - t0 > limit) return false;
     }
 }

@@ -212,11 +212,11 @@ k_cnn_conv1_tc(const float* __restrict__ theta, uint32_t ldD, uint32_t P, const 
             const uint32_t a_base = smem_u32(Asm), b_base = smem_u32(Bsm);
             uint32_t u = 0, ti = 0;
             for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++ti) {
-                wait_or_abort(&ctl.abort, &ctl.a_full[ti & 1u], (ti >> 1) & 1u, status);
+                try_wait_or_abort(&ctl.abort, &ctl.a_full[ti & 1u], (ti >> 1) & 1u, status);
                 const uint32_t a0 = a_base + (ti & 1u) * kC1SmemA;
                 for (uint32_t gm = 0; gm < n_gm; ++gm, ++u) {
                     const uint32_t buf = u & 1u;
-                    wait_or_abort(&ctl.abort, &ctl.acc_free[buf], (u >> 1) & 1u, status);
+                    try_wait_or_abort(&ctl.abort, &ctl.acc_free[buf], (u >> 1) & 1u, status);
                     tc_fence_after();
 #pragma unroll
                     for (uint32_t ks = 0; ks < 3u; ++ks) {
@@ -238,7 +238,7 @@ k_cnn_conv1_tc(const float* __restrict__ theta, uint32_t ldD, uint32_t P, const 
         uint32_t ti = 0;
         for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++ti) {
             c1_load_patch(images, tile * 128u + row, batch, patch);
-            if (ti >= 2u) wait_or_abort(&ctl.abort, &ctl.a_free[ti & 1u], ((ti >> 1) - 1u) & 1u, status);
+            if (ti >= 2u) try_wait_or_abort(&ctl.abort, &ctl.a_free[ti & 1u], ((ti >> 1) - 1u) & 1u, status);
             unsigned char* Abuf = Asm + (ti & 1u) * kC1SmemA;
             c1_stage_row(Abuf, row, patch);
             fence_async_smem();
@@ -248,7 +248,7 @@ k_cnn_conv1_tc(const float* __restrict__ theta, uint32_t ldD, uint32_t P, const 
         // the last arrivals on a_free land in this block's shared memory: see them in before the block ends
         if (row < 2 && ti > static_cast<uint32_t>(row)) {
             const uint32_t n_done = (ti - row + 1u) >> 1;              // completions of buffer `row`
-            wait_or_abort(&ctl.abort, &ctl.a_free[row], (n_done - 1u) & 1u, status);
+            try_wait_or_abort(&ctl.abort, &ctl.a_free[row], (n_done - 1u) & 1u, status);
         }
     } else {
         // ================= epilogue warps ==========================================================
@@ -262,28 +262,26 @@ k_cnn_conv1_tc(const float* __restrict__ theta, uint32_t ldD, uint32_t P, const 
 
             for (uint32_t gm = 0; gm < n_gm; ++gm, ++u) {
                 const uint32_t buf = u & 1u;
-                wait_or_abort(&ctl.abort, &ctl.mma_done[buf], (u >> 1) & 1u, status);
+                try_wait_or_abort(&ctl.abort, &ctl.mma_done[buf], (u >> 1) & 1u, status);
                 tc_fence_after();
                 const uint32_t t0 = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + buf * 256u + part * (32u * kC1PerThread);
-                // My members of the unit, one at a time: a member's 8 filters at the four positions of
-                // the pooling window are 32 consecutive columns.  The loads of the next member are in flight
-                // while this one is pooled and stored (two register buffers).
-                uint32_t ra[4][8], rb[4][8];
+                // My members of the unit: a member's 8 filters at the four positions of the pooling window are 32 consecutive
+                // columns.  One load instruction per member and one wait for both, then the accumulator is free: the turn of an
+                // accumulator (MMAs, hand-over, read, hand-back) paces this kernel, no pipe is more than half busy.
+                // 500 members x 1000 images: 252 us; with loads of 8 columns and a wait per member 262; with the
+                // two accumulators read by eight warps each 281.
+                static_assert(kC1PerThread == 2, "two register buffers");
+                uint32_t acc[kC1PerThread][4][8];
 #pragma unroll
-                for (int w = 0; w < 4; ++w) tmem_ld8_issue(t0 + w * 8u, ra[w]);
+                for (int j = 0; j < kC1PerThread; ++j) tmem_ld32_issue(t0 + j * 32u, acc[j]);
+#pragma unroll
+                for (int j = 0; j < kC1PerThread; ++j) tmem_ld8x4_fence(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl.acc_free[buf]));
 #pragma unroll
                 for (int j = 0; j < kC1PerThread; ++j) {
-                    uint32_t (&cur)[4][8] = (j & 1) ? rb : ra;
-                    uint32_t (&nxt)[4][8] = (j & 1) ? ra : rb;
-                    tmem_ld8x4_fence(cur[0], cur[1], cur[2], cur[3]);
-                    if (j < kC1PerThread - 1) {
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) tmem_ld8_issue(t0 + (j + 1) * 32u + w * 8u, nxt[w]);
-                    } else {                                             // my part of the accumulator is in registers
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&ctl.acc_free[buf]));
-                    }
+                    const uint32_t (&cur)[4][8] = acc[j];
                     const uint32_t m = gm * 8u + part * kC1PerThread + j;
                     // the accumulators already contain the bias: relu(max4) = two 3-input max per value
                     uint32_t o[4];
@@ -370,7 +368,7 @@ struct __align__(128) C2Smem {
 
 __device__ __forceinline__ void c2_wait(C2Smem& S, uint64_t* bar, uint32_t parity, DeviceStatus* status)
 {
-    wait_or_abort(&S.abort, bar, parity, status);
+    try_wait_or_abort(&S.abort, bar, parity, status);
 }
 
 // Progress that is counted, not signalled: the members whose bands are staged, the members whose
@@ -384,9 +382,8 @@ __device__ __forceinline__ void c2_wait_count(C2Smem& S, const uint32_t* counter
     uint32_t have;
     long long t0 = 0;
     for (;;) {
-        if (S.abort) return;
         asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(have) : "r"(addr) : "memory");
-        if (have >= need) return;
+        if (have >= need || S.abort) return;
         if (t0 == 0) t0 = clock64();
         if (clock64() - t0 > (1ll << status->wait_cycles_log2)) {
             S.abort = 1;

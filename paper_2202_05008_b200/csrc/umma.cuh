@@ -102,6 +102,15 @@ __device__ __forceinline__ void wait_or_abort(volatile int* abort_flag, uint64_t
     }
 }
 
+// The same for a wait whose phase has often completed already: only one that has to sleep asks whether there is anything to wait
+// for.  (Convolutions, 500 members x 1000 images: 580 us instead of 598 a generation.  The recurrent roll-out, where
+// nearly every wait sleeps, is 0.4 % faster without the extra try.)
+__device__ __forceinline__ void try_wait_or_abort(volatile int* abort_flag, uint64_t* bar, uint32_t parity,
+                                                  DeviceStatus* status)
+{
+    if (!mbar_try_wait(smem_u32(bar), parity)) wait_or_abort(abort_flag, bar, parity, status);
+}
+
 // asynchronous TMEM load of 16 columns; the registers are valid after tmem_ld16_fence on them
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* u)
 {
@@ -124,6 +133,18 @@ __device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t* u)
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7])
+                 : "r"(taddr) : "memory");
+}
+// asynchronous TMEM load of 32 columns into r[0..3][0..7]; valid after tmem_ld8x4_fence on them
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&r)[4][8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(r[0][0]), "=r"(r[0][1]), "=r"(r[0][2]), "=r"(r[0][3]), "=r"(r[0][4]), "=r"(r[0][5]), "=r"(r[0][6]), "=r"(r[0][7]),
+                   "=r"(r[1][0]), "=r"(r[1][1]), "=r"(r[1][2]), "=r"(r[1][3]), "=r"(r[1][4]), "=r"(r[1][5]), "=r"(r[1][6]), "=r"(r[1][7]),
+                   "=r"(r[2][0]), "=r"(r[2][1]), "=r"(r[2][2]), "=r"(r[2][3]), "=r"(r[2][4]), "=r"(r[2][5]), "=r"(r[2][6]), "=r"(r[2][7]),
+                   "=r"(r[3][0]), "=r"(r[3][1]), "=r"(r[3][2]), "=r"(r[3][3]), "=r"(r[3][4]), "=r"(r[3][5]), "=r"(r[3][6]), "=r"(r[3][7])
                  : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld8x4_fence(uint32_t* a, uint32_t* b, uint32_t* c, uint32_t* d)
