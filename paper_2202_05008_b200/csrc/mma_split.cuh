@@ -10,10 +10,12 @@
 // the same 128x16x8 product from registers in 16 clocks of the four sub-cores (8.1 clocks per m16n8k16 and
 // sub-core, measured) and the result is there after 22 (28 for another pipe).
 //
-// tanh.  tanh(x) = 1 - 2 r, r = 1 / (1 + 2^p), p = 2 log2(e) x.  The activation that travels is r (between 0 and 1, so
-// its low part needs no scaling), and the layers are rewritten once, when the weights are loaded, to give p from r:
-//     p = f (b + sum_k w_k) + sum_k (-2 f w_k) r_k        f = 2 log2(e)
-// so a tanh is an exponential, an addition and a reciprocal.  r is as accurate as the 1 - 2 r it stands for.
+// tanh.  A layer's weights and biases are taken times f = 2 log2(e) when they are loaded, so its sums are p = f x and
+//     tanh x = (e - 1) / (e + 1),  e = 2^p:
+// e - 1 is exact where e is near 1, so a small tanh keeps its relative accuracy as far as the exponential has it.  It
+// travels times 2^13: the low part of an activation is then in fp16's normal range down to 2^-16 of the largest.  (Carrying
+// r = 1 / (1 + 2^p) instead, with the layers rewritten for it, saves a few instructions, but r is near 1/2 for small
+// activations: the products then cancel, and the states were 2 to 5 times as far from the 64-bit ones.)
 //
 // Activations of a layer lie in shared memory as the B operand, [column][unit] fp16, a column = one episode and
 // part.  Two packings of the columns of an n-tile (8 columns) are used:
@@ -77,6 +79,11 @@ __device__ __forceinline__ uint32_t transpose8(uint32_t x)
 }
 
 constexpr float kF = 2.885390082f;                           // 2 log2(e)
+// What a factor f lacks: the fp32 f is short by 1.3e-8, and the tensor core cuts its sums off, which leaves a result 3e-8 short
+// on average.  (Both are systematic, and a roll-out adds them up: without, the states of 28-64-64-64-8 shrink by 4e-8 per step
+// and the fitness is off by 5e-7; with, by less than 5e-9 and 2e-7 to 1e-7.)
+constexpr float kRest = 1.3e-8f + 3.0e-8f;
+constexpr float kAct = 8192.0f, kActInv = 1.0f / 8192.0f;    // scale of the activations (a start state of 5.8, the largest normal, fits fp16)
 constexpr float kLo = 2048.0f, kLoInv = 1.0f / 2048.0f;      // scale of the weights' low parts
 
 // a and b, a in the low half: hi parts in one word, the negated low parts in the other
@@ -112,11 +119,14 @@ __device__ __forceinline__ uint32_t finite_magnitude(float w)
     const uint32_t m = __float_as_uint(w) & 0x7FFFFFFFu;
     return m < 0x7F800000u ? m : 0u;
 }
-__device__ __forceinline__ void split_weights(float a, float b, uint32_t& hi, uint32_t& lo)
+// k wa and k wb, a in the low half, with k2 = k kRest and the roundings of the products in the low parts
+__device__ __forceinline__ void split_weights(float wa, float wb, float k, float k2, uint32_t& hi, uint32_t& lo)
 {
+    const float a = wa * k, b = wb * k;
     const __half2 h = __floats2half2_rn(a, b);
     const float2 f = __half22float2(h);
-    const __half2 l = __floats2half2_rn((a - f.x) * kLo, (b - f.y) * kLo);
+    const float ra = fmaf(wa, k2, fmaf(wa, k, -a)), rb = fmaf(wb, k2, fmaf(wb, k, -b));
+    const __half2 l = __floats2half2_rn(((a - f.x) + ra) * kLo, ((b - f.y) + rb) * kLo);
     hi = *reinterpret_cast<const uint32_t*>(&h);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
@@ -140,28 +150,12 @@ __device__ __forceinline__ void load_tile(const float* W, int ni, int no, int ro
             if (row < no && col < ni) w.x = p[0];
             if (row < no && col + 1 < ni) w.y = p[1];
         }
-        split_weights(sc.weight(w.x) * k, sc.weight(w.y) * k, h[i], l[i]);
+        split_weights(sc.weight(w.x), sc.weight(w.y), k, k * kRest, h[i], l[i]);
     }
     hi = make_uint4(h[0], h[1], h[2], h[3]);
     lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// f (bias + sum of a row's weights) of `unit`; the four lanes of a group add a quarter of the row each
-__device__ __forceinline__ float folded_bias(const float* W, const float* B, int ni, int no, int unit, int lane, const Scale& sc)
-{
-    float s = 0.f;
-    if (unit < no) {
-        if ((lane & 3) == 0) s = B[unit];
-        for (int k = lane & 3; k < ni; k += 4) s += sc.weight(W[static_cast<size_t>(unit) * ni + k]);
-    }
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    return kF * s;
-}
-
-// r = 1 / (1 + 2^p).  The special-function unit takes 8 clocks per warp for an exponential and 16 for a reciprocal, so two
-// values share one: 1/a = b / (a b).  p is held below 60 there so that the product stays finite (r is 0 to fp32 from
-// 2^-24 on: 1 - 2 r rounds to 1).
 __device__ __forceinline__ float ex2_fast(float p)
 {
     float e;
@@ -174,14 +168,41 @@ __device__ __forceinline__ float rcp_fast(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ float logistic2(float p) { return rcp_fast(ex2_fast(p) + 1.0f); }
-__device__ __forceinline__ void logistic2(float& p, float& q)
+// kAct tanh(p / f).  p is held below 40, where the tanh is 1 to fp32 long since, so that e stays finite.
+__device__ __forceinline__ float hold(float p)
 {
-    asm("min.NaN.f32 %0, %0, 0f42700000;\n\tmin.NaN.f32 %1, %1, 0f42700000;" : "+f"(p), "+f"(q));
-    const float a = ex2_fast(p) + 1.0f, b = ex2_fast(q) + 1.0f;
+    asm("min.NaN.f32 %0, %0, 0f42200000;" : "+f"(p));
+    return p;
+}
+__device__ __forceinline__ float tanh_one(float p)
+{
+    const float e = ex2_fast(hold(p));
+    return fmaf(kAct, e, -kAct) * rcp_fast(e + 1.0f);
+}
+// Two of them with one reciprocal, 1/a = b / (a b): the special-function unit takes 8 clocks per warp for an exponential and 16
+// for a reciprocal.  Two more multiplications, each with its rounding.
+__device__ __forceinline__ void tanh_two(float& p, float& q)
+{
+    const float e = ex2_fast(hold(p)), d = ex2_fast(hold(q));
+    const float a = e + 1.0f, b = d + 1.0f;
     const float r = rcp_fast(a * b);
-    p = r * b;
-    q = r * a;
+    p = fmaf(kAct, e, -kAct) * b * r;
+    q = fmaf(kAct, d, -kAct) * a * r;
+}
+// With the Taylor polynomial to x^9 below |x| = 0.3, where what it leaves out is below 6e-8 of x.  For k_rollout_mlp_mma,
+// which also takes policies without a wide layer whose sums would hide the exponential's error near 1 (28-20-8: states 1.0
+// to 1.2 times as far from the 64-bit ones as with tanhf on the fp32 pipe, 0.8 to 0.95 with the polynomial; 28-64-64-64-8,
+// 512 members: 485 us a generation instead of 465).
+__device__ __forceinline__ float tanh_fine(float p)
+{
+    constexpr double f = 2.885390081777927, g = 1.0 / (f * f);                // z = p^2 = x^2 / g
+    const float z = p * p, k = p * static_cast<float>(8192.0 / f);
+    float c = fmaf(z, static_cast<float>(62.0 / 2835.0 * g * g * g * g), static_cast<float>(-17.0 / 315.0 * g * g * g));
+    c = fmaf(c, z, static_cast<float>(2.0 / 15.0 * g * g));
+    c = fmaf(c, z, static_cast<float>(-1.0 / 3.0 * g));
+    c = fmaf(c, z * k, k);
+    const float h = tanh_one(p);
+    return fabsf(p) < static_cast<float>(0.3 * f) ? c : h;
 }
 
 // Activations of an episode packing: columns of the operand, values per lane, sums of 16 units.
@@ -202,18 +223,18 @@ template <> struct Units<4> {
         mma_k16(h, wh, b[0], b[1]);
         mma_k16(l, wl, b[0], b[1]);
     }
-    // up = Scale::up, up_lo = up / 2048, b0 and b1: biases of units g and g + 8
-    __device__ __forceinline__ void sums(float up, float up_lo, float b0, float b1, float* v) const
+    // up = Scale::up / kAct, b0 and b1: f times the biases of units g and g + 8.  The small products are added up first.
+    __device__ __forceinline__ void sums(float up, float b0, float b1, float* v) const
     {
-        v[0] = fmaf(up_lo, l[0] - l[1], fmaf(up, h[0] - h[1], b0));
-        v[1] = fmaf(up_lo, l[2] - l[3], fmaf(up, h[2] - h[3], b1));
+        v[0] = fmaf(up, h[0], fmaf(up, fmaf(kLoInv, l[0] - l[1], -h[1]), b0));
+        v[1] = fmaf(up, h[2], fmaf(up, fmaf(kLoInv, l[2] - l[3], -h[3]), b1));
     }
     // eight outputs (hi parts of their weights in rows 0-7 of the tile, low parts in rows 8-15): output g
-    static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float up_lo, float bias, float* v)
+    static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float bias, float* v)
     {
         float c[4];
         mma_k16_first(c, w, b[0], b[1]);
-        v[0] = fmaf(up_lo, c[2] - c[3], fmaf(up, c[0] - c[1], bias));
+        v[0] = fmaf(up, c[0], fmaf(up, fmaf(kLoInv, c[2] - c[3], -c[1]), bias));
     }
     // address of this lane's row for store() and load(): 16 units from byte 32 k on
     static __device__ __forceinline__ uint32_t row(uint32_t base, uint32_t pitch, int lane)
@@ -262,18 +283,18 @@ template <> struct Units<8> {
         mma_k16(hl, wh, b[2], b[3]);
         mma_k16(lh, wl, b[0], b[1]);
     }
-    __device__ __forceinline__ void sums(float up, float up_lo, float b0, float b1, float* v) const
+    __device__ __forceinline__ void sums(float up, float b0, float b1, float* v) const
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = fmaf(up_lo, lh[i], fmaf(up, hh[i] - hl[i], i < 2 ? b0 : b1));
+        for (int i = 0; i < 4; ++i) v[i] = fmaf(up, hh[i], fmaf(up, fmaf(kLoInv, lh[i], -hl[i]), i < 2 ? b0 : b1));
     }
-    static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float up_lo, float bias, float* v)
+    static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float bias, float* v)
     {
         float c[4], d[4];
         mma_k16_first(c, w, b[0], b[1]);
         mma_k16_first(d, w, b[2], b[3]);
-        v[0] = fmaf(up_lo, c[2], fmaf(up, c[0] - d[0], bias));
-        v[1] = fmaf(up_lo, c[3], fmaf(up, c[1] - d[1], bias));
+        v[0] = fmaf(up, c[0], fmaf(up, fmaf(kLoInv, c[2], -d[0]), bias));
+        v[1] = fmaf(up, c[1], fmaf(up, fmaf(kLoInv, c[3], -d[1]), bias));
     }
     static __device__ __forceinline__ uint32_t row(uint32_t base, uint32_t pitch, int lane)
     {
@@ -301,10 +322,16 @@ template <> struct Units<8> {
     }
 };
 
-template <int EB> __device__ __forceinline__ void logistic_units(float* v)
+enum class Tanh { kOwn, kShared, kFine };                // a reciprocal each, one for two, with the polynomial
+
+template <int EB, Tanh KIND> __device__ __forceinline__ void tanh_units(float* v)
 {
 #pragma unroll
-    for (int i = 0; i < Units<EB>::kValues; i += 2) logistic2(v[i], v[i + 1]);
+    for (int i = 0; i < Units<EB>::kValues; i += 2) {
+        if (KIND == Tanh::kShared) tanh_two(v[i], v[i + 1]);
+        else if (KIND == Tanh::kFine) { v[i] = tanh_fine(v[i]); v[i + 1] = tanh_fine(v[i + 1]); }
+        else { v[i] = tanh_one(v[i]); v[i + 1] = tanh_one(v[i + 1]); }
+    }
 }
 
 }  // namespace ms

@@ -59,6 +59,9 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 {
     using U = Units<EB>;
     constexpr int NV = U::kValues, NH = NV / 2;                      // NH: values of one unit in a lane
+    // The special-function unit is what several cart-pole members on an SM wait for (5-64-64-1, 256 members: 778 us with shared
+    // reciprocals, 797 without), the issue slots what tanh-linear ones do (28-128-128-8, 4,096: 12.06 and 11.64 ms).
+    constexpr Tanh kTanh = CART ? Tanh::kShared : Tanh::kOwn;
     constexpr int MW = RT == 1 && KT > 4 ? 8 : 4;                    // warps at most
     constexpr uint32_t kPitch = (KT + 1) / 2 * 64 + 16;              // bytes per column of the hidden operand (read two tiles at a time)
     // first the parameters (RT = 2: of the first layer only), then (RT = 2) the low parts of the second layer, [warp][tile][k]
@@ -111,9 +114,9 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         __syncthreads();
     }
     const Scale sc(peak);
-    const float up = sc.up, up_lo = sc.up * kLoInv;
+    const float up = sc.up * kActInv;
 
-    // ---- weights into registers, rewritten for r (see mma_split.cuh) ---------------------------------------
+    // ---- weights into registers, times f (see mma_split.cuh) ---------------------------------------
     const float* W1 = stage;
     const float* B1 = W1 + n1 * nin;
     const float* W2 = (RT == 1 ? stage : row) + w2_at;
@@ -123,28 +126,25 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     const bool pairs = ((n1 | w2_at) & 1) == 0;                      // the second layer's rows can be read two weights at a time
     uint4 w2h[RT][KT], w2l[RT == 1 ? KT : 1];
     uint4 w1h[CART ? 1 : RT][2], w1l[CART ? 1 : RT][2], w3[CART ? 1 : RT];           // w3: the action layer's own inputs (see Units::eight)
-    float w1c[CART ? RT : 1][10], w3c[RT][2], b1[RT][2], b2[RT][2], b3, bd[2];
+    float w1c[CART ? RT : 1][10], w3c[RT][2], b1[RT][2], b2[RT][2], b3;
     uint4* const w2l_s = reinterpret_cast<uint4*>(stage) + warp * (RT * KT * 32) + lane;
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
         const int tile = tile0 + r, u0 = 16 * tile + g, u1 = u0 + 8;              // this lane's two units
-        b2[r][0] = folded_bias(W2, B2, n1, n2, u0, lane, sc);
-        b2[r][1] = folded_bias(W2, B2, n1, n2, u1, lane, sc);
+        b2[r][0] = u0 < n2 ? kF * B2[u0] : 0.f; b2[r][1] = u1 < n2 ? kF * B2[u1] : 0.f;
+        b1[r][0] = u0 < n1 ? kF * B1[u0] : 0.f; b1[r][1] = u1 < n1 ? kF * B1[u1] : 0.f;
         if constexpr (CART) {                                        // the observation is taken as it is, in fp32
-            b1[r][0] = u0 < n1 ? kF * B1[u0] : 0.f; b1[r][1] = u1 < n1 ? kF * B1[u1] : 0.f;
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
                 w1c[r][k] = u0 < n1 ? kF * W1[u0 * 5 + k] : 0.f;
                 w1c[r][5 + k] = u1 < n1 ? kF * W1[u1 * 5 + k] : 0.f;
             }
-            w3c[r][0] = u0 < n2 ? -2.0f * kF * W3[u0] : 0.f; w3c[r][1] = u1 < n2 ? -2.0f * kF * W3[u1] : 0.f;
+            w3c[r][0] = u0 < n2 ? kF * kActInv * W3[u0] : 0.f; w3c[r][1] = u1 < n2 ? kF * kActInv * W3[u1] : 0.f;
         } else {
-            b1[r][0] = folded_bias(W1, B1, nin, n1, u0, lane, sc);
-            b1[r][1] = folded_bias(W1, B1, nin, n1, u1, lane, sc);
 #pragma unroll
-            for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, sc, -2.0f * kF, w1h[r][k], w1l[r][k]);
+            for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, sc, kF, w1h[r][k], w1l[r][k]);
             uint4 lo3;
-            load_tile(W3, n2, nout, 0, 16 * tile, lane, sc, -2.0f * kF, w3[r], lo3);
+            load_tile(W3, n2, nout, 0, 16 * tile, lane, sc, kF, w3[r], lo3);
             w3[r].y = lo3.x; w3[r].w = lo3.z;
         }
     }
@@ -154,38 +154,24 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             uint4 lo;
-            load_tile(W2, n1, n2, 16 * (tile0 + r), 16 * k, lane, sc, -2.0f * kF, w2h[r][k], lo, pairs);
+            load_tile(W2, n1, n2, 16 * (tile0 + r), 16 * k, lane, sc, kF, w2h[r][k], lo, pairs);
             if constexpr (RT == 1) w2l[k] = lo;
             else w2l_s[32 * (r * KT + k)] = lo;
         }
     if constexpr (CART) {
-        float sum = 0.f;
-        for (int k = lane; k < n2; k += 32) sum += W3[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-        b3 = kF * (B3[0] + sum);
+        b3 = kF * B3[0];
     } else {
-        b3 = folded_bias(W3, B3, n2, nout, g, lane, sc);
-        // x' = tanh(A x + B a), x = 1 - 2 r, a = s - 2 s r
+        b3 = kF * B3[g];
+        // x' = tanh(A x + B a)
         const Scale one(0u);
         const float* A = a.task_const;
         const float* Bm = a.task_const + kTlNx * kTlNx;
         for (int i = warp; i < static_cast<int>(kDynTiles); i += nw) {
             uint4 hi, lo;
-            if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, 16 * (i / 3), 16 * (i % 3), lane, one, -2.0f * kF, hi, lo);
-            else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3), 0, lane, one, -2.0f * kF * a.action_scale, hi, lo);
+            if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, 16 * (i / 3), 16 * (i % 3), lane, one, kF, hi, lo);
+            else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3), 0, lane, one, kF * a.action_scale, hi, lo);
             dyn[i * 64 + lane] = hi;
             dyn[i * 64 + 32 + lane] = lo;
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int unit = 16 * warp + g + 8 * i;
-            float sa = 0.f, sb = 0.f;
-            if (unit < static_cast<int>(kTlNx)) {
-                for (uint32_t k = 0; k < kTlNx; ++k) sa += A[unit * kTlNx + k];
-                for (uint32_t k = 0; k < kTlNa; ++k) sb += Bm[unit * kTlNa + k];
-            }
-            bd[i] = kF * fmaf(a.action_scale, sb, sa);
         }
     }
 
@@ -220,7 +206,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
             for (int i = 0; i < NV; ++i) {
                 const int unit = 16 * warp + g + (i >= NH ? 8 : 0);
                 xcur[i] = unit < static_cast<int>(kTlNx) ? x0s[unit][U::episode(i, t)] : 0.f;
-                v[i] = fmaf(-0.5f, xcur[i], 0.5f);
+                v[i] = kAct * xcur[i];
             }
             U::store(x_row + 32u * warp, v);
         }
@@ -258,11 +244,11 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
                 for (int r = 0; r < RT; ++r) acc[r].add(w1h[r][1], w1l[r][1], b[1]);
 #pragma unroll
-                for (int r = 0; r < RT; ++r) acc[r].sums(up, up_lo, b1[r][0], b1[r][1], v[r]);
+                for (int r = 0; r < RT; ++r) acc[r].sums(up, b1[r][0], b1[r][1], v[r]);
             }
 #pragma unroll
             for (int r = 0; r < RT; ++r) {
-                logistic_units<EB>(v[r]);
+                tanh_units<EB, kTanh>(v[r]);
                 if (RT == 1 || tile0 + r < KT) U::store(h1_row + 32u * (tile0 + r), v[r]);
             }
         }
@@ -302,8 +288,8 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                 float v[RT][NV];
 #pragma unroll
                 for (int r = 0; r < RT; ++r) {
-                    acc[r].sums(up, up_lo, b2[r][0], b2[r][1], v[r]);
-                    logistic_units<EB>(v[r]);
+                    acc[r].sums(up, b2[r][0], b2[r][1], v[r]);
+                    tanh_units<EB, kTanh>(v[r]);
                 }
                 if constexpr (CART) {
                     float p[NH];
@@ -320,7 +306,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
                     for (int r = 0; r < RT; ++r) U::transpose(v[r], b[r]);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) U::eight(w3[r], b[r], up, up_lo, 0.f, p[r]);
+                    for (int r = 0; r < RT; ++r) U::eight(w3[r], b[r], up, 0.f, p[r]);
                     if constexpr (RT == 2) { p[0][0] += p[RT - 1][0]; p[0][1] += p[RT - 1][1]; }
                     if constexpr (EB == 4) part_t[warp][lane] = p[0][0];
                     else *reinterpret_cast<float2*>(&part_t[warp][2 * lane]) = make_float2(p[0][0], p[0][1]);
@@ -345,7 +331,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                 float pre = p[0];
 #pragma unroll
                 for (int off = EB; off < 32; off <<= 1) pre += __shfl_xor_sync(0xffffffffu, pre, off);
-                const float force = fmaf(-2.0f * a.action_scale, logistic2(pre + b3), a.action_scale);
+                const float force = a.action_scale * kActInv * tanh_one(pre + b3);
                 cartpole_finish(cpc, ahead, force, cps, snc, csc);
                 if (lane < EB) { obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd; }
                 if (step < traced && lane < nE)
@@ -374,7 +360,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
             acc.first(tiles[0], tiles[32], b[0]);
             acc.add(tiles[64], tiles[96], b[1]);
 #pragma unroll
-            for (int i = 0; i < NH; ++i) v[i] = logistic2(((p[0][i] + p[1][i]) + (p[2][i] + p[3][i])) + b3);
+            for (int i = 0; i < NH; ++i) v[i] = tanh_one(((p[0][i] + p[1][i]) + (p[2][i] + p[3][i])) + b3);
             uint32_t hi, lo;
             split_two(v[0], EB == 4 ? 0.f : v[NH - 1], hi, lo);
             if constexpr (EB == 4) { b[0][0] = transpose8(__byte_perm(hi, lo, 0x5410)); b[0][1] = 0u; }
@@ -382,16 +368,16 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
             if (warp == 0) {                                      // the action's share of the reward
 #pragma unroll
                 for (int i = 0; i < NH; ++i) {
-                    const float act = fmaf(-2.0f * a.action_scale, v[i], a.action_scale);
+                    const float act = a.action_scale * kActInv * v[i];
                     if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
                 }
             }
             acc.add(tiles[128], tiles[160], b[0]);
-            acc.sums(1.0f, kLoInv, bd[0], bd[1], v);
-            logistic_units<EB>(v);
+            acc.sums(kActInv, 0.f, 0.f, v);
+            tanh_units<EB, kTanh>(v);
             U::store(xout + 32u * warp, v);
 #pragma unroll
-            for (int i = 0; i < NV; ++i) xcur[i] = fmaf(-2.0f, v[i], 1.0f);        // padding rows: p = 0, exactly 0
+            for (int i = 0; i < NV; ++i) xcur[i] = kActInv * v[i];              // padding rows: p = 0, exactly 0
             if (step < traced) {
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
@@ -447,7 +433,7 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
     uint32_t most = 0;
     for (uint32_t i = lane; i < a.ldD; i += 32u) most = max(most, finite_magnitude(stage[i]));
     const Scale sc(__reduce_max_sync(0xffffffffu, most));
-    const float up_lo = sc.up * kLoInv;
+    const float up = sc.up * kActInv;
     const uint32_t traced = a.trace ? a.trace_T : 0u;
 
     const float* W1 = stage;
@@ -462,19 +448,19 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
         for (int k = 0; k < 5; ++k) w1[i][k] = u < n1 ? kF * W1[u * 5 + k] : 0.f;
         w1[i][5] = u < n1 ? kF * B1[u] : 0.f;
-        b2[i] = folded_bias(W2, B2, n1, n2, u, lane, sc);
+        b2[i] = u < n2 ? kF * B2[u] : 0.f;
     }
     uint4 w2h, w2l;
-    load_tile(W2, n1, n2, 0, 0, lane, sc, -2.0f * kF, w2h, w2l);
+    load_tile(W2, n1, n2, 0, 0, lane, sc, kF, w2h, w2l);
     uint32_t w3h[2], w3l[2];
-    const float f = -2.0f * kF * sc.down;
+    const float f = kF * sc.down;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int col = 2 * t + 8 * k;
-        split_weights(col < n2 ? f * sc.weight(W3[col]) : 0.f, col + 1 < n2 ? f * sc.weight(W3[col + 1]) : 0.f, w3h[k], w3l[k]);
+        split_weights(col < n2 ? sc.weight(W3[col]) : 0.f, col + 1 < n2 ? sc.weight(W3[col + 1]) : 0.f, f, f * kRest, w3h[k], w3l[k]);
     }
     const uint4 w3 = make_uint4(w3h[0], w3l[0], w3h[1], w3l[1]);        // the one output in every row (see Units::eight)
-    const float b3 = folded_bias(W3, W3 + n2, n2, 1, 0, lane, sc);
+    const float b3 = kF * W3[n2];
 
     const CartpoleFast c = cartpole_fast_const(a.tp);
     CpState s = cartpole_reset(key, status->generation, e0 + min(t, nE - 1), a.tp[EVO_CP_INIT_RANGE]);
@@ -491,18 +477,18 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
             p = fmaf(w1[i][1], s.xd, p);
             p = fmaf(w1[i][4], s.thd, p);
             p = fmaf(w1[i][3], sn, p);
-            v[i] = logistic2(fmaf(w1[i][2], cs, p));
+            v[i] = tanh_one(fmaf(w1[i][2], cs, p));
         }
         U::transpose(v, b);
         U h2;
         h2.first(w2h, w2l, b);
         const CpAhead ahead = cartpole_ahead(c, s, sn, cs);
         if (step > 0u) ret = fmaf(cs, __expf(-s.x * s.x), ret);       // reward of the step before, on its post-step state
-        h2.sums(sc.up, up_lo, b2[0], b2[1], v);
-        v[0] = logistic2(v[0]); v[1] = logistic2(v[1]);               // a reciprocal each: the unit is idle, the chain shorter
+        h2.sums(up, b2[0], b2[1], v);
+        v[0] = tanh_one(v[0]); v[1] = tanh_one(v[1]);                 // a reciprocal each: the unit is idle, the chain shorter
         U::transpose(v, b);
-        U::eight(w3, b, sc.up, up_lo, b3, v);
-        cartpole_finish(c, ahead, fmaf(-2.0f * a.action_scale, logistic2(v[0]), a.action_scale), s, sn, cs);
+        U::eight(w3, b, up, b3, v);
+        cartpole_finish(c, ahead, a.action_scale * kActInv * tanh_one(v[0]), s, sn, cs);
         if (step < traced && lane < nE)
             *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + lane) * a.trace_T + step) * 4) =
                 make_float4(s.x, s.xd, s.th, s.thd);

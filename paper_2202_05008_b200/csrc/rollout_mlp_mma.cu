@@ -70,7 +70,7 @@ __device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint3
         U::load(row + 32u * k, b);
         acc.add(tiles[k * 64u], tiles[k * 64u + 32u], b[0]);
     }
-    acc.sums(up, up * kLoInv, b0, b1, v);
+    acc.sums(up, b0, b1, v);
 }
 
 template <int EB, bool CART>
@@ -127,34 +127,25 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
             }
             for (uint32_t i = warp; i < p.mt[l] * p.kt[l]; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, sc, -2.0f * kF, hi, lo);
+                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, sc, kF, hi, lo);
                 tiles[(p.tile0[l] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[l] + i) * 64u + 32u + lane] = lo;
             }
-            for (uint32_t i = 8u * warp; i < p.mt[l] * 16u; i += blockDim.x / 4u) {
-                const float b = folded_bias(W, B, ni, no, static_cast<int>(i) + g, lane, sc);
-                if (t == 0) bias[p.bias0[l] + i + g] = b;
-            }
+            for (uint32_t i = tid; i < p.mt[l] * 16u; i += blockDim.x)
+                bias[p.bias0[l] + i] = static_cast<int>(i) < no ? kF * __ldg(B + i) : 0.f;
         }
-        if (!CART) {                                                 // x' = tanh(A x + B a), x = 1 - 2 r, a = s - 2 s r
+        if (!CART) {                                                 // x' = tanh(A x + B a)
             const Scale one(0u);
             const float* A = a.task_const;
             const float* Bm = a.task_const + kTlNx * kTlNx;
             for (uint32_t i = warp; i < 6u; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, one, -2.0f * kF, hi, lo);
-                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, one, -2.0f * kF * a.action_scale, hi, lo);
+                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, one, kF, hi, lo);
+                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, one, kF * a.action_scale, hi, lo);
                 tiles[(p.tile0[layers] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[layers] + i) * 64u + 32u + lane] = lo;
             }
-            for (uint32_t i = tid; i < 32u; i += blockDim.x) {
-                float sa = 0.f, sb = 0.f;
-                if (i < kTlNx) {
-                    for (uint32_t k = 0; k < kTlNx; ++k) sa += A[i * kTlNx + k];
-                    for (uint32_t k = 0; k < kTlNa; ++k) sb += Bm[i * kTlNa + k];
-                }
-                bias[p.bias0[layers] + i] = kF * fmaf(a.action_scale, sb, sa);
-            }
+            for (uint32_t i = tid; i < 32u; i += blockDim.x) bias[p.bias0[layers] + i] = 0.f;
             for (uint32_t i = tid; i < 2u * xbuf_bytes / 4u; i += blockDim.x)
                 reinterpret_cast<uint32_t*>(mma_smem + (xbuf - smem_u32(mma_smem)))[i] = 0u;
         }
@@ -188,7 +179,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                 const int e = EB == 4 ? t : 2 * t + (i & 1);
                 v[i] = row < kTlNx ? x0s[row][e] : 0.f;
                 if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
-                v[i] = fmaf(-0.5f, v[i], 0.5f);
+                v[i] *= kAct;
             }
             Units<EB>::store(Units<EB>::row(xbuf, kXPitch, lane) + 32u * m, v);
         }
@@ -223,9 +214,9 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                         }
                     } else {
                         const float* bb = bias + p.bias0[l] + 16u * m + g;
-                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], sc.up, v);
+                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], sc.up * kActInv, v);
                     }
-                    logistic_units<EB>(v);
+                    tanh_units<EB, Tanh::kFine>(v);
                     if (!last) {
                         Units<EB>::store(Units<EB>::row(out, p.pitch, lane) + 32u * m, v);
                     } else if (CART) {
@@ -237,7 +228,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                         Units<EB>::store(Units<EB>::row(xin, kXPitch, lane) + 64u, v);
 #pragma unroll
                         for (int i = 0; i < NV / 2; ++i) {
-                            const float act = fmaf(-2.0f * a.action_scale, v[i], a.action_scale);
+                            const float act = a.action_scale * kActInv * v[i];
                             if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
                         }
                     }
@@ -247,7 +238,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
         }
         if (CART) {
             if (!layer_warp) {
-                cartpole_finish(cpc, ahead, fmaf(-2.0f * a.action_scale, act[te], a.action_scale), cps, snc, csc);
+                cartpole_finish(cpc, ahead, a.action_scale * kActInv * act[te], cps, snc, csc);
                 ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
                 if (lane < EB) {
                     obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
@@ -260,11 +251,11 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
             for (uint32_t m = warp; m < 2u; m += nw) {
                 float v[NV];
                 unit_sums<EB>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane,
-                              bias[p.bias0[layers] + 16u * m + g], bias[p.bias0[layers] + 16u * m + g + 8u], 1.0f, v);
-                logistic_units<EB>(v);
+                              bias[p.bias0[layers] + 16u * m + g], bias[p.bias0[layers] + 16u * m + g + 8u], kActInv, v);
+                tanh_units<EB, Tanh::kFine>(v);
                 Units<EB>::store(Units<EB>::row(xout, kXPitch, lane) + 32u * m, v);
 #pragma unroll
-                for (int i = 0; i < NV; ++i) v[i] = fmaf(-2.0f, v[i], 1.0f);
+                for (int i = 0; i < NV; ++i) v[i] *= kActInv;
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
                     const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
