@@ -169,9 +169,10 @@ __device__ __forceinline__ CpState cartpole_step_fast(const CartpoleConst& c, co
 //     T = F + m l w^2 s       w' = q (g M s - c T)       M x'' = T - m l c w'
 // the angles of the first two Runge-Kutta stages are known without F (the second is half a step of the present
 // angular velocity on), and so are q and the products with s and c there.  The stages' velocities of the
-// cart cancel into x += h x' + h^2/6 (x1'' + x2'' + x3''), the same for the angle.
-struct CartpoleFast { float gm, ml, den0, den1, h, h2, w6, w6m, hh6, hh6m; };
-struct CpAhead { float n0, bq1, t01, mlc1, s2, c2, bq2, aq2, mls2, mlc2, th0, x0; };      // what the coming step knows without F
+// cart cancel into x += h (x' + h/6 (x1'' + x2'' + x3'')), the same for the angle: one rounding of the size of x.  (With
+// x + h x' taken ahead of the force there are two, and x and the angle were 1.5 times as far from the 64-bit ones.)
+struct CartpoleFast { float gm, ml, den0, den1, h, h2, w6, w6m; };
+struct CpAhead { float n0, bq1, t01, mlc1, s2, c2, bq2, aq2, mls2, mlc2; };      // what the coming step knows without F
 
 __device__ __forceinline__ CartpoleFast cartpole_fast_const(const float* tp)
 {
@@ -182,7 +183,6 @@ __device__ __forceinline__ CartpoleFast cartpole_fast_const(const float* tp)
     c.den0 = tp[EVO_CP_POLE_HALF_LENGTH] * (4.0f / 3.0f) * total;
     c.den1 = -c.ml;
     c.h = tp[EVO_CP_DT]; c.h2 = 0.5f * c.h; c.w6 = c.h * (1.0f / 6.0f); c.w6m = c.w6 / total;
-    c.hh6 = c.h * c.w6; c.hh6m = c.h * c.w6m;
     return c;
 }
 
@@ -222,8 +222,6 @@ __device__ __forceinline__ CpAhead cartpole_ahead(const CartpoleFast& c, const C
     p.aq2 = q2 * (c.gm * p.s2);
     p.mls2 = c.ml * p.s2;
     p.mlc2 = c.ml * p.c2;
-    p.th0 = fmaf(c.h, s.thd, s.th);
-    p.x0 = fmaf(c.h, s.xd, s.x);
     return p;
 }
 
@@ -252,8 +250,8 @@ __device__ __forceinline__ void cartpole_finish(const CartpoleFast& c, const CpA
     const float x3 = fmaf(-c.ml * c3, w3, t3);
     const float x4 = fmaf(-c.ml * c4, w4, t4);
     const float x23 = x2 + x3, w23 = w2 + w3;
-    s.th = fmaf(c.hh6, w1 + w23, p.th0);
-    s.x = fmaf(c.hh6m, x1 + x23, p.x0);
+    s.th = fmaf(c.h, fmaf(c.w6, w1 + w23, s.thd), s.th);
+    s.x = fmaf(c.h, fmaf(c.w6m, x1 + x23, s.xd), s.x);
     s.xd = fmaf(c.w6m, fmaf(2.0f, x23, x1 + x4), s.xd);
     s.thd = fmaf(c.w6, fmaf(2.0f, w23, w1 + w4), s.thd);
     const float kf = kr - kRound;

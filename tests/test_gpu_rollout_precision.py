@@ -30,7 +30,7 @@ def _traces(w, theta, T, kernel):
 
 @pytest.mark.parametrize("sizes,pop,episodes", [
     ((28, 128, 128, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 8), 64, 8), ((28, 64, 64, 64, 8), 64, 4),
-    ((28, 20, 8), 64, 8)])
+    ((28, 20, 8), 64, 8), ((5, 16, 16, 1), 64, 4), ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 8)])
 def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, pop, episodes):
     base, T = (W.CFG2, max(STEPS)) if sizes[0] == 5 else (W.CFG4, max(STEPS))
     # (the oracle computes with the task constants as fp32 numbers, which the kernels get)
