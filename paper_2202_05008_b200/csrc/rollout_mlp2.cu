@@ -100,12 +100,15 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     if (!fetch_row(a, status, &bar, &copy_ok, stage, row, RT == 1 ? a.ldD : static_cast<uint32_t>((w2_at + 3) & ~3), member, eb)) return;
     const uint32_t generation = status->generation;
     {
+        // (of the parameters only: what a caller's matrix has in its padding columns is nobody's)
         uint32_t most = 0;
-        const float4* all = reinterpret_cast<const float4*>(RT == 1 ? stage : row);
-        for (uint32_t i = tid; i < a.ldD / 4u; i += blockDim.x) {
-            const float4 w = all[i];
+        const float* all = RT == 1 ? stage : row;
+        const uint32_t n_params = static_cast<uint32_t>(w2_at + (n1 + 1) * n2 + (n2 + 1) * nout);
+        for (uint32_t i = tid; i < n_params / 4u; i += blockDim.x) {
+            const float4 w = reinterpret_cast<const float4*>(all)[i];
             most = max(max(most, max(finite_magnitude(w.x), finite_magnitude(w.y))), max(finite_magnitude(w.z), finite_magnitude(w.w)));
         }
+        if (tid < static_cast<int>(n_params & 3u)) most = max(most, finite_magnitude(all[(n_params & ~3u) + tid]));
         most = __reduce_max_sync(0xffffffffu, most);
         if (lane == 0) atomicMax(&peak, most);
         for (uint32_t i = tid; i < sizeof(h1) / 4u; i += blockDim.x) reinterpret_cast<uint32_t*>(h1)[i] = 0u;
@@ -431,7 +434,7 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
     dep_wait();
     if (!fetch_row(a, status, &bar, &copy_ok, stage, a.theta + static_cast<size_t>(member) * a.ldD, a.ldD, member, eb)) return;
     uint32_t most = 0;
-    for (uint32_t i = lane; i < a.ldD; i += 32u) most = max(most, finite_magnitude(stage[i]));
+    for (int i = lane; i < 6 * n1 + (n1 + 1) * n2 + n2 + 1; i += 32) most = max(most, finite_magnitude(stage[i]));      // (not the padding)
     const Scale sc(__reduce_max_sync(0xffffffffu, most));
     const float up = sc.up * kActInv;
     const uint32_t traced = a.trace ? a.trace_T : 0u;
