@@ -96,33 +96,33 @@ __device__ __forceinline__ void split_two(float a, float b, uint32_t& hi, uint32
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(neg_lo) : "f"(y), "f"(x));
 }
 
-// Weights beyond the fp16 range: a member that has any keeps all of its weights and biases times a power of two that
-// brings -2 f w of the largest finite one below it; p is multiplied back.  `peak` = the bit pattern of that
-// magnitude.  Infinities are taken as that magnitude (the tanh behind is saturated); NaN stays NaN.
-struct Scale {
-    float down, up, limit;
-    __device__ __forceinline__ explicit Scale(uint32_t peak)
-    {
-        const int e = static_cast<int>(peak >> 23) - 127, d = e <= 12 ? 0 : e - 12;
-        down = __uint_as_float(static_cast<uint32_t>(127 - d) << 23);
-        up = __uint_as_float(static_cast<uint32_t>(127 + d) << 23);
-        limit = __uint_as_float(max(peak, 0x46000000u));                 // 8,192 or the peak
-    }
-    __device__ __forceinline__ float weight(float w) const
-    {
-        asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(w) : "f"(-limit), "f"(limit));
-        return w;
-    }
-};
-__device__ __forceinline__ uint32_t finite_magnitude(float w)
+// Weights beyond the fp16 range: a unit that has any keeps its weights times 2^-n, which brings f w of the largest below it, and
+// its sums are multiplied back.  What the other weights lose is then below 2^-22 of the largest, as it is in the unit's
+// sum; other units, and the biases, are not touched.  The kernels look at a member's largest weight first: nearly always there is
+// nothing to scale, and a step then does without the units' factors.  Infinities count, and are taken, as the largest finite number (the tanh
+// behind them saturates); NaN stays NaN.
+__device__ __forceinline__ uint32_t magnitude(float w)                    // bit pattern
 {
     const uint32_t m = __float_as_uint(w) & 0x7FFFFFFFu;
-    return m < 0x7F800000u ? m : 0u;
+    return m > 0x7F800000u ? 0u : min(m, 0x7F7FFFFFu);
 }
-// k wa and k wb, a in the low half, with k2 = k kRest and the roundings of the products in the low parts
-__device__ __forceinline__ void split_weights(float wa, float wb, float k, float k2, uint32_t& hi, uint32_t& lo)
+__device__ __forceinline__ int scale_exponent(uint32_t peak)              // n: 0 for weights below 8,192
 {
-    const float a = wa * k, b = wb * k;
+    return max(static_cast<int>(peak >> 23) - (127 + 12), 0);
+}
+__device__ __forceinline__ float scale_down(int n) { return __uint_as_float(static_cast<uint32_t>(127 - n) << 23); }
+__device__ __forceinline__ float scale_up(int n) { return __uint_as_float(static_cast<uint32_t>(127 + n) << 23) * kActInv; }      // and the activations' scale
+__device__ __forceinline__ float finite(float w)
+{
+    asm("max.NaN.f32 %0, %0, %1;\n\tmin.NaN.f32 %0, %0, %2;" : "+f"(w) : "f"(-3.402823466e38f), "f"(3.402823466e38f));
+    return w;
+}
+// f x; a finite x stays finite
+__device__ __forceinline__ float times_f(float x) { return isinf(x) ? x : finite(kF * x); }
+// k wa and k wb, a in the low half, with kRest and the roundings of the products in the low parts
+__device__ __forceinline__ void split_weights(float wa, float wb, float k, uint32_t& hi, uint32_t& lo)
+{
+    const float a = wa * k, b = wb * k, k2 = k * kRest;
     const __half2 h = __floats2half2_rn(a, b);
     const float2 f = __half22float2(h);
     const float ra = fmaf(wa, k2, fmaf(wa, k, -a)), rb = fmaf(wb, k2, fmaf(wb, k, -b));
@@ -131,27 +131,52 @@ __device__ __forceinline__ void split_weights(float wa, float wb, float k, float
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// This lane's part of the 16x16 weight tile at (row0, col0) of a row-major [no][ni] matrix, times `factor`, as the A
-// operand; zeros outside the matrix.  `pairs`: ni is even and W 8-byte aligned.
-__device__ __forceinline__ void load_tile(const float* W, int ni, int no, int row0, int col0, int lane, const Scale& sc,
-                                          float factor, uint4& hi, uint4& lo, bool pairs = false)
+// This lane's part of a 16x16 tile at (row0, col0) of a row-major [no][ni] matrix: w[i] = columns 2t and 2t + 1 (i < 2) or
+// 2t + 8 and 2t + 9 of row g (i even) or g + 8; zeros outside the matrix.  `pairs`: ni is even and W 8-byte aligned.
+__device__ __forceinline__ void read_tile(const float* W, int ni, int no, int row0, int col0, int lane, bool pairs, float2 (&w)[4])
 {
     const int g = lane >> 2, t = lane & 3;
-    const float k = factor * sc.down;
-    uint32_t h[4], l[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {                       // rows g, g + 8; columns 2t, then 2t + 8
+    for (int i = 0; i < 4; ++i) {
         const int row = row0 + g + 8 * (i & 1), col = col0 + 2 * t + 8 * (i >> 1);
         const float* p = W + static_cast<size_t>(row) * ni + col;
-        float2 w = make_float2(0.f, 0.f);
+        w[i] = make_float2(0.f, 0.f);
         if (pairs) {
-            if (row < no && col < ni) w = *reinterpret_cast<const float2*>(p);
+            if (row < no && col < ni) w[i] = *reinterpret_cast<const float2*>(p);
         } else {
-            if (row < no && col < ni) w.x = p[0];
-            if (row < no && col + 1 < ni) w.y = p[1];
+            if (row < no && col < ni) w[i].x = p[0];
+            if (row < no && col + 1 < ni) w[i].y = p[1];
         }
-        split_weights(sc.weight(w.x), sc.weight(w.y), k, k * kRest, h[i], l[i]);
     }
+}
+// Exponents of rows g and g + 8 of the `kt` tiles from row0 on.
+__device__ __forceinline__ void row_exponents(const float* W, int ni, int no, int row0, int kt, int lane, int& n0, int& n1)
+{
+    uint32_t m0 = 0, m1 = 0;
+    for (int k = 0; k < kt; ++k) {
+        float2 w[4];
+        read_tile(W, ni, no, row0, 16 * k, lane, false, w);
+        m0 = max(max(m0, max(magnitude(w[0].x), magnitude(w[0].y))), max(magnitude(w[2].x), magnitude(w[2].y)));
+        m1 = max(max(m1, max(magnitude(w[1].x), magnitude(w[1].y))), max(magnitude(w[3].x), magnitude(w[3].y)));
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+        m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, off));
+        m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, off));
+    }
+    n0 = scale_exponent(m0);
+    n1 = scale_exponent(m1);
+}
+// A tile times f (and `times`) as the A operand; n0, n1: the exponents of rows g and g + 8.
+__device__ __forceinline__ void load_tile(const float* W, int ni, int no, int row0, int col0, int lane, int n0, int n1,
+                                          uint4& hi, uint4& lo, bool pairs = false, float times = 1.0f)
+{
+    float2 w[4];
+    read_tile(W, ni, no, row0, col0, lane, pairs, w);
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        split_weights(finite(times * w[i].x), finite(times * w[i].y), kF * scale_down(i & 1 ? n1 : n0), h[i], l[i]);
     hi = make_uint4(h[0], h[1], h[2], h[3]);
     lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
@@ -190,9 +215,10 @@ __device__ __forceinline__ void tanh_two(float& p, float& q)
     q = fmaf(kAct, d, -kAct) * a * r;
 }
 // With the Taylor polynomial to x^9 below |x| = 0.3, where what it leaves out is below 6e-8 of x.  For k_rollout_mlp_mma,
-// which also takes policies without a wide layer whose sums would hide the exponential's error near 1 (28-20-8: states 1.0
-// to 1.2 times as far from the 64-bit ones as with tanhf on the fp32 pipe, 0.8 to 0.95 with the polynomial; 28-64-64-64-8,
-// 512 members: 485 us a generation instead of 465).
+// which also takes policies with layers so narrow that their sums do not hide the exponential's error near 1.  State error
+// against that of tanhf on the fp32 pipe, after 1 / 20 / 200 steps: 28-20-8 without it 1.05 / 1.05 / 1.18, with it 0.95 / 0.82 / 0.92;
+// 28-64-10-10-8 without 1.04 / 1.12 / 1.16; 28-64-64-64-8 without 0.91 / 0.84 / 0.86.  It costs that last one 4 % (485 us a
+// generation of 512 members instead of 465), so a policy has it whose narrowest hidden layer is below 49 units.
 __device__ __forceinline__ float tanh_fine(float p)
 {
     constexpr double f = 2.885390081777927, g = 1.0 / (f * f);                // z = p^2 = x^2 / g
@@ -223,11 +249,11 @@ template <> struct Units<4> {
         mma_k16(h, wh, b[0], b[1]);
         mma_k16(l, wl, b[0], b[1]);
     }
-    // up = Scale::up / kAct, b0 and b1: f times the biases of units g and g + 8.  The small products are added up first.
-    __device__ __forceinline__ void sums(float up, float b0, float b1, float* v) const
+    // p of units g and g + 8: their scale_up, f times their biases.  The small products are added up first.
+    __device__ __forceinline__ void sums(float up0, float up1, float b0, float b1, float* v) const
     {
-        v[0] = fmaf(up, h[0], fmaf(up, fmaf(kLoInv, l[0] - l[1], -h[1]), b0));
-        v[1] = fmaf(up, h[2], fmaf(up, fmaf(kLoInv, l[2] - l[3], -h[3]), b1));
+        v[0] = fmaf(up0, h[0], fmaf(up0, fmaf(kLoInv, l[0] - l[1], -h[1]), b0));
+        v[1] = fmaf(up1, h[2], fmaf(up1, fmaf(kLoInv, l[2] - l[3], -h[3]), b1));
     }
     // eight outputs (hi parts of their weights in rows 0-7 of the tile, low parts in rows 8-15): output g
     static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float bias, float* v)
@@ -283,10 +309,13 @@ template <> struct Units<8> {
         mma_k16(hl, wh, b[2], b[3]);
         mma_k16(lh, wl, b[0], b[1]);
     }
-    __device__ __forceinline__ void sums(float up, float b0, float b1, float* v) const
+    __device__ __forceinline__ void sums(float up0, float up1, float b0, float b1, float* v) const
     {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = fmaf(up, hh[i], fmaf(up, fmaf(kLoInv, lh[i], -hl[i]), i < 2 ? b0 : b1));
+        for (int i = 0; i < 4; ++i) {
+            const float up = i < 2 ? up0 : up1;
+            v[i] = fmaf(up, hh[i], fmaf(up, fmaf(kLoInv, lh[i], -hl[i]), i < 2 ? b0 : b1));
+        }
     }
     static __device__ __forceinline__ void eight(const uint4& w, const uint32_t* b, float up, float bias, float* v)
     {

@@ -19,6 +19,8 @@
 #include "noise.cuh"
 #include "tasks.cuh"
 
+#include <type_traits>
+
 namespace evo {
 namespace {
 
@@ -77,6 +79,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     __shared__ uint4 dyn[CART ? 1 : kDynTiles * 64];                 // ... task matrices in operand order
     __shared__ float x0s[CART ? 1 : kTlNx][EB];                      // ... start states
     __shared__ float rets[2][EB];
+    __shared__ float ups[2 * 16 * MW * RT + 8];                      // scale_up of the units of both hidden layers, then of the actions
 
     // (the shuffle tells the compiler that the warp number is the same in all lanes)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -106,9 +109,9 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         const uint32_t n_params = static_cast<uint32_t>(w2_at + (n1 + 1) * n2 + (n2 + 1) * nout);
         for (uint32_t i = tid; i < n_params / 4u; i += blockDim.x) {
             const float4 w = reinterpret_cast<const float4*>(all)[i];
-            most = max(max(most, max(finite_magnitude(w.x), finite_magnitude(w.y))), max(finite_magnitude(w.z), finite_magnitude(w.w)));
+            most = max(max(most, max(magnitude(w.x), magnitude(w.y))), max(magnitude(w.z), magnitude(w.w)));
         }
-        if (tid < static_cast<int>(n_params & 3u)) most = max(most, finite_magnitude(all[(n_params & ~3u) + tid]));
+        if (tid < static_cast<int>(n_params & 3u)) most = max(most, magnitude(all[(n_params & ~3u) + tid]));
         most = __reduce_max_sync(0xffffffffu, most);
         if (lane == 0) atomicMax(&peak, most);
         for (uint32_t i = tid; i < sizeof(h1) / 4u; i += blockDim.x) reinterpret_cast<uint32_t*>(h1)[i] = 0u;
@@ -116,8 +119,8 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         else for (uint32_t i = tid; i < sizeof(part_t) / 4u; i += blockDim.x) (&part_t[0][0])[i] = 0.f;
         __syncthreads();
     }
-    const Scale sc(peak);
-    const float up = sc.up * kActInv;
+    const int most = scale_exponent(peak);
+    const bool scaled = most != 0;
 
     // ---- weights into registers, times f (see mma_split.cuh) ---------------------------------------
     const float* W1 = stage;
@@ -130,49 +133,61 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     uint4 w2h[RT][KT], w2l[RT == 1 ? KT : 1];
     uint4 w1h[CART ? 1 : RT][2], w1l[CART ? 1 : RT][2], w3[CART ? 1 : RT];           // w3: the action layer's own inputs (see Units::eight)
     float w1c[CART ? RT : 1][10], w3c[RT][2], b1[RT][2], b2[RT][2], b3;
+    float* const ups1 = ups + 16 * tile0 + g, *const ups2 = ups1 + 16 * MW * RT, *const ups3 = ups + 2 * 16 * MW * RT + g;
     uint4* const w2l_s = reinterpret_cast<uint4*>(stage) + warp * (RT * KT * 32) + lane;
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
         const int tile = tile0 + r, u0 = 16 * tile + g, u1 = u0 + 8;              // this lane's two units
-        b2[r][0] = u0 < n2 ? kF * B2[u0] : 0.f; b2[r][1] = u1 < n2 ? kF * B2[u1] : 0.f;
-        b1[r][0] = u0 < n1 ? kF * B1[u0] : 0.f; b1[r][1] = u1 < n1 ? kF * B1[u1] : 0.f;
+        b2[r][0] = u0 < n2 ? times_f(B2[u0]) : 0.f; b2[r][1] = u1 < n2 ? times_f(B2[u1]) : 0.f;
+        b1[r][0] = u0 < n1 ? times_f(B1[u0]) : 0.f; b1[r][1] = u1 < n1 ? times_f(B1[u1]) : 0.f;
         if constexpr (CART) {                                        // the observation is taken as it is, in fp32
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                w1c[r][k] = u0 < n1 ? kF * W1[u0 * 5 + k] : 0.f;
-                w1c[r][5 + k] = u1 < n1 ? kF * W1[u1 * 5 + k] : 0.f;
+                w1c[r][k] = u0 < n1 ? times_f(W1[u0 * 5 + k]) : 0.f;
+                w1c[r][5 + k] = u1 < n1 ? times_f(W1[u1 * 5 + k]) : 0.f;
             }
             w3c[r][0] = u0 < n2 ? kF * kActInv * W3[u0] : 0.f; w3c[r][1] = u1 < n2 ? kF * kActInv * W3[u1] : 0.f;
         } else {
+            int s0 = 0, s1 = 0, s3 = 0, none;
+            if (scaled) {
+                row_exponents(W1, nin, n1, 16 * tile, 2, lane, s0, s1);
+                row_exponents(W3, n2, nout, 0, mt2, lane, s3, none);
+                ups1[16 * r] = scale_up(s0); ups1[16 * r + 8] = scale_up(s1); ups3[0] = scale_up(s3);
+            }
 #pragma unroll
-            for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, sc, kF, w1h[r][k], w1l[r][k]);
+            for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, s0, s1, w1h[r][k], w1l[r][k]);
             uint4 lo3;
-            load_tile(W3, n2, nout, 0, 16 * tile, lane, sc, kF, w3[r], lo3);
+            load_tile(W3, n2, nout, 0, 16 * tile, lane, s3, 0, w3[r], lo3);
             w3[r].y = lo3.x; w3[r].w = lo3.z;
         }
     }
     if constexpr (RT > 1) __syncthreads();                           // every warp has read the first layer out of `stage`
 #pragma unroll
-    for (int r = 0; r < RT; ++r)
+    for (int r = 0; r < RT; ++r) {
+        int s0 = 0, s1 = 0;
+        if (scaled) {
+            row_exponents(W2, n1, n2, 16 * (tile0 + r), KT, lane, s0, s1);
+            ups2[16 * r] = scale_up(s0); ups2[16 * r + 8] = scale_up(s1);
+        }
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             uint4 lo;
-            load_tile(W2, n1, n2, 16 * (tile0 + r), 16 * k, lane, sc, kF, w2h[r][k], lo, pairs);
+            load_tile(W2, n1, n2, 16 * (tile0 + r), 16 * k, lane, s0, s1, w2h[r][k], lo, pairs);
             if constexpr (RT == 1) w2l[k] = lo;
             else w2l_s[32 * (r * KT + k)] = lo;
         }
+    }
     if constexpr (CART) {
-        b3 = kF * B3[0];
+        b3 = times_f(B3[0]);
     } else {
-        b3 = kF * B3[g];
+        b3 = times_f(B3[g]);
         // x' = tanh(A x + B a)
-        const Scale one(0u);
         const float* A = a.task_const;
         const float* Bm = a.task_const + kTlNx * kTlNx;
         for (int i = warp; i < static_cast<int>(kDynTiles); i += nw) {
             uint4 hi, lo;
-            if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, 16 * (i / 3), 16 * (i % 3), lane, one, kF, hi, lo);
-            else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3), 0, lane, one, kF * a.action_scale, hi, lo);
+            if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, 16 * (i / 3), 16 * (i % 3), lane, 0, 0, hi, lo);
+            else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3), 0, lane, 0, 0, hi, lo, false, a.action_scale);
             dyn[i * 64 + lane] = hi;
             dyn[i * 64 + 32 + lane] = lo;
         }
@@ -218,181 +233,189 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 
     // ---- time loop ------------------------------------------------------------------------------------------
     uint32_t xin = x_row, xout = x_row + kXBytes;
-    for (uint32_t step = 0; step < a.T; ++step) {
-        if (tile0 < mt1) {
-            float v[RT][NV];
-            if constexpr (CART) {
-                float o[5][NH];
+    // (kActInv where nothing is scaled, but as a constant it becomes immediate operands: 28-128-128-8, 4,096 members then take 12.1 us
+    // a step, and 11.5 us with a register)
+    const float up = scale_up(most);
+    auto roll = [&](auto with_scales) {
+        constexpr bool kScaled = decltype(with_scales)::value;
+        for (uint32_t step = 0; step < a.T; ++step) {
+            if (tile0 < mt1) {
+                float v[RT][NV];
+                if constexpr (CART) {
+                    float o[5][NH];
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    if constexpr (EB == 4) o[k][0] = obs[k][t];
-                    else { const float2 q = *reinterpret_cast<const float2*>(&obs[k][2 * t]); o[k][0] = q.x; o[k][1] = q.y; }
+                    for (int k = 0; k < 5; ++k) {
+                        if constexpr (EB == 4) o[k][0] = obs[k][t];
+                        else { const float2 q = *reinterpret_cast<const float2*>(&obs[k][2 * t]); o[k][0] = q.x; o[k][1] = q.y; }
+                    }
+#pragma unroll
+                    for (int r = 0; r < RT; ++r)
+#pragma unroll
+                        for (int i = 0; i < NV; ++i) {
+                            float s = b1[r][i / NH];
+#pragma unroll
+                            for (int k = 0; k < 5; ++k) s = fmaf(w1c[r][5 * (i / NH) + k], o[k][i % NH], s);
+                            v[r][i] = s;
+                        }
+                } else {
+                    U acc[RT];
+                    uint32_t b[2][4];
+                    U::load(xin, b);
+                    if (U::kLoadTiles == 1) U::load(xin + 32u, b + 1);
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) acc[r].first(w1h[r][0], w1l[r][0], b[0]);
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) acc[r].add(w1h[r][1], w1l[r][1], b[1]);
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) acc[r].sums(kScaled ? ups1[16 * r] : up, kScaled ? ups1[16 * r + 8] : up, b1[r][0], b1[r][1], v[r]);
                 }
 #pragma unroll
-                for (int r = 0; r < RT; ++r)
+                for (int r = 0; r < RT; ++r) {
+                    tanh_units<EB, kTanh>(v[r]);
+                    if (RT == 1 || tile0 + r < KT) U::store(h1_row + 32u * (tile0 + r), v[r]);
+                }
+            }
+            __syncthreads();
+            CpAhead ahead;
+            {
+                U acc[RT];
+                if (tile0 < mt2) {
+                    uint32_t b[2][2][4];                                 // the operands of two tiles, those of the next two on their way
+                    U::load(h1_row, b[0]);
+                    if (U::kLoadTiles == 1 && KT > 1) U::load(h1_row + 32u, b[0] + 1);
+#pragma unroll
+                    for (int k = 0; k < KT; ++k) {
+                        uint32_t (&now)[2][4] = b[(k >> 1) & 1], (&next)[2][4] = b[((k >> 1) + 1) & 1];
+                        if (!(k & 1) && k + 2 < KT) {
+                            U::load(h1_row + 32u * k + 64u, next);
+                            if (U::kLoadTiles == 1 && k + 3 < KT) U::load(h1_row + 32u * k + 96u, next + 1);
+                        }
+#pragma unroll
+                        for (int r = 0; r < RT; ++r) {
+                            const uint4 lo = RT == 1 ? w2l[RT == 1 ? k : 0] : w2l_s[32 * (r * KT + k)];
+                            if (k == 0) acc[r].first(w2h[r][k], lo, now[0]);
+                            else acc[r].add(w2h[r][k], lo, now[k & 1]);
+                        }
+                    }
+                }
+                if (!CART) {                                             // under the MMAs: reward on the pre-step state (0 in other warps, padding rows)
 #pragma unroll
                     for (int i = 0; i < NV; ++i) {
-                        float s = b1[r][i / NH];
-#pragma unroll
-                        for (int k = 0; k < 5; ++k) s = fmaf(w1c[r][5 * (i / NH) + k], o[k][i % NH], s);
-                        v[r][i] = s;
+                        if (EB == 4 || !(i & 1)) ret = fmaf(-xcur[i], xcur[i], ret); else ret2 = fmaf(-xcur[i], xcur[i], ret2);
                     }
-            } else {
-                U acc[RT];
+                } else if (tw) {
+                    ahead = cartpole_ahead(cpc, cps, snc, csc);
+                    if (step > 0u) ret = fmaf(csc, __expf(-cps.x * cps.x), ret);        // reward of the step before, on its post-step state
+                }
+                if (tile0 < mt2) {
+                    float v[RT][NV];
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) {
+                        acc[r].sums(kScaled ? ups2[16 * r] : up, kScaled ? ups2[16 * r + 8] : up, b2[r][0], b2[r][1], v[r]);
+                        tanh_units<EB, kTanh>(v[r]);
+                    }
+                    if constexpr (CART) {
+                        float p[NH];
+#pragma unroll
+                        for (int i = 0; i < NH; ++i) {
+                            p[i] = fmaf(w3c[0][1], v[0][NH + i], w3c[0][0] * v[0][i]);
+                            if constexpr (RT == 2) p[i] = fmaf(w3c[RT - 1][1], v[RT - 1][NH + i], fmaf(w3c[RT - 1][0], v[RT - 1][i], p[i]));
+                        }
+                        if constexpr (EB == 4) part_c[warp][lane] = p[0];
+                        else *reinterpret_cast<float2*>(&part_c[warp][2 * lane]) = make_float2(p[0], p[1]);
+                    } else {                                             // the action layer's share of the warp's units
+                        uint32_t b[RT][4];
+                        float p[RT][2];
+#pragma unroll
+                        for (int r = 0; r < RT; ++r) U::transpose(v[r], b[r]);
+#pragma unroll
+                        for (int r = 0; r < RT; ++r) U::eight(w3[r], b[r], kScaled ? ups3[0] : up, 0.f, p[r]);
+                        if constexpr (RT == 2) { p[0][0] += p[RT - 1][0]; p[0][1] += p[RT - 1][1]; }
+                        if constexpr (EB == 4) part_t[warp][lane] = p[0][0];
+                        else *reinterpret_cast<float2*>(&part_t[warp][2 * lane]) = make_float2(p[0][0], p[0][1]);
+                    }
+                }
+            }
+            __syncthreads();
+            if constexpr (CART) {
+                if (tw) {
+                    // the shares of episode te, [warp][g]: this lane adds a quarter (an eighth) of them
+                    float p[EB];
+#pragma unroll
+                    for (int i = 0; i < EB; ++i) p[i] = (&part_c[0][0])[lane + 32 * i];
+                    if constexpr (MW > 4) {
+#pragma unroll
+                        for (int i = 0; i < EB; ++i) p[i] += (&part_c[MW - 4][0])[lane + 32 * i];
+                    }
+#pragma unroll
+                    for (int n = EB / 2; n > 0; n >>= 1)
+#pragma unroll
+                        for (int i = 0; i < n; ++i) p[i] += p[i + n];
+                    float pre = p[0];
+#pragma unroll
+                    for (int off = EB; off < 32; off <<= 1) pre += __shfl_xor_sync(0xffffffffu, pre, off);
+                    const float force = a.action_scale * kActInv * tanh_one(pre + b3);
+                    cartpole_finish(cpc, ahead, force, cps, snc, csc);
+                    if (lane < EB) { obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd; }
+                    if (step < traced && lane < nE)
+                        *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
+                            make_float4(cps.x, cps.xd, cps.th, cps.thd);
+                }
+            } else if (tw) {                                              // action (in both warps), then x' = tanh(A x + B a)
+                float v[NV], p[4][NH];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    if constexpr (EB == 4) p[w][0] = part_t[w][lane];
+                    else { const float2 q = *reinterpret_cast<const float2*>(&part_t[w][2 * lane]); p[w][0] = q.x; p[w][1] = q.y; }
+                }
+                if constexpr (MW > 4) {
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) {
+                        if constexpr (EB == 4) p[w][0] += part_t[MW - 4 + w][lane];
+                        else { const float2 q = *reinterpret_cast<const float2*>(&part_t[MW - 4 + w][2 * lane]); p[w][0] += q.x; p[w][1] += q.y; }
+                    }
+                }
+                U acc;
+                const uint4* tiles = dyn + 192 * warp + lane;
                 uint32_t b[2][4];
                 U::load(xin, b);
                 if (U::kLoadTiles == 1) U::load(xin + 32u, b + 1);
+                acc.first(tiles[0], tiles[32], b[0]);
+                acc.add(tiles[64], tiles[96], b[1]);
 #pragma unroll
-                for (int r = 0; r < RT; ++r) acc[r].first(w1h[r][0], w1l[r][0], b[0]);
-#pragma unroll
-                for (int r = 0; r < RT; ++r) acc[r].add(w1h[r][1], w1l[r][1], b[1]);
-#pragma unroll
-                for (int r = 0; r < RT; ++r) acc[r].sums(up, b1[r][0], b1[r][1], v[r]);
-            }
-#pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                tanh_units<EB, kTanh>(v[r]);
-                if (RT == 1 || tile0 + r < KT) U::store(h1_row + 32u * (tile0 + r), v[r]);
-            }
-        }
-        __syncthreads();
-        CpAhead ahead;
-        {
-            U acc[RT];
-            if (tile0 < mt2) {
-                uint32_t b[2][2][4];                                 // the operands of two tiles, those of the next two on their way
-                U::load(h1_row, b[0]);
-                if (U::kLoadTiles == 1 && KT > 1) U::load(h1_row + 32u, b[0] + 1);
-#pragma unroll
-                for (int k = 0; k < KT; ++k) {
-                    uint32_t (&now)[2][4] = b[(k >> 1) & 1], (&next)[2][4] = b[((k >> 1) + 1) & 1];
-                    if (!(k & 1) && k + 2 < KT) {
-                        U::load(h1_row + 32u * k + 64u, next);
-                        if (U::kLoadTiles == 1 && k + 3 < KT) U::load(h1_row + 32u * k + 96u, next + 1);
-                    }
-#pragma unroll
-                    for (int r = 0; r < RT; ++r) {
-                        const uint4 lo = RT == 1 ? w2l[RT == 1 ? k : 0] : w2l_s[32 * (r * KT + k)];
-                        if (k == 0) acc[r].first(w2h[r][k], lo, now[0]);
-                        else acc[r].add(w2h[r][k], lo, now[k & 1]);
-                    }
-                }
-            }
-            if (!CART) {                                             // under the MMAs: reward on the pre-step state (0 in other warps, padding rows)
-#pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    if (EB == 4 || !(i & 1)) ret = fmaf(-xcur[i], xcur[i], ret); else ret2 = fmaf(-xcur[i], xcur[i], ret2);
-                }
-            } else if (tw) {
-                ahead = cartpole_ahead(cpc, cps, snc, csc);
-                if (step > 0u) ret = fmaf(csc, __expf(-cps.x * cps.x), ret);        // reward of the step before, on its post-step state
-            }
-            if (tile0 < mt2) {
-                float v[RT][NV];
-#pragma unroll
-                for (int r = 0; r < RT; ++r) {
-                    acc[r].sums(up, b2[r][0], b2[r][1], v[r]);
-                    tanh_units<EB, kTanh>(v[r]);
-                }
-                if constexpr (CART) {
-                    float p[NH];
+                for (int i = 0; i < NH; ++i) v[i] = tanh_one(((p[0][i] + p[1][i]) + (p[2][i] + p[3][i])) + b3);
+                uint32_t hi, lo;
+                split_two(v[0], EB == 4 ? 0.f : v[NH - 1], hi, lo);
+                if constexpr (EB == 4) { b[0][0] = transpose8(__byte_perm(hi, lo, 0x5410)); b[0][1] = 0u; }
+                else { b[0][0] = transpose8(hi); b[0][1] = 0u; b[0][2] = transpose8(lo); b[0][3] = 0u; }
+                if (warp == 0) {                                      // the action's share of the reward
 #pragma unroll
                     for (int i = 0; i < NH; ++i) {
-                        p[i] = fmaf(w3c[0][1], v[0][NH + i], w3c[0][0] * v[0][i]);
-                        if constexpr (RT == 2) p[i] = fmaf(w3c[RT - 1][1], v[RT - 1][NH + i], fmaf(w3c[RT - 1][0], v[RT - 1][i], p[i]));
+                        const float act = a.action_scale * kActInv * v[i];
+                        if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
                     }
-                    if constexpr (EB == 4) part_c[warp][lane] = p[0];
-                    else *reinterpret_cast<float2*>(&part_c[warp][2 * lane]) = make_float2(p[0], p[1]);
-                } else {                                             // the action layer's share of the warp's units
-                    uint32_t b[RT][4];
-                    float p[RT][2];
+                }
+                acc.add(tiles[128], tiles[160], b[0]);
+                acc.sums(kActInv, kActInv, 0.f, 0.f, v);
+                tanh_units<EB, kTanh>(v);
+                U::store(xout + 32u * warp, v);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) U::transpose(v[r], b[r]);
+                for (int i = 0; i < NV; ++i) xcur[i] = kActInv * v[i];              // padding rows: p = 0, exactly 0
+                if (step < traced) {
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) U::eight(w3[r], b[r], up, 0.f, p[r]);
-                    if constexpr (RT == 2) { p[0][0] += p[RT - 1][0]; p[0][1] += p[RT - 1][1]; }
-                    if constexpr (EB == 4) part_t[warp][lane] = p[0][0];
-                    else *reinterpret_cast<float2*>(&part_t[warp][2 * lane]) = make_float2(p[0][0], p[0][1]);
+                    for (int i = 0; i < NV; ++i) {
+                        const int unit = 16 * warp + g + (i >= NH ? 8 : 0), e = U::episode(i, t);
+                        if (e < nE && unit < static_cast<int>(kTlNx))
+                            a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + unit] = xcur[i];
+                    }
                 }
             }
+            const uint32_t x = xin; xin = xout; xout = x;
+            __syncthreads();
         }
-        __syncthreads();
-        if constexpr (CART) {
-            if (tw) {
-                // the shares of episode te, [warp][g]: this lane adds a quarter (an eighth) of them
-                float p[EB];
-#pragma unroll
-                for (int i = 0; i < EB; ++i) p[i] = (&part_c[0][0])[lane + 32 * i];
-                if constexpr (MW > 4) {
-#pragma unroll
-                    for (int i = 0; i < EB; ++i) p[i] += (&part_c[MW - 4][0])[lane + 32 * i];
-                }
-#pragma unroll
-                for (int n = EB / 2; n > 0; n >>= 1)
-#pragma unroll
-                    for (int i = 0; i < n; ++i) p[i] += p[i + n];
-                float pre = p[0];
-#pragma unroll
-                for (int off = EB; off < 32; off <<= 1) pre += __shfl_xor_sync(0xffffffffu, pre, off);
-                const float force = a.action_scale * kActInv * tanh_one(pre + b3);
-                cartpole_finish(cpc, ahead, force, cps, snc, csc);
-                if (lane < EB) { obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd; }
-                if (step < traced && lane < nE)
-                    *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
-                        make_float4(cps.x, cps.xd, cps.th, cps.thd);
-            }
-        } else if (tw) {                                              // action (in both warps), then x' = tanh(A x + B a)
-            float v[NV], p[4][NH];
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                if constexpr (EB == 4) p[w][0] = part_t[w][lane];
-                else { const float2 q = *reinterpret_cast<const float2*>(&part_t[w][2 * lane]); p[w][0] = q.x; p[w][1] = q.y; }
-            }
-            if constexpr (MW > 4) {
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    if constexpr (EB == 4) p[w][0] += part_t[MW - 4 + w][lane];
-                    else { const float2 q = *reinterpret_cast<const float2*>(&part_t[MW - 4 + w][2 * lane]); p[w][0] += q.x; p[w][1] += q.y; }
-                }
-            }
-            U acc;
-            const uint4* tiles = dyn + 192 * warp + lane;
-            uint32_t b[2][4];
-            U::load(xin, b);
-            if (U::kLoadTiles == 1) U::load(xin + 32u, b + 1);
-            acc.first(tiles[0], tiles[32], b[0]);
-            acc.add(tiles[64], tiles[96], b[1]);
-#pragma unroll
-            for (int i = 0; i < NH; ++i) v[i] = tanh_one(((p[0][i] + p[1][i]) + (p[2][i] + p[3][i])) + b3);
-            uint32_t hi, lo;
-            split_two(v[0], EB == 4 ? 0.f : v[NH - 1], hi, lo);
-            if constexpr (EB == 4) { b[0][0] = transpose8(__byte_perm(hi, lo, 0x5410)); b[0][1] = 0u; }
-            else { b[0][0] = transpose8(hi); b[0][1] = 0u; b[0][2] = transpose8(lo); b[0][3] = 0u; }
-            if (warp == 0) {                                      // the action's share of the reward
-#pragma unroll
-                for (int i = 0; i < NH; ++i) {
-                    const float act = a.action_scale * kActInv * v[i];
-                    if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
-                }
-            }
-            acc.add(tiles[128], tiles[160], b[0]);
-            acc.sums(kActInv, 0.f, 0.f, v);
-            tanh_units<EB, kTanh>(v);
-            U::store(xout + 32u * warp, v);
-#pragma unroll
-            for (int i = 0; i < NV; ++i) xcur[i] = kActInv * v[i];              // padding rows: p = 0, exactly 0
-            if (step < traced) {
-#pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    const int unit = 16 * warp + g + (i >= NH ? 8 : 0), e = U::episode(i, t);
-                    if (e < nE && unit < static_cast<int>(kTlNx))
-                        a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + unit] = xcur[i];
-                }
-            }
-        }
-        const uint32_t x = xin; xin = xout; xout = x;
-        __syncthreads();
-    }
+    };
+    if (!scaled) roll(std::false_type{});
+    else roll(std::true_type{});
 
     // ---- block return: fixed order ----------------------------------------------------------------------------
     if constexpr (CART) {
@@ -434,9 +457,8 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
     dep_wait();
     if (!fetch_row(a, status, &bar, &copy_ok, stage, a.theta + static_cast<size_t>(member) * a.ldD, a.ldD, member, eb)) return;
     uint32_t most = 0;
-    for (int i = lane; i < 6 * n1 + (n1 + 1) * n2 + n2 + 1; i += 32) most = max(most, finite_magnitude(stage[i]));      // (not the padding)
-    const Scale sc(__reduce_max_sync(0xffffffffu, most));
-    const float up = sc.up * kActInv;
+    for (int i = lane; i < 6 * n1 + (n1 + 1) * n2 + n2 + 1; i += 32) most = max(most, magnitude(stage[i]));      // (not the padding)
+    const bool scaled = scale_exponent(__reduce_max_sync(0xffffffffu, most)) != 0;
     const uint32_t traced = a.trace ? a.trace_T : 0u;
 
     const float* W1 = stage;
@@ -449,53 +471,62 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
     for (int i = 0; i < 2; ++i) {
         const int u = g + 8 * i;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) w1[i][k] = u < n1 ? kF * W1[u * 5 + k] : 0.f;
-        w1[i][5] = u < n1 ? kF * B1[u] : 0.f;
-        b2[i] = u < n2 ? kF * B2[u] : 0.f;
+        for (int k = 0; k < 5; ++k) w1[i][k] = u < n1 ? times_f(W1[u * 5 + k]) : 0.f;
+        w1[i][5] = u < n1 ? times_f(B1[u]) : 0.f;
+        b2[i] = u < n2 ? times_f(B2[u]) : 0.f;
     }
     uint4 w2h, w2l;
-    load_tile(W2, n1, n2, 0, 0, lane, sc, kF, w2h, w2l);
+    int s0 = 0, s1 = 0, s3 = 0;
+    if (scaled) {
+        row_exponents(W2, n1, n2, 0, 1, lane, s0, s1);
+        s3 = scale_exponent(__reduce_max_sync(0xffffffffu, lane < n2 ? magnitude(W3[lane]) : 0u));
+    }
+    load_tile(W2, n1, n2, 0, 0, lane, s0, s1, w2h, w2l);
     uint32_t w3h[2], w3l[2];
-    const float f = kF * sc.down;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int col = 2 * t + 8 * k;
-        split_weights(col < n2 ? sc.weight(W3[col]) : 0.f, col + 1 < n2 ? sc.weight(W3[col + 1]) : 0.f, f, f * kRest, w3h[k], w3l[k]);
+        split_weights(col < n2 ? finite(W3[col]) : 0.f, col + 1 < n2 ? finite(W3[col + 1]) : 0.f, kF * scale_down(s3), w3h[k], w3l[k]);
     }
     const uint4 w3 = make_uint4(w3h[0], w3l[0], w3h[1], w3l[1]);        // the one output in every row (see Units::eight)
-    const float b3 = kF * W3[n2];
+    const float b3 = times_f(W3[n2]);
 
     const CartpoleFast c = cartpole_fast_const(a.tp);
     CpState s = cartpole_reset(key, status->generation, e0 + min(t, nE - 1), a.tp[EVO_CP_INIT_RANGE]);
     float sn, cs, ret = 0.f;
     sincos_fast(s.th, sn, cs);
 
-    for (uint32_t step = 0; step < a.T; ++step) {
-        float v[2];
-        uint32_t b[2];
+    auto roll = [&](auto with_scales) {
+        constexpr bool kScaled = decltype(with_scales)::value;
+        for (uint32_t step = 0; step < a.T; ++step) {
+            float v[2];
+            uint32_t b[2];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            // the velocity and the angle come last out of a step, so they go in last here
-            float p = fmaf(w1[i][0], s.x, w1[i][5]);
-            p = fmaf(w1[i][1], s.xd, p);
-            p = fmaf(w1[i][4], s.thd, p);
-            p = fmaf(w1[i][3], sn, p);
-            v[i] = tanh_one(fmaf(w1[i][2], cs, p));
+            for (int i = 0; i < 2; ++i) {
+                // the velocity and the angle come last out of a step, so they go in last here
+                float p = fmaf(w1[i][0], s.x, w1[i][5]);
+                p = fmaf(w1[i][1], s.xd, p);
+                p = fmaf(w1[i][4], s.thd, p);
+                p = fmaf(w1[i][3], sn, p);
+                v[i] = tanh_one(fmaf(w1[i][2], cs, p));
+            }
+            U::transpose(v, b);
+            U h2;
+            h2.first(w2h, w2l, b);
+            const CpAhead ahead = cartpole_ahead(c, s, sn, cs);
+            if (step > 0u) ret = fmaf(cs, __expf(-s.x * s.x), ret);       // reward of the step before, on its post-step state
+            h2.sums(kScaled ? scale_up(s0) : kActInv, kScaled ? scale_up(s1) : kActInv, b2[0], b2[1], v);
+            v[0] = tanh_one(v[0]); v[1] = tanh_one(v[1]);                 // a reciprocal each: the unit is idle, the chain shorter
+            U::transpose(v, b);
+            U::eight(w3, b, kScaled ? scale_up(s3) : kActInv, b3, v);
+            cartpole_finish(c, ahead, a.action_scale * kActInv * tanh_one(v[0]), s, sn, cs);
+            if (step < traced && lane < nE)
+                *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + lane) * a.trace_T + step) * 4) =
+                    make_float4(s.x, s.xd, s.th, s.thd);
         }
-        U::transpose(v, b);
-        U h2;
-        h2.first(w2h, w2l, b);
-        const CpAhead ahead = cartpole_ahead(c, s, sn, cs);
-        if (step > 0u) ret = fmaf(cs, __expf(-s.x * s.x), ret);       // reward of the step before, on its post-step state
-        h2.sums(up, b2[0], b2[1], v);
-        v[0] = tanh_one(v[0]); v[1] = tanh_one(v[1]);                 // a reciprocal each: the unit is idle, the chain shorter
-        U::transpose(v, b);
-        U::eight(w3, b, up, b3, v);
-        cartpole_finish(c, ahead, a.action_scale * kActInv * tanh_one(v[0]), s, sn, cs);
-        if (step < traced && lane < nE)
-            *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + lane) * a.trace_T + step) * 4) =
-                make_float4(s.x, s.xd, s.th, s.thd);
-    }
+    };
+    if (scaled) roll(std::true_type{});
+    else roll(std::false_type{});
     ret = fmaf(cs, __expf(-s.x * s.x), ret);
     float v = t < nE ? ret : 0.f;
     v += __shfl_xor_sync(0xffffffffu, v, 1);

@@ -20,13 +20,15 @@
 #include "noise.cuh"
 #include "tasks.cuh"
 
+#include <type_traits>
+
 namespace evo {
 namespace {
 
 using namespace ms;
 
 constexpr uint32_t kXPitch = 48 * 2 + 16;           // bytes per column of the [x 28 | 0 4 | a 8 | 0 8] operand
-constexpr size_t kMaxSmem = 220u * 1024u;
+constexpr size_t kMaxSmem = 222u * 1024u;
 
 struct Plan {
     uint32_t mt[EVO_MAX_LAYERS + 1], kt[EVO_MAX_LAYERS + 1];   // 16-unit and 16-input tiles of a layer; last entry: dynamics
@@ -34,13 +36,14 @@ struct Plan {
     uint32_t bias0[EVO_MAX_LAYERS + 1];             // first float of a layer's biases
     uint32_t tiles, biases, pitch;                  // pitch: bytes per column of the hidden operands
     uint32_t warps;                                 // layer warps
+    bool     fine;                                  // tanh with the polynomial (see tanh_fine)
     size_t   smem;
 };
 
-// p of 16 units: tiles = the units' weight tiles in operand order, b0/b1 their biases (units g, g + 8)
-template <int EB>
-__device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint32_t in, uint32_t pitch, int lane, float b0,
-                                          float b1, float up, float* v)
+// p of 16 units: tiles = the units' weight tiles in operand order, bias and (SCALED) exponent of units g and g + 8, up = kActInv
+template <int EB, bool SCALED>
+__device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint32_t in, uint32_t pitch, int lane, float b0, float b1,
+                                          const uint8_t* exponent, float up, float* v)
 {
     using U = Units<EB>;
     U acc;
@@ -70,10 +73,10 @@ __device__ __forceinline__ void unit_sums(const uint4* tiles, uint32_t kt, uint3
         U::load(row + 32u * k, b);
         acc.add(tiles[k * 64u], tiles[k * 64u + 32u], b[0]);
     }
-    acc.sums(up, b0, b1, v);
+    acc.sums(SCALED ? scale_up(exponent[0]) : up, SCALED ? scale_up(exponent[8]) : up, b0, b1, v);
 }
 
-template <int EB, bool CART>
+template <int EB, bool CART, bool FINE>
 __global__ void __launch_bounds__(288)
 k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
 {
@@ -83,7 +86,8 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     __shared__ uint32_t peaks[9];
     uint4* tiles = reinterpret_cast<uint4*>(mma_smem);
     float* bias = reinterpret_cast<float*>(mma_smem + static_cast<size_t>(p.tiles) * 1024u);
-    float* w_in = bias + p.biases;                                   // cart-pole: [unit][8] = five weights, bias
+    uint8_t* exponents = reinterpret_cast<uint8_t*>(bias + p.biases);
+    float* w_in = bias + p.biases + p.biases / 4u;                                   // cart-pole: [unit][8] = five weights, bias
     const uint32_t buf0 = smem_u32(w_in + (CART ? p.mt[0] * 128u : 0u));
     const uint32_t buf_bytes = Units<EB>::kRows * p.pitch;
     const uint32_t xbuf = buf0 + 2u * buf_bytes;                     // tanh-linear: two state operands
@@ -104,13 +108,14 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     uint32_t n_params = 0;
     for (uint32_t l = 0; l < layers; ++l) n_params += (a.sizes[l] + 1u) * a.sizes[l + 1];
     uint32_t most = 0;
-    for (uint32_t i = tid; i < n_params; i += blockDim.x) most = max(most, finite_magnitude(__ldg(th + i)));
+    for (uint32_t i = tid; i < n_params; i += blockDim.x) most = max(most, magnitude(__ldg(th + i)));
     most = __reduce_max_sync(0xffffffffu, most);
     if (lane == 0) peaks[warp] = most;
     __syncthreads();
     most = 0;
     for (uint32_t i = 0; i < blockDim.x / 32u; ++i) most = max(most, peaks[i]);
-    const Scale sc(most);
+    const int largest = scale_exponent(most);
+    const bool scaled = largest != 0;
     {
         uint32_t off = 0;
         for (uint32_t l = 0; l < layers; ++l) {
@@ -121,31 +126,40 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
             if (CART && l == 0) {
                 for (uint32_t i = tid; i < p.mt[0] * 128u; i += blockDim.x) {
                     const int u = static_cast<int>(i >> 3), k = static_cast<int>(i & 7u);
-                    w_in[i] = (u < no && k < 6) ? kF * (k < 5 ? __ldg(W + u * 5 + k) : __ldg(B + u)) : 0.f;
+                    w_in[i] = (u < no && k < 6) ? times_f(k < 5 ? __ldg(W + u * 5 + k) : __ldg(B + u)) : 0.f;
                 }
                 continue;
             }
+            if (scaled) {
+                for (uint32_t m = warp; m < p.mt[l]; m += blockDim.x >> 5) {
+                    int n0, n1;
+                    row_exponents(W, ni, no, 16 * static_cast<int>(m), static_cast<int>(p.kt[l]), lane, n0, n1);
+                    if (t < 2) exponents[p.bias0[l] + 16u * m + g + 8u * t] = static_cast<uint8_t>(t ? n1 : n0);
+                }
+                __syncthreads();
+            }
             for (uint32_t i = warp; i < p.mt[l] * p.kt[l]; i += blockDim.x >> 5) {
+                const uint8_t* n = exponents + p.bias0[l] + 16u * (i / p.kt[l]) + g;
                 uint4 hi, lo;
-                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, sc, kF, hi, lo);
+                load_tile(W, ni, no, 16 * static_cast<int>(i / p.kt[l]), 16 * static_cast<int>(i % p.kt[l]), lane, scaled ? n[0] : 0,
+                          scaled ? n[8] : 0, hi, lo);
                 tiles[(p.tile0[l] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[l] + i) * 64u + 32u + lane] = lo;
             }
             for (uint32_t i = tid; i < p.mt[l] * 16u; i += blockDim.x)
-                bias[p.bias0[l] + i] = static_cast<int>(i) < no ? kF * __ldg(B + i) : 0.f;
+                bias[p.bias0[l] + i] = static_cast<int>(i) < no ? times_f(__ldg(B + i)) : 0.f;
         }
         if (!CART) {                                                 // x' = tanh(A x + B a)
-            const Scale one(0u);
             const float* A = a.task_const;
             const float* Bm = a.task_const + kTlNx * kTlNx;
             for (uint32_t i = warp; i < 6u; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, one, kF, hi, lo);
-                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, one, kF * a.action_scale, hi, lo);
+                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, 0, 0, hi, lo);
+                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, 0, 0, hi, lo, false, a.action_scale);
                 tiles[(p.tile0[layers] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[layers] + i) * 64u + 32u + lane] = lo;
             }
-            for (uint32_t i = tid; i < 32u; i += blockDim.x) bias[p.bias0[layers] + i] = 0.f;
+            for (uint32_t i = tid; i < 32u; i += blockDim.x) { bias[p.bias0[layers] + i] = 0.f; exponents[p.bias0[layers] + i] = 0; }
             for (uint32_t i = tid; i < 2u * xbuf_bytes / 4u; i += blockDim.x)
                 reinterpret_cast<uint32_t*>(mma_smem + (xbuf - smem_u32(mma_smem)))[i] = 0u;
         }
@@ -187,89 +201,95 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     }
 
     // ---- time loop -----------------------------------------------------------------------------------------
-    for (uint32_t step = 0; step < a.T; ++step) {
-        const uint32_t xin = xbuf + (step & 1u) * xbuf_bytes, xout = xbuf + ((step + 1u) & 1u) * xbuf_bytes;
-        CpAhead ahead{};
-        if (CART && !layer_warp) ahead = cartpole_ahead(cpc, cps, snc, csc);
-        for (uint32_t l = 0; l < layers; ++l) {
-            const bool last = l + 1u == layers;
-            const uint32_t in = l == 0u ? xin : buf0 + ((l + 1u) & 1u) * buf_bytes, out = buf0 + (l & 1u) * buf_bytes;
-            const uint32_t in_pitch = l == 0u ? kXPitch : p.pitch;
-            if (layer_warp) {
-                for (uint32_t m = warp; m < p.mt[l]; m += nw) {
-                    float v[NV];
-                    if (CART && l == 0u) {
-                        const float* wa = w_in + (16u * m + g) * 8u;
-                        const float4 w0 = *reinterpret_cast<const float4*>(wa), w1 = *reinterpret_cast<const float4*>(wa + 64);
-                        const float2 q0 = *reinterpret_cast<const float2*>(wa + 4), q1 = *reinterpret_cast<const float2*>(wa + 68);
+    const float up = scale_up(largest);                              // kActInv where nothing is scaled, in a register
+    auto roll = [&](auto with_scales) {
+        constexpr bool kScaled = decltype(with_scales)::value;
+        for (uint32_t step = 0; step < a.T; ++step) {
+            const uint32_t xin = xbuf + (step & 1u) * xbuf_bytes, xout = xbuf + ((step + 1u) & 1u) * xbuf_bytes;
+            CpAhead ahead{};
+            if (CART && !layer_warp) ahead = cartpole_ahead(cpc, cps, snc, csc);
+            for (uint32_t l = 0; l < layers; ++l) {
+                const bool last = l + 1u == layers;
+                const uint32_t in = l == 0u ? xin : buf0 + ((l + 1u) & 1u) * buf_bytes, out = buf0 + (l & 1u) * buf_bytes;
+                const uint32_t in_pitch = l == 0u ? kXPitch : p.pitch;
+                if (layer_warp) {
+                    for (uint32_t m = warp; m < p.mt[l]; m += nw) {
+                        float v[NV];
+                        if (CART && l == 0u) {
+                            const float* wa = w_in + (16u * m + g) * 8u;
+                            const float4 w0 = *reinterpret_cast<const float4*>(wa), w1 = *reinterpret_cast<const float4*>(wa + 64);
+                            const float2 q0 = *reinterpret_cast<const float2*>(wa + 4), q1 = *reinterpret_cast<const float2*>(wa + 68);
 #pragma unroll
-                        for (int i = 0; i < NV; ++i) {
-                            const int e = EB == 4 ? t : 2 * t + (i & 1);
-                            const bool up = i >= NV / 2;
-                            float s = fmaf(up ? w1.x : w0.x, obs[0][e], up ? q1.y : q0.y);
-                            s = fmaf(up ? w1.y : w0.y, obs[1][e], s);
-                            s = fmaf(up ? w1.z : w0.z, obs[2][e], s);
-                            s = fmaf(up ? w1.w : w0.w, obs[3][e], s);
-                            v[i] = fmaf(up ? q1.x : q0.x, obs[4][e], s);
+                            for (int i = 0; i < NV; ++i) {
+                                const int e = EB == 4 ? t : 2 * t + (i & 1);
+                                const bool up = i >= NV / 2;
+                                float s = fmaf(up ? w1.x : w0.x, obs[0][e], up ? q1.y : q0.y);
+                                s = fmaf(up ? w1.y : w0.y, obs[1][e], s);
+                                s = fmaf(up ? w1.z : w0.z, obs[2][e], s);
+                                s = fmaf(up ? w1.w : w0.w, obs[3][e], s);
+                                v[i] = fmaf(up ? q1.x : q0.x, obs[4][e], s);
+                            }
+                        } else {
+                            const uint32_t at = p.bias0[l] + 16u * m + g;
+                            unit_sums<EB, kScaled>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bias[at], bias[at + 8u], exponents + at, up, v);
                         }
-                    } else {
-                        const float* bb = bias + p.bias0[l] + 16u * m + g;
-                        unit_sums<EB>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bb[0], bb[8], sc.up * kActInv, v);
+                        tanh_units<EB, FINE ? Tanh::kFine : Tanh::kOwn>(v);
+                        if (!last) {
+                            Units<EB>::store(Units<EB>::row(out, p.pitch, lane) + 32u * m, v);
+                        } else if (CART) {
+                            if (g == 0) {
+                                if (EB == 4) act[t] = v[0];
+                                else { act[2 * t] = v[0]; act[2 * t + 1] = v[1]; }
+                            }
+                        } else {                                         // the action, and its share of the reward (units 8..15 are padding)
+                            Units<EB>::store(Units<EB>::row(xin, kXPitch, lane) + 64u, v);
+#pragma unroll
+                            for (int i = 0; i < NV / 2; ++i) {
+                                const float act = a.action_scale * kActInv * v[i];
+                                if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
+                            }
+                        }
                     }
-                    tanh_units<EB, Tanh::kFine>(v);
-                    if (!last) {
-                        Units<EB>::store(Units<EB>::row(out, p.pitch, lane) + 32u * m, v);
-                    } else if (CART) {
-                        if (g == 0) {
-                            if (EB == 4) act[t] = v[0];
-                            else { act[2 * t] = v[0]; act[2 * t + 1] = v[1]; }
-                        }
-                    } else {                                         // the action, and its share of the reward (units 8..15 are padding)
-                        Units<EB>::store(Units<EB>::row(xin, kXPitch, lane) + 64u, v);
+                }
+                __syncthreads();
+            }
+            if (CART) {
+                if (!layer_warp) {
+                    cartpole_finish(cpc, ahead, a.action_scale * kActInv * act[te], cps, snc, csc);
+                    ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
+                    if (lane < EB) {
+                        obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
+                        if (step < traced && te < nE)
+                            *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
+                                make_float4(cps.x, cps.xd, cps.th, cps.thd);
+                    }
+                }
+            } else {
+                for (uint32_t m = warp; m < 2u; m += nw) {
+                    float v[NV];
+                    const uint32_t at = p.bias0[layers] + 16u * m + g;
+                    unit_sums<EB, kScaled>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane, bias[at], bias[at + 8u], exponents + at, kActInv, v);
+                    tanh_units<EB, FINE ? Tanh::kFine : Tanh::kOwn>(v);
+                    Units<EB>::store(Units<EB>::row(xout, kXPitch, lane) + 32u * m, v);
 #pragma unroll
-                        for (int i = 0; i < NV / 2; ++i) {
-                            const float act = a.action_scale * kActInv * v[i];
-                            if (i == 0) ret = fmaf(-0.01f * act, act, ret); else ret2 = fmaf(-0.01f * act, act, ret2);
+                    for (int i = 0; i < NV; ++i) v[i] *= kActInv;
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) {
+                        const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
+                        const int e = EB == 4 ? t : 2 * t + (i & 1);
+                        if (step + 1u < a.T) {                           // reward of the next step: its pre-step state (padding rows are 0)
+                            if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
                         }
+                        if (step < traced && e < nE && row < kTlNx)
+                            a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + row] = v[i];
                     }
                 }
             }
             __syncthreads();
         }
-        if (CART) {
-            if (!layer_warp) {
-                cartpole_finish(cpc, ahead, a.action_scale * kActInv * act[te], cps, snc, csc);
-                ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
-                if (lane < EB) {
-                    obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
-                    if (step < traced && te < nE)
-                        *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
-                            make_float4(cps.x, cps.xd, cps.th, cps.thd);
-                }
-            }
-        } else {
-            for (uint32_t m = warp; m < 2u; m += nw) {
-                float v[NV];
-                unit_sums<EB>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane,
-                              bias[p.bias0[layers] + 16u * m + g], bias[p.bias0[layers] + 16u * m + g + 8u], kActInv, v);
-                tanh_units<EB, Tanh::kFine>(v);
-                Units<EB>::store(Units<EB>::row(xout, kXPitch, lane) + 32u * m, v);
-#pragma unroll
-                for (int i = 0; i < NV; ++i) v[i] *= kActInv;
-#pragma unroll
-                for (int i = 0; i < NV; ++i) {
-                    const uint32_t row = 16u * m + g + (i >= NV / 2 ? 8u : 0u);
-                    const int e = EB == 4 ? t : 2 * t + (i & 1);
-                    if (step + 1u < a.T) {                           // reward of the next step: its pre-step state (padding rows are 0)
-                        if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
-                    }
-                    if (step < traced && e < nE && row < kTlNx)
-                        a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + row] = v[i];
-                }
-            }
-        }
-        __syncthreads();
-    }
+    };
+    if (scaled) roll(std::true_type{});
+    else roll(std::false_type{});
 
     // ---- block return: fixed order --------------------------------------------------------------------------
     if (CART) {
@@ -294,11 +314,14 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     }
 }
 
+template <int EB, bool CART>
+auto pick_kernel(bool fine) { return fine ? k_rollout_mlp_mma<EB, CART, true> : k_rollout_mlp_mma<EB, CART, false>; }
+
 Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB)
 {
     Plan p = {};
     const bool cart = task == EVO_TASK_CARTPOLE;
-    uint32_t widest = 0;
+    uint32_t widest = 0, narrowest = n_layers > 1u ? ~0u : 0u;
     for (uint32_t l = 0; l < n_layers; ++l) {
         p.mt[l] = (sizes[l + 1] + 15u) / 16u;
         p.kt[l] = l == 0u ? 2u : (sizes[l] + 15u) / 16u;
@@ -306,7 +329,9 @@ Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t
         p.tile0[l] = p.tiles;
         if (!(cart && l == 0u)) { p.tiles += p.mt[l] * p.kt[l]; p.biases += p.mt[l] * 16u; }
         if (p.mt[l] > widest) widest = p.mt[l];
+        if (l + 1u < n_layers && p.mt[l] < narrowest) narrowest = p.mt[l];
     }
+    p.fine = narrowest < 4u;
     p.tile0[n_layers] = p.tiles;
     p.bias0[n_layers] = p.biases;
     p.mt[n_layers] = 2; p.kt[n_layers] = 3;
@@ -314,7 +339,7 @@ Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t
     p.pitch = (widest + 1u) / 2u * 64u + 16u;           // operands are read two tiles at a time
     p.warps = widest < 8u ? widest : 8u;
     const uint32_t rows = EB == 4u ? 8u : 16u;
-    p.smem = static_cast<size_t>(p.tiles) * 1024u + p.biases * 4u + (cart ? p.mt[0] * 512u : 0u) + 2u * rows * p.pitch +
+    p.smem = static_cast<size_t>(p.tiles) * 1024u + p.biases * 5u + (cart ? p.mt[0] * 512u : 0u) + 2u * rows * p.pitch +
              (cart ? 0u : 2u * rows * kXPitch + 32u);         // (the last column's third tile is read with the 32 bytes behind it)
     return p;
 }
@@ -334,8 +359,8 @@ int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatu
     const Plan p = make_plan(a.task, a.n_layers, a.sizes, a.EB);
     if (p.smem > kMaxSmem) return -2;
     const bool cart = a.task == EVO_TASK_CARTPOLE;
-    auto kernel = a.EB == 4u ? (cart ? k_rollout_mlp_mma<4, true> : k_rollout_mlp_mma<4, false>)
-                             : (cart ? k_rollout_mlp_mma<8, true> : k_rollout_mlp_mma<8, false>);
+    auto kernel = a.EB == 4u ? (cart ? pick_kernel<4, true>(p.fine) : pick_kernel<4, false>(p.fine))
+                             : (cart ? pick_kernel<8, true>(p.fine) : pick_kernel<8, false>(p.fine));
     if (!a.attr_done &&
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) != cudaSuccess)
         return -1;

@@ -91,8 +91,8 @@ def test_two_row_tiles_per_warp(sizes, episodes):
 @pytest.mark.parametrize("sizes,pop", [((28, 128, 128, 8), 4), ((28, 128, 128, 8), 300), ((5, 64, 64, 1), 4), ((5, 16, 16, 1), 4),
                                        ((28, 32, 32, 32, 8), 4)])
 def test_weights_far_beyond_the_fp16_range(sizes, pop):
-    """A member with a weight of 1e7 keeps its other weights to 22 bits of the largest one; the tanh behind the big one is
-    saturated, so the fitness agrees with the oracle, which uses every weight as it is."""
+    """The unit with a weight of 1e7 keeps its other weights to 22 bits of that one, every other unit keeps its own as they are, so
+    the fitness agrees with the oracle, which uses every weight as it is."""
     base = W.CFG2 if sizes[0] == 5 else W.CFG4
     w = base.with_(pop_size=pop, episodes=4, horizon=20, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
     theta = W.random_parameters(5, pop, w.param_dim, scale=0.05)

@@ -28,25 +28,70 @@ def _traces(w, theta, T, kernel):
     return trace.cpu().numpy().astype(np.float64)
 
 
-@pytest.mark.parametrize("sizes,pop,episodes", [
-    ((28, 128, 128, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 8), 64, 8), ((28, 64, 64, 64, 8), 64, 4),
-    ((28, 20, 8), 64, 8), ((5, 16, 16, 1), 64, 4), ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 8)])
-def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, pop, episodes):
-    base, T = (W.CFG2, max(STEPS)) if sizes[0] == 5 else (W.CFG4, max(STEPS))
+def _workload(sizes, pop, episodes):
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
     # (the oracle computes with the task constants as fp32 numbers, which the kernels get)
-    w = base.with_(pop_size=pop, episodes=episodes, horizon=T, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes),
-                   task_param=tuple(float(np.float32(x)) for x in base.task_param))
-    rng = np.random.default_rng(sum(sizes) + pop)
-    noise = rng.standard_normal((pop // 2, w.param_dim)) * 0.1                 # a population in mid-training
+    return base.with_(pop_size=pop, episodes=episodes, horizon=max(STEPS), layer_sizes=sizes, param_dim=W.mlp_param_count(sizes),
+                      task_param=tuple(float(np.float32(x)) for x in base.task_param))
+
+
+def _population(w, seed):
+    """A population in mid-training."""
+    rng = np.random.default_rng(seed)
+    noise = rng.standard_normal((w.pop_size // 2, w.param_dim)) * 0.1
     centre = rng.standard_normal(w.param_dim) * 0.05
-    theta = np.empty((pop, w.param_dim), np.float32)
+    theta = np.empty((w.pop_size, w.param_dim), np.float32)
     theta[0::2], theta[1::2] = centre + noise, centre - noise
-    members = list(range(32)) + list(range(pop - 32, pop))
-    want = np.array(oracle_fitness(w, theta[members], 0, T, want_trace=True)[1])
+    return theta
+
+
+def _check_against_fp32(w, theta):
+    members = list(range(32)) + list(range(w.pop_size - 32, w.pop_size))
+    want = np.array(oracle_fitness(w, theta[members], 0, w.horizon, want_trace=True)[1])
     rms = np.sqrt((want ** 2).mean(axis=(0, 1, 2)))
     at = [t - 1 for t in STEPS]
     err = {}
     for kernel in (ROLLOUT_AUTO, ROLLOUT_GENERIC):
-        e = (_traces(w, theta, T, kernel)[members][:, :, at] - want[:, :, at]) / rms
-        err[kernel] = np.exp(np.log(np.sqrt((e ** 2).mean(axis=(1, 3)))).mean(axis=0))       # one per step
-    assert (err[ROLLOUT_AUTO] < 1.2 * err[ROLLOUT_GENERIC]).all(), (err[ROLLOUT_AUTO] / err[ROLLOUT_GENERIC]).round(2)
+        e = (_traces(w, theta, w.horizon, kernel)[members][:, :, at] - want[:, :, at]) / rms
+        err[kernel] = np.exp(np.log(np.sqrt((e ** 2).mean(axis=(1, 3))) + 1e-30).mean(axis=0))       # one per step
+    ratio = err[ROLLOUT_AUTO] / err[ROLLOUT_GENERIC]
+    assert (ratio < 1.2).all(), ratio.round(2)
+
+
+@pytest.mark.parametrize("sizes,pop,episodes", [
+    ((28, 128, 128, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 8), 64, 8), ((28, 64, 64, 64, 8), 64, 4),
+    ((28, 20, 8), 64, 8), ((5, 16, 16, 1), 64, 4), ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 8)])
+def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, pop, episodes):
+    w = _workload(sizes, pop, episodes)
+    _check_against_fp32(w, _population(w, sum(sizes) + pop))
+
+
+@pytest.mark.parametrize("sizes,pop,episodes", [
+    ((28, 64, 64, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 64, 8), 64, 8), ((5, 16, 16, 1), 64, 4),
+    ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 4)])
+def test_a_huge_weight_takes_nothing_from_the_others(sizes, pop, episodes):
+    """One weight or bias beyond the fp16 range per member, from 2e4 to 1e30, anywhere in the policy."""
+    w = _workload(sizes, pop, episodes)
+    theta = _population(w, 1 + sum(sizes))
+    rng = np.random.default_rng(pop)
+    for m in range(pop):
+        theta[m, rng.integers(w.param_dim)] = rng.choice((-1.0, 1.0)) * rng.choice((2.0e4, 1.0e7, 1.0e12, 1.0e30))
+    _check_against_fp32(w, theta)
+
+
+@pytest.mark.parametrize("sizes", [(28, 24, 40, 8), (28, 24, 24, 24, 8), (5, 16, 16, 1), (5, 30, 40, 1), (5, 16, 16, 16, 1)])
+def test_infinite_weights_saturate(sizes):
+    w = _workload(sizes, 64, 4).with_(pop_size=8, horizon=3)
+    theta = _population(w, 9)[:8]
+    second = sizes[0] * sizes[1] + sizes[1]
+    theta[0, 3], theta[1, second + 1], theta[2, second + sizes[1] * sizes[2]] = np.inf, -np.inf, np.inf      # both layers, a bias
+    theta[3, second + 1], theta[3, second + 2] = np.inf, np.nan
+    fit = {}
+    for kernel in (ROLLOUT_AUTO, ROLLOUT_GENERIC):
+        s = Solver(w, rollout_kernel=kernel)
+        rows = s.padded_rows(8)
+        rows[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+        fit[kernel] = s.rollout(rows).cpu().numpy()
+        s.close()
+    np.testing.assert_allclose(fit[ROLLOUT_AUTO], fit[ROLLOUT_GENERIC], rtol=1e-5)
+    assert np.isnan(fit[ROLLOUT_AUTO]).tolist() == [False] * 3 + [True] + [False] * 4
