@@ -30,6 +30,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "internal.h"
+
 namespace evo {
 namespace ms {
 
@@ -99,8 +101,8 @@ __device__ __forceinline__ void split_two(float a, float b, uint32_t& hi, uint32
 // Weights beyond the fp16 range: a unit that has any keeps its weights times 2^-n, which brings f w of the largest below it, and
 // its sums are multiplied back.  What the other weights lose is then below 2^-22 of the largest, as it is in the unit's
 // sum; other units, and the biases, are not touched.  The kernels look at a member's largest weight first: nearly always there is
-// nothing to scale, and a step then does without the units' factors.  Infinities count, and are taken, as the largest finite number (the tanh
-// behind them saturates); NaN stays NaN.
+// nothing to scale, and a step then does without the units' factors.  Infinities count, and are taken, as the largest finite
+// number (the tanh behind them saturates); NaN stays NaN.
 __device__ __forceinline__ uint32_t magnitude(float w)                    // bit pattern
 {
     const uint32_t m = __float_as_uint(w) & 0x7FFFFFFFu;
@@ -149,15 +151,15 @@ __device__ __forceinline__ void read_tile(const float* W, int ni, int no, int ro
         }
     }
 }
-// Exponents of rows g and g + 8 of the `kt` tiles from row0 on.
-__device__ __forceinline__ void row_exponents(const float* W, int ni, int no, int row0, int kt, int lane, int& n0, int& n1)
+// Exponents of rows g and g + 8 of the `kt` tiles from row0 on, of the matrix times `times`.
+__device__ __forceinline__ void row_exponents(const float* W, int ni, int no, int row0, int kt, int lane, int& n0, int& n1, float times = 1.0f)
 {
     uint32_t m0 = 0, m1 = 0;
     for (int k = 0; k < kt; ++k) {
         float2 w[4];
         read_tile(W, ni, no, row0, 16 * k, lane, false, w);
-        m0 = max(max(m0, max(magnitude(w[0].x), magnitude(w[0].y))), max(magnitude(w[2].x), magnitude(w[2].y)));
-        m1 = max(max(m1, max(magnitude(w[1].x), magnitude(w[1].y))), max(magnitude(w[3].x), magnitude(w[3].y)));
+        m0 = max(max(m0, max(magnitude(times * w[0].x), magnitude(times * w[0].y))), max(magnitude(times * w[2].x), magnitude(times * w[2].y)));
+        m1 = max(max(m1, max(magnitude(times * w[1].x), magnitude(times * w[1].y))), max(magnitude(times * w[3].x), magnitude(times * w[3].y)));
     }
 #pragma unroll
     for (int off = 1; off < 4; off <<= 1) {
@@ -179,6 +181,27 @@ __device__ __forceinline__ void load_tile(const float* W, int ni, int no, int ro
         split_weights(finite(times * w[i].x), finite(times * w[i].y), kF * scale_down(i & 1 ? n1 : n0), h[i], l[i]);
     hi = make_uint4(h[0], h[1], h[2], h[3]);
     lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// The tanh-linear task's dynamics x' = tanh(A x + s B a) as operand tiles: tile i of six, three (two of A, one of B) for each 16 rows,
+// and the exponents of its rows where anything is scaled.  Entries of B stay below 2.1 (normals over sqrt(8)), so s does
+// not have to be looked at more closely below 2,048.
+__device__ __forceinline__ bool scales_dynamics(float action_scale) { return !(fabsf(action_scale) < 2048.0f); }
+__device__ __forceinline__ void load_dynamics(const float* task_const, float action_scale, int i, int lane, bool scaled, int& n0, int& n1,
+                                              uint4& hi, uint4& lo)
+{
+    const float* A = task_const;
+    const float* B = task_const + kTlNx * kTlNx;
+    const int row0 = 16 * (i / 3);
+    n0 = n1 = 0;
+    if (scaled) {
+        int b0, b1;
+        row_exponents(A, kTlNx, kTlNx, row0, 2, lane, n0, n1);
+        row_exponents(B, kTlNa, kTlNx, row0, 1, lane, b0, b1, action_scale);
+        n0 = max(n0, b0); n1 = max(n1, b1);
+    }
+    if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, row0, 16 * (i % 3), lane, n0, n1, hi, lo);
+    else load_tile(B, kTlNa, kTlNx, row0, 0, lane, n0, n1, hi, lo, false, action_scale);
 }
 
 __device__ __forceinline__ float ex2_fast(float p)

@@ -79,7 +79,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     __shared__ uint4 dyn[CART ? 1 : kDynTiles * 64];                 // ... task matrices in operand order
     __shared__ float x0s[CART ? 1 : kTlNx][EB];                      // ... start states
     __shared__ float rets[2][EB];
-    __shared__ float ups[2 * 16 * MW * RT + 8];                      // scale_up of the units of both hidden layers, then of the actions
+    __shared__ float ups[2 * 16 * MW * RT + 8 + (CART ? 0 : 32)];    // scale_up of the units of both hidden layers, the actions, the states
 
     // (the shuffle tells the compiler that the warp number is the same in all lanes)
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -120,7 +120,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         __syncthreads();
     }
     const int most = scale_exponent(peak);
-    const bool scaled = most != 0;
+    const bool scaled = most != 0 || (!CART && scales_dynamics(a.action_scale));
 
     // ---- weights into registers, times f (see mma_split.cuh) ---------------------------------------
     const float* W1 = stage;
@@ -181,13 +181,11 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         b3 = times_f(B3[0]);
     } else {
         b3 = times_f(B3[g]);
-        // x' = tanh(A x + B a)
-        const float* A = a.task_const;
-        const float* Bm = a.task_const + kTlNx * kTlNx;
         for (int i = warp; i < static_cast<int>(kDynTiles); i += nw) {
             uint4 hi, lo;
-            if (i % 3 < 2) load_tile(A, kTlNx, kTlNx, 16 * (i / 3), 16 * (i % 3), lane, 0, 0, hi, lo);
-            else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3), 0, lane, 0, 0, hi, lo, false, a.action_scale);
+            int s0, s1;
+            load_dynamics(a.task_const, a.action_scale, i, lane, scaled, s0, s1, hi, lo);
+            if (scaled) { ups3[8 + 16 * (i / 3)] = scale_up(s0); ups3[16 + 16 * (i / 3)] = scale_up(s1); }
             dyn[i * 64 + lane] = hi;
             dyn[i * 64 + 32 + lane] = lo;
         }
@@ -396,7 +394,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                     }
                 }
                 acc.add(tiles[128], tiles[160], b[0]);
-                acc.sums(kActInv, kActInv, 0.f, 0.f, v);
+                acc.sums(kScaled ? ups3[8 + 16 * warp] : kActInv, kScaled ? ups3[16 + 16 * warp] : kActInv, 0.f, 0.f, v);
                 tanh_units<EB, kTanh>(v);
                 U::store(xout + 32u * warp, v);
 #pragma unroll

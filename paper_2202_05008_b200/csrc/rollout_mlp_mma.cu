@@ -87,7 +87,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     uint4* tiles = reinterpret_cast<uint4*>(mma_smem);
     float* bias = reinterpret_cast<float*>(mma_smem + static_cast<size_t>(p.tiles) * 1024u);
     uint8_t* exponents = reinterpret_cast<uint8_t*>(bias + p.biases);
-    float* w_in = bias + p.biases + p.biases / 4u;                                   // cart-pole: [unit][8] = five weights, bias
+    float* w_in = bias + p.biases + p.biases / 4u;                   // cart-pole: [unit][8] = five weights, bias
     const uint32_t buf0 = smem_u32(w_in + (CART ? p.mt[0] * 128u : 0u));
     const uint32_t buf_bytes = Units<EB>::kRows * p.pitch;
     const uint32_t xbuf = buf0 + 2u * buf_bytes;                     // tanh-linear: two state operands
@@ -115,7 +115,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
     most = 0;
     for (uint32_t i = 0; i < blockDim.x / 32u; ++i) most = max(most, peaks[i]);
     const int largest = scale_exponent(most);
-    const bool scaled = largest != 0;
+    const bool scaled = largest != 0 || (!CART && scales_dynamics(a.action_scale));
     {
         uint32_t off = 0;
         for (uint32_t l = 0; l < layers; ++l) {
@@ -149,17 +149,16 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
             for (uint32_t i = tid; i < p.mt[l] * 16u; i += blockDim.x)
                 bias[p.bias0[l] + i] = static_cast<int>(i) < no ? times_f(__ldg(B + i)) : 0.f;
         }
-        if (!CART) {                                                 // x' = tanh(A x + B a)
-            const float* A = a.task_const;
-            const float* Bm = a.task_const + kTlNx * kTlNx;
+        if (!CART) {
             for (uint32_t i = warp; i < 6u; i += blockDim.x >> 5) {
                 uint4 hi, lo;
-                if (i % 3u < 2u) load_tile(A, kTlNx, kTlNx, 16 * (i / 3u), 16 * (i % 3u), lane, 0, 0, hi, lo);
-                else load_tile(Bm, kTlNa, kTlNx, 16 * (i / 3u), 0, lane, 0, 0, hi, lo, false, a.action_scale);
+                int n0, n1;
+                load_dynamics(a.task_const, a.action_scale, static_cast<int>(i), lane, scaled, n0, n1, hi, lo);
                 tiles[(p.tile0[layers] + i) * 64u + lane] = hi;
                 tiles[(p.tile0[layers] + i) * 64u + 32u + lane] = lo;
+                if (t < 2) exponents[p.bias0[layers] + 16u * (i / 3u) + g + 8u * t] = static_cast<uint8_t>(t ? n1 : n0);
             }
-            for (uint32_t i = tid; i < 32u; i += blockDim.x) { bias[p.bias0[layers] + i] = 0.f; exponents[p.bias0[layers] + i] = 0; }
+            for (uint32_t i = tid; i < 32u; i += blockDim.x) bias[p.bias0[layers] + i] = 0.f;
             for (uint32_t i = tid; i < 2u * xbuf_bytes / 4u; i += blockDim.x)
                 reinterpret_cast<uint32_t*>(mma_smem + (xbuf - smem_u32(mma_smem)))[i] = 0u;
         }
@@ -231,7 +230,8 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                             }
                         } else {
                             const uint32_t at = p.bias0[l] + 16u * m + g;
-                            unit_sums<EB, kScaled>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bias[at], bias[at + 8u], exponents + at, up, v);
+                            unit_sums<EB, kScaled>(tiles + (p.tile0[l] + m * p.kt[l]) * 64u, p.kt[l], in, in_pitch, lane, bias[at],
+                                                   bias[at + 8u], exponents + at, up, v);
                         }
                         tanh_units<EB, FINE ? Tanh::kFine : Tanh::kOwn>(v);
                         if (!last) {
@@ -268,7 +268,8 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                 for (uint32_t m = warp; m < 2u; m += nw) {
                     float v[NV];
                     const uint32_t at = p.bias0[layers] + 16u * m + g;
-                    unit_sums<EB, kScaled>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane, bias[at], bias[at + 8u], exponents + at, kActInv, v);
+                    unit_sums<EB, kScaled>(tiles + (p.tile0[layers] + m * 3u) * 64u, 3u, xin, kXPitch, lane, bias[at], bias[at + 8u],
+                                           exponents + at, kActInv, v);
                     tanh_units<EB, FINE ? Tanh::kFine : Tanh::kOwn>(v);
                     Units<EB>::store(Units<EB>::row(xout, kXPitch, lane) + 32u * m, v);
 #pragma unroll

@@ -95,3 +95,21 @@ def test_infinite_weights_saturate(sizes):
         s.close()
     np.testing.assert_allclose(fit[ROLLOUT_AUTO], fit[ROLLOUT_GENERIC], rtol=1e-5)
     assert np.isnan(fit[ROLLOUT_AUTO]).tolist() == [False] * 3 + [True] + [False] * 4
+
+
+@pytest.mark.parametrize("sizes,pop", [((28, 24, 40, 8), 64), ((28, 128, 100, 8), 300), ((28, 24, 24, 24, 8), 64)])
+@pytest.mark.parametrize("scale", [-1.0e3, 3.0e3, 1.0e6, 1.0e15])
+def test_large_action_scales(sizes, pop, scale):
+    """Actions that saturate the dynamics: a state near a sign change is either sign's in any arithmetic, so most members agree with
+    the oracle to fp32 rounding and every one is finite."""
+    w = _workload(sizes, pop, 4).with_(horizon=8, action_scale=scale)
+    theta = _population(w, 5)
+    s = Solver(w)
+    rows = s.padded_rows(pop)
+    rows[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    fit = s.rollout(rows).cpu().numpy()
+    assert s.sync_status() == 0 and np.isfinite(fit).all()
+    want, _ = oracle_fitness(w, theta[:64], 0, 8)
+    err = np.abs(fit[:64] - want) / np.abs(want)
+    assert np.median(err) < 1e-5, np.sort(err)
+    s.close()
