@@ -112,10 +112,7 @@ k_rollout_mlp_generic(const RolloutMlpArgs a, const DeviceStatus* __restrict__ s
                 obs[0 * EB + tid] = cps.x;  obs[1 * EB + tid] = cps.xd;
                 obs[2 * EB + tid] = cs;     obs[3 * EB + tid] = sn;
                 obs[4 * EB + tid] = cps.thd;
-                if (a.trace && t < a.trace_T) {
-                    float* tr = a.trace + ((static_cast<size_t>(member) * a.E + e0 + tid) * a.trace_T + t) * 4;
-                    tr[0] = cps.x; tr[1] = cps.xd; tr[2] = cps.th; tr[3] = cps.thd;
-                }
+                if (a.trace && t < a.trace_T) trace_state(a, status, member, e0 + tid, t, cps);
             }
             __syncthreads();
         } else {
@@ -139,8 +136,7 @@ k_rollout_mlp_generic(const RolloutMlpArgs a, const DeviceStatus* __restrict__ s
                 const uint32_t i = item / nE, e = item % nE;
                 const float xv = nxt[i * EB + e];
                 obs[i * EB + e] = xv;
-                if (a.trace && t < a.trace_T)
-                    a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + t) * kTlNx + i] = xv;
+                if (a.trace && t < a.trace_T) trace_component(a, status, member, e0 + e, t, i, xv);
             }
             __syncthreads();
         }

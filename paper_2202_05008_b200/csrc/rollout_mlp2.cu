@@ -355,9 +355,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                     const float force = a.action_scale * kActInv * tanh_one(pre + b3);
                     cartpole_finish(cpc, ahead, force, cps, snc, csc);
                     if (lane < EB) { obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd; }
-                    if (step < traced && lane < nE)
-                        *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
-                            make_float4(cps.x, cps.xd, cps.th, cps.thd);
+                    if (step < traced && lane < nE) trace_state(a, status, member, e0 + te, step, cps);
                 }
             } else if (tw) {                                              // action (in both warps), then x' = tanh(A x + B a)
                 float v[NV], p[4][NH];
@@ -403,8 +401,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
                     for (int i = 0; i < NV; ++i) {
                         const int unit = 16 * warp + g + (i >= NH ? 8 : 0), e = U::episode(i, t);
-                        if (e < nE && unit < static_cast<int>(kTlNx))
-                            a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + unit] = xcur[i];
+                        if (e < nE && unit < static_cast<int>(kTlNx)) trace_component(a, status, member, e0 + e, step, unit, xcur[i]);
                     }
                 }
             }
@@ -518,9 +515,7 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
             U::transpose(v, b);
             U::eight(w3, b, kScaled ? scale_up(s3) : kActInv, b3, v);
             cartpole_finish(c, ahead, a.action_scale * kActInv * tanh_one(v[0]), s, sn, cs);
-            if (step < traced && lane < nE)
-                *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + lane) * a.trace_T + step) * 4) =
-                    make_float4(s.x, s.xd, s.th, s.thd);
+            if (step < traced && lane < nE) trace_state(a, status, member, e0 + lane, step, s);
         }
     };
     if (scaled) roll(std::true_type{});

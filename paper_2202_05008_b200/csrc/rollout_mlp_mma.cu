@@ -259,9 +259,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                     ret = fmaf(csc, __expf(-cps.x * cps.x), ret);         // reward on the post-step state
                     if (lane < EB) {
                         obs[0][te] = cps.x; obs[1][te] = cps.xd; obs[2][te] = csc; obs[3][te] = snc; obs[4][te] = cps.thd;
-                        if (step < traced && te < nE)
-                            *reinterpret_cast<float4*>(a.trace + ((static_cast<size_t>(member) * a.E + e0 + te) * a.trace_T + step) * 4) =
-                                make_float4(cps.x, cps.xd, cps.th, cps.thd);
+                        if (step < traced && te < nE) trace_state(a, status, member, e0 + te, step, cps);
                     }
                 }
             } else {
@@ -281,8 +279,7 @@ k_rollout_mlp_mma(const RolloutMlpArgs a, const Plan p, DeviceStatus* status)
                         if (step + 1u < a.T) {                           // reward of the next step: its pre-step state (padding rows are 0)
                             if (EB == 4 || !(i & 1)) ret = fmaf(-v[i], v[i], ret); else ret2 = fmaf(-v[i], v[i], ret2);
                         }
-                        if (step < traced && e < nE && row < kTlNx)
-                            a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + step) * kTlNx + row] = v[i];
+                        if (step < traced && e < nE && row < kTlNx) trace_component(a, status, member, e0 + e, step, row, v[i]);
                     }
                 }
             }

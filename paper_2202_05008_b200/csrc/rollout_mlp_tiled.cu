@@ -348,11 +348,7 @@ k_rollout_mlp_tiled(const RolloutMlpArgs a, DeviceStatus* status)
                     obs[0 * EB + tid] = cps.x;  obs[1 * EB + tid] = cps.xd;
                     obs[2 * EB + tid] = cs;     obs[3 * EB + tid] = sn;
                     obs[4 * EB + tid] = cps.thd;
-                    if (tracing && t < a.trace_T && tid < nE) {
-                        float4* tr = reinterpret_cast<float4*>(
-                            a.trace + ((static_cast<size_t>(member) * a.E + e0 + tid) * a.trace_T + t) * 4);
-                        *tr = make_float4(cps.x, cps.xd, cps.th, cps.thd);
-                    }
+                    if (tracing && t < a.trace_T && tid < nE) trace_state(a, status, member, e0 + tid, t, cps);
                 }
             }
             __syncthreads();
@@ -383,8 +379,7 @@ k_rollout_mlp_tiled(const RolloutMlpArgs a, DeviceStatus* status)
                 __syncthreads();
                 for (int item = tid; item < static_cast<int>(kTlNx) * nE; item += THREADS) {
                     const int i = item / nE, e = item % nE;
-                    a.trace[((static_cast<size_t>(member) * a.E + e0 + e) * a.trace_T + t) * kTlNx + i] =
-                        obs_next[i * EB + e];
+                    trace_component(a, status, member, e0 + e, t, i, obs_next[i * EB + e]);
                 }
             }
             __syncthreads();
@@ -533,11 +528,7 @@ k_rollout_cartpole_ws(const RolloutMlpArgs a, DeviceStatus* status)
                 o[0 * EB + tid] = cps[g].x;  o[1 * EB + tid] = cps[g].xd;
                 o[2 * EB + tid] = cs;        o[3 * EB + tid] = sn;
                 o[4 * EB + tid] = cps[g].thd;
-                if (tracing && t < a.trace_T && tid < (g ? nB : nA)) {
-                    float4* tr = reinterpret_cast<float4*>(
-                        a.trace + ((static_cast<size_t>(member) * a.E + e0 + g * EB + tid) * a.trace_T + t) * 4);
-                    *tr = make_float4(cps[g].x, cps[g].xd, cps[g].th, cps[g].thd);
-                }
+                if (tracing && t < a.trace_T && tid < (g ? nB : nA)) trace_state(a, status, member, e0 + g * EB + tid, t, cps[g]);
             }
             __syncwarp();
         };

@@ -27,6 +27,21 @@ __device__ __forceinline__ CartpoleConst cartpole_const(const float* tp)
 
 struct CpState { float x, xd, th, thd; };
 
+// post-step state of a cart-pole, or component i of a tanh-linear state, into the trace of the roll-out
+__device__ __forceinline__ void trace_state(const RolloutMlpArgs& a, const DeviceStatus* status, uint32_t member, uint32_t episode, uint32_t step,
+                                            const CpState& s)
+{
+    const size_t at = ((static_cast<size_t>(member) * a.E + episode) * a.trace_T + step) * 4u;
+    if (EVO_IN_BOUNDS(status, EVO_SITE_TRACE, at + 3u, static_cast<size_t>(a.P) * a.E * a.trace_T * 4u))
+        *reinterpret_cast<float4*>(a.trace + at) = make_float4(s.x, s.xd, s.th, s.thd);
+}
+__device__ __forceinline__ void trace_component(const RolloutMlpArgs& a, const DeviceStatus* status, uint32_t member, uint32_t episode,
+                                                uint32_t step, uint32_t i, float value)
+{
+    const size_t at = ((static_cast<size_t>(member) * a.E + episode) * a.trace_T + step) * kTlNx + i;
+    if (EVO_IN_BOUNDS(status, EVO_SITE_TRACE, at, static_cast<size_t>(a.P) * a.E * a.trace_T * kTlNx)) a.trace[at] = value;
+}
+
 // time derivative of (x, x', theta, theta') for the uniform-rod cart-pole, theta = 0 upright
 __device__ __forceinline__ CpState cartpole_deriv(const CartpoleConst& c, const CpState& s, float force)
 {
