@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/evo.h"
+#include "spread.h"
 
 namespace evo {
 
@@ -154,20 +155,19 @@ int launch_rollout_paint(cudaStream_t st, const float* theta, uint32_t ldD, uint
 // everything before it.  A kernel lets its successor be set up with dep_trigger().  After a kernel that
 // never triggers, or after a copy, the launch is an ordinary one.
 // ------------------------------------------------------------------------------------------
-// Dynamic shared memory for a grid of `blocks` that fits the SMs at fewer blocks each than could be resident: asking
-// for a little more than the (r + 1)-th part of an SM's memory holds every SM at its even share r.  Without it the blocks
-// of a grid that becomes resident while the kernel before it still occupies some SMs crowd the others (256
-// blocks of a cart-pole roll-out: 1.95 ms in a stream of generations against 1.45 ms alone).
-inline size_t spread_over_sms(size_t bytes, uint64_t blocks)
+// Dynamic shared memory for a grid of `blocks` that fits the SMs at fewer blocks each than could be resident (see spread_bytes).
+// Without it the blocks of a grid that becomes resident while the kernel before it still occupies some SMs crowd the others
+// (256 blocks of a cart-pole roll-out: 1.95 ms in a stream of generations against 1.45 ms alone).
+template <class Kernel>
+inline size_t spread_over_sms(Kernel kernel, size_t bytes, uint64_t blocks)
 {
-    static const int sms = [] {
-        int dev = 0, n = 0;
-        return cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? n : 148;
-    }();
-    const uint64_t share = (blocks + sms - 1u) / sms;
-    if (share < 1u || share > 8u) return bytes;
-    const size_t least = 228u * 1024u / (share + 1u) - 1024u + 16u;      // a block also takes 1 KB for the system
-    return bytes < least ? least : bytes;
+    int dev = 0, sms = 0, sm_bytes = 0;
+    cudaFuncAttributes attr;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&attr, kernel) != cudaSuccess)
+        return bytes;
+    return spread_bytes(bytes, attr.sharedSizeBytes + 1024u, blocks, static_cast<uint32_t>(sms), static_cast<size_t>(sm_bytes));
 }
 
 #ifdef __CUDACC__

@@ -574,7 +574,7 @@ int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* 
         const size_t first = ((a.sizes[0] + 1u) * a.sizes[1] + 3u) * sizeof(float), low = warps * 2u * kt * 512u;
         bytes = first > low ? first : low;
     }
-    bytes = spread_over_sms(bytes, blocks);
+    bytes = spread_over_sms(kernel, bytes, blocks);
     if (!a.attr_done &&
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return -1;
     return launch_dependent(kernel, dim3(a.P, a.n_eb), dim3(32u * warps), bytes, st, a, status) == cudaSuccess ? 1 : -1;
