@@ -49,3 +49,36 @@ def test_tell_shapes(P, D, noise_mode, clipup):
             assert rel_err(s.center().cpu().numpy(), c0 + vel) < 1e-5
     assert s.counters() == (2, 2)
     s.close()
+
+
+@pytest.mark.parametrize("P,D", [(64, 257), (1024, 600), (4098, 70), (1024, 70000)])      # ranks inside and outside, one and several splits
+@pytest.mark.parametrize("noise_mode", [W.NOISE_STORED, W.NOISE_REGENERATED])
+@pytest.mark.parametrize("clipup,adapt", [(False, False), (True, False), (False, True), (True, True)])
+def test_a_nan_between_two_good_tells_changes_nothing(P, D, noise_mode, clipup, adapt):
+    """Centre, moments and sigma keep their bits over a tell with a NaN fitness, which is reported; the next good tell is that of a
+    solver which never saw one (same state, same generation)."""
+    w = W.Workload("nan", P, D, seed=P, sigma=0.1, optimizer=W.OPT_CLIPUP if clipup else W.OPT_ADAM,
+                   sigma_mode=W.SIGMA_PGPE if adapt else W.SIGMA_CONSTANT)
+    rng = np.random.default_rng(D)
+    good = [torch.tensor(rng.standard_normal(P).astype(np.float32), device="cuda") for _ in range(2)]
+    state = lambda s: [x.clone() for x in (s.center(), *s.moments(), s.sigma())]
+    s = Solver(w, noise_mode=noise_mode)
+    s.ask(); s.tell(good[0])
+    before = state(s)
+    bad = good[1].clone()
+    bad[int(rng.integers(P))] = float("nan")
+    s.ask(); s.tell(bad)
+    for a, b in zip(before, state(s)):
+        assert torch.equal(a, b)
+    assert s.sync_status() == 5 and s.sync_status() == 0                       # EVO_ERR_NONFINITE, then cleared
+    assert s.counters() == (2, 1)
+    s.ask(); s.tell(good[1])
+    assert s.sync_status() == 0
+    t = Solver(w, noise_mode=noise_mode)
+    t.set_state(center=before[0], m=before[1], v=before[2], generation=2, adam_step=1)
+    t.set_sigma(before[3])
+    t.ask(); t.tell(good[1])
+    for a, b in zip(state(s), state(t)):
+        assert torch.equal(a, b)
+    assert not torch.equal(before[0], s.center()) and s.counters() == t.counters() == (3, 2)
+    s.close(); t.close()
