@@ -697,9 +697,10 @@ static int launch_tell(cudaStream_t st, const TellArgs& a, uint32_t mode, double
     const uint32_t pps = (a.H + a.splits - 1u) / a.splits;
     const dim3 grid(tell_blocks(a.ldD), (a.H + pps - 1u) / pps);       // splits that own at least one pair
     // Every column block repeats the ranking of its split's members, P comparisons each: worth it while the repetition costs
-    // less than a launch (a few microseconds; 570 column blocks x 1,024 members would add about 10).
+    // less than a launch.  A generation of ask and tell, ranked inside / by k_rank: 128 members x 2,000 columns 12.8 / 14.8 us, 200 x 6,000
+    // (24 column blocks) 13.9 / 14.7, 256 x 4,609 14.4 / 15.1, 300 x 4,000 15.0 / 14.2, 512 x 4,000 16.2 / 15.5, 2,048 x 8,000 62.8 / 42.4.
     const bool whole = 2u * a.H == a.P && a.pair0 == 0u;
-    const bool ranks = whole && a.P <= kRankInTell && pps <= kTellPairs && static_cast<uint64_t>(grid.x) * a.P <= 65536u;
+    const bool ranks = whole && a.P <= kRankInTell && pps <= kTellPairs && static_cast<uint64_t>(grid.x) * a.P <= 5000u;
     int launches = 1;
     if (!ranks) {
         if (launch_rank(st, a.fitness, a.P, a.rank, a.u, a.status) < 0) return -1;

@@ -82,3 +82,13 @@ def test_a_nan_between_two_good_tells_changes_nothing(P, D, noise_mode, clipup, 
         assert torch.equal(a, b)
     assert not torch.equal(before[0], s.center()) and s.counters() == t.counters() == (3, 2)
     s.close(); t.close()
+
+
+@pytest.mark.parametrize("P,D,launches", [(16, 385, 1), (64, 5994, 1), (200, 6000, 1), (300, 6000, 2), (2048, 8000, 2), (2048, 600, 2)])
+def test_a_tell_ranks_inside_the_gradient_kernel_only_while_that_is_cheaper(P, D, launches):
+    s = Solver(W.Workload("tell", P, D, seed=1, sigma=0.1))
+    s.ask()
+    before = s.launch_count()
+    s.tell(torch.randn(P, device="cuda"))
+    assert s.launch_count() - before == launches and s.sync_status() == 0
+    s.close()
