@@ -92,3 +92,13 @@ def test_a_tell_ranks_inside_the_gradient_kernel_only_while_that_is_cheaper(P, D
     s.tell(torch.randn(P, device="cuda"))
     assert s.launch_count() - before == launches and s.sync_status() == 0
     s.close()
+
+
+@pytest.mark.parametrize("D,launches", [(12288, 1), (12320, 2)])
+def test_clipup_moves_many_columns_in_a_kernel_of_its_own(D, launches):
+    s = Solver(W.Workload("tell", 8, D, seed=1, sigma=0.1, optimizer=W.OPT_CLIPUP))
+    s.ask()
+    before = s.launch_count()
+    s.tell(torch.randn(8, device="cuda"))
+    assert s.launch_count() - before == launches and s.sync_status() == 0
+    s.close()
