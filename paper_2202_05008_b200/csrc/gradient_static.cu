@@ -45,7 +45,7 @@ static double* static_scratch_for_current_device(cudaError_t* err)
 static uint32_t static_splits(uint32_t H, uint32_t ldS)
 {
     const uint32_t blocks_x = (ldS / 4u + 255u) / 256u;
-    uint32_t s = (148u * 32u + blocks_x - 1u) / blocks_x;
+    uint32_t s = (kSms * 32u + blocks_x - 1u) / blocks_x;
     if (s > 64u) s = 64u;
     const uint32_t most = (H + 15u) / 16u;
     return s > most ? most : s;

@@ -48,6 +48,7 @@ constexpr size_t kCanaryBytes = 0;
 #endif
 constexpr int kMaxRegions = 24;
 
+constexpr uint32_t kSms = 148;   // of a B200: the plans that size workspaces are functions of the configuration alone
 constexpr uint32_t kTlNx = 28;   // tanh-linear task: state width
 constexpr uint32_t kTlNa = 8;    // tanh-linear task: action width
 constexpr uint32_t kCnnParams = 5994;

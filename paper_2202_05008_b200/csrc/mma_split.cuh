@@ -52,10 +52,6 @@ __device__ __forceinline__ void mma_k16_first(float (&c)[4], const uint4& a, uin
 }
 
 // 8x8 fp16 matrices from shared memory, row addresses from lanes 0-7, 8-15, ...
-__device__ __forceinline__ void ldsm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
-}
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -83,7 +79,7 @@ __device__ __forceinline__ uint32_t transpose8(uint32_t x)
 constexpr float kF = 2.885390082f;                           // 2 log2(e)
 // What a factor f lacks: the fp32 f is short by 1.3e-8, and the tensor core cuts its sums off, which leaves a result 3e-8 short
 // on average.  (Both are systematic, and a roll-out adds them up: without, the states of 28-64-64-64-8 shrink by 4e-8 per step
-// and the fitness is off by 5e-7; with, by less than 5e-9 and 2e-7 to 1e-7.)
+// and the fitness is off by 5e-7; with, by less than 1e-8 per step, and by 2e-7.)
 constexpr float kRest = 1.3e-8f + 3.0e-8f;
 constexpr float kAct = 8192.0f, kActInv = 1.0f / 8192.0f;    // scale of the activations (a start state of 5.8, the largest normal, fits fp16)
 constexpr float kLo = 2048.0f, kLoInv = 1.0f / 2048.0f;      // scale of the weights' low parts

@@ -226,7 +226,7 @@ void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
     if (k == MlpKernel::kGeneric || k == MlpKernel::kNone) {
         eb = cfg.episodes < 32u ? cfg.episodes : 32u;
         // few members: split the episodes of a member over more blocks to fill the SMs
-        while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * 148u)
+        while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * kSms)
             eb = (eb + 1u) / 2u;
     }
     *EB = eb;

@@ -53,8 +53,8 @@ __device__ __forceinline__ bool fetch_row(const RolloutMlpArgs& a, DeviceStatus*
 // KT: 16-unit tiles of the first hidden layer (rounded up to 1, 2, 3, 4, 6 or 8); RT: row tiles per warp.  With one row tile
 // a warp has all of its weights in registers, the shortest chain, but a wide member then takes eight warps of 128
 // registers and two members fill an SM.  RT = 2: four warps, the low parts of the second layer in shared memory,
-// three members per SM.  28-128-128-8, 4 episodes, per step of one / two / three resident members: RT = 1 0.86 / 1.08 us
-// (three do not fit), RT = 2 0.88 / 1.09 / 1.31 us; 28-96-40-8, 250 members: RT = 1 0.69 us, RT = 2 0.86 us.
+// three members per SM.  28-128-128-8, 4 episodes, per step of one / two / three resident members: RT = 1 0.76 / 0.97 us
+// (three do not fit), RT = 2 0.81 / 1.07 / 1.26 us; 28-96-40-8, 250 members: RT = 1 0.63 us, RT = 2 0.80 us.
 template <int EB, bool CART, int KT, int RT>
 __global__ void __launch_bounds__(RT == 1 && KT > 4 ? 256 : 128, RT == 2 ? 3 : KT > 4 ? 2 : 4)
 k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
@@ -563,7 +563,7 @@ int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* 
         return launch_dependent(k_rollout_cart_solo, dim3(a.P, a.n_eb), dim3(32), bytes, st, a, status) == cudaSuccess ? 1 : -1;
     // Wide policies: all weights in registers as long as no SM gets more than the two members that then fit.
     const uint64_t blocks = static_cast<uint64_t>(a.P) * a.n_eb;
-    const bool wide = tiles > 4u, two_tiles = wide && blocks > 2u * 148u;
+    const bool wide = tiles > 4u, two_tiles = wide && blocks > 2u * kSms;
     uint32_t kt = (a.sizes[1] + 15u) / 16u;
     if (wide) kt = two_tiles && kt <= 4u ? 4u : kt <= 6u ? 6u : 8u;
     auto kernel = a.EB == 4u ? (cart ? pick_kernel<4, true>(kt, two_tiles) : pick_kernel<4, false>(kt, two_tiles))

@@ -260,7 +260,7 @@ static PaintSplit paint_split(uint32_t P, uint32_t W, uint32_t H)
     PaintSplit s;
     s.rects_x = (W + kRectW - 1u) / kRectW;
     s.rects = s.rects_x * ((H + kRectH - 1u) / kRectH);
-    const uint64_t share = static_cast<uint64_t>(s.rects) * P / (148u * 24u);
+    const uint64_t share = static_cast<uint64_t>(s.rects) * P / (kSms * 24u);
     s.per_block = share < 4u ? 4u : share > s.rects ? (s.rects + 3u) / 4u * 4u : static_cast<uint32_t>(share) / 4u * 4u;
     s.blocks = (s.rects + s.per_block - 1u) / s.per_block;
     return s;

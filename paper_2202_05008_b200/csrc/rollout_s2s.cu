@@ -815,7 +815,7 @@ static uint32_t s2s_mma_chunk(uint32_t P, uint32_t B)
 {
     const uint32_t tiles = (B + 7u) / 8u;
     uint32_t chunks = (tiles + kMmaTiles - 1u) / kMmaTiles;
-    while (chunks < tiles && static_cast<uint64_t>(P) * chunks < 2u * 148u) ++chunks;
+    while (chunks < tiles && static_cast<uint64_t>(P) * chunks < 2u * kSms) ++chunks;
     return (tiles + chunks - 1u) / chunks * 8u;
 }
 

@@ -111,7 +111,7 @@ int launch_ask(cudaStream_t st, const float* center, const float* sigma_vec, uin
     // Eight pairs per thread reuse the centre; a small problem is one wave whose length is what a thread does, so it takes fewer.
     const uint32_t bx = (quads + 255u) / 256u;
     uint32_t ppt = 8u;
-    while (ppt > 1u && static_cast<uint64_t>(bx) * ((H + ppt - 1u) / ppt) < 148u * 6u) ppt /= 2u;
+    while (ppt > 1u && static_cast<uint64_t>(bx) * ((H + ppt - 1u) / ppt) < kSms * 6u) ppt /= 2u;
     dim3 grid(bx, (H + ppt - 1u) / ppt);
     if (grid.y > 65535u) grid.y = 65535u;
     return launch_dependent(k_ask, grid, dim3(256), 0, st, center, sigma_vec, philox_key(k0, k1), status, pair0, H, D, ldD,
@@ -659,10 +659,10 @@ static uint32_t tell_blocks(uint32_t ldD) { return (ldD / 4u + kTellQuads - 1u) 
 
 uint32_t gradient_splits(uint32_t H, uint32_t ldD)
 {
-    // Four waves of eight blocks per SM (with two the last one shows: 131,072 columns, 8,192 pairs 745 us against 660), as long
-    // as every pair lane keeps two rounds of loads; a pure function of the shape.
+    // 32 blocks per SM in all, six waves and more (with half as many the last one shows: 131,072 columns, 8,192 pairs 745 us against 660),
+    // as long as every pair lane keeps two rounds of loads; a pure function of the shape.
     const uint32_t bx = tell_blocks(ldD);
-    uint32_t s = (148u * 32u + bx - 1u) / bx;
+    uint32_t s = (kSms * 32u + bx - 1u) / bx;
     if (s > 64u) s = 64u;
     const uint32_t most = (H + 2u * kGradRows * kTellLanes - 1u) / (2u * kGradRows * kTellLanes);
     if (s > most) s = most;

@@ -64,7 +64,7 @@ def test_cfg2_T200_sampled_members(kernel):
     _rollout_check(W.CFG2, 200, [0, 1, 77, 128, 255], kernel)
 
 
-# AUTO = the tensor-core kernel (wide layers as split-fp16 tcgen05 MMAs), TILED = the fp32-pipe kernel
+# AUTO = the tensor-core kernel (layers as split-fp16 mma.sync products), TILED = the fp32-pipe kernel
 @pytest.mark.parametrize("kernel", [ROLLOUT_GENERIC, ROLLOUT_TILED, ROLLOUT_AUTO])
 def test_cfg4_T200_sampled_members(kernel):
     _rollout_check(W.CFG4, 200, [0, 1, 591, 592, 2047, 4095], kernel)
@@ -72,8 +72,8 @@ def test_cfg4_T200_sampled_members(kernel):
 
 @pytest.mark.parametrize("pop,episodes", [(2, 4), (6, 3), (10, 6), (1186, 4), (6, 9)])
 def test_cfg4_tensor_core_kernel_ragged_members_and_episodes(pop, episodes):
-    """Populations that do not fill the four teams of a block, episode counts that leave a partial
-    episode block, and more items than resident teams (1186 > 2 * 592: teams loop three times)."""
+    """Populations from two members to more blocks than are resident at a time, episode counts that leave a partial episode
+    block of four or of eight."""
     w = W.CFG4.with_(pop_size=pop, episodes=episodes)
     members = sorted({0, 1, pop // 2, pop - 1})
     T = 40 if pop > 100 else 120
@@ -97,9 +97,8 @@ def test_cfg4_action_scale_and_later_generation(kernel):
 
 
 def test_cfg4_tensor_core_kernel_with_weights_beyond_the_fp16_range():
-    """The tensor-core kernel holds the wide layers as fp16 pairs; a weight beyond +-65,504 is clamped
-    to that when staged.  The tanh behind it is saturated either way, so the fitness still agrees with
-    the oracle (which uses the weight as it is), and nothing turns into an infinity."""
+    """The tensor-core kernel holds the layers as fp16 pairs; the weights of a unit that has one beyond their range are scaled by a
+    power of two.  The fitness still agrees with the oracle (which uses the weights as they are), and nothing turns into an infinity."""
     w = W.CFG4.with_(pop_size=4, horizon=60)
     theta = W.random_parameters(11, 4, w.param_dim, scale=0.05)
     theta[0, 5] = 1.0e7                      # first layer, unit 0
