@@ -106,3 +106,9 @@ def test_weights_far_beyond_the_fp16_range(sizes, pop):
     fit_o, _ = oracle_fitness(w, theta[:4], 0, 20)
     assert rel_err(fit[:4], fit_o, floor=1.0) < FIT_TOL
     s.close()
+
+
+@pytest.mark.parametrize("sizes,episodes", [((28, 384, 96, 8), 4), ((5, 112, 384, 1), 8), ((5, 256, 192, 1), 4)])
+def test_policies_that_just_fit_the_shared_memory(sizes, episodes):
+    """221 to 222 KB of operand tiles, biases and exponents; with a larger one the runtime-shape kernel would run."""
+    check(sizes, episodes, 12, scale=0.02 if sizes[0] == 28 else 0.1)
