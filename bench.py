@@ -449,10 +449,8 @@ def roofline_of(w, workload_key, noise, stages, work, peaks, sm_count, max_mhz, 
              "frac": achieved / peaks["bf16_tflops"], "peak_source": peaks["source"], "traffic": None}
     else:
         achieved = stages["rollout"]["TFLOP/s"]
-        # control tasks: two hidden layers of up to 128 units (one warp per member where they have at most 16), else any depth
-        two = len(w.layer_sizes) == 4 and max(w.layer_sizes[1:3]) <= 128
-        control = "k_rollout_mlp_mma" if not two else (
-            "k_rollout_cart_solo" if w.task_kind == W.TASK_CARTPOLE and max(w.layer_sizes[1:3]) <= 16 else "k_rollout_mlp2")
+        # control tasks (all of these have two hidden layers of up to 128 units): one warp per member where they have at most 16
+        control = "k_rollout_cart_solo" if w.task_kind == W.TASK_CARTPOLE and max(w.layer_sizes[1:3]) <= 16 else "k_rollout_mlp2"
         kernel = "k_paint" if w.task_kind == W.TASK_PAINT else control
         r = {"kernel": kernel,
              "bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",

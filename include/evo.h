@@ -55,8 +55,8 @@ enum { EVO_TASK_NONE = 0, EVO_TASK_CARTPOLE = 1, EVO_TASK_TANH_LINEAR = 2, EVO_T
  * kernels with the weights in registers (two hidden layers, each at most as wide as a compiled shape:
  * 16/32/64/128 for the cart-pole, 128 for the tanh-linear task); UNSUPPORTED at evo_rollout if none
  * fits.  AUTO: the layers on the tensor cores as pairs of fp16 numbers (fp32-accurate), the weights
- * of two hidden layers of up to 128 units in registers, those of any other policy in shared memory as
- * long as they fit; else GENERIC. */
+ * of one to four hidden layers of up to 128 units in registers (but where only some of the layers are wide
+ * and the population large), those of any other policy in shared memory as long as they fit; else GENERIC. */
 enum { EVO_ROLLOUT_AUTO = 0, EVO_ROLLOUT_GENERIC = 1, EVO_ROLLOUT_TILED = 2 };
 enum { EVO_OPT_ADAM = 0, EVO_OPT_CLIPUP = 1 };
 enum { EVO_SIGMA_CONSTANT = 0, EVO_SIGMA_PGPE = 1 };

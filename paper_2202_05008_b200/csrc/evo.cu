@@ -311,6 +311,7 @@ evo_status evo_rollout(evo_solver* s, const float* d_theta, float* d_fitness, fl
     a.trace = d_trace;
     a.task_const = reinterpret_cast<const float*>(s->ws + L.task_const);
     a.P = s->local_pop;
+    a.pop = c.pop_size;
     a.ldD = L.ldD;
     a.n_layers = c.n_layers;
     a.max_width = 0;

@@ -61,6 +61,7 @@ struct RolloutMlpArgs {
     float*       trace;          // nullable
     const float* task_const;     // tanh-linear: A[28][28] then B[28][8]
     uint32_t P, ldD;
+    uint32_t pop;                // the whole population, of which P may be a shard: what chooses the kernel
     uint32_t n_layers;
     uint32_t sizes[EVO_MAX_LAYERS + 1];
     uint32_t max_width;

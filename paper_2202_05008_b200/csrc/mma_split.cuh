@@ -233,11 +233,11 @@ __device__ __forceinline__ void tanh_two(float& p, float& q)
     p = fmaf(kAct, e, -kAct) * b * r;
     q = fmaf(kAct, d, -kAct) * a * r;
 }
-// With the Taylor polynomial to x^9 below |x| = 0.3, where what it leaves out is below 6e-8 of x.  For k_rollout_mlp_mma,
-// which also takes policies with layers so narrow that their sums do not hide the exponential's error near 1.  State error
+// With the Taylor polynomial to x^9 below |x| = 0.3, where what it leaves out is below 6e-8 of x.  For k_rollout_mlp_deep and
+// k_rollout_mlp_mma, which also take policies with layers so narrow that their sums do not hide the exponential's error near 1.  State error
 // against that of tanhf on the fp32 pipe, after 1 / 20 / 200 steps: 28-20-8 without it 1.05 / 1.05 / 1.18, with it 0.95 / 0.82 / 0.92;
-// 28-64-10-10-8 without 1.04 / 1.12 / 1.16; 28-64-64-64-8 without 0.91 / 0.84 / 0.86.  It costs that last one 4 % (485 us a
-// generation of 512 members instead of 465), so a policy has it whose narrowest hidden layer is below 49 units.
+// 28-64-10-10-8 without 1.04 / 1.12 / 1.16; 28-64-64-64-8 without 0.91 / 0.84 / 0.86.  It costs k_rollout_mlp_mma 4 % with that last
+// one (485 us a generation of 512 members instead of 465), so a policy has it whose narrowest hidden layer is below 49 units.
 __device__ __forceinline__ float tanh_fine(float p)
 {
     constexpr double f = 2.885390081777927, g = 1.0 / (f * f);                // z = p^2 = x^2 / g

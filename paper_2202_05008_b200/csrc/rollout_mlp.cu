@@ -8,6 +8,7 @@
 //
 //   k_rollout_mlp_generic   any layer count / widths (runtime), the reference device path
 //   k_rollout_mlp2          two hidden layers, split-fp16 tensor-core products, weights in registers
+//   k_rollout_mlp_deep      one, three or four hidden layers, likewise
 //   k_rollout_mlp_mma       any layer count, the same products, weights in shared memory
 //   k_rollout_mlp_tiled<..> compile-time shapes with register-tiled layers on the fp32 pipe
 #include "internal.h"
@@ -195,16 +196,18 @@ uint32_t rollout_mlp_tiled_eb(int shape, uint32_t episodes);
 int launch_rollout_mlp_tiled(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 uint32_t rollout_mlp2_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
+uint32_t rollout_mlp_deep_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t episodes);
+int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
-// The kernel of a policy: AUTO takes the register-resident one where the policy has two hidden layers of up to 128
-// units, for any other number of layers and wider ones the one with the weights in shared memory as long
-// as they fit it, and else the runtime-shape kernel, which reads them through the caches.
-enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kSharedMemory };
+// The kernel of a policy: AUTO takes a register-resident one where the policy has one to four hidden layers of up to 128
+// units (beside an exception, see rollout_mlp_deep_eb), for other numbers of layers and wider ones the one with the weights in
+// shared memory as long as they fit it, and else the runtime-shape kernel, which reads them through the caches.
+enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kDeep, kSharedMemory };
 
-static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t episodes,
-                               uint32_t* EB)
+static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t pop,
+                               uint32_t episodes, uint32_t* EB)
 {
     if (choice == EVO_ROLLOUT_TILED) {
         const int shape = rollout_mlp_tiled_shape(task, n_layers, sizes);
@@ -214,6 +217,7 @@ static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t*
     }
     if (choice == EVO_ROLLOUT_AUTO) {
         if ((*EB = rollout_mlp2_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kRegisters;
+        if ((*EB = rollout_mlp_deep_eb(task, n_layers, sizes, pop, episodes)) != 0u) return MlpKernel::kDeep;
         if ((*EB = rollout_mlp_mma_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kSharedMemory;
     }
     return MlpKernel::kGeneric;
@@ -222,7 +226,7 @@ static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t*
 void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
 {
     uint32_t eb = 0;
-    const MlpKernel k = choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.episodes, &eb);
+    const MlpKernel k = choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.pop_size, cfg.episodes, &eb);
     if (k == MlpKernel::kGeneric || k == MlpKernel::kNone) {
         eb = cfg.episodes < 32u ? cfg.episodes : 32u;
         // few members: split the episodes of a member over more blocks to fill the SMs
@@ -250,12 +254,16 @@ int launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a_in, uint32_t ker
     uint32_t eb = 0;
     int launches = 0;
     a.fitness = fitness;
-    switch (choose_kernel(a.task, a.n_layers, a.sizes, kernel_choice, a.E, &eb)) {
+    switch (choose_kernel(a.task, a.n_layers, a.sizes, kernel_choice, a.pop, a.E, &eb)) {
     case MlpKernel::kNone:
         return -2;
     case MlpKernel::kRegisters:
         launches = launch_rollout_mlp2(st, a, status);
         if (launches < 0 || a.n_eb == 1u) return launches;            // one block per member writes the fitness itself
+        break;
+    case MlpKernel::kDeep:
+        launches = launch_rollout_mlp_deep(st, a, status);
+        if (launches < 0 || a.n_eb == 1u) return launches;
         break;
     case MlpKernel::kSharedMemory:
         launches = launch_rollout_mlp_mma(st, a, status);

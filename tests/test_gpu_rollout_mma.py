@@ -112,3 +112,47 @@ def test_weights_far_beyond_the_fp16_range(sizes, pop):
 def test_policies_that_just_fit_the_shared_memory(sizes, episodes):
     """221 to 222 KB of operand tiles, biases and exponents; with a larger one the runtime-shape kernel would run."""
     check(sizes, episodes, 12, scale=0.02 if sizes[0] == 28 else 0.1)
+
+
+@pytest.mark.parametrize("sizes", [(28, 128, 8), (28, 3, 8), (28, 64, 17, 49, 8), (28, 128, 128, 128, 8), (28, 65, 16, 100, 8), (28, 5, 128, 64, 8),
+                                   (28, 64, 33, 64, 49, 8), (28, 128, 64, 65, 128, 8),
+                                   (5, 128, 1), (5, 64, 64, 64, 1), (5, 65, 128, 3, 1), (5, 50, 64, 49, 64, 1), (5, 16, 65, 64, 128, 1)])
+@pytest.mark.parametrize("episodes", [3, 8, 11])
+def test_one_three_and_four_hidden_layers_with_the_weights_in_registers(sizes, episodes):
+    check(sizes, episodes, 40, scale=0.05 if sizes[0] == 28 else 0.25)
+
+
+@pytest.mark.parametrize("sizes", [(28, 128, 8), (28, 64, 64, 64, 8), (28, 128, 100, 128, 8), (28, 64, 40, 64, 30, 8), (28, 128, 128, 128, 128, 8),
+                                   (5, 60, 1), (5, 64, 64, 64, 1), (5, 128, 30, 100, 64, 1)])
+@pytest.mark.parametrize("episodes", [4, 5])
+def test_weights_far_beyond_the_fp16_range_in_every_layer(sizes, episodes):
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=len(sizes) // 2 * 2, episodes=episodes, horizon=20, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
+    theta = W.random_parameters(7, w.pop_size, w.param_dim, scale=0.05)
+    at = 0
+    for m, (a, b) in enumerate(zip(sizes[:-1], sizes[1:])):      # member m: the last unit of layer m has one
+        theta[m % w.pop_size, at + a * b - 1] = 1.0e6
+        at += (a + 1) * b
+    s = Solver(w)
+    arg = s.padded_rows(w.pop_size)
+    arg[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    fit = s.rollout(arg).cpu().numpy()
+    assert s.sync_status() == 0 and np.isfinite(fit).all()
+    fit_o, _ = oracle_fitness(w, theta, 0, 20)
+    assert rel_err(fit, fit_o, floor=1.0) < FIT_TOL
+    s.close()
+
+
+@pytest.mark.parametrize("sizes,pop,episodes", [((28, 120, 20, 10, 8), 300, 4), ((28, 100, 30, 100, 8), 300, 8), ((5, 90, 20, 20, 20, 1), 150, 16)])
+def test_deep_wide_policies_of_more_blocks_than_the_gpu_holds(sizes, pop, episodes):
+    """Either side of the line between weights in registers and in shared memory."""
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=pop, episodes=episodes, horizon=12, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes), sigma=0.05)
+    s = Solver(w)
+    theta = s.ask().cpu().numpy()
+    fit = s.rollout().cpu().numpy()
+    assert s.sync_status() == 0
+    members = [0, 1, 147, 148, pop - 1]
+    fit_o, _ = oracle_fitness(w, theta[members], 0, 12)
+    assert rel_err(fit[members], fit_o, floor=1.0) < FIT_TOL
+    s.close()
