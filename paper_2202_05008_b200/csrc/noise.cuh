@@ -27,12 +27,13 @@ __host__ __device__ __forceinline__ PhiloxKey philox_key(uint32_t k0, uint32_t k
     return k;
 }
 
-// counter = (item, row, generation, stream)
+// counter = (item, row, generation, stream); FIRST: rounds that have been done
+template <int FIRST = 0>
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                                const PhiloxKey& key)
 {
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
+    for (int r = FIRST; r < 10; ++r) {
         const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * c0;      // one wide multiply each
         const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * c2;
         const uint32_t hi0 = static_cast<uint32_t>(p0 >> 32), lo0 = static_cast<uint32_t>(p0);
@@ -43,6 +44,30 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
         c3 = lo0;
     }
     return make_uint4(c0, c1, c2, c3);
+}
+
+// The generator for many rows of one (item, generation, stream): of the first three rounds' six products four do not depend on the
+// row.  What is left of those rounds are two products and four exclusive ors with these words.
+struct PhiloxItem { uint32_t a, b, c, d, e; };
+
+__device__ __forceinline__ PhiloxItem philox_item(uint32_t item, uint32_t generation, uint32_t stream, const PhiloxKey& key)
+{
+    const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * item, p1 = static_cast<uint64_t>(0xCD9E8D57u) * generation;
+    const uint64_t q1 = static_cast<uint64_t>(0xCD9E8D57u) * (static_cast<uint32_t>(p0 >> 32) ^ stream ^ key.r[1]);
+    const uint64_t s0 = static_cast<uint64_t>(0xD2511F53u) * (static_cast<uint32_t>(q1 >> 32) ^ static_cast<uint32_t>(p1) ^ key.r[2]);
+    PhiloxItem x;
+    x.a = static_cast<uint32_t>(p1 >> 32) ^ key.r[0];
+    x.b = static_cast<uint32_t>(p0) ^ key.r[3];
+    x.c = static_cast<uint32_t>(q1) ^ key.r[4];
+    x.d = static_cast<uint32_t>(s0 >> 32) ^ key.r[5];
+    x.e = static_cast<uint32_t>(s0);
+    return x;
+}
+__device__ __forceinline__ uint4 philox4x32_10(const PhiloxItem& x, uint32_t row, const PhiloxKey& key)
+{
+    const uint64_t p = static_cast<uint64_t>(0xD2511F53u) * (x.a ^ row);
+    const uint64_t q = static_cast<uint64_t>(0xCD9E8D57u) * (static_cast<uint32_t>(p >> 32) ^ x.b);
+    return philox4x32_10<3>(static_cast<uint32_t>(q >> 32) ^ x.c, static_cast<uint32_t>(q), static_cast<uint32_t>(p) ^ x.d, x.e, key);
 }
 
 __device__ __forceinline__ float uniform_open(uint32_t r)   // (0, 1]
@@ -155,7 +180,10 @@ __device__ __forceinline__ void cossin_of_v24(uint32_t ja, uint32_t jb, float (&
 // Both transforms of a quad in packed arithmetic.  Instruction issue bounded the generator; asking for 8 GB of parameters takes
 // 165 instructions per four normals now where two scalar transforms took 231, and the multiply pipe bounds it (a wide
 // multiply of the counters holds it for 4 clocks, a packed operation for 2).  1,000,003 columns x 1,000 pairs,
-// recomputed noise: ask 2.01 -> 1.67 ms; 131,072 x 8,192, stored noise (12.9 GB written): 2.17 -> 1.81 ms.
+// recomputed noise: ask 2.01 -> 1.67 ms; 131,072 x 8,192, stored noise (12.9 GB written): 2.17 -> 1.81 ms.  Then four of the counters'
+// products per column instead of per row (PhiloxItem), and four packed operations instead of eight for the two members: a generation
+// of the former, ask and tell, 3,133 -> 3,093 us.  Slower: the upper halves of the products from the idle fp64 pipe,
+// by multiply-adds rounded towards zero beside 2^84 (two, four, seven of the last rounds: 3,168, 3,242, 3,317 us).
 __device__ __forceinline__ float4 normal4(uint4 r)
 {
     float ra, rb, c[2], s[2];

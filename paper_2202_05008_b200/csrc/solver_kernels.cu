@@ -76,20 +76,23 @@ k_ask(const float* __restrict__ center, const float* __restrict__ sigma_vec, Phi
     const float4 c = reinterpret_cast<const float4*>(center)[quad];
     const float4 sg = reinterpret_cast<const float4*>(sigma_vec)[quad];      // one sigma per dimension
     const bool full = d0 + 4u <= D;
+    const PhiloxItem item = philox_item(quad, generation, 0u, key);
+    const fp2 c2[2] = { fp2_make(c.x, c.y), fp2_make(c.z, c.w) }, s2[2] = { fp2_make(sg.x, sg.y), fp2_make(sg.z, sg.w) };
+    const fp2 n2[2] = { fp2_make(-sg.x, -sg.y), fp2_make(-sg.z, -sg.w) };
     for (uint32_t j = blockIdx.y * pairs_per_thread; j < H; j += gridDim.y * pairs_per_thread) {
         const uint32_t jend = min(j + pairs_per_thread, H);
         for (uint32_t jj = j; jj < jend; ++jj) {
-            float4 z = stream_normal4(key, 0u, generation, pair0 + jj, quad);   // counters use the global pair
+            float4 z = normal4(philox4x32_10(item, pair0 + jj, key));         // counters use the global pair
             if (!full) {                       // ragged tail and padding columns carry zeros
                 if (d0 + 0u >= D) z.x = 0.f;
                 if (d0 + 1u >= D) z.y = 0.f;
                 if (d0 + 2u >= D) z.z = 0.f;
                 if (d0 + 3u >= D) z.w = 0.f;
             }
-            const float4 tp = make_float4(__fmaf_rn(sg.x, z.x, c.x), __fmaf_rn(sg.y, z.y, c.y),
-                                          __fmaf_rn(sg.z, z.z, c.z), __fmaf_rn(sg.w, z.w, c.w));
-            const float4 tm = make_float4(__fmaf_rn(-sg.x, z.x, c.x), __fmaf_rn(-sg.y, z.y, c.y),
-                                          __fmaf_rn(-sg.z, z.z, c.z), __fmaf_rn(-sg.w, z.w, c.w));
+            const fp2 z2[2] = { fp2_make(z.x, z.y), fp2_make(z.z, z.w) };
+            float4 tp, tm;
+            fp2_split(fp2_fma(s2[0], z2[0], c2[0]), tp.x, tp.y); fp2_split(fp2_fma(s2[1], z2[1], c2[1]), tp.z, tp.w);
+            fp2_split(fp2_fma(n2[0], z2[0], c2[0]), tm.x, tm.y); fp2_split(fp2_fma(n2[1], z2[1], c2[1]), tm.z, tm.w);
             float* row = theta + static_cast<size_t>(2u * jj) * ldD + d0;
             if (EVO_IN_BOUNDS(status, EVO_SITE_ASK_THETA, static_cast<size_t>(2u * jj + 1u) * ldD + d0 + 3u,
                               static_cast<size_t>(2u * H) * ldD)) {
@@ -246,12 +249,11 @@ __device__ __forceinline__ void acc_fma(Acc4& a, double wd, const float4& e)
     a.z = fma(wd, static_cast<double>(e.z), a.z);
     a.w = fma(wd, static_cast<double>(e.w), a.w);
 }
-__device__ __forceinline__ void sig_fma(float4& a, float sj, const float4& e)
+__device__ __forceinline__ void sig_fma(fp2 (&a)[2], float sj, const float4& e)
 {
-    a.x = fmaf(sj, fmaf(e.x, e.x, -1.0f), a.x);
-    a.y = fmaf(sj, fmaf(e.y, e.y, -1.0f), a.y);
-    a.z = fmaf(sj, fmaf(e.z, e.z, -1.0f), a.z);
-    a.w = fmaf(sj, fmaf(e.w, e.w, -1.0f), a.w);
+    const fp2 s = fp2_both(sj), z[2] = { fp2_make(e.x, e.y), fp2_make(e.z, e.w) };
+#pragma unroll
+    for (int i = 0; i < 2; ++i) a[i] = fp2_fma(s, fp2_fma(z[i], z[i], fp2_both(-1.0f)), a[i]);
 }
 
 __device__ __forceinline__ double power(double b, uint32_t n)
@@ -449,8 +451,10 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
     const uint32_t j1 = min(H, j0 + pairs_per_split);
     const uint32_t first = j0 + lane;
     const float2* up = reinterpret_cast<const float2*>(u) + pair0;    // u is global, eps rows are the shard's
+    PhiloxItem item;
+    if (REGEN) item = philox_item(quad, generation, 0u, key);
     auto noise = [&](uint32_t j) -> float4 {
-        if (REGEN) return stream_normal4(key, 0u, generation, pair0 + j, quad);
+        if (REGEN) return normal4(philox4x32_10(item, pair0 + j, key));
         return __ldcs(reinterpret_cast<const float4*>(eps + static_cast<size_t>(j) * ldD) + quad);
     };
     constexpr bool kPrefetch = RANK && !REGEN;             // the first rows of stored noise are on their way while the ranks are counted
@@ -495,7 +499,7 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
     }
 
     Acc4 acc = { 0., 0., 0., 0. }, acc2 = acc;             // two chains of sums
-    float4 sacc = make_float4(0.f, 0.f, 0.f, 0.f), sacc2 = sacc;
+    fp2 sacc[2] = { 0ull, 0ull }, sacc2[2] = { 0ull, 0ull };
     if (live) {
         auto weight = [&](uint32_t j) { return RANK ? uu_s[j - j0] : __ldg(up + j); };
         auto add = [&](int i, const float2& uu, const float4& z) {
@@ -527,16 +531,18 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
                 if (j + i * kTellLanes < j1) add(i, weight(j + i * kTellLanes), noise(j + i * kTellLanes));
         }
         acc.x += acc2.x; acc.y += acc2.y; acc.z += acc2.z; acc.w += acc2.w;
-        if (SIGMA) { sacc.x += sacc2.x; sacc.y += sacc2.y; sacc.z += sacc2.z; sacc.w += sacc2.w; }
+        if (SIGMA) { sacc[0] = fp2_add(sacc[0], sacc2[0]); sacc[1] = fp2_add(sacc[1], sacc2[1]); }
     }
+    float sr[4];
+    fp2_split(sacc[0], sr[0], sr[1]);
+    fp2_split(sacc[1], sr[2], sr[3]);
     // the pair lanes in order
     if (lane > 0) {
         sums[lane - 1u][q][0] = acc.x; sums[lane - 1u][q][1] = acc.y; sums[lane - 1u][q][2] = acc.z; sums[lane - 1u][q][3] = acc.w;
-        if (SIGMA) { ssums[lane - 1u][q][0] = sacc.x; ssums[lane - 1u][q][1] = sacc.y; ssums[lane - 1u][q][2] = sacc.z; ssums[lane - 1u][q][3] = sacc.w; }
+        if (SIGMA) { ssums[lane - 1u][q][0] = sr[0]; ssums[lane - 1u][q][1] = sr[1]; ssums[lane - 1u][q][2] = sr[2]; ssums[lane - 1u][q][3] = sr[3]; }
     }
     __syncthreads();
     double r[4] = { acc.x, acc.y, acc.z, acc.w };
-    float sr[4] = { sacc.x, sacc.y, sacc.z, sacc.w };
     if (lane == 0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
