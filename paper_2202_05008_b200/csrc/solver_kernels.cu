@@ -675,6 +675,22 @@ uint32_t gradient_splits(uint32_t H, uint32_t ldD)
     return s < 1u ? 1u : s;
 }
 
+// The splits of a launch with stored noise, out of at most `most`: as many waves of blocks as it takes, each as long as a block's pairs and what
+// a block costs besides, about 20 pairs (its first loads, the sums of its lanes, the partial sums' way through memory).  tell, with all
+// splits / with these, sigma constant and adapted: 300 members x 40,256 columns 23.2 / 21.6 and 25.7 / 22.6 us, 500 x 60,000 28.6 / 23.6 and 33.8 / 29.7,
+// 600 x 90,000 40.0 / 31.8 and 52.3 / 42.1, 200 x 100,000 27.6 / 23.8 and 32.7 / 21.0; 131,072 x 16,384 and few columns keep theirs.  Recomputed
+// noise is bound by issue and keeps all (300 x 40,256 29.2 / 29.2, 1,000 x 48,000 52.3 / 56.1, 600 x 90,000 58.4 / 56.3).
+static uint32_t whole_waves(uint32_t bx, uint32_t H, uint32_t most, uint32_t places)
+{
+    uint32_t best = most;
+    uint64_t least = ~0ull;
+    for (uint32_t s = most; s >= 1u; --s) {
+        const uint64_t time = (static_cast<uint64_t>(bx) * s + places - 1u) / places * ((H + s - 1u) / s + 20u);
+        if (time < least) { least = time; best = s; }
+    }
+    return best;
+}
+
 size_t clipup_norm_doubles(uint32_t ldD) { return 3u * (tell_blocks(ldD) + 1u); }
 size_t tell_counter_words(uint32_t ldD) { return tell_blocks(ldD) + 1u; }
 
@@ -702,7 +718,8 @@ static cudaError_t launch_tell_kernel(cudaStream_t st, const TellArgs& a, const 
 // ranks + gradient sums (+ the step, unless mode is kStepSums)
 static int launch_tell(cudaStream_t st, const TellArgs& a, uint32_t mode, double* grad_sum, float* sigma_sum)
 {
-    const uint32_t pps = (a.H + a.splits - 1u) / a.splits;
+    const uint32_t splits = a.eps ? whole_waves(tell_blocks(a.ldD), a.H, a.splits, kSms * (a.sigma_partial ? 3u : 5u)) : a.splits;
+    const uint32_t pps = (a.H + splits - 1u) / splits;
     const dim3 grid(tell_blocks(a.ldD), (a.H + pps - 1u) / pps);       // splits that own at least one pair
     // Every column block repeats the ranking of its split's members, P comparisons each: worth it while the repetition costs
     // less than a launch.  A generation of ask and tell, ranked inside / by k_rank: 128 members x 2,000 columns 12.8 / 14.8 us, 200 x 6,000

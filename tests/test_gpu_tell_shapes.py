@@ -102,3 +102,10 @@ def test_clipup_moves_many_columns_in_a_kernel_of_its_own(D, launches):
     s.tell(torch.randn(8, device="cuda"))
     assert s.launch_count() - before == launches and s.sync_status() == 0
     s.close()
+
+
+@pytest.mark.parametrize("P,D", [(300, 40256), (202, 60001), (1000, 20000)])
+@pytest.mark.parametrize("noise_mode", [W.NOISE_STORED, W.NOISE_REGENERATED])
+def test_tells_of_fewer_splits_than_there_is_room_for(P, D, noise_mode):
+    """Column blocks times splits just above a wave or two of blocks: the launch takes fewer, longer splits."""
+    test_tell_shapes(P, D, noise_mode, clipup=False)
