@@ -192,15 +192,17 @@ __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, ui
 {
     dep_wait();
     dep_trigger();
-    const uint32_t m = blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t m = blockIdx.x * 8u + (threadIdx.x >> 5), lane = threadIdx.x & 31u;         // a warp per member
     if (m >= P) return;
     float s = 0.f;
-    for (uint32_t t = 0; t < n_chunks; ++t) s += partial[static_cast<size_t>(m) * n_chunks + t];
-    fitness[m] = -s * inv_count;
+    for (uint32_t t = lane; t < n_chunks; t += 32u) s += partial[static_cast<size_t>(m) * n_chunks + t];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0u) fitness[m] = -s * inv_count;
 }
 
 // ------------------------------------------------------------------------------------------
-// Narrow cells (h = 32, 64, 96) on warp-level tensor-core products.  Block = (member, up to 64 queries); a warp owns 8
+// Narrow cells (h = 32, 64, 96) on warp-level tensor-core products.  A block takes (member, up to 8 TILES queries) at a time; a warp owns 8
 // hidden units with all four of their gates, rows (input | forget) and (cell | output) of two 16-row operand tiles that
 // it keeps in registers for a whole phase, so a lane's accumulators are the four pre-activations of its
 // (unit, two queries) and the cell state never leaves its registers.  The hidden state travels through shared memory
@@ -209,10 +211,8 @@ __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, ui
 // The gates in fp32: sigma(x) = 1 / (1 + 2^(-x log2 e)), tanh(x) = 2 sigma(2 x) - 1.  The special-function unit, which takes 8
 // clocks per warp for an exponential and 16 for a reciprocal, bounds the kernel, so a cell's four gates share one
 // reciprocal and two cells share that of tanh(c): 64 clocks per cell and step.  The CUDA-core version took one
-// fp32 multiply-add per weight and query on top: h = 64, 2 digits, 300 members x 100 queries: 765 us, here 88 us.
+// fp32 multiply-add per weight and query on top: h = 64, 2 digits, 300 members x 100 queries: 765 us, here 75 us.
 // ------------------------------------------------------------------------------------------
-constexpr int kMmaTiles = 8;                     // n-tiles of 8 queries per block
-
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1)
 {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -273,160 +273,197 @@ __device__ __forceinline__ uint4 readout_tile(const float* oW, int k, int lane)
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-template <int H>
-__global__ void __launch_bounds__(4 * H)
-k_s2s_mma(const S2sArgs a, uint32_t chunk_q)
+// A block has `chunk` n-tiles of a member, or (RUNS) a run of the n-tiles of all members, which are dealt out evenly to the blocks and
+// worked off in pieces of one member and up to TILES tiles.
+template <int H, int TILES, bool RUNS>
+__global__ void __launch_bounds__(4 * H, H == 32 ? 6 : H == 64 ? 2 : 1)
+k_s2s_mma(const S2sArgs a, uint32_t chunk)
 {
-    constexpr int KH = H / 16, KT = KH + 1, kWarps = H / 8, kQ = 8 * kMmaTiles;
+    constexpr int KH = H / 16, KT = KH + 1, kWarps = H / 8, kQ = 8 * TILES;
     constexpr uint32_t kPitch = (H + 16) * 2 + 16;               // bytes per query of the operand: rows of 8 queries fall in distinct banks
     __shared__ __align__(16) unsigned char bop[2 * kQ * kPitch + 32];      // two buffers (the last row's last k-tile is read with the 16 bytes behind it)
     __shared__ __align__(16) uint4 out_w[KH * 32];               // read-out weights in operand order
     __shared__ float out_b[16];
     __shared__ uint8_t enc[kQ][kS2sMaxTe], dec[kQ][kS2sMaxTd], tgt[kQ][kS2sMaxTd];
-    __shared__ float loss_w[kWarps];
+    __shared__ float losses[RUNS ? TILES : kWarps];             // of a run's tiles (which block has a tile changes nothing), or of the warps
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t4 = lane & 3;
-    const uint32_t member = blockIdx.x, q0 = blockIdx.y * chunk_q;
-    const uint32_t nq = min(chunk_q, a.B - q0), nt = (nq + 7u) / 8u;
     const uint32_t Te = 2 * a.nd + 1, Td = a.nd + 1, T = Te + Td;
     const PhiloxKey key = philox_key(a.k0, a.k1);
     dep_wait();
     dep_trigger();
-    const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
     constexpr size_t cell = static_cast<size_t>(4) * H * kVocab + static_cast<size_t>(4) * H * H + 4u * H;
-
-    if (tid < kQ) s2s_query(key, a.status->generation, q0 + min(static_cast<uint32_t>(tid), nq - 1u), a.nd, enc[tid], dec[tid], tgt[tid]);
-    for (uint32_t i = tid; i < sizeof(bop) / 16u; i += 4 * H) reinterpret_cast<uint4*>(bop)[i] = make_uint4(0u, 0u, 0u, 0u);
-    {
-        const float* oW = p + 2 * cell;
-        for (int i = tid; i < KH * 32; i += 4 * H) out_w[i] = readout_tile<H>(oW, i >> 5, i & 31);
-        if (tid < 16) out_b[tid] = tid < kVocab ? __ldg(oW + kVocab * H + tid) : 0.f;
+    uint32_t at, run_end, nt;                                    // this block's run, in tiles of all members; tiles of the piece
+    if (!RUNS) {
+        const uint32_t per_member = (a.n_chunks + chunk - 1u) / chunk, m = blockIdx.x / per_member;
+        at = m * a.n_chunks + (blockIdx.x % per_member) * chunk;
+        run_end = min(at + chunk, (m + 1u) * a.n_chunks);
+    } else {
+        const uint64_t all = static_cast<uint64_t>(a.P) * a.n_chunks;
+        at = static_cast<uint32_t>(all * blockIdx.x / gridDim.x);
+        run_end = static_cast<uint32_t>(all * (blockIdx.x + 1u) / gridDim.x);
     }
-    __syncthreads();
-    auto write_token = [&](uint32_t buf, uint32_t n, uint32_t tok) {
-        uint32_t w[8];
-        const uint32_t one = (tok & 1u) ? 0x3F800000u : 0x00003F80u;      // bf16 1.0 in the upper / lower half
-#pragma unroll
-        for (uint32_t i = 0; i < 8u; ++i) w[i] = (i == (tok >> 1)) ? one : 0u;
-        w[6] |= 0x00003F80u;                                      // input 12: the constant 1 of the bias
-        uint4* dst = reinterpret_cast<uint4*>(bop + buf * (kQ * kPitch) + n * kPitch + H * 2);
-        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    };
-    if (tid < kQ) write_token(0u, tid, enc[tid][0]);
+    do {
+        const uint32_t member = at / a.n_chunks, tile0 = at % a.n_chunks;
+        nt = run_end - at;
+        if (RUNS) {
+            const uint32_t left = min(nt, a.n_chunks - tile0), pieces = (left + TILES - 1u) / TILES;
+            nt = (left + pieces - 1u) / pieces;
+        }
+        const uint32_t q0 = tile0 * 8u, nq = min(nt * 8u, a.B - q0);
+        const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
+        if (RUNS) __syncthreads();                                   // the piece before is done with shared memory
 
-    float c[kMmaTiles][2];
-#pragma unroll
-    for (int j = 0; j < kMmaTiles; ++j) c[j][0] = c[j][1] = 0.f;
-    float loss = 0.f;
-    const uint32_t bop0 = smem_u32(bop), ld_row = (lane & 7) * kPitch + 16u * (lane >> 3), st_row = lane * kPitch + 16u * warp;
-    const int u = 8 * warp + g;                                   // this lane's hidden unit
-
-    for (uint32_t phase = 0; phase < 2u; ++phase) {
-        const float* Wx = p + (phase ? cell : 0);
-        const float* Wh = Wx + static_cast<size_t>(4) * H * kVocab;
-        const float* bb = Wh + static_cast<size_t>(4) * H * H;
-        uint4 w[2][KT];
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-#pragma unroll
-            for (int k = 0; k < KT; ++k) {
-                uint32_t v[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int gate = 2 * m + (j & 1), row = gate * H + u, col = 2 * t4 + 8 * (j >> 1);
-                    const float s = gate == 2 ? 2.0f : 1.0f;      // the cell gate is doubled (exact in bf16)
-                    if (k < KH) {
-                        const float2 x = __ldg(reinterpret_cast<const float2*>(Wh + static_cast<size_t>(row) * H + 16 * k + col));
-                        v[j] = pack_bf16(s * x.x, s * x.y);
-                    } else {
-                        const float x = col < kVocab ? __ldg(Wx + row * kVocab + col) : col == kVocab ? __ldg(bb + row) : 0.f;
-                        const float y = col < kVocab ? __ldg(Wx + row * kVocab + col + 1) : 0.f;
-                        v[j] = pack_bf16(s * x, s * y);
-                    }
-                }
-                w[m][k] = make_uint4(v[0], v[1], v[2], v[3]);
-            }
-        __syncthreads();
-        for (uint32_t t = phase ? Te : 0u; t < (phase ? T : Te); ++t) {
-            const uint32_t src = bop0 + (t & 1u) * (kQ * kPitch), dst = bop0 + ((t + 1u) & 1u) * (kQ * kPitch);
-#pragma unroll
-            for (int j4 = 0; j4 < kMmaTiles; j4 += 4) {
-                if (static_cast<uint32_t>(j4) < nt) {
-                    uint32_t hp[4];
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        const int j = j4 + jj;
-                        hp[jj] = 0u;
-                        if (static_cast<uint32_t>(j) < nt) {
-                            float x[4], y[4];                     // (input, forget) and (cell, output) of two queries
-                            const uint32_t row = src + j * 8u * kPitch + ld_row;
-#pragma unroll
-                            for (int k = 0; k < KT; k += 2) {
-                                uint32_t b0, b1, b2, b3;
-                                asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                             : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
-                                if (k == 0) { mma_bf16_first(x, w[0][0], b0, b1); mma_bf16_first(y, w[1][0], b0, b1); }
-                                else { mma_bf16(x, w[0][k], b0, b1); mma_bf16(y, w[1][k], b0, b1); }
-                                if (k + 1 < KT) { mma_bf16(x, w[0][k + 1 < KT ? k + 1 : k], b2, b3); mma_bf16(y, w[1][k + 1 < KT ? k + 1 : k], b2, b3); }
-                            }
-                            const float o0 = lstm_cell(x[0], x[2], y[0], y[2], c[j][0]);
-                            const float o1 = lstm_cell(x[1], x[3], y[1], y[3], c[j][1]);
-                            float t0, t1;
-                            tanh_two(c[j][0], c[j][1], t0, t1);
-                            hp[jj] = pack_bf16(o0 * t0, o1 * t1);
-                        }
-                    }
-                    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
-                                 :: "r"(dst + j4 * 8u * kPitch + st_row), "r"(hp[0]), "r"(hp[1]), "r"(hp[2]), "r"(hp[3]) : "memory");
-                }
-            }
-            if (t + 1u < T && tid < kQ) write_token((t + 1u) & 1u, tid, t + 1u < Te ? enc[tid][t + 1u] : dec[tid][t + 1u - Te]);
-            __syncthreads();
-            if (t >= Te) {
-                // read-out and cross-entropy of this position, an n-tile per warp; the next step's products need the same buffer
-                for (uint32_t j = warp; j < nt; j += kWarps) {
-                    float l[4];
-                    const uint32_t row = dst + j * 8u * kPitch + ld_row;
-#pragma unroll
-                    for (int k = 0; k < KH; k += 2) {
-                        uint32_t b0, b1, b2, b3;
-                        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                     : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
-                        if (k == 0) mma_bf16_first(l, out_w[lane], b0, b1);
-                        else mma_bf16(l, out_w[k * 32 + lane], b0, b1);
-                        mma_bf16(l, out_w[k * 32 + 32 + lane], b2, b3);
-                    }
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {                 // query 2 t4 + i: token g and, for g < 4, token g + 8
-                        const uint32_t n = j * 8u + 2u * t4 + i;
-                        const int target = tgt[n][t - Te];
-                        const float l0 = l[i] + out_b[g], l1 = g < kVocab - 8 ? l[2 + i] + out_b[g + 8] : -INFINITY;
-                        float mx = fmaxf(l0, l1), at = target == g ? l0 : target == g + 8 ? l1 : 0.f;
-#pragma unroll
-                        for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-                        float se = expf(l0 - mx) + (g < kVocab - 8 ? expf(l1 - mx) : 0.f);
-#pragma unroll
-                        for (int off = 4; off < 32; off <<= 1) {
-                            se += __shfl_xor_sync(0xffffffffu, se, off);
-                            at += __shfl_xor_sync(0xffffffffu, at, off);
-                        }
-                        if (g == 0 && n < nq) loss += (mx + logf(se)) - at;
-                    }
-                }
-            }
+        float loss = 0.f;
+        if (RUNS && tid < TILES) losses[tid] = 0.f;
+        if (tid < kQ) s2s_query(key, a.status->generation, q0 + min(static_cast<uint32_t>(tid), nq - 1u), a.nd, enc[tid], dec[tid], tgt[tid]);
+        for (uint32_t i = tid; i < sizeof(bop) / 16u; i += 4 * H) reinterpret_cast<uint4*>(bop)[i] = make_uint4(0u, 0u, 0u, 0u);
+        {
+            const float* oW = p + 2 * cell;
+            for (int i = tid; i < KH * 32; i += 4 * H) out_w[i] = readout_tile<H>(oW, i >> 5, i & 31);
+            if (tid < 16) out_b[tid] = tid < kVocab ? __ldg(oW + kVocab * H + tid) : 0.f;
         }
         __syncthreads();
-    }
+        auto write_token = [&](uint32_t buf, uint32_t n, uint32_t tok) {
+            uint32_t w[8];
+            const uint32_t one = (tok & 1u) ? 0x3F800000u : 0x00003F80u;      // bf16 1.0 in the upper / lower half
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
-    if (lane == 0) loss_w[warp] = loss;
-    __syncthreads();
-    if (tid == 0) {
-        float total = 0.f;
-        for (int i = 0; i < kWarps; ++i) total += loss_w[i];
-        a.partial[static_cast<size_t>(member) * a.n_chunks + blockIdx.y] = total;
-    }
+            for (uint32_t i = 0; i < 8u; ++i) w[i] = (i == (tok >> 1)) ? one : 0u;
+            w[6] |= 0x00003F80u;                                      // input 12: the constant 1 of the bias
+            uint4* dst = reinterpret_cast<uint4*>(bop + buf * (kQ * kPitch) + n * kPitch + H * 2);
+            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        };
+        if (tid < kQ) write_token(0u, tid, enc[tid][0]);
+
+        float c[TILES][2];
+#pragma unroll
+        for (int j = 0; j < TILES; ++j) c[j][0] = c[j][1] = 0.f;
+        const uint32_t bop0 = smem_u32(bop), ld_row = (lane & 7) * kPitch + 16u * (lane >> 3), st_row = lane * kPitch + 16u * warp;
+        const int u = 8 * warp + g;                                   // this lane's hidden unit
+
+        for (uint32_t phase = 0; phase < 2u; ++phase) {
+            const float* Wx = p + (phase ? cell : 0);
+            const float* Wh = Wx + static_cast<size_t>(4) * H * kVocab;
+            const float* bb = Wh + static_cast<size_t>(4) * H * H;
+            uint4 w[2][KT];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int k = 0; k < KT; ++k) {
+                    uint32_t v[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int gate = 2 * m + (j & 1), row = gate * H + u, col = 2 * t4 + 8 * (j >> 1);
+                        const float s = gate == 2 ? 2.0f : 1.0f;      // the cell gate is doubled (exact in bf16)
+                        if (k < KH) {
+                            const float2 x = __ldg(reinterpret_cast<const float2*>(Wh + static_cast<size_t>(row) * H + 16 * k + col));
+                            v[j] = pack_bf16(s * x.x, s * x.y);
+                        } else {
+                            const float x = col < kVocab ? __ldg(Wx + row * kVocab + col) : col == kVocab ? __ldg(bb + row) : 0.f;
+                            const float y = col < kVocab ? __ldg(Wx + row * kVocab + col + 1) : 0.f;
+                            v[j] = pack_bf16(s * x, s * y);
+                        }
+                    }
+                    w[m][k] = make_uint4(v[0], v[1], v[2], v[3]);
+                }
+            __syncthreads();
+            for (uint32_t t = phase ? Te : 0u; t < (phase ? T : Te); ++t) {
+                const uint32_t src = bop0 + (t & 1u) * (kQ * kPitch), dst = bop0 + ((t + 1u) & 1u) * (kQ * kPitch);
+#pragma unroll
+                for (int j4 = 0; j4 < TILES; j4 += 4) {
+                    if (static_cast<uint32_t>(j4) < nt) {
+                        uint32_t hp[4];
+#pragma unroll
+                        for (int jj = 0; jj < 4; ++jj) {
+                            const int j = j4 + jj;
+                            hp[jj] = 0u;
+                            if (j < TILES && static_cast<uint32_t>(j) < nt) {
+                                float x[4], y[4];                     // (input, forget) and (cell, output) of two queries
+                                const uint32_t row = src + j * 8u * kPitch + ld_row;
+#pragma unroll
+                                for (int k = 0; k < KT; k += 2) {
+                                    uint32_t b0, b1, b2, b3;
+                                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                                 : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
+                                    if (k == 0) { mma_bf16_first(x, w[0][0], b0, b1); mma_bf16_first(y, w[1][0], b0, b1); }
+                                    else { mma_bf16(x, w[0][k], b0, b1); mma_bf16(y, w[1][k], b0, b1); }
+                                    if (k + 1 < KT) { mma_bf16(x, w[0][k + 1 < KT ? k + 1 : k], b2, b3); mma_bf16(y, w[1][k + 1 < KT ? k + 1 : k], b2, b3); }
+                                }
+                                const float o0 = lstm_cell(x[0], x[2], y[0], y[2], c[j % TILES][0]);
+                                const float o1 = lstm_cell(x[1], x[3], y[1], y[3], c[j % TILES][1]);
+                                float t0, t1;
+                                tanh_two(c[j % TILES][0], c[j % TILES][1], t0, t1);
+                                hp[jj] = pack_bf16(o0 * t0, o1 * t1);
+                            }
+                        }
+                        if (j4 + 4 <= TILES)
+                            asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};"
+                                         :: "r"(dst + j4 * 8u * kPitch + st_row), "r"(hp[0]), "r"(hp[1]), "r"(hp[2]), "r"(hp[3]) : "memory");
+                        else                                          // (rows of lanes 16 to 31 are not used)
+                            asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};"
+                                         :: "r"(dst + j4 * 8u * kPitch + st_row), "r"(hp[0]), "r"(hp[1]) : "memory");
+                    }
+                }
+                if (t + 1u < T && tid < kQ) write_token((t + 1u) & 1u, tid, t + 1u < Te ? enc[tid][t + 1u] : dec[tid][t + 1u - Te]);
+                __syncthreads();
+                if (t >= Te) {
+                    // read-out and cross-entropy of this position, an n-tile per warp; the next step's products need the same buffer
+                    for (uint32_t j = warp; j < nt; j += kWarps) {
+                        float l[4];
+                        if (RUNS) loss = 0.f;
+                        const uint32_t row = dst + j * 8u * kPitch + ld_row;
+#pragma unroll
+                        for (int k = 0; k < KH; k += 2) {
+                            uint32_t b0, b1, b2, b3;
+                            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                                         : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 32u * k));
+                            if (k == 0) mma_bf16_first(l, out_w[lane], b0, b1);
+                            else mma_bf16(l, out_w[k * 32 + lane], b0, b1);
+                            mma_bf16(l, out_w[k * 32 + 32 + lane], b2, b3);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {                 // query 2 t4 + i: token g and, for g < 4, token g + 8
+                            const uint32_t n = j * 8u + 2u * t4 + i;
+                            const int target = tgt[n][t - Te];
+                            const float l0 = l[i] + out_b[g], l1 = g < kVocab - 8 ? l[2 + i] + out_b[g + 8] : -INFINITY;
+                            float mx = fmaxf(l0, l1), hit = target == g ? l0 : target == g + 8 ? l1 : 0.f;
+#pragma unroll
+                            for (int off = 4; off < 32; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+                            float se = expf(l0 - mx) + (g < kVocab - 8 ? expf(l1 - mx) : 0.f);
+#pragma unroll
+                            for (int off = 4; off < 32; off <<= 1) {
+                                se += __shfl_xor_sync(0xffffffffu, se, off);
+                                hit += __shfl_xor_sync(0xffffffffu, hit, off);
+                            }
+                            if (g == 0 && n < nq) loss += (mx + logf(se)) - hit;
+                        }
+                        if (RUNS) {
+                            loss += __shfl_xor_sync(0xffffffffu, loss, 1);
+                            loss += __shfl_xor_sync(0xffffffffu, loss, 2);
+                            if (lane == 0) losses[j] += loss;
+                        }
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        float* const out = a.partial + static_cast<size_t>(member) * a.n_chunks + tile0;
+        if constexpr (RUNS) {
+            if (tid < static_cast<int>(nt)) out[tid] = losses[tid];
+        } else {                                                     // a chunk's sum stands at its first tile
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
+            if (lane == 0) losses[warp] = loss;
+            __syncthreads();
+            if (tid < static_cast<int>(nt)) {
+                float total = 0.f;
+                for (int i = 0; i < kWarps; ++i) total += losses[i];
+                out[tid] = tid == 0 ? total : 0.f;
+            }
+        }
+        at += nt;
+    } while (RUNS && at < run_end);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -800,14 +837,23 @@ bool s2s_supported(uint32_t h, uint32_t nd, uint32_t B)
 
 static uint32_t s2s_chunks(uint32_t B, bool tc) { return tc ? (B + kTcQ - 1) / kTcQ : (B + kSimpleQ - 1) / kSimpleQ; }
 
-// Queries per block of the narrow kernel: up to 64, spread evenly over the fewest chunks, in whole n-tiles; a small population
-// takes smaller chunks (down to one tile of 8) until there are two blocks for every SM.
-static uint32_t s2s_mma_chunk(uint32_t P, uint32_t B)
+// Chunks of up to 64 queries, spread evenly over the fewest chunks, in whole n-tiles; a small population takes smaller ones (down to
+// one tile) until there are two blocks for every SM.  More blocks of wide cells than the SMs hold at once (two blocks of 64 units, one of 96) would
+// leave the last wave nearly empty or end in many of them: each SM then gets its runs.  300 members x 100 queries, 2 digits, chunks / runs:
+// 64 units 85 / 77 us, 96 units 181 / 149; 296 members x 104: 68 / 64 and 151 / 133; 600 x 56: 94 / 96 and 192 / 168.  Cells of 32 units
+// hold six blocks to an SM and lose: 300 x 100 40 / 51.  Runs of 64 units are worked off in pieces of up to 14 tiles; as blocks of a
+// single chunk that instance is slower for its length (148 x 8 17.5 / 23.1).
+static cudaError_t launch_s2s_mma(cudaStream_t st, const S2sArgs& a)
 {
-    const uint32_t tiles = (B + 7u) / 8u;
-    uint32_t chunks = (tiles + kMmaTiles - 1u) / kMmaTiles;
-    while (chunks < tiles && static_cast<uint64_t>(P) * chunks < 2u * kSms) ++chunks;
-    return (tiles + chunks - 1u) / chunks * 8u;
+    const uint32_t tiles = a.n_chunks;
+    uint32_t chunks = (tiles + 7u) / 8u;
+    while (chunks < tiles && static_cast<uint64_t>(a.P) * chunks < 2u * kSms) ++chunks;
+    const uint32_t chunk = (tiles + chunks - 1u) / chunks, places = kSms * (a.h == 64u ? 2u : 1u);
+    const uint64_t blocks = static_cast<uint64_t>(a.P) * ((tiles + chunk - 1u) / chunk);
+    if (a.h != 32u && blocks > places)
+        return launch_dependent(a.h == 64u ? k_s2s_mma<64, 14, true> : k_s2s_mma<96, 8, true>, dim3(places), dim3(4u * a.h), 0, st, a, 0u);
+    return launch_dependent(a.h == 32u ? k_s2s_mma<32, 8, false> : a.h == 64u ? k_s2s_mma<64, 8, false> : k_s2s_mma<96, 8, false>, dim3(static_cast<uint32_t>(blocks)),
+                            dim3(4u * a.h), 0, st, a, chunk);
 }
 
 size_t s2s_scratch_bytes(uint32_t P, uint32_t B)
@@ -828,8 +874,7 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
     a.theta = theta; a.ldD = ldD; a.P = P; a.h = h; a.nd = nd; a.B = B;
     a.k0 = k0; a.k1 = k1; a.status = status;
     a.partial = static_cast<float*>(scratch);
-    const uint32_t chunk_q = mma ? s2s_mma_chunk(P, B) : 0u;
-    a.n_chunks = mma ? (B + chunk_q - 1u) / chunk_q : s2s_chunks(B, tc);
+    a.n_chunks = mma ? (B + 7u) / 8u : s2s_chunks(B, tc);
     a.logits = logits;
     if (tc) {
         static int sm_count = 0;
@@ -844,15 +889,14 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
         const uint32_t grid = items < static_cast<uint32_t>(sm_count) ? items : static_cast<uint32_t>(sm_count);
         k_s2s_tc<<<grid, kTcThreads, sizeof(S2sSmem), st>>>(a, status);
     } else if (mma) {
-        auto kernel = h == 32u ? k_s2s_mma<32> : h == 64u ? k_s2s_mma<64> : k_s2s_mma<96>;
-        if (launch_dependent(kernel, dim3(P, a.n_chunks), dim3(4u * h), 0, st, a, chunk_q) != cudaSuccess) return -1;
+        if (launch_s2s_mma(st, a) != cudaSuccess) return -1;
     } else {
         dim3 grid(P, a.n_chunks);
         k_s2s_simple<<<grid, 128, 0, st>>>(a);
     }
     if (cudaGetLastError() != cudaSuccess) return -1;
     const float inv = 1.0f / (static_cast<float>(B) * static_cast<float>(nd + 1));
-    if (launch_dependent(k_s2s_finalize, dim3((P + 255u) / 256u), dim3(256), 0, st, a.partial, P, a.n_chunks, inv, fitness) != cudaSuccess)
+    if (launch_dependent(k_s2s_finalize, dim3((P + 7u) / 8u), dim3(256), 0, st, a.partial, P, a.n_chunks, inv, fitness) != cudaSuccess)
         return -1;
     return 2;
 }

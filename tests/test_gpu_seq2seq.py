@@ -162,3 +162,18 @@ def test_narrow_cells_on_tensor_cores_match_oracle(h, nd, B, P):
     want = _oracle_fits(w, theta[members], 0)
     for i, m in enumerate(members):
         assert abs(float(fa[m]) - want[i][0]) < FIT_TOL
+
+
+@pytest.mark.parametrize("h", [32, 64, 96])
+@pytest.mark.parametrize("nd,B,P", [(1, 100, 300), (1, 400, 60), (1, 112, 296), (1, 9, 750)])
+def test_runs_of_tiles_that_begin_and_end_inside_a_member(h, nd, B, P):
+    """The blocks' runs of n-tiles: of several members, of a part of one, in one piece and several; every member against the
+    CUDA-core kernel (both round the same operands; left are accumulation order and gates to about 3e-7)."""
+    w = _workload(h, nd, B, P=P, sigma=0.2)
+    a, b = Solver(w), Solver(w, rollout_kernel=ROLLOUT_GENERIC)
+    a.ask(); b.ask()
+    fa = a.rollout().clone(); again = a.rollout(); fb = b.rollout()
+    assert a.sync_status() == 0 and b.sync_status() == 0
+    assert torch.equal(fa, again)
+    assert torch.max(torch.abs(fa - fb)) < FIT_TOL
+    a.close(); b.close()
