@@ -34,7 +34,7 @@ def build_library(force: bool = False, verbose: bool = False, debug: bool = Fals
     if not force and not is_stale(lib):
         return lib
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "--shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3"] + \
+           "--threads", "0", "--shared", "-Xcompiler", "-fPIC", "-Xptxas", "-v" if verbose else "-O3"] + \
           (["-DEVO_DEBUG"] if debug else []) + ["-o", lib] + [os.path.join(CSRC, s) for s in SOURCES]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if verbose:
