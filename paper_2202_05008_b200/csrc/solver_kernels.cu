@@ -249,11 +249,22 @@ __device__ __forceinline__ void acc_fma(Acc4& a, double wd, const float4& e)
     a.z = fma(wd, static_cast<double>(e.z), a.z);
     a.w = fma(wd, static_cast<double>(e.w), a.w);
 }
+// PACKED: where issue bounds (recomputed noise)
+template <bool PACKED>
 __device__ __forceinline__ void sig_fma(fp2 (&a)[2], float sj, const float4& e)
 {
-    const fp2 s = fp2_both(sj), z[2] = { fp2_make(e.x, e.y), fp2_make(e.z, e.w) };
+    const float ev[4] = { e.x, e.y, e.z, e.w };
 #pragma unroll
-    for (int i = 0; i < 2; ++i) a[i] = fp2_fma(s, fp2_fma(z[i], z[i], fp2_both(-1.0f)), a[i]);
+    for (int i = 0; i < 2; ++i) {
+        if (PACKED) {
+            const fp2 z = fp2_make(ev[2 * i], ev[2 * i + 1]);
+            a[i] = fp2_fma(fp2_both(sj), fp2_fma(z, z, fp2_both(-1.0f)), a[i]);
+        } else {
+            float x, y;
+            fp2_split(a[i], x, y);
+            a[i] = fp2_make(fmaf(sj, fmaf(ev[2 * i], ev[2 * i], -1.0f), x), fmaf(sj, fmaf(ev[2 * i + 1], ev[2 * i + 1], -1.0f), y));
+        }
+    }
 }
 
 __device__ __forceinline__ double power(double b, uint32_t n)
@@ -504,7 +515,7 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
         auto weight = [&](uint32_t j) { return RANK ? uu_s[j - j0] : __ldg(up + j); };
         auto add = [&](int i, const float2& uu, const float4& z) {
             acc_fma(i & 1 ? acc2 : acc, static_cast<double>(uu.x) - static_cast<double>(uu.y), z);            // (exact difference)
-            if (SIGMA) sig_fma(i & 1 ? sacc2 : sacc, 0.5f * (uu.x + uu.y), z);
+            if (SIGMA) sig_fma<REGEN>(i & 1 ? sacc2 : sacc, 0.5f * (uu.x + uu.y), z);
         };
         uint32_t j = first;
         if constexpr (kPrefetch) {
