@@ -293,21 +293,17 @@ k_s2s_mma(const S2sArgs a, uint32_t chunk)
     dep_wait();
     dep_trigger();
     constexpr size_t cell = static_cast<size_t>(4) * H * kVocab + static_cast<size_t>(4) * H * H + 4u * H;
-    uint32_t at, run_end, nt;                                    // this block's run, in tiles of all members; tiles of the piece
-    if (!RUNS) {
-        const uint32_t per_member = (a.n_chunks + chunk - 1u) / chunk, m = blockIdx.x / per_member;
-        at = m * a.n_chunks + (blockIdx.x % per_member) * chunk;
-        run_end = min(at + chunk, (m + 1u) * a.n_chunks);
-    } else {
+    uint32_t member = blockIdx.x, tile0 = blockIdx.y * chunk, nt = min(chunk, a.n_chunks - tile0);     // first n-tile and n-tiles of the piece
+    uint32_t at = 0, run_end = 0;                                // this block's run, in tiles of all members
+    if (RUNS) {
         const uint64_t all = static_cast<uint64_t>(a.P) * a.n_chunks;
         at = static_cast<uint32_t>(all * blockIdx.x / gridDim.x);
         run_end = static_cast<uint32_t>(all * (blockIdx.x + 1u) / gridDim.x);
     }
     do {
-        const uint32_t member = at / a.n_chunks, tile0 = at % a.n_chunks;
-        nt = run_end - at;
         if (RUNS) {
-            const uint32_t left = min(nt, a.n_chunks - tile0), pieces = (left + TILES - 1u) / TILES;
+            member = at / a.n_chunks; tile0 = at % a.n_chunks;
+            const uint32_t left = min(run_end - at, a.n_chunks - tile0), pieces = (left + TILES - 1u) / TILES;
             nt = (left + pieces - 1u) / pieces;
         }
         const uint32_t q0 = tile0 * 8u, nq = min(nt * 8u, a.B - q0);
@@ -849,11 +845,11 @@ static cudaError_t launch_s2s_mma(cudaStream_t st, const S2sArgs& a)
     uint32_t chunks = (tiles + 7u) / 8u;
     while (chunks < tiles && static_cast<uint64_t>(a.P) * chunks < 2u * kSms) ++chunks;
     const uint32_t chunk = (tiles + chunks - 1u) / chunks, places = kSms * (a.h == 64u ? 2u : 1u);
-    const uint64_t blocks = static_cast<uint64_t>(a.P) * ((tiles + chunk - 1u) / chunk);
-    if (a.h != 32u && blocks > places)
+    chunks = (tiles + chunk - 1u) / chunk;
+    if (a.h != 32u && static_cast<uint64_t>(a.P) * chunks > places)
         return launch_dependent(a.h == 64u ? k_s2s_mma<64, 14, true> : k_s2s_mma<96, 8, true>, dim3(places), dim3(4u * a.h), 0, st, a, 0u);
-    return launch_dependent(a.h == 32u ? k_s2s_mma<32, 8, false> : a.h == 64u ? k_s2s_mma<64, 8, false> : k_s2s_mma<96, 8, false>, dim3(static_cast<uint32_t>(blocks)),
-                            dim3(4u * a.h), 0, st, a, chunk);
+    return launch_dependent(a.h == 32u ? k_s2s_mma<32, 8, false> : a.h == 64u ? k_s2s_mma<64, 8, false> : k_s2s_mma<96, 8, false>,
+                            dim3(a.P, chunks), dim3(4u * a.h), 0, st, a, chunk);
 }
 
 size_t s2s_scratch_bytes(uint32_t P, uint32_t B)
