@@ -22,15 +22,18 @@
 //                 back into the B operand, the tensor cores work on the other half.  The rows of the
 //                 sigmoid gates are halved when staged, so every non-linearity is one tanh of the
 //                 special-function unit; that unit (5 tanh per cell and step) is what bounds the
-//                 kernel, not the tensor cores.  The decoder's read-out is done by the same warps, as warp-level
-//                 products on the B operand while the next step's MMAs are in flight (on the CUDA cores a
-//                 generation of 1,024 members x 128 queries took 659 us, so 645); its logits are kept and
+//                 kernel, not the tensor cores.  The decoder's read-out runs on the CUDA cores from
+//                 the B operand while the next step's MMAs are in flight: as warp-level products a generation of
+//                 1,024 members x 128 queries takes 641 us instead of 655, but these cut their sums off
+//                 where additions round (logits of 128 positive terms: relative error 3.4e-7 RMS, all of one sign,
+//                 against 0.7e-7 without bias).  The logits are kept and
 //                 the cross-entropy is taken once per item.  The next cell's weights are prefetched
 //                 into L2 while the current phase computes.  Every wait is bounded.
 #include "internal.h"
 #include "async.cuh"
 #include "noise.cuh"
 #include "umma.cuh"
+#include "fp32x2.cuh"
 
 namespace evo {
 
@@ -259,20 +262,6 @@ __device__ __forceinline__ void tanh_two(float c0, float c1, float& t0, float& t
     t1 = fmaf(2.0f, r * a, -1.0f);
 }
 
-// A lane's part of 16 inputs (tile k) of the read-out matrix [12][H], as the 16-row operand of a warp-level product
-template <int H>
-__device__ __forceinline__ uint4 readout_tile(const float* oW, int k, int lane)
-{
-    const int r = lane >> 2;
-    uint32_t w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {                                // rows r, r + 8; inputs 2 t, 2 t + 1 and the two 8 further
-        const int row = r + 8 * (j & 1), col = 16 * k + 2 * (lane & 3) + 8 * (j >> 1);
-        w[j] = row < kVocab ? pack_bf16(__ldg(oW + row * H + col), __ldg(oW + row * H + col + 1)) : 0u;
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // A block has `chunk` n-tiles of a member, or (RUNS) a run of the n-tiles of all members, which are dealt out evenly to the blocks and
 // worked off in pieces of one member and up to TILES tiles.
 template <int H, int TILES, bool RUNS>
@@ -316,7 +305,16 @@ k_s2s_mma(const S2sArgs a, uint32_t chunk)
         for (uint32_t i = tid; i < sizeof(bop) / 16u; i += 4 * H) reinterpret_cast<uint4*>(bop)[i] = make_uint4(0u, 0u, 0u, 0u);
         {
             const float* oW = p + 2 * cell;
-            for (int i = tid; i < KH * 32; i += 4 * H) out_w[i] = readout_tile<H>(oW, i >> 5, i & 31);
+            for (int i = tid; i < KH * 32; i += 4 * H) {
+                const int k = (i >> 5) * 16 + 2 * (i & 3), r = (i & 31) >> 2;
+                uint32_t v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {                    // rows r, r + 8; inputs k, k + 1 and k + 8, k + 9
+                    const int row = r + 8 * (j & 1), col = k + 8 * (j >> 1);
+                    v[j] = row < kVocab ? pack_bf16(__ldg(oW + row * H + col), __ldg(oW + row * H + col + 1)) : 0u;
+                }
+                out_w[i] = make_uint4(v[0], v[1], v[2], v[3]);
+            }
             if (tid < 16) out_b[tid] = tid < kVocab ? __ldg(oW + kVocab * H + tid) : 0.f;
         }
         __syncthreads();
@@ -471,6 +469,7 @@ constexpr int kTcSub = 1;                                  // warps per TMEM lan
 constexpr int kTcHalfThreads = 128 * kTcSub;
 constexpr int kTcEpiThreads = 2 * kTcHalfThreads;          // half 0's warps first, then half 1's
 constexpr int kTcCols = 64 / kTcSub;                       // queries per epilogue thread
+constexpr int kTcOutPerThread = kVocab * 64 / kTcHalfThreads;   // read-out: tokens per thread
 constexpr int kTcThreads = kTcEpiThreads + 32;             // + the MMA warp
 constexpr int kTcKBlocks = 18;                             // K = 128 (h) + 16 (one-hot, 1, padding) in groups of 8
 constexpr uint32_t kTcALbo = 64 * 128 + 16;                // 64 row groups of 8 x 16 bytes between K groups, +16 bytes
@@ -484,8 +483,8 @@ constexpr uint32_t kTcCellFloats = 4 * kTcH * kVocab + 4 * kTcH * kTcH + 4 * kTc
 struct __align__(128) S2sSmem {
     unsigned char A[kTcABytes];                            // [Wh | Wx | b | 0] as core matrices
     unsigned char Bop[kTcBBytes];                          // [h; onehot; 1; 0] of the 128 queries
-    uint4 oW[kTcH / 16][32];                               // read-out weights in operand order
-    float ob[16];
+    float oW[16][kVocab][8];                               // read-out weights [K group][token][k], bf16-rounded
+    float ob[kVocab];
     float lg[kS2sMaxTd][kTcQ][kVocab];                     // logits of every answer position
     uint8_t enc[kTcQ][kS2sMaxTe + 1], dec[kTcQ][kS2sMaxTd + 1], tgt[kTcQ][kS2sMaxTd + 1];
     float loss_w[kTcThreads / 32];
@@ -646,8 +645,15 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         }
         for (uint32_t i = tid; i < 16u * kTcBLbo / 16u; i += kTcThreads)
             reinterpret_cast<uint4*>(S.Bop)[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (tid < kTcH / 16 * 32) S.oW[tid >> 5][lane] = readout_tile<kTcH>(p + 2u * kTcCellFloats, tid >> 5, lane);
-        if (tid < 16u) S.ob[tid] = tid < kVocab ? p[2u * kTcCellFloats + kVocab * kTcH + tid] : 0.f;
+        for (uint32_t i = tid; i < kVocab * 16u; i += kTcThreads) {       // (token, K group) -> 8 weights
+            const uint32_t o = i >> 4, kb = i & 15u;
+            const float4* src = reinterpret_cast<const float4*>(p + 2u * kTcCellFloats + o * kTcH + kb * 8u);
+            const float4 w0 = __ldg(src), w1 = __ldg(src + 1);
+            float* dst = S.oW[kb][o];
+            dst[0] = bf16_round(w0.x); dst[1] = bf16_round(w0.y); dst[2] = bf16_round(w0.z); dst[3] = bf16_round(w0.w);
+            dst[4] = bf16_round(w1.x); dst[5] = bf16_round(w1.y); dst[6] = bf16_round(w1.z); dst[7] = bf16_round(w1.w);
+        }
+        if (tid < kVocab) S.ob[tid] = p[2u * kTcCellFloats + kVocab * kTcH + tid];
         s2s_stage_weights(S, p, tid);
         __syncthreads();                                        // tokens are there
         if (tid < kTcQ) s2s_write_onehot(S, tid, S.enc[tid][0]);
@@ -763,29 +769,35 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
                     fence_async_smem();
                     tc_fence_before();
                     if (t >= Te) {
-                        // read-out from the state just written (all warps of the half must have written it),
-                        // while the tensor cores work on the next step
+                        // read-out on the CUDA cores from the state just written (all warps of the
+                        // half must have written it), while the tensor cores work on the next step
                         half_barrier(half);
                         if (t + 1u < T && lane == 0) mbar_arrive(smem_u32(&S.hready[half]));
+                        const uint32_t s = tid & 63u, o0 = ((tid % kTcHalfThreads) >> 6) * kTcOutPerThread;
+                        float2 acc[kTcOutPerThread];
 #pragma unroll
-                        for (uint32_t i = 0; i < 2u; ++i) {      // 16 queries per warp
-                            const uint32_t n0 = half * 64u + (warp & 3u) * 16u + i * 8u;
-                            const uint32_t row = smem_u32(S.Bop) + (lane >> 3) * kTcBLbo + (n0 + (lane & 7u)) * 16u;
-                            float l[4];
+                        for (int o = 0; o < kTcOutPerThread; ++o) acc[o] = make_float2(0.f, 0.f);
+                        const unsigned char* hrow = S.Bop + (half * 64u + s) * 16u;
+#pragma unroll 4
+                        for (uint32_t kb = 0; kb < 16u; ++kb) {
+                            const uint4 hv = *reinterpret_cast<const uint4*>(hrow + kb * kTcBLbo);
+                            const uint32_t hw[4] = { hv.x, hv.y, hv.z, hv.w };
+                            float2 x[4];
 #pragma unroll
-                            for (uint32_t k = 0; k < kTcH / 16; k += 2) {
-                                uint32_t b0, b1, b2, b3;
-                                asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                             : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3) : "r"(row + 2u * k * kTcBLbo));
-                                if (k == 0) mma_bf16_first(l, S.oW[0][lane], b0, b1);
-                                else mma_bf16(l, S.oW[k][lane], b0, b1);
-                                mma_bf16(l, S.oW[k + 1][lane], b2, b3);
+                            for (int i = 0; i < 4; ++i)
+                                x[i] = make_float2(__uint_as_float(hw[i] << 16), __uint_as_float(hw[i] & 0xFFFF0000u));
+#pragma unroll
+                            for (int o = 0; o < kTcOutPerThread; ++o) {
+                                const float4 w0 = *reinterpret_cast<const float4*>(&S.oW[kb][o0 + o][0]);
+                                const float4 w1 = *reinterpret_cast<const float4*>(&S.oW[kb][o0 + o][4]);
+                                ffma2(acc[o], make_float2(w0.x, w0.y), x[0]);
+                                ffma2(acc[o], make_float2(w0.z, w0.w), x[1]);
+                                ffma2(acc[o], make_float2(w1.x, w1.y), x[2]);
+                                ffma2(acc[o], make_float2(w1.z, w1.w), x[3]);
                             }
-                            const uint32_t o = lane >> 2, q = n0 + 2u * (lane & 3u);
-                            float (&lg)[kTcQ][kVocab] = S.lg[t - Te];
-                            lg[q][o] = l[0] + S.ob[o]; lg[q + 1u][o] = l[1] + S.ob[o];
-                            if (o < kVocab - 8u) { lg[q][o + 8u] = l[2] + S.ob[o + 8u]; lg[q + 1u][o + 8u] = l[3] + S.ob[o + 8u]; }
                         }
+#pragma unroll
+                        for (int o = 0; o < kTcOutPerThread; ++o) S.lg[t - Te][half * 64u + s][o0 + o] = (acc[o].x + acc[o].y) + S.ob[o0 + o];
                         // the next epilogue overwrites the state: everyone must be done reading it
                         half_barrier(half);
                     } else {

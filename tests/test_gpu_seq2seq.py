@@ -59,6 +59,39 @@ def test_tensor_core_kernel_matches_oracle(B):
     assert np.std(fit) > 1e-3                                    # members really differ
 
 
+def test_the_read_out_is_as_exact_as_a_chain_of_fp32_additions():
+    """Gates and cells saturated by their biases: every hidden state is +-bf16(tanh 1) = +-195/256 exactly, whatever the query.  Only the
+    logit of '=' (never an answer) has weights, all of its terms positive: the loss of every position is that logit (30 and
+    more, so that the others add nothing to the exponentials), a sum of 128 products that fp32 holds exactly.  Its error may be no larger than that of two chains of 64 rounded additions (RMS; 1,024
+    members scatter by 2 %), and without their rounding's bias: a mean within 4 of its standard errors."""
+    h, P = 128, 1024
+    w = _workload(h, 1, 1, P=P)
+    rng = np.random.default_rng(2)
+    sign = rng.choice((-1.0, 1.0), (P, h)).astype(np.float32)
+    weights = (np.exp2(rng.uniform(-10.0, 2.0, (P, h))).astype(np.float32).view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+    theta = np.zeros((P, w.param_dim), np.float32)
+    cell = 4 * h * 12 + 4 * h * h + 4 * h
+    for at in (cell - 4 * h, 2 * cell - 4 * h):                  # the biases: input 1, forget 0, cell +-1, output 1
+        theta[:, at:at + h], theta[:, at + h:at + 2 * h] = 64.0, -64.0
+        theta[:, at + 2 * h:at + 3 * h], theta[:, at + 3 * h:at + 4 * h] = 64.0 * sign, 64.0
+    theta[:, 2 * cell + 11 * h:2 * cell + 12 * h] = weights * sign
+    s = Solver(w)
+    rows = s.padded_rows(P)
+    rows[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    fit = s.rollout(rows).cpu().numpy()
+    assert s.sync_status() == 0
+    s.close()
+    terms = weights * np.float32(195.0 / 256.0)
+    chains = np.zeros((P, 2), np.float32)
+    for k in range(0, h, 2):
+        chains = chains + terms[:, k:k + 2]
+    exact = terms.astype(np.float64).sum(1)
+    chain_err, err = (chains[:, 0] + chains[:, 1]) / exact - 1.0, -fit.astype(np.float64) / exact - 1.0
+    rms = lambda x: float(np.sqrt((x * x).mean()))
+    assert rms(err) <= 1.05 * rms(chain_err), (rms(err), rms(chain_err))
+    assert abs(err.mean()) <= 4.0 * err.std() / math.sqrt(P), (err.mean(), err.std())
+
+
 @pytest.mark.parametrize("kernel", [ROLLOUT_TILED, ROLLOUT_GENERIC])
 def test_kernels_against_the_unrounded_oracle(kernel):
     """Against the fp64 oracle with NO bf16 rounding (the mode pinned to torch.nn.LSTM): bound =
