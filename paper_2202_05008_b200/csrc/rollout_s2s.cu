@@ -268,13 +268,12 @@ template <int H, int TILES, bool RUNS>
 __global__ void __launch_bounds__(4 * H, H == 32 ? 6 : H == 64 ? 2 : 1)
 k_s2s_mma(const S2sArgs a, uint32_t chunk)
 {
-    constexpr int KH = H / 16, KT = KH + 1, kWarps = H / 8, kQ = 8 * TILES;
+    constexpr int KH = H / 16, KT = KH + 1, kWarps = H / 8, kQ = 8 * TILES, kOwn = (TILES + kWarps - 1) / kWarps;
     constexpr uint32_t kPitch = (H + 16) * 2 + 16;               // bytes per query of the operand: rows of 8 queries fall in distinct banks
     __shared__ __align__(16) unsigned char bop[2 * kQ * kPitch + 32];      // two buffers (the last row's last k-tile is read with the 16 bytes behind it)
     __shared__ __align__(16) uint4 out_w[KH * 32];               // read-out weights in operand order
     __shared__ float out_b[16];
     __shared__ uint8_t enc[kQ][kS2sMaxTe], dec[kQ][kS2sMaxTd], tgt[kQ][kS2sMaxTd];
-    __shared__ float losses[RUNS ? TILES : kWarps];             // of a run's tiles (which block has a tile changes nothing), or of the warps
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g = lane >> 2, t4 = lane & 3;
     const uint32_t Te = 2 * a.nd + 1, Td = a.nd + 1, T = Te + Td;
@@ -299,8 +298,9 @@ k_s2s_mma(const S2sArgs a, uint32_t chunk)
         const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
         if (RUNS) __syncthreads();                                   // the piece before is done with shared memory
 
-        float loss = 0.f;
-        if (RUNS && tid < TILES) losses[tid] = 0.f;
+        float loss[kOwn];                                            // of the n-tiles that this warp reads out
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) loss[i] = 0.f;
         if (tid < kQ) s2s_query(key, a.status->generation, q0 + min(static_cast<uint32_t>(tid), nq - 1u), a.nd, enc[tid], dec[tid], tgt[tid]);
         for (uint32_t i = tid; i < sizeof(bop) / 16u; i += 4 * H) reinterpret_cast<uint4*>(bop)[i] = make_uint4(0u, 0u, 0u, 0u);
         {
@@ -403,9 +403,11 @@ k_s2s_mma(const S2sArgs a, uint32_t chunk)
                 __syncthreads();
                 if (t >= Te) {
                     // read-out and cross-entropy of this position, an n-tile per warp; the next step's products need the same buffer
-                    for (uint32_t j = warp; j < nt; j += kWarps) {
+#pragma unroll
+                    for (int own = 0; own < kOwn; ++own) {
+                        const uint32_t j = warp + own * kWarps;
+                        if (j >= nt) break;
                         float l[4];
-                        if (RUNS) loss = 0.f;
                         const uint32_t row = dst + j * 8u * kPitch + ld_row;
 #pragma unroll
                         for (int k = 0; k < KH; k += 2) {
@@ -430,31 +432,20 @@ k_s2s_mma(const S2sArgs a, uint32_t chunk)
                                 se += __shfl_xor_sync(0xffffffffu, se, off);
                                 hit += __shfl_xor_sync(0xffffffffu, hit, off);
                             }
-                            if (g == 0 && n < nq) loss += (mx + logf(se)) - hit;
-                        }
-                        if (RUNS) {
-                            loss += __shfl_xor_sync(0xffffffffu, loss, 1);
-                            loss += __shfl_xor_sync(0xffffffffu, loss, 2);
-                            if (lane == 0) losses[j] += loss;
+                            if (g == 0 && n < nq) loss[own] += (mx + logf(se)) - hit;
                         }
                     }
                 }
             }
             __syncthreads();
         }
-        float* const out = a.partial + static_cast<size_t>(member) * a.n_chunks + tile0;
-        if constexpr (RUNS) {
-            if (tid < static_cast<int>(nt)) out[tid] = losses[tid];
-        } else {                                                     // a chunk's sum stands at its first tile
+        // a sum per n-tile, whichever block had it: the form of the launch (a shard may take another) changes no bit of the fitness
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
-            if (lane == 0) losses[warp] = loss;
-            __syncthreads();
-            if (tid < static_cast<int>(nt)) {
-                float total = 0.f;
-                for (int i = 0; i < kWarps; ++i) total += losses[i];
-                out[tid] = tid == 0 ? total : 0.f;
-            }
+        for (int own = 0; own < kOwn; ++own) {
+            const uint32_t j = warp + own * kWarps;
+            loss[own] += __shfl_xor_sync(0xffffffffu, loss[own], 1);
+            loss[own] += __shfl_xor_sync(0xffffffffu, loss[own], 2);
+            if (lane == 0 && j < nt) a.partial[static_cast<size_t>(member) * a.n_chunks + tile0 + j] = loss[own];
         }
         at += nt;
     } while (RUNS && at < run_end);

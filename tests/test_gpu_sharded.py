@@ -158,6 +158,25 @@ def test_sharded_supervised_rollout_matches_unsharded():
     assert torch.equal(fit_sh, fit_full)
 
 
+@pytest.mark.parametrize("h", [32, 64, 96, 128])
+@pytest.mark.parametrize("batch", [9, 100, 300])
+def test_sharded_seq2seq_rollout_matches_unsharded(h, batch):
+    """Shards so small that they split a member's queries otherwise than the whole population does."""
+    w = W.SEQ2SEQ.with_(pop_size=592, param_dim=W.seq2seq_param_count(h), layer_sizes=(h,), batch=batch, task_param=(2.0,), sigma=0.2)
+    full = binding.Solver(w)
+    shards = _shards(w, 8)
+    full.ask()
+    fit_full = full.rollout().clone()
+    for s in shards:
+        s.ask()
+    fit_sh = torch.cat([s.rollout().clone() for s in shards])
+    assert torch.equal(fit_sh, fit_full)
+    assert all(s.sync_status() == 0 for s in shards) and full.sync_status() == 0
+    for s in shards:
+        s.close()
+    full.close()
+
+
 def test_sharded_solver_order_and_argument_errors():
     w = W.CFG1.with_(pop_size=16)
     with pytest.raises(RuntimeError):
