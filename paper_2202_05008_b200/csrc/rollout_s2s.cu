@@ -190,18 +190,21 @@ k_s2s_simple(const S2sArgs a)
     }
 }
 
+// LANES per member.  One: the sums of its chunks in order.  Four: every fourth sum each, then the lanes as a tree, for the many sums (one
+// per 8 queries) of k_s2s_mma.
+template <int LANES>
 __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, uint32_t n_chunks, float inv_count,
                                float* __restrict__ fitness)
 {
     dep_wait();
     dep_trigger();
-    const uint32_t m = blockIdx.x * 8u + (threadIdx.x >> 5), lane = threadIdx.x & 31u;         // a warp per member
-    if (m >= P) return;
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, m = i / LANES, lane = i % LANES;
     float s = 0.f;
-    for (uint32_t t = lane; t < n_chunks; t += 32u) s += partial[static_cast<size_t>(m) * n_chunks + t];
+    if (m < P)
+        for (uint32_t t = lane; t < n_chunks; t += LANES) s += partial[static_cast<size_t>(m) * n_chunks + t];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0u) fitness[m] = -s * inv_count;
+    for (int off = LANES / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (m < P && lane == 0u) fitness[m] = -s * inv_count;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -895,7 +898,9 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
     }
     if (cudaGetLastError() != cudaSuccess) return -1;
     const float inv = 1.0f / (static_cast<float>(B) * static_cast<float>(nd + 1));
-    if (launch_dependent(k_s2s_finalize, dim3((P + 7u) / 8u), dim3(256), 0, st, a.partial, P, a.n_chunks, inv, fitness) != cudaSuccess)
+    const uint32_t members = mma ? 64u : 256u;                    // per block of 256 threads
+    if (launch_dependent(mma ? k_s2s_finalize<4> : k_s2s_finalize<1>, dim3((P + members - 1u) / members), dim3(256), 0, st, a.partial, P,
+                         a.n_chunks, inv, fitness) != cudaSuccess)
         return -1;
     return 2;
 }

@@ -59,13 +59,12 @@ def test_tensor_core_kernel_matches_oracle(B):
     assert np.std(fit) > 1e-3                                    # members really differ
 
 
-def test_the_read_out_is_as_exact_as_a_chain_of_fp32_additions():
+def _saturated_fitness(P, batch):
     """Gates and cells saturated by their biases: every hidden state is +-bf16(tanh 1) = +-195/256 exactly, whatever the query.  Only the
-    logit of '=' (never an answer) has weights, all of its terms positive: the loss of every position is that logit (30 and
-    more, so that the others add nothing to the exponentials), a sum of 128 products that fp32 holds exactly.  Its error may be no larger than that of two chains of 64 rounded additions (RMS; 1,024
-    members scatter by 2 %), and without their rounding's bias: a mean within 4 of its standard errors."""
-    h, P = 128, 1024
-    w = _workload(h, 1, 1, P=P)
+    logit of '=' (never an answer) has weights, all of its terms positive: the loss of every position is that logit (28 and
+    more, so that the others add nothing to the exponentials), a sum of 128 products that fp32 holds exactly.  Fitness and products."""
+    h = 128
+    w = _workload(h, 1, batch, P=P)
     rng = np.random.default_rng(2)
     sign = rng.choice((-1.0, 1.0), (P, h)).astype(np.float32)
     weights = (np.exp2(rng.uniform(-10.0, 2.0, (P, h))).astype(np.float32).view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
@@ -81,15 +80,32 @@ def test_the_read_out_is_as_exact_as_a_chain_of_fp32_additions():
     fit = s.rollout(rows).cpu().numpy()
     assert s.sync_status() == 0
     s.close()
-    terms = weights * np.float32(195.0 / 256.0)
+    return fit, weights * np.float32(195.0 / 256.0)
+
+
+def test_the_read_out_is_as_exact_as_a_chain_of_fp32_additions():
+    """Its error may be no larger than that of two chains of 64 rounded additions (RMS; 1,024 members scatter by 2 %), and without their
+    rounding's bias: a mean within 4 of its standard errors."""
+    P = 1024
+    fit, terms = _saturated_fitness(P, 1)
     chains = np.zeros((P, 2), np.float32)
-    for k in range(0, h, 2):
+    for k in range(0, 128, 2):
         chains = chains + terms[:, k:k + 2]
     exact = terms.astype(np.float64).sum(1)
     chain_err, err = (chains[:, 0] + chains[:, 1]) / exact - 1.0, -fit.astype(np.float64) / exact - 1.0
     rms = lambda x: float(np.sqrt((x * x).mean()))
     assert rms(err) <= 1.05 * rms(chain_err), (rms(err), rms(chain_err))
     assert abs(err.mean()) <= 4.0 * err.std() / math.sqrt(P), (err.mean(), err.std())
+
+
+def test_chunks_of_128_queries_are_summed_in_order():
+    """All chunks have the same sum, which the fitness of one chunk gives exactly (a division by 256)."""
+    chunk = _saturated_fitness(256, 128)[0] * np.float32(-256.0)
+    total = np.zeros(256, np.float32)
+    for _ in range(5):
+        total = total + chunk
+    want = -total * (np.float32(1.0) / (np.float32(640.0) * np.float32(2.0)))
+    assert np.array_equal(_saturated_fitness(256, 640)[0], want)
 
 
 @pytest.mark.parametrize("kernel", [ROLLOUT_TILED, ROLLOUT_GENERIC])
