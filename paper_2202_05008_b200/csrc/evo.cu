@@ -25,6 +25,7 @@ struct evo_solver {
     const float*   d_target;
     uint64_t     launches;
     uint32_t     k0, k1;
+    S2sSplit     s2s;              // how a roll-out of narrow seq2seq cells is split
     bool         rollout_prepared;  // per-kernel attributes are set by the solver's first roll-out only
 };
 
@@ -194,6 +195,9 @@ evo_status evo_create(const evo_config* cfg_in, void* d_workspace, size_t worksp
     s->d_target = nullptr;
     s->launches = 0;
     s->rollout_prepared = false;
+    if (s->cfg.task_kind == EVO_TASK_SEQ2SEQ_ADD)
+        s->s2s = s2s_split(s->cfg.layer_sizes[0], s->local_pop, (s->cfg.batch + 7u) / 8u,
+                           static_cast<uint32_t>(s->cfg.task_param[EVO_S2S_DIGITS]), kSms);
     s->k0 = static_cast<uint32_t>(s->cfg.seed & 0xFFFFFFFFull);
     s->k1 = static_cast<uint32_t>(s->cfg.seed >> 32);
     const Layout& L = s->lay;
@@ -298,7 +302,7 @@ evo_status evo_rollout(evo_solver* s, const float* d_theta, float* d_fitness, fl
         // d_trace, when given, receives the logits [P][batch][digits+1][12] (CUDA-core kernel)
         const int n = launch_rollout_s2s(s->stream, d_theta, L.ldD, s->local_pop, c.layer_sizes[0],
                                          static_cast<uint32_t>(c.task_param[EVO_S2S_DIGITS]), c.batch, s->k0, s->k1,
-                                         c.rollout_kernel, s->ws + L.cnn_scratch, d_fitness, d_trace,
+                                         c.rollout_kernel, s->s2s, s->ws + L.cnn_scratch, d_fitness, d_trace,
                                          reinterpret_cast<DeviceStatus*>(s->ws + L.status));
         if (n < 0) return n == -2 ? EVO_ERR_UNSUPPORTED : EVO_ERR_CUDA;
         s->launches += n;

@@ -6,6 +6,7 @@
 
 #include "../../include/evo.h"
 #include "spread.h"
+#include "s2s_split.h"
 
 namespace evo {
 
@@ -138,7 +139,7 @@ bool s2s_supported(uint32_t h, uint32_t nd, uint32_t B);
 size_t s2s_scratch_bytes(uint32_t P, uint32_t B);
 // logits (nullable): [P][B][nd+1][12], written by the CUDA-core kernel only
 int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32_t P, uint32_t h, uint32_t nd,
-                       uint32_t B, uint32_t k0, uint32_t k1, uint32_t kernel_choice,
+                       uint32_t B, uint32_t k0, uint32_t k1, uint32_t kernel_choice, const S2sSplit& split,
                        void* scratch, float* fitness, float* logits, DeviceStatus* status);
 
 bool paint_supported(uint32_t param_dim, uint32_t W, uint32_t H);

@@ -266,7 +266,7 @@ __device__ __forceinline__ void tanh_two(float c0, float c1, float& t0, float& t
 }
 
 // A block has `chunk` n-tiles of a member, or (RUNS) a run of the n-tiles of all members, which are dealt out evenly to the blocks and
-// worked off in pieces of one member and up to TILES tiles.
+// worked off in pieces of one member and up to TILES tiles.  s2s_split.h chooses.
 template <int H, int TILES, bool RUNS>
 __global__ void __launch_bounds__(4 * H, H == 32 ? 6 : H == 64 ? 2 : 1)
 k_s2s_mma(const S2sArgs a, uint32_t chunk)
@@ -839,23 +839,13 @@ bool s2s_supported(uint32_t h, uint32_t nd, uint32_t B)
 
 static uint32_t s2s_chunks(uint32_t B, bool tc) { return tc ? (B + kTcQ - 1) / kTcQ : (B + kSimpleQ - 1) / kSimpleQ; }
 
-// Chunks of up to 64 queries, spread evenly over the fewest chunks, in whole n-tiles; a small population takes smaller ones (down to
-// one tile) until there are two blocks for every SM.  More blocks of wide cells than the SMs hold at once (two blocks of 64 units, one of 96) would
-// leave the last wave nearly empty or end in many of them: each SM then gets its runs.  300 members x 100 queries, 2 digits, chunks / runs:
-// 64 units 85 / 77 us, 96 units 181 / 149; 296 members x 104: 68 / 64 and 151 / 133; 600 x 56: 94 / 96 and 192 / 168.  Cells of 32 units
-// hold six blocks to an SM and lose: 300 x 100 40 / 51.  Runs of 64 units are worked off in pieces of up to 14 tiles; as blocks of a
-// single chunk that instance is slower for its length (148 x 8 17.5 / 23.1).
-static cudaError_t launch_s2s_mma(cudaStream_t st, const S2sArgs& a)
+static cudaError_t launch_s2s_mma(cudaStream_t st, const S2sArgs& a, const S2sSplit& split)
 {
-    const uint32_t tiles = a.n_chunks;
-    uint32_t chunks = (tiles + 7u) / 8u;
-    while (chunks < tiles && static_cast<uint64_t>(a.P) * chunks < 2u * kSms) ++chunks;
-    const uint32_t chunk = (tiles + chunks - 1u) / chunks, places = kSms * (a.h == 64u ? 2u : 1u);
-    chunks = (tiles + chunk - 1u) / chunk;
-    if (a.h != 32u && static_cast<uint64_t>(a.P) * chunks > places)
-        return launch_dependent(a.h == 64u ? k_s2s_mma<64, 14, true> : k_s2s_mma<96, 8, true>, dim3(places), dim3(4u * a.h), 0, st, a, 0u);
+    if (split.chunk == 0u)
+        return launch_dependent(a.h == 64u ? k_s2s_mma<64, kS2sRunTiles64, true> : k_s2s_mma<96, kS2sRunTiles96, true>, dim3(split.places),
+                                dim3(4u * a.h), 0, st, a, 0u);
     return launch_dependent(a.h == 32u ? k_s2s_mma<32, 8, false> : a.h == 64u ? k_s2s_mma<64, 8, false> : k_s2s_mma<96, 8, false>,
-                            dim3(a.P, chunks), dim3(4u * a.h), 0, st, a, chunk);
+                            dim3(a.P, split.chunks), dim3(4u * a.h), 0, st, a, split.chunk);
 }
 
 size_t s2s_scratch_bytes(uint32_t P, uint32_t B)
@@ -864,7 +854,7 @@ size_t s2s_scratch_bytes(uint32_t P, uint32_t B)
 }
 
 int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32_t P, uint32_t h, uint32_t nd,
-                       uint32_t B, uint32_t k0, uint32_t k1, uint32_t kernel_choice,
+                       uint32_t B, uint32_t k0, uint32_t k1, uint32_t kernel_choice, const S2sSplit& split,
                        void* scratch, float* fitness, float* logits, DeviceStatus* status)
 {
     const bool want_tc = kernel_choice != EVO_ROLLOUT_GENERIC;
@@ -891,7 +881,7 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
         const uint32_t grid = items < static_cast<uint32_t>(sm_count) ? items : static_cast<uint32_t>(sm_count);
         k_s2s_tc<<<grid, kTcThreads, sizeof(S2sSmem), st>>>(a, status);
     } else if (mma) {
-        if (launch_s2s_mma(st, a) != cudaSuccess) return -1;
+        if (launch_s2s_mma(st, a, split) != cudaSuccess) return -1;
     } else {
         dim3 grid(P, a.n_chunks);
         k_s2s_simple<<<grid, 128, 0, st>>>(a);

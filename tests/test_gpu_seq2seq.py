@@ -214,10 +214,12 @@ def test_narrow_cells_on_tensor_cores_match_oracle(h, nd, B, P):
 
 
 @pytest.mark.parametrize("h", [32, 64, 96])
-@pytest.mark.parametrize("nd,B,P", [(1, 100, 300), (1, 400, 60), (1, 112, 296), (1, 9, 750)])
+@pytest.mark.parametrize("nd,B,P", [(1, 100, 300), (1, 400, 60), (1, 112, 296), (1, 9, 750), (2, 400, 250), (3, 133, 302)])
 def test_runs_of_tiles_that_begin_and_end_inside_a_member(h, nd, B, P):
-    """The blocks' runs of n-tiles: of several members, of a part of one, in one piece and several; every member against the
-    CUDA-core kernel (both round the same operands; left are accumulation order and gates to about 3e-7)."""
+    """The blocks' runs of n-tiles: of several members, of a part of one, in one piece and several (of one member too: 133 and 400 queries);
+    every member against the CUDA-core kernel.  Both round the same operands; left are accumulation order, gates to about 3e-7 and, by these,
+    a hidden state here and there that rounds to the neighbouring bf16 value: 5e-3 of one position's loss at most were seen,
+    where a position lost or taken from another query changes its loss by 0.1 and more."""
     w = _workload(h, nd, B, P=P, sigma=0.2)
     a, b = Solver(w), Solver(w, rollout_kernel=ROLLOUT_GENERIC)
     a.ask(); b.ask()
@@ -225,4 +227,5 @@ def test_runs_of_tiles_that_begin_and_end_inside_a_member(h, nd, B, P):
     assert a.sync_status() == 0 and b.sync_status() == 0
     assert torch.equal(fa, again)
     assert torch.max(torch.abs(fa - fb)) < FIT_TOL
+    assert torch.max(torch.abs(fa - fb)) < 2e-2 / (B * (nd + 1))
     a.close(); b.close()
