@@ -38,7 +38,7 @@ inline S2sSplit s2s_split(uint32_t units, uint32_t members, uint32_t tiles, uint
     s.chunks = (tiles + s.chunk - 1u) / s.chunk;
     s.places = sms * (units == 64u ? 2u : 1u);
     const uint64_t blocks = static_cast<uint64_t>(members) * s.chunks, all = static_cast<uint64_t>(members) * tiles;
-    if ((units != 64u && units != 96u) || blocks <= s.places) return s;
+    if ((units != 64u && units != 96u) || blocks <= s.places || all > 0xFFFFFFFFull) return s;       // (a run counts its tiles in 32 bits)
     const uint64_t steps = 3u * digits + 2u, piece = 50u + 2u * steps;
     const uint64_t waves3 = 3u * (blocks / s.places) + (blocks % s.places == 0u ? 0u : units == 64u && blocks % s.places <= sms ? 2u : 3u);
     const uint64_t chunked = waves3 * (piece * s.chunks + 2u * steps * tiles);     // x 3 chunks

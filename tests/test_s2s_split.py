@@ -53,6 +53,12 @@ def test_every_tile_has_its_block(lib, units):
             assert chunk <= 8 and chunk * chunks >= tiles > chunk * (chunks - 1)
 
 
+def test_runs_count_their_tiles_in_32_bits(lib):
+    """One tile fewer than 2^32 and as many: the latter in chunks."""
+    assert _split(lib, 64, 65537, 65535)[0] == 0
+    assert _split(lib, 64, 65536, 65536)[0] == 8
+
+
 # units, digits, queries, members, whether runs are faster
 MEASURED = [(64, 1, 47, 52, True), (64, 2, 100, 300, True), (64, 2, 100, 600, True), (64, 2, 64, 298, True), (64, 2, 8, 400, False), (64, 2, 24, 1000, False),
             (64, 2, 40, 400, False), (64, 2, 56, 100, False), (64, 2, 56, 1000, False), (64, 2, 64, 1000, False), (64, 3, 15, 192, False),
