@@ -26,6 +26,7 @@ struct evo_solver {
     uint64_t     launches;
     uint32_t     k0, k1;
     S2sSplit     s2s;              // how a roll-out of narrow seq2seq cells is split
+    bool         deep;             // the control policy runs on k_rollout_mlp_deep
     bool         rollout_prepared;  // per-kernel attributes are set by the solver's first roll-out only
 };
 
@@ -198,6 +199,12 @@ evo_status evo_create(const evo_config* cfg_in, void* d_workspace, size_t worksp
     if (s->cfg.task_kind == EVO_TASK_SEQ2SEQ_ADD)
         s->s2s = s2s_split(s->cfg.layer_sizes[0], s->local_pop, (s->cfg.batch + 7u) / 8u,
                            static_cast<uint32_t>(s->cfg.task_param[EVO_S2S_DIGITS]), kSms);
+    s->deep = false;
+    if (s->cfg.task_kind == EVO_TASK_CARTPOLE || s->cfg.task_kind == EVO_TASK_TANH_LINEAR) {
+        const int deep = rollout_mlp_prepare(s->cfg, s->lay.EB, s->lay.n_eb);
+        if (deep < 0) { delete s; return EVO_ERR_CUDA; }
+        s->deep = deep != 0;
+    }
     s->k0 = static_cast<uint32_t>(s->cfg.seed & 0xFFFFFFFFull);
     s->k1 = static_cast<uint32_t>(s->cfg.seed >> 32);
     const Layout& L = s->lay;
@@ -315,7 +322,7 @@ evo_status evo_rollout(evo_solver* s, const float* d_theta, float* d_fitness, fl
     a.trace = d_trace;
     a.task_const = reinterpret_cast<const float*>(s->ws + L.task_const);
     a.P = s->local_pop;
-    a.pop = c.pop_size;
+    a.deep = s->deep ? 1u : 0u;
     a.ldD = L.ldD;
     a.n_layers = c.n_layers;
     a.max_width = 0;

@@ -1,5 +1,6 @@
 // Internal declarations shared by the host API (evo.cu) and the kernel files.
 #pragma once
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -7,6 +8,7 @@
 #include "../../include/evo.h"
 #include "spread.h"
 #include "s2s_split.h"
+#include "mlp_choice.h"
 
 namespace evo {
 
@@ -62,7 +64,7 @@ struct RolloutMlpArgs {
     float*       trace;          // nullable
     const float* task_const;     // tanh-linear: A[28][28] then B[28][8]
     uint32_t P, ldD;
-    uint32_t pop;                // the whole population, of which P may be a shard: what chooses the kernel
+    uint32_t deep;               // whether k_rollout_mlp_deep takes the policy (see rollout_mlp_prepare)
     uint32_t n_layers;
     uint32_t sizes[EVO_MAX_LAYERS + 1];
     uint32_t max_width;
@@ -124,6 +126,9 @@ int  launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a, uint32_t kerne
                         float* fitness, DeviceStatus* status);
 bool rollout_mlp_supported(const evo_config& cfg);
 void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb);
+// What of the choice of a kernel takes the device: 1: k_rollout_mlp_deep, 0: another one, -1: an error of the runtime
+int rollout_mlp_prepare(const evo_config& cfg, uint32_t EB, uint32_t n_eb);
+int rollout_mlp_mma_resident(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB);
 
 size_t cnn_scratch_bytes(uint32_t P, uint32_t batch);
 size_t cnn_tc_scratch_bytes(uint32_t P, uint32_t batch);
@@ -171,6 +176,22 @@ inline size_t spread_over_sms(Kernel kernel, size_t bytes, uint64_t blocks)
         cudaFuncGetAttributes(&attr, kernel) != cudaSuccess)
         return bytes;
     return spread_bytes(bytes, attr.sharedSizeBytes + 1024u, blocks, static_cast<uint32_t>(sms), static_cast<size_t>(sm_bytes));
+}
+
+// Registers of a thread and static shared memory of a block; `known` holds them once they were asked for (15 us).
+template <class Kernel>
+inline bool kernel_needs(Kernel kernel, std::atomic<uint64_t>& known, uint32_t* regs, size_t* smem)
+{
+    uint64_t k = known.load(std::memory_order_relaxed);
+    if (k == 0u) {
+        cudaFuncAttributes attr;
+        if (cudaFuncGetAttributes(&attr, kernel) != cudaSuccess) return false;
+        k = static_cast<uint64_t>(attr.sharedSizeBytes) << 32 | static_cast<uint32_t>(attr.numRegs);
+        known.store(k, std::memory_order_relaxed);
+    }
+    *regs = static_cast<uint32_t>(k);
+    *smem = static_cast<size_t>(k >> 32);
+    return true;
 }
 
 #ifdef __CUDACC__

@@ -1,0 +1,43 @@
+// Which kernel a control policy of three or four hidden layers of up to 128 units runs on, without CUDA so that it can be tested anywhere.
+#pragma once
+#include <cstddef>
+#include <cstdint>
+
+namespace evo {
+
+// Blocks of a kernel that an SM of compute capability 10.0 holds at once: 64 K registers and 64 warps in four parts (registers in units of
+// 256 per warp), 228 KB of shared memory in units of 128 bytes, 1 KB of which the system takes per block.
+inline uint32_t resident_blocks(uint32_t regs, size_t smem, uint32_t threads)
+{
+    const uint32_t warps = (threads + 31u) / 32u, per_warp = (regs + 7u) / 8u * 256u;
+    const uint32_t fit = 16384u / per_warp < 16u ? 16384u / per_warp : 16u;
+    const uint32_t by_regs = 4u * fit / warps, by_smem = static_cast<uint32_t>(228u * 1024u / ((smem + 1024u + 127u) / 128u * 128u));
+    const uint32_t n = by_regs < by_smem ? by_regs : by_smem;
+    return n < 32u ? n : 32u;
+}
+
+// Waves of blocks, with `resident` of them on an SM at once: a last wave that leaves SMs room takes 0.6 of a whole one and, for each
+// block, its share of the other 0.4.
+inline double mlp_waves(uint64_t blocks, uint32_t sms, uint32_t resident)
+{
+    const uint64_t share = (blocks + sms - 1u) / sms, rest = share % resident;
+    return static_cast<double>(share / resident) + (rest ? 0.6 + 0.4 * static_cast<double>(rest) / resident : 0.0);
+}
+
+// Whether k_rollout_mlp_deep (weights in registers) is faster than k_rollout_mlp_mma (weights in shared memory; resident_mma = 0: they do not
+// fit).  Its blocks are as large as the widest layer and hold many registers, so fewer of them fit an SM; wave for wave it is the
+// faster one by a factor that depends on the layers, on whether one is wide (above 64 units) and on the episodes of a block (eb).  These
+// are the limits below: how many times the waves of the other it may take.  Measured in 258 policies of 6 to 128 units, both tasks, 4 and 8
+// episodes, 100 to 2,000 members (4,068 roll-outs): 0.2 % more time in the mean than with the faster kernel of the two, and 16 take 1 to 8 % longer
+// here than with the other.  Examples, 50 steps, deep / mma: 28-57-53-52-8, 592 members x 4 episodes 69 / 130 us;
+// 28-8-68-20-8, 592 x 8 183 / 121; 5-14-13-110-1, 444 x 8 172 / 120; 5-6-9-14-50-1, 740 x 8 165 / 140; 28-8-102-8-12-8, 2,000 x 4 774 / 365;
+// 28-109-10-119-115-8, 300 x 8 271 / 475.
+inline bool mlp_deep_pays(uint32_t hidden, bool wide, uint32_t eb, uint64_t blocks, uint32_t sms, uint32_t resident_deep, uint32_t resident_mma)
+{
+    if (hidden == 1u || resident_mma == 0u) return true;
+    if (resident_deep == 0u) return false;
+    const double limit = hidden == 3u ? (!wide ? 2.0 : eb == 4u ? 1.7 : 1.45) : wide ? 2.4 : eb == 4u ? 1.95 : 1.65;
+    return mlp_waves(blocks, sms, resident_deep) <= limit * mlp_waves(blocks, sms, resident_mma);
+}
+
+}  // namespace evo

@@ -196,17 +196,18 @@ uint32_t rollout_mlp_tiled_eb(int shape, uint32_t episodes);
 int launch_rollout_mlp_tiled(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 uint32_t rollout_mlp2_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
-uint32_t rollout_mlp_deep_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t episodes);
+uint32_t rollout_mlp_deep_eb(uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
+int rollout_mlp_deep_pays(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t EB, uint32_t n_eb);
 int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
 // The kernel of a policy: AUTO takes a register-resident one where the policy has one to four hidden layers of up to 128
-// units (beside an exception, see rollout_mlp_deep_eb), for other numbers of layers and wider ones the one with the weights in
+// units (three and four where that is the faster one, see mlp_choice.h), for other numbers of layers and wider ones the one with the weights in
 // shared memory as long as they fit it, and else the runtime-shape kernel, which reads them through the caches.
 enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kDeep, kSharedMemory };
 
-static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, uint32_t pop,
+static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, bool deep,
                                uint32_t episodes, uint32_t* EB)
 {
     if (choice == EVO_ROLLOUT_TILED) {
@@ -217,7 +218,7 @@ static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t*
     }
     if (choice == EVO_ROLLOUT_AUTO) {
         if ((*EB = rollout_mlp2_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kRegisters;
-        if ((*EB = rollout_mlp_deep_eb(task, n_layers, sizes, pop, episodes)) != 0u) return MlpKernel::kDeep;
+        if (deep && (*EB = rollout_mlp_deep_eb(n_layers, sizes, episodes)) != 0u) return MlpKernel::kDeep;
         if ((*EB = rollout_mlp_mma_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kSharedMemory;
     }
     return MlpKernel::kGeneric;
@@ -226,7 +227,8 @@ static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t*
 void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
 {
     uint32_t eb = 0;
-    const MlpKernel k = choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, cfg.pop_size, cfg.episodes, &eb);
+    // (both kernels that a policy may be left to have the same episodes per block)
+    const MlpKernel k = choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, true, cfg.episodes, &eb);
     if (k == MlpKernel::kGeneric || k == MlpKernel::kNone) {
         eb = cfg.episodes < 32u ? cfg.episodes : 32u;
         // few members: split the episodes of a member over more blocks to fill the SMs
@@ -235,6 +237,13 @@ void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
     }
     *EB = eb;
     *n_eb = (cfg.episodes + eb - 1u) / eb;
+}
+
+int rollout_mlp_prepare(const evo_config& cfg, uint32_t EB, uint32_t n_eb)
+{
+    uint32_t eb = 0;
+    if (choose_kernel(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.rollout_kernel, true, cfg.episodes, &eb) != MlpKernel::kDeep) return 0;
+    return rollout_mlp_deep_pays(cfg.task_kind, cfg.n_layers, cfg.layer_sizes, cfg.pop_size, EB, n_eb);
 }
 
 static size_t generic_smem_bytes(const RolloutMlpArgs& a, bool with_weights)
@@ -254,7 +263,7 @@ int launch_rollout_mlp(cudaStream_t st, const RolloutMlpArgs& a_in, uint32_t ker
     uint32_t eb = 0;
     int launches = 0;
     a.fitness = fitness;
-    switch (choose_kernel(a.task, a.n_layers, a.sizes, kernel_choice, a.pop, a.E, &eb)) {
+    switch (choose_kernel(a.task, a.n_layers, a.sizes, kernel_choice, a.deep != 0u, a.E, &eb)) {
     case MlpKernel::kNone:
         return -2;
     case MlpKernel::kRegisters:

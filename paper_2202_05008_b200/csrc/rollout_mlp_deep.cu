@@ -406,48 +406,64 @@ uint32_t tiles_of(uint32_t units) { return (units + 15u) / 16u; }
 
 }  // namespace
 
-// Episodes per block; 0: not a policy for this kernel.  Its blocks are as large as the widest layer, all layers' products as long as the
-// widest's input needs, in steps of four tiles; two (four hidden layers: one) of the wide ones fit an SM.  So once more of them are to run than
-// fit, a policy that is wide in one layer only is left to k_rollout_mlp_mma, whose blocks are small then.  The measure is the tiles of the
-// matrices between hidden layers.  512 blocks of 8 episodes, this kernel / the other, 100 steps: 28-120-20-10-8 (18 tiles; 400 blocks, 200 steps) 605 / 492 us,
-// 28-120-40-20-8 (30) 361 / 467, 28-100-30-100-8 (28) 397 / 510, 5-120-40-20-1 (30) 358 / 319, 5-100-90-100-1 (84) 439 / 630, 28-90-70-30-30-8 (44)
-// 574 / 547, 28-100-50-30-60-8 (44; 400 blocks of 4 episodes, 200 steps) 608 / 937.  While they fit: 28-120-20-10-8, 200 members 337 / 446, 5-10-120-10-10-1, 128 members 239 / 453.
-uint32_t rollout_mlp_deep_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t episodes)
+namespace {
+
+struct DeepLaunch { void (*kernel)(const RolloutMlpArgs, DeviceStatus*); uint32_t threads; size_t bytes; bool wide, fine; };
+
+DeepLaunch deep_launch(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB)
 {
+    const bool cart = task == EVO_TASK_CARTPOLE;
     const uint32_t hidden = n_layers - 1u;
-    if (n_layers != 2u && n_layers != 4u && n_layers != 5u) return 0u;
-    uint32_t widest = 0, between = 0;
+    uint32_t warps = 1;
+    DeepLaunch d;
+    d.fine = false;
     for (uint32_t l = 1; l <= hidden; ++l) {
-        if (tiles_of(sizes[l]) > widest) widest = tiles_of(sizes[l]);
-        if (l > 1u) between += tiles_of(sizes[l - 1u]) * tiles_of(sizes[l]);
+        if (tiles_of(sizes[l]) > warps) warps = tiles_of(sizes[l]);
+        d.fine = d.fine || sizes[l] < 49u;
     }
-    if (widest > 8u) return 0u;
-    const uint32_t eb = episodes > 4u ? 8u : 4u;
-    const uint64_t blocks = static_cast<uint64_t>(pop) * ((episodes + eb - 1u) / eb);
-    if (widest > 4u && hidden > 1u && blocks > static_cast<uint64_t>(kSms) * (hidden == 3u ? 2u : 1u) &&
-        between < (hidden == 4u ? (eb == 4u ? 44u : 64u) : task == EVO_TASK_CARTPOLE ? 44u : 24u)) return 0u;
-    return eb;
+    d.wide = warps > 4u;
+    if (!cart && warps < 2u) warps = 2u;
+    d.threads = 32u * warps;
+    d.kernel = EB == 4u ? (cart ? pick_kernel<4, true>(hidden, d.wide, d.fine) : pick_kernel<4, false>(hidden, d.wide, d.fine))
+                        : (cart ? pick_kernel<8, true>(hidden, d.wide, d.fine) : pick_kernel<8, false>(hidden, d.wide, d.fine));
+    d.bytes = static_cast<size_t>(warps) * (hidden - 1u) * (d.wide ? 8u : 4u) * 512u;
+    return d;
+}
+
+}  // namespace
+
+// Episodes per block; 0: not a policy for this kernel.
+uint32_t rollout_mlp_deep_eb(uint32_t n_layers, const uint32_t* sizes, uint32_t episodes)
+{
+    if (n_layers != 2u && n_layers != 4u && n_layers != 5u) return 0u;
+    for (uint32_t l = 1; l < n_layers; ++l)
+        if (tiles_of(sizes[l]) > 8u) return 0u;
+    return episodes > 4u ? 8u : 4u;
+}
+
+// Whether the policy (one of this kernel) is faster here than on k_rollout_mlp_mma, for the whole population, of which the solver may have a
+// shard; -1: the runtime's error
+int rollout_mlp_deep_pays(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t EB, uint32_t n_eb)
+{
+    if (n_layers == 2u) return 1;
+    static std::atomic<uint64_t> known[2][2][2][2][2];
+    const DeepLaunch d = deep_launch(task, n_layers, sizes, EB);
+    uint32_t regs;
+    size_t fixed;
+    if (!kernel_needs(d.kernel, known[EB == 8u][task == EVO_TASK_CARTPOLE][n_layers == 5u][d.wide][d.fine], &regs, &fixed)) return -1;
+    const int mma = rollout_mlp_mma_resident(task, n_layers, sizes, EB);
+    if (mma < 0) return -1;
+    return mlp_deep_pays(n_layers - 1u, d.wide, EB, static_cast<uint64_t>(pop) * n_eb, kSms, resident_blocks(regs, d.bytes + fixed, d.threads),
+                         static_cast<uint32_t>(mma));
 }
 
 int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status)
 {
-    const bool cart = a.task == EVO_TASK_CARTPOLE;
-    const uint32_t hidden = a.n_layers - 1u;
-    uint32_t warps = 1;
-    bool fine = false;
-    for (uint32_t l = 1; l <= hidden; ++l) {
-        if (tiles_of(a.sizes[l]) > warps) warps = tiles_of(a.sizes[l]);
-        fine = fine || a.sizes[l] < 49u;
-    }
-    const bool wide = warps > 4u;
-    if (!cart && warps < 2u) warps = 2u;
-    auto kernel = a.EB == 4u ? (cart ? pick_kernel<4, true>(hidden, wide, fine) : pick_kernel<4, false>(hidden, wide, fine))
-                             : (cart ? pick_kernel<8, true>(hidden, wide, fine) : pick_kernel<8, false>(hidden, wide, fine));
-    size_t bytes = static_cast<size_t>(warps) * (hidden - 1u) * (wide ? 8u : 4u) * 512u;
-    bytes = spread_over_sms(kernel, bytes, static_cast<uint64_t>(a.P) * a.n_eb);
+    const DeepLaunch d = deep_launch(a.task, a.n_layers, a.sizes, a.EB);
+    const size_t bytes = spread_over_sms(d.kernel, d.bytes, static_cast<uint64_t>(a.P) * a.n_eb);
     if (!a.attr_done &&
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return -1;
-    return launch_dependent(kernel, dim3(a.P, a.n_eb), dim3(32u * warps), bytes, st, a, status) == cudaSuccess ? 1 : -1;
+        cudaFuncSetAttribute(d.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return -1;
+    return launch_dependent(d.kernel, dim3(a.P, a.n_eb), dim3(d.threads), bytes, st, a, status) == cudaSuccess ? 1 : -1;
 }
 
 }  // namespace evo

@@ -354,6 +354,21 @@ uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* si
     return make_plan(task, n_layers, sizes, eb).smem <= kMaxSmem ? eb : 0u;
 }
 
+// Blocks that an SM holds at once; 0: the weights do not fit, -1: the runtime's error
+int rollout_mlp_mma_resident(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB)
+{
+    const Plan p = make_plan(task, n_layers, sizes, EB);
+    if (p.smem > kMaxSmem) return 0;
+    const bool cart = task == EVO_TASK_CARTPOLE;
+    auto kernel = EB == 4u ? (cart ? pick_kernel<4, true>(p.fine) : pick_kernel<4, false>(p.fine))
+                           : (cart ? pick_kernel<8, true>(p.fine) : pick_kernel<8, false>(p.fine));
+    static std::atomic<uint64_t> known[2][2][2];
+    uint32_t regs;
+    size_t fixed;
+    if (!kernel_needs(kernel, known[EB == 8u][cart][p.fine], &regs, &fixed)) return -1;
+    return static_cast<int>(resident_blocks(regs, p.smem + fixed, 32u * (p.warps + (cart ? 1u : 0u))));
+}
+
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status)
 {
     const Plan p = make_plan(a.task, a.n_layers, a.sizes, a.EB);
