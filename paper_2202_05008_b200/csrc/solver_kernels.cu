@@ -4,6 +4,8 @@
 #include "internal.h"
 #include "noise.cuh"
 
+#include <type_traits>
+
 namespace evo {
 
 // ------------------------------------------------------------------------------------------
@@ -226,8 +228,8 @@ int launch_rank(cudaStream_t st, const float* fitness, uint32_t P, int32_t* rank
 // ill-conditioned where |g| is near adam_eps, so the cancellation error of an fp32 sum (~1e-7 of RMS(g)) would
 // move those coordinates by far more than the 1e-5 parity bound.  The stored-noise form is HBM-bound (4 bytes
 // per term; 4.3 GB in 621 us), so the fp64 arithmetic is hidden.  REGEN recomputes eps from the Philox counters instead of
-// reading it.  SIGMA also accumulates the PGPE sigma gradient sum_j ((u[2j]+u[2j+1])/2) (eps^2 - 1) in fp32 (a plain step on
-// sigma follows, which is not ill-conditioned like Adam's normalised step).
+// reading it.  SIGMA also accumulates the PGPE sigma gradient sum_j ((u[2j]+u[2j+1])/2) (eps^2 - 1), whose partial sums are fp32 (a plain
+// step on sigma follows, which is not ill-conditioned like Adam's normalised step).
 //
 // The block that finds itself the last of its columns (a counter, no waiting) adds the splits' partial sums and takes the step
 // for them; the last of those closes the tell.  RANK: each block also ranks the members of its own pairs.  A tell of a
@@ -249,23 +251,38 @@ __device__ __forceinline__ void acc_fma(Acc4& a, double wd, const float4& e)
     a.z = fma(wd, static_cast<double>(e.z), a.z);
     a.w = fma(wd, static_cast<double>(e.w), a.w);
 }
-// PACKED: where issue bounds (recomputed noise)
-template <bool PACKED>
-__device__ __forceinline__ void sig_fma(fp2 (&a)[2], float sj, const float4& e)
-{
-    const float ev[4] = { e.x, e.y, e.z, e.w };
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        if (PACKED) {
-            const fp2 z = fp2_make(ev[2 * i], ev[2 * i + 1]);
-            a[i] = fp2_fma(fp2_both(sj), fp2_fma(z, z, fp2_both(-1.0f)), a[i]);
-        } else {
-            float x, y;
-            fp2_split(a[i], x, y);
-            a[i] = fp2_make(fmaf(sj, fmaf(ev[2 * i], ev[2 * i], -1.0f), x), fmaf(sj, fmaf(ev[2 * i + 1], ev[2 * i + 1], -1.0f), y));
-        }
+// A thread's sums of the sigma gradient.  Stored noise streams and leaves the fp64 pipe time: sums in fp64, one rounding when they leave the thread.
+// In fp32 their error grew with the pairs of a split, of which there are fewer than room for (see whole_waves): relative RMS
+// error of the gradient with all splits / with these / these in fp64, 300 members x 40,256 columns 7.8 / 8.4 / 5.2e-8, 4,096 x 20,872 10.2 / 14.6 /
+// 6.4e-8, 16,384 x 131,072 21 / 25 / 6.6e-8.
+struct SigmaSums64 {
+    Acc4 a = { 0., 0., 0., 0. };
+    __device__ __forceinline__ static void term(double& s, double w, float e) { const double z = e; s = fma(w, fma(z, z, -1.0), s); }
+    __device__ __forceinline__ void add(int, const float2& uu, const float4& e)
+    {
+        const double d = 0.5 * (static_cast<double>(uu.x) + static_cast<double>(uu.y));
+        term(a.x, d, e.x); term(a.y, d, e.y); term(a.z, d, e.z); term(a.w, d, e.w);
     }
-}
+    __device__ __forceinline__ void sums(float (&r)[4]) const
+    {
+        r[0] = static_cast<float>(a.x); r[1] = static_cast<float>(a.y); r[2] = static_cast<float>(a.z); r[3] = static_cast<float>(a.w);
+    }
+};
+// Recomputed noise is bound by issue: packed fp32, two chains.
+struct SigmaSums32 {
+    fp2 a[2][2] = { { 0ull, 0ull }, { 0ull, 0ull } };
+    __device__ __forceinline__ void add(int i, const float2& uu, const float4& e)
+    {
+        const fp2 s = fp2_both(0.5f * (uu.x + uu.y)), z[2] = { fp2_make(e.x, e.y), fp2_make(e.z, e.w) };
+#pragma unroll
+        for (int k = 0; k < 2; ++k) a[i & 1][k] = fp2_fma(s, fp2_fma(z[k], z[k], fp2_both(-1.0f)), a[i & 1][k]);
+    }
+    __device__ __forceinline__ void sums(float (&r)[4]) const
+    {
+        fp2_split(fp2_add(a[0][0], a[1][0]), r[0], r[1]);
+        fp2_split(fp2_add(a[0][1], a[1][1]), r[2], r[3]);
+    }
+};
 
 __device__ __forceinline__ double power(double b, uint32_t n)
 {
@@ -510,12 +527,12 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
     }
 
     Acc4 acc = { 0., 0., 0., 0. }, acc2 = acc;             // two chains of sums
-    fp2 sacc[2] = { 0ull, 0ull }, sacc2[2] = { 0ull, 0ull };
+    std::conditional_t<REGEN, SigmaSums32, SigmaSums64> sacc;
     if (live) {
         auto weight = [&](uint32_t j) { return RANK ? uu_s[j - j0] : __ldg(up + j); };
         auto add = [&](int i, const float2& uu, const float4& z) {
             acc_fma(i & 1 ? acc2 : acc, static_cast<double>(uu.x) - static_cast<double>(uu.y), z);            // (exact difference)
-            if (SIGMA) sig_fma<REGEN>(i & 1 ? sacc2 : sacc, 0.5f * (uu.x + uu.y), z);
+            if (SIGMA) sacc.add(i, uu, z);
         };
         uint32_t j = first;
         if constexpr (kPrefetch) {
@@ -542,11 +559,9 @@ k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __r
                 if (j + i * kTellLanes < j1) add(i, weight(j + i * kTellLanes), noise(j + i * kTellLanes));
         }
         acc.x += acc2.x; acc.y += acc2.y; acc.z += acc2.z; acc.w += acc2.w;
-        if (SIGMA) { sacc[0] = fp2_add(sacc[0], sacc2[0]); sacc[1] = fp2_add(sacc[1], sacc2[1]); }
     }
     float sr[4];
-    fp2_split(sacc[0], sr[0], sr[1]);
-    fp2_split(sacc[1], sr[2], sr[3]);
+    sacc.sums(sr);
     // the pair lanes in order
     if (lane > 0) {
         sums[lane - 1u][q][0] = acc.x; sums[lane - 1u][q][1] = acc.y; sums[lane - 1u][q][2] = acc.z; sums[lane - 1u][q][3] = acc.w;
