@@ -453,9 +453,12 @@ __device__ __forceinline__ bool last_to_arrive(uint32_t* counter, uint32_t n, ui
     return *shared_flag != 0u;
 }
 
+// Blocks of k_tell that an SM holds
+constexpr uint32_t tell_resident(bool regen, bool sigma, bool rank) { return sigma || rank || regen ? 3u : 5u; }
+
 // counters: [0, column blocks) splits that have arrived, [column blocks] columns
 template <bool REGEN, bool SIGMA, bool RANK>
-__global__ void __launch_bounds__(256, SIGMA || RANK || REGEN ? 3 : 5)
+__global__ void __launch_bounds__(256, tell_resident(REGEN, SIGMA, RANK))
 k_tell(const float* __restrict__ fitness, int32_t* __restrict__ rank, float* __restrict__ u, const float* __restrict__ eps,
        PhiloxKey key, uint32_t pair0, uint32_t H, uint32_t P, uint32_t D, uint32_t pairs_per_split, double* __restrict__ partial,
        float* __restrict__ sigma_partial, uint32_t* __restrict__ counters, const StepArgs a)
@@ -744,7 +747,8 @@ static cudaError_t launch_tell_kernel(cudaStream_t st, const TellArgs& a, const 
 // ranks + gradient sums (+ the step, unless mode is kStepSums)
 static int launch_tell(cudaStream_t st, const TellArgs& a, uint32_t mode, double* grad_sum, float* sigma_sum)
 {
-    const uint32_t splits = a.eps ? whole_waves(tell_blocks(a.ldD), a.H, a.splits, kSms * (a.sigma_partial ? 3u : 5u)) : a.splits;
+    // (places without ranks: what is ranked inside is one wave, or has a single split)
+    const uint32_t splits = a.eps ? whole_waves(tell_blocks(a.ldD), a.H, a.splits, kSms * tell_resident(false, a.sigma_partial != nullptr, false)) : a.splits;
     const uint32_t pps = (a.H + splits - 1u) / splits;
     const dim3 grid(tell_blocks(a.ldD), (a.H + pps - 1u) / pps);       // splits that own at least one pair
     // Every column block repeats the ranking of its split's members, P comparisons each: worth it while the repetition costs
