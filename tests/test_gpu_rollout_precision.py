@@ -60,7 +60,11 @@ def _check_against_fp32(w, theta):
 
 @pytest.mark.parametrize("sizes,pop,episodes", [
     ((28, 128, 128, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 8), 64, 8), ((28, 64, 64, 64, 8), 64, 4),
-    ((28, 20, 8), 64, 8), ((5, 16, 16, 1), 64, 4), ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 8)])
+    ((28, 20, 8), 64, 8), ((5, 16, 16, 1), 64, 4), ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 8),
+    # one, three and four hidden layers with the weights in registers, wide ones and such that take the other tanh
+    ((28, 128, 8), 64, 4), ((28, 49, 8), 64, 4), ((28, 128, 128, 128, 8), 64, 4), ((28, 100, 90, 80, 8), 64, 8), ((28, 70, 20, 100, 8), 64, 4),
+    ((28, 52, 56, 60, 8), 64, 8), ((28, 64, 64, 64, 64, 8), 64, 4), ((28, 128, 128, 128, 128, 8), 64, 8), ((28, 100, 66, 70, 90, 8), 64, 4),
+    ((5, 100, 1), 64, 8), ((5, 128, 128, 128, 1), 64, 8), ((5, 64, 64, 64, 64, 1), 64, 8), ((5, 128, 128, 128, 128, 1), 64, 4), ((5, 128, 20, 20, 1), 64, 4)])
 def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, pop, episodes):
     w = _workload(sizes, pop, episodes)
     _check_against_fp32(w, _population(w, sum(sizes) + pop))
@@ -68,7 +72,8 @@ def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, po
 
 @pytest.mark.parametrize("sizes,pop,episodes", [
     ((28, 64, 64, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 64, 8), 64, 8), ((5, 16, 16, 1), 64, 4),
-    ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 4)])
+    ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 4),
+    ((28, 128, 8), 64, 8), ((28, 128, 128, 128, 8), 64, 4), ((28, 100, 128, 70, 128, 8), 64, 8), ((5, 128, 100, 128, 1), 64, 8)])
 def test_a_huge_weight_takes_nothing_from_the_others(sizes, pop, episodes):
     """One weight or bias beyond the fp16 range per member, from 2e4 to 1e30, anywhere in the policy."""
     w = _workload(sizes, pop, episodes)
