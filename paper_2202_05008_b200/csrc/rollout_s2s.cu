@@ -190,8 +190,8 @@ k_s2s_simple(const S2sArgs a)
     }
 }
 
-// LANES per member.  One: the sums of its chunks in order.  Four: every fourth sum each, then the lanes as a tree, for the many sums (one
-// per 8 queries) of k_s2s_mma.
+// LANES per member.  One: the sums of its chunks in order.  Four: every fourth sum each, then the lanes as a tree, for the sums of k_s2s_mma (one
+// per 8 queries) where they are more than four.
 template <int LANES>
 __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, uint32_t n_chunks, float inv_count,
                                float* __restrict__ fitness)
@@ -888,8 +888,9 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
     }
     if (cudaGetLastError() != cudaSuccess) return -1;
     const float inv = 1.0f / (static_cast<float>(B) * static_cast<float>(nd + 1));
-    const uint32_t members = mma ? 64u : 256u;                    // per block of 256 threads
-    if (launch_dependent(mma ? k_s2s_finalize<4> : k_s2s_finalize<1>, dim3((P + members - 1u) / members), dim3(256), 0, st, a.partial, P,
+    const bool four = mma && a.n_chunks > 4u;
+    const uint32_t members = four ? 64u : 256u;                   // per block of 256 threads
+    if (launch_dependent(four ? k_s2s_finalize<4> : k_s2s_finalize<1>, dim3((P + members - 1u) / members), dim3(256), 0, st, a.partial, P,
                          a.n_chunks, inv, fitness) != cudaSuccess)
         return -1;
     return 2;
