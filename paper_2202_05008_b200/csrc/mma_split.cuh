@@ -236,8 +236,10 @@ __device__ __forceinline__ void tanh_two(float& p, float& q)
 // With the Taylor polynomial to x^9 below |x| = 0.3, where what it leaves out is below 6e-8 of x.  For k_rollout_mlp_deep and
 // k_rollout_mlp_mma, which also take policies with layers so narrow that their sums do not hide the exponential's error near 1.  State error
 // against that of tanhf on the fp32 pipe, after 1 / 20 / 200 steps: 28-20-8 without it 1.05 / 1.05 / 1.18, with it 0.95 / 0.82 / 0.92;
-// 28-64-10-10-8 without 1.04 / 1.12 / 1.16; 28-64-64-64-8 without 0.91 / 0.84 / 0.86.  It costs k_rollout_mlp_mma 4 % with that last
-// one (485 us a generation of 512 members instead of 465), so a policy has it whose narrowest hidden layer is below 49 units.
+// 28-64-10-10-8 without 1.04 / 1.12 / 1.16; 28-64-64-64-8 without 0.91 / 0.84 / 0.86.  In k_rollout_mlp_deep after 5 / 20 / 60 steps: 28-40-8
+// without 0.95 / 1.09 / 1.09, 28-48-8 0.96 / 1.01 / 1.01, 28-56-8 0.93 / 0.96 / 0.98, 28-40-40-40-8 0.94 / 1.05 / 1.03, 28-56-56-56-8 0.89 / 0.94 / 0.93,
+// all with it 0.74 to 0.82.  It costs there 4 to 12 % (28-64-64-64-8, 512 members, 200 steps 222 -> 244 us; 128 members 143 -> 148), so a
+// policy has it whose narrowest hidden layer is below 49 units.
 __device__ __forceinline__ float tanh_fine(float p)
 {
     constexpr double f = 2.885390081777927, g = 1.0 / (f * f);                // z = p^2 = x^2 / g

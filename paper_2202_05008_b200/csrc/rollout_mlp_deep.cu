@@ -7,8 +7,8 @@
 // barrier per layer; the action layer needs no pass of its own (a warp turns its last units into an operand, and partial sums meet).
 //
 // What bounds it: the serial chain of a step, HIDDEN + 1 barriers long, with as many members per SM as the registers hold
-// (28-64-64-64-8, 4 episodes: 0.76 us a step with one member on an SM, 1.16 us with up to four).  k_rollout_mlp_mma, which
-// reads the operands of every layer from shared memory in runtime loops, takes 1.74 and 2.24 us.  With the low parts in
+// (28-64-64-64-8, 4 episodes: 0.71 us a step with one member on an SM, 1.11 us with up to four).  k_rollout_mlp_mma, which
+// reads the operands of every layer from shared memory in runtime loops, takes 1.69 and 2.21 us.  With the low parts in
 // registers too the compiler has none left to work with: 0.86 and 1.19 us, and 4.1 against 2.9 us for 16 episodes of 512 members.
 //
 // Paper: Section 2 (roll-out loop, central seeds), Section 4 (get_actions over the population with parameters as

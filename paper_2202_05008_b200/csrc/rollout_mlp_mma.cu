@@ -6,8 +6,7 @@
 // memory in operand order: a 16x16 tile is one 128-bit load per lane and part.  A warp takes 16 units of a
 // layer (several if the layer has more than the block's warps), applies bias and tanh to its accumulators in
 // registers, and writes the two fp16 parts of the result as the next layer's B operand.  A layer so costs one
-// barrier (28-64-64-64-8, 4 episodes, were it to run here: 1.57 us a step, 620 clocks for each of its five products, with one member on
-// an SM; 2.07 us with four).  The dynamics of the tanh-linear task
+// barrier (28-64-64-64-8, 4 episodes, were it to run here: 1.69 us a step with one member on an SM, 2.21 us with four).  The dynamics of the tanh-linear task
 // are one more layer ([A | B] on the state with the action behind it); the cart-pole's five inputs are taken
 // in fp32, and a warp of its own steps the task, which works on the coming step while the layers run.
 //

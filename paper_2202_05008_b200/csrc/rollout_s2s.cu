@@ -217,7 +217,7 @@ __global__ void k_s2s_finalize(const float* __restrict__ partial, uint32_t P, ui
 // The gates in fp32: sigma(x) = 1 / (1 + 2^(-x log2 e)), tanh(x) = 2 sigma(2 x) - 1.  The special-function unit, which takes 8
 // clocks per warp for an exponential and 16 for a reciprocal, bounds the kernel, so a cell's four gates share one
 // reciprocal and two cells share that of tanh(c): 64 clocks per cell and step.  The CUDA-core version took one
-// fp32 multiply-add per weight and query on top: h = 64, 2 digits, 300 members x 100 queries: 765 us, here 75 us.
+// fp32 multiply-add per weight and query on top: h = 64, 2 digits, 300 members x 100 queries: 765 us, here 67 us.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1)
 {
