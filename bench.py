@@ -88,22 +88,22 @@ def stage_work(w, stored):
 # that digest; once a kernel's source changes its entry reads null until it is captured again.
 CSRC = os.path.join(ROOT, "paper_2202_05008_b200", "csrc")
 NCU_TRAFFIC = {
-    ("cfg4", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 3.526500e+08,
+    ("cfg4", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 3.523800e+08,
                          "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
-                         "digest": "ae8637185501763c", "capture": "T = 200 (the parameters are read once, whatever the horizon)"},
+                         "digest": "1b67439b175a725e", "capture": "T = 200 (the parameters are read once, whatever the horizon)"},
     ("cfg2", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 4.790000e+06,
                          "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
-                         "digest": "ae8637185501763c", "capture": "full size"},
-    ("cfg3", "stored"): {"kernel": "k_cnn_conv2_tc", "bytes": 1.568400e+08,
+                         "digest": "1b67439b175a725e", "capture": "full size"},
+    ("cfg3", "stored"): {"kernel": "k_cnn_conv2_tc", "bytes": 1.565100e+08,
                          "files": ['rollout_cnn_tc.cu', 'umma.cuh', 'async.cuh', 'fp32x2.cuh', 'internal.h'],
-                         "digest": "62b6b22dac9c41d2", "capture": "full size"},
-    ("cfg5", "stored"): {"kernel": "k_ask", "bytes": 1.012202e+11,
+                         "digest": "92dd5c5bb53fc0c1", "capture": "full size"},
+    ("cfg5", "stored"): {"kernel": "k_ask", "bytes": 1.011830e+11,
                          "files": ['solver_kernels.cu', 'noise.cuh', 'internal.h'],
-                         "digest": "9817b3dd7b04751f",
+                         "digest": "d063f1ff879f2067",
                          "capture": "D = 32,768 capture scaled by 32 (columns are independent)"},
-    ("cfg5", "regenerated"): {"kernel": "k_ask", "bytes": 6.683488e+10,
+    ("cfg5", "regenerated"): {"kernel": "k_ask", "bytes": 6.683520e+10,
                               "files": ['solver_kernels.cu', 'noise.cuh', 'internal.h'],
-                              "digest": "9817b3dd7b04751f", "capture": "D = 32,768 capture scaled by 32"},
+                              "digest": "d063f1ff879f2067", "capture": "D = 32,768 capture scaled by 32"},
 }
 NCU_TRAFFIC[("cfg4", "regenerated")] = NCU_TRAFFIC[("cfg4", "stored")]
 NCU_TRAFFIC[("cfg2", "regenerated")] = NCU_TRAFFIC[("cfg2", "stored")]
