@@ -590,6 +590,8 @@ __device__ __forceinline__ void half_barrier(uint32_t half)
     else      asm volatile("bar.sync 1, %0;" :: "n"(kTcHalfThreads) : "memory");
 }
 
+// FULL: every item has 128 queries, and the loops do not ask (1,036 members, 3 digits: 454 us; the other instance takes 465).
+template <bool FULL>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_s2s_tc(const S2sArgs a, DeviceStatus* status)
 {
@@ -598,6 +600,8 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
     const uint32_t Te = 2 * a.nd + 1, Td = a.nd + 1, T = Te + Td;
     const uint32_t n_items = a.P * a.n_chunks;
+    // chunks of equal size, so that blocks have equal work
+    const uint32_t per_chunk = FULL ? kTcQ : ((a.B + a.n_chunks - 1u) / a.n_chunks + 7u) & ~7u;
     const PhiloxKey key = philox_key(a.k0, a.k1);
 
     if (tid == 0) {
@@ -623,13 +627,18 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
 
     for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const uint32_t member = item / a.n_chunks, chunk = item % a.n_chunks;
-        const uint32_t q0 = chunk * kTcQ;
-        const uint32_t nq = min(static_cast<uint32_t>(kTcQ), a.B - q0);
+        const uint32_t q0 = chunk * per_chunk;
+        const uint32_t nq = FULL ? kTcQ : min(per_chunk, a.B - q0);
+        // The halves share the queries evenly, to eights, and what holds none is left out: a half, eight queries of it, a warp's read-out.
+        // Every item was worked off as 128 queries before.  1,036 members, 3 digits: 40 queries 456 -> 330 us, 64 456 -> 348, 100 457 -> 449,
+        // 130 (two items of 65 instead of 128 and 2) 852 -> 672, 300 1,275 -> 1,217.
+        const uint32_t nq0 = FULL ? 64u : min(nq, (nq + 15u) / 16u * 8u), n_halves = FULL || nq > nq0 ? 2u : 1u, nq_half = half ? nq - nq0 : nq0;
         const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
 
         // ---- per-item setup: queries, zero state, read-out weights, encoder weights ------------
         if (chunk != staged_chunk) {
-            if (tid < kTcQ) s2s_query(key, a.status->generation, q0 + min(tid, nq - 1u), a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
+            if (tid < kTcQ)
+                s2s_query(key, a.status->generation, q0 + min(tid < 64u ? tid : nq0 + tid - 64u, nq - 1u), a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
             staged_chunk = chunk;
         }
         if (is_mma) {                                            // the decoder's weights will be wanted next
@@ -637,8 +646,8 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
             constexpr uint32_t piece = kTcCellFloats * 4u / 32u;       // 9,024 bytes per lane
             prefetch_l2(next + lane * piece, piece);
         }
-        for (uint32_t i = tid; i < 16u * kTcBLbo / 16u; i += kTcThreads)
-            reinterpret_cast<uint4*>(S.Bop)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (FULL)
+            for (uint32_t i = tid; i < 16u * kTcBLbo / 16u; i += kTcThreads) reinterpret_cast<uint4*>(S.Bop)[i] = make_uint4(0u, 0u, 0u, 0u);
         for (uint32_t i = tid; i < kVocab * 16u; i += kTcThreads) {       // (token, K group) -> 8 weights
             const uint32_t o = i >> 4, kb = i & 15u;
             const float4* src = reinterpret_cast<const float4*>(p + 2u * kTcCellFloats + o * kTcH + kb * 8u);
@@ -683,27 +692,34 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
                 for (uint32_t t = t0; t < t1; ++t) {
 #pragma unroll
                     for (uint32_t x = 0; x < 2u; ++x) {
-                        if (t > 0) {                             // step 0 reads the state the setup wrote
+                        if (x >= n_halves) break;
+                        if (t > 0) {                             // step 0 reads the tokens that the setup wrote
                             uint32_t& n = x ? n_wait1 : n_wait;
                             wait_or_abort(&S.abort, &S.hready[x], n & 1u, status);
                             ++n;
                         }
                         tc_fence_after();
                         if (elect_one()) {
+                            auto issue = [&](uint32_t g, uint32_t kk, uint32_t accumulate) {
+                                const uint64_t ad = umma_smem_desc(a_base + 2u * kk * kTcALbo + g * 16u * 128u, kTcALbo, 128u);
+                                const uint64_t bd = umma_smem_desc(b_base + 2u * kk * kTcBLbo + x * 8u * 128u, kTcBLbo, 128u);
+                                umma_bf16(tmem + x * 256u + g * 64u, ad, bd, idesc, accumulate);
+                            };
+                            if (!FULL && t == 0u) {              // the start state is zero: token and bias only (the last K-step)
 #pragma unroll
-                            for (uint32_t g = 0; g < 4u; ++g)
+                                for (uint32_t g = 0; g < 4u; ++g) issue(g, kTcKBlocks / 2 - 1, 0u);
+                            } else {
 #pragma unroll
-                                for (uint32_t kk = 0; kk < kTcKBlocks / 2; ++kk) {
-                                    const uint64_t ad = umma_smem_desc(a_base + 2u * kk * kTcALbo + g * 16u * 128u, kTcALbo, 128u);
-                                    const uint64_t bd = umma_smem_desc(b_base + 2u * kk * kTcBLbo + x * 8u * 128u, kTcBLbo, 128u);
-                                    umma_bf16(tmem + x * 256u + g * 64u, ad, bd, idesc, kk);
-                                }
+                                for (uint32_t g = 0; g < 4u; ++g)
+#pragma unroll
+                                    for (uint32_t kk = 0; kk < kTcKBlocks / 2; ++kk) issue(g, kk, kk);
+                            }
                             umma_commit(smem_u32(&S.full[x]));
                         }
                         __syncwarp();
                     }
                 }
-            } else {
+            } else if (half < n_halves) {
                 // ================= epilogue warps ======================================================
                 const uint32_t tq = tmem + (static_cast<uint32_t>((warp & 3u) * 32u) << 16) + half * 256u + sub * kTcCols;
                 for (uint32_t t = t0; t < t1; ++t) {
@@ -754,6 +770,7 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
                             *reinterpret_cast<uint16_t*>(dst + j * 16 + 16) = static_cast<uint16_t>(hb >> 16);
                         }
                         if (ch + 1u < kTcCols / 8u) tmem_ld8x4_fence(g0[nxt], g1[nxt], g2[nxt], g3[nxt]);
+                        if (!FULL && sub * kTcCols + (ch + 1u) * 8u >= nq_half) break;
                     }
                     // the coming step's token (none after the last step)
                     if (t + 1u < T && sub == 0u && r < 64u) {
@@ -768,12 +785,13 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
                         half_barrier(half);
                         if (t + 1u < T && lane == 0) mbar_arrive(smem_u32(&S.hready[half]));
                         const uint32_t s = tid & 63u, o0 = ((tid % kTcHalfThreads) >> 6) * kTcOutPerThread;
+                        const uint32_t kb_end = FULL || (s & 32u) < nq_half ? 16u : 0u;             // (logits of no query are not looked at)
                         float2 acc[kTcOutPerThread];
 #pragma unroll
                         for (int o = 0; o < kTcOutPerThread; ++o) acc[o] = make_float2(0.f, 0.f);
                         const unsigned char* hrow = S.Bop + (half * 64u + s) * 16u;
 #pragma unroll 4
-                        for (uint32_t kb = 0; kb < 16u; ++kb) {
+                        for (uint32_t kb = 0; kb < kb_end; ++kb) {
                             const uint4 hv = *reinterpret_cast<const uint4*>(hrow + kb * kTcBLbo);
                             const uint32_t hw[4] = { hv.x, hv.y, hv.z, hv.w };
                             float2 x[4];
@@ -805,7 +823,8 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         __syncthreads();
         for (uint32_t idx = tid; idx < Td * kTcQ; idx += kTcThreads) {
             const uint32_t pos = idx / kTcQ, q = idx % kTcQ;
-            if (q < nq) loss += token_loss(S.lg[pos][q], S.tgt[q][pos]);
+            const uint32_t row = q < nq0 ? q : 64u + q - nq0;
+            if (q < nq) loss += token_loss(S.lg[pos][row], S.tgt[row][pos]);
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
@@ -875,11 +894,11 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
             if (cudaGetDevice(&dev) != cudaSuccess) return -1;
             if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
         }
-        if (cudaFuncSetAttribute(k_s2s_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(sizeof(S2sSmem))) != cudaSuccess) return -1;
+        auto kernel = B % kTcQ == 0u ? k_s2s_tc<true> : k_s2s_tc<false>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(S2sSmem))) != cudaSuccess) return -1;
         const uint32_t items = P * a.n_chunks;
         const uint32_t grid = items < static_cast<uint32_t>(sm_count) ? items : static_cast<uint32_t>(sm_count);
-        k_s2s_tc<<<grid, kTcThreads, sizeof(S2sSmem), st>>>(a, status);
+        kernel<<<grid, kTcThreads, sizeof(S2sSmem), st>>>(a, status);
     } else if (mma) {
         if (launch_s2s_mma(st, a, split) != cudaSuccess) return -1;
     } else {
