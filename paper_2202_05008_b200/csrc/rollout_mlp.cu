@@ -202,8 +202,8 @@ int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStat
 uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes);
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
-// The kernel of a policy: AUTO takes a register-resident one where the policy has one to four hidden layers of up to 128
-// units (three and four where that is the faster one, see mlp_choice.h), for other numbers of layers and wider ones the one with the weights in
+// The kernel of a policy: AUTO takes a register-resident one where the policy has one to four hidden layers of up to 192
+// units (three and four, and any above 128 units, where that is the faster one, see mlp_choice.h), for other numbers of layers and wider ones the one with the weights in
 // shared memory as long as they fit it, and else the runtime-shape kernel, which reads them through the caches.
 enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kDeep, kSharedMemory };
 

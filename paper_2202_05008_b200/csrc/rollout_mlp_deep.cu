@@ -1,5 +1,5 @@
-// Control roll-outs of policies with one, three or four hidden layers of up to 128 units, on warp-level tensor-core products
-// (mma_split.cuh) with the weights in REGISTERS for all T steps: what k_rollout_mlp2 is for two hidden layers.
+// Control roll-outs of policies with one, three or four hidden layers of up to 192 units (and of two, one of them above 128), on warp-level
+// tensor-core products (mma_split.cuh) with the weights in REGISTERS for all T steps: what k_rollout_mlp2 is for two hidden layers.
 //
 // Block = (member, EB episodes).  A warp owns 16 units of every layer: it keeps the operand tiles of the first layer, the hi parts of
 // its rows of the matrices between hidden layers, and the action layer's columns of its own units in registers; the low parts of the
@@ -10,6 +10,10 @@
 // (28-64-64-64-8, 4 episodes: 0.71 us a step with one member on an SM, 1.11 us with up to four).  k_rollout_mlp_mma, which
 // reads the operands of every layer from shared memory in runtime loops, takes 1.69 and 2.21 us.  With the low parts in
 // registers too the compiler has none left to work with: 0.86 and 1.19 us, and 4.1 against 2.9 us for 16 episodes of 512 members.
+//
+// Above 128 units (KT = 12) a block has up to twelve warps and an SM to itself.  100 members, 4 episodes, us a step, with k_rollout_mlp_mma behind:
+// 28-160-8 0.47 / 1.34, 5-190-180-1 1.15 / 3.00, 5-145-52-48-1 1.31 / 2.22, 28-150-60-60-60-8 1.51 / 2.60; 28-180-180-180-8 1.97 / 66.7 (the runtime-shape
+// kernel: its weights do not fit the shared memory).
 //
 // Paper: Section 2 (roll-out loop, central seeds), Section 4 (get_actions over the population with parameters as
 // data; stateless task step; identical initial observations).
@@ -28,19 +32,22 @@ using namespace ms;
 
 constexpr uint32_t kXPitch = 32 * 2 + 16;           // bytes per column of the state operand [x 28 | 0 4]
 constexpr uint32_t kDynTiles = 6;                   // [A | B] in operand tiles: two of 16 rows x three of 16 inputs
+constexpr int kMaxDynamic = 198 * 1024;             // shared memory besides the static arrays, which take up to 28.2 KB
+constexpr size_t kMaxLowBytes = 190u * 1024u;
 
-// HIDDEN: hidden layers; KT: 16-unit tiles of the widest, 4 or 8; FINE: see tanh_fine.
+// HIDDEN: hidden layers; KT: 16-unit tiles of the widest, 4, 8 or 12; FINE: see tanh_fine.
 template <int EB, bool CART, int HIDDEN, int KT, bool FINE>
-__global__ void __launch_bounds__(32 * KT, KT == 4 ? 4 : HIDDEN <= 3 ? 2 : 1)
+__global__ void __launch_bounds__(32 * KT, KT == 4 ? 4 : KT == 8 && HIDDEN <= 3 ? 2 : 1)
 k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
 {
     using U = Units<EB>;
     constexpr int NV = U::kValues, NH = NV / 2;                      // NH: values of one unit in a lane
     constexpr int NM = HIDDEN - 1, NS = NM > 0 ? NM : 1;             // matrices between hidden layers (and room for them)
+    constexpr int RM = KT == 12 && NM > 2 ? 2 : NS;                  // of which the hi parts are in registers (48 a matrix and thread)
     constexpr Tanh kTanh = FINE ? Tanh::kFine : Tanh::kOwn;
     constexpr uint32_t kPitch = KT / 2 * 64 + 16;                    // bytes per column of a hidden operand (read two tiles at a time)
     constexpr uint32_t kHidBytes = U::kRows * kPitch;
-    extern __shared__ __align__(16) uint4 lows[];                    // low parts of the matrices, [warp][matrix][tile][lane]
+    extern __shared__ __align__(16) uint4 lows[];                    // low parts of the matrices, [warp][matrix][tile][lane]; KT = 12: see below
     __shared__ uint32_t peak;
     __shared__ __align__(16) unsigned char hid[NM > 1 ? 2 : 1][kHidBytes];               // outputs of the hidden layers, in turn
     __shared__ __align__(16) float obs[CART ? 5 : 1][EB];            // cart-pole: observation
@@ -98,11 +105,27 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
     const float* W3 = row + w3_at;
     const float* B3 = W3 + nout * nl;
     const int u0 = 16 * warp + g, u1 = u0 + 8;                       // this lane's two units of every layer
-    uint4 wh[NS][KT];
+    uint4 wh[RM][KT];
     uint4 w1h[2], w1l[2], w3 = make_uint4(0u, 0u, 0u, 0u);           // w3: the action layer's own inputs (see Units::eight)
     float w1c[10], w3c[2], bias[HIDDEN][2], b3;
     float* const ups1 = ups + u0, *const ups3 = ups + HIDDEN * 16 * KT + g;              // ups1: + 16 KT per layer
-    uint4* const wl = lows + warp * (NM * KT * 32) + lane;
+    // KT = 12: [matrix][warp][tile][lane], only what the layers have, tiles in fours; behind them the hi parts of a matrix that are not in registers
+    uint4* wl[NS];
+    uint4* whs = nullptr;
+    {
+        uint4* to = lows + (KT == 12 ? 0 : warp * (NM * KT * 32)) + lane;
+#pragma unroll
+        for (int m = 0; m < NS; ++m) {
+            if constexpr (KT == 12) {
+                const int tiles = m < NM ? (mt[m] + 3) & ~3 : 0, rows = m < NM ? mt[m + 1 < HIDDEN ? m + 1 : m] : 0;
+                wl[m] = to + 32 * warp * tiles;
+                to += 32 * rows * tiles;
+                if (m >= RM) { whs = to + 32 * warp * tiles; to += 32 * rows * tiles; }
+            } else {
+                wl[m] = to + 32 * m * KT;
+            }
+        }
+    }
     bias[0][0] = u0 < n[0] ? times_f(B1[u0]) : 0.f; bias[0][1] = u1 < n[0] ? times_f(B1[u1]) : 0.f;
     if constexpr (CART) {                                            // the observation is taken as it is, in fp32
 #pragma unroll
@@ -146,9 +169,13 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
         }
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
-            uint4 lo;
-            load_tile(W, n[m], n[m + 1], 16 * warp, 16 * k, lane, s0, s1, wh[m][k], lo, pairs);
-            wl[32 * (m * KT + k)] = lo;
+            uint4 hi, lo;
+            load_tile(W, n[m], n[m + 1], 16 * warp, 16 * k, lane, s0, s1, hi, lo, pairs);
+            if (m < RM) wh[m < RM ? m : 0][k] = hi;
+            if (KT < 12 || (warp < mt[m + 1] && k < ((mt[m] + 3) & ~3))) {
+                wl[m][32 * k] = lo;
+                if (m >= RM) whs[32 * k] = hi;
+            }
         }
     }
 
@@ -269,15 +296,19 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
                             U::load(in + 32u * k + 64u, next);
                             if (U::kLoadTiles == 1) U::load(in + 32u * k + 96u, next + 1);
                         }
-                        const uint4 lo = wl[32 * (m * KT + k)];
-                        if (k == 0) acc.first(wh[m][k], lo, now[0]);
-                        else acc.add(wh[m][k], lo, now[k & 1]);
+                        const uint4 lo = wl[m][32 * k], hi = m < RM ? wh[m < RM ? m : 0][k] : whs[32 * k];
+                        if (k == 0) acc.first(hi, lo, now[0]);
+                        else acc.add(hi, lo, now[k & 1]);
                     };
 #pragma unroll
                     for (int k = 0; k < 4; ++k) products(k);
                     if (KT > 4 && mt[m] > 4) {                           // (not behind a narrow layer of a wide policy)
 #pragma unroll
-                        for (int k = 4; k < KT; ++k) products(k);
+                        for (int k = 4; k < (KT < 8 ? KT : 8); ++k) products(k);
+                        if (KT > 8 && mt[m] > 8) {
+#pragma unroll
+                            for (int k = 8; k < KT; ++k) products(k);
+                        }
                     }
                 }
                 if (m == 0) meanwhile();
@@ -297,10 +328,10 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
                     float p[EB];
 #pragma unroll
                     for (int i = 0; i < EB; ++i) p[i] = (&part_c[0][0])[lane + 32 * i];
-                    if constexpr (KT > 4) {
 #pragma unroll
-                        for (int i = 0; i < EB; ++i) p[i] += (&part_c[KT - 4][0])[lane + 32 * i];
-                    }
+                    for (int w = 4; w < KT; w += 4)
+#pragma unroll
+                        for (int i = 0; i < EB; ++i) p[i] += (&part_c[w][0])[lane + 32 * i];
 #pragma unroll
                     for (int k = EB / 2; k > 0; k >>= 1)
 #pragma unroll
@@ -319,9 +350,10 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
                 for (int w = 0; w < 4; ++w) {
                     if constexpr (EB == 4) p[w][0] = part_t[w][lane];
                     else { const float2 q = *reinterpret_cast<const float2*>(&part_t[w][2 * lane]); p[w][0] = q.x; p[w][1] = q.y; }
-                    if constexpr (KT > 4) {
-                        if constexpr (EB == 4) p[w][0] += part_t[KT - 4 + w][lane];
-                        else { const float2 q = *reinterpret_cast<const float2*>(&part_t[KT - 4 + w][2 * lane]); p[w][0] += q.x; p[w][1] += q.y; }
+#pragma unroll
+                    for (int more = 4; more < KT; more += 4) {
+                        if constexpr (EB == 4) p[w][0] += part_t[more + w][lane];
+                        else { const float2 q = *reinterpret_cast<const float2*>(&part_t[more + w][2 * lane]); p[w][0] += q.x; p[w][1] += q.y; }
                     }
                 }
                 U acc;
@@ -390,25 +422,33 @@ k_rollout_mlp_deep(const RolloutMlpArgs a, DeviceStatus* status)
     }
 }
 
+using DeepKernel = void (*)(const RolloutMlpArgs, DeviceStatus*);
+
+// size: 0 up to 64 units, 1 up to 128, 2 up to 192
 template <int EB, bool CART, int HIDDEN>
-auto pick_width(bool wide, bool fine)
+DeepKernel pick_size(uint32_t size, bool fine)
 {
-    if (wide) return fine ? k_rollout_mlp_deep<EB, CART, HIDDEN, 8, true> : k_rollout_mlp_deep<EB, CART, HIDDEN, 8, false>;
-    return fine ? k_rollout_mlp_deep<EB, CART, HIDDEN, 4, true> : k_rollout_mlp_deep<EB, CART, HIDDEN, 4, false>;
+    if (size == 2u) return fine ? k_rollout_mlp_deep<EB, CART, HIDDEN, 12, true> : k_rollout_mlp_deep<EB, CART, HIDDEN, 12, false>;
+    if constexpr (HIDDEN == 2) return nullptr;                       // (k_rollout_mlp2)
+    else {
+        if (size == 1u) return fine ? k_rollout_mlp_deep<EB, CART, HIDDEN, 8, true> : k_rollout_mlp_deep<EB, CART, HIDDEN, 8, false>;
+        return fine ? k_rollout_mlp_deep<EB, CART, HIDDEN, 4, true> : k_rollout_mlp_deep<EB, CART, HIDDEN, 4, false>;
+    }
 }
 template <int EB, bool CART>
-auto pick_kernel(uint32_t hidden, bool wide, bool fine)
+DeepKernel pick_kernel(uint32_t hidden, uint32_t size, bool fine)
 {
-    return hidden == 1u ? pick_width<EB, CART, 1>(wide, fine) : hidden == 3u ? pick_width<EB, CART, 3>(wide, fine) : pick_width<EB, CART, 4>(wide, fine);
+    switch (hidden) {
+        case 1u: return pick_size<EB, CART, 1>(size, fine);
+        case 2u: return pick_size<EB, CART, 2>(size, fine);
+        case 3u: return pick_size<EB, CART, 3>(size, fine);
+        default: return pick_size<EB, CART, 4>(size, fine);
+    }
 }
 
 uint32_t tiles_of(uint32_t units) { return (units + 15u) / 16u; }
 
-}  // namespace
-
-namespace {
-
-struct DeepLaunch { void (*kernel)(const RolloutMlpArgs, DeviceStatus*); uint32_t threads; size_t bytes; bool wide, fine; };
+struct DeepLaunch { DeepKernel kernel; uint32_t threads; size_t bytes; uint32_t size; bool fine; };
 
 DeepLaunch deep_launch(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t EB)
 {
@@ -421,12 +461,16 @@ DeepLaunch deep_launch(uint32_t task, uint32_t n_layers, const uint32_t* sizes, 
         if (tiles_of(sizes[l]) > warps) warps = tiles_of(sizes[l]);
         d.fine = d.fine || sizes[l] < 49u;
     }
-    d.wide = warps > 4u;
+    d.size = warps > 8u ? 2u : warps > 4u ? 1u : 0u;
     if (!cart && warps < 2u) warps = 2u;
     d.threads = 32u * warps;
-    d.kernel = EB == 4u ? (cart ? pick_kernel<4, true>(hidden, d.wide, d.fine) : pick_kernel<4, false>(hidden, d.wide, d.fine))
-                        : (cart ? pick_kernel<8, true>(hidden, d.wide, d.fine) : pick_kernel<8, false>(hidden, d.wide, d.fine));
-    d.bytes = static_cast<size_t>(warps) * (hidden - 1u) * (d.wide ? 8u : 4u) * 512u;
+    d.kernel = EB == 4u ? (cart ? pick_kernel<4, true>(hidden, d.size, d.fine) : pick_kernel<4, false>(hidden, d.size, d.fine))
+                        : (cart ? pick_kernel<8, true>(hidden, d.size, d.fine) : pick_kernel<8, false>(hidden, d.size, d.fine));
+    d.bytes = static_cast<size_t>(warps) * (hidden - 1u) * (d.size == 1u ? 8u : 4u) * 512u;
+    if (d.size == 2u) {                                              // the layers' own tiles; the third matrix with its hi parts
+        d.bytes = 0;
+        for (uint32_t m = 1; m < hidden; ++m) d.bytes += tiles_of(sizes[m + 1]) * ((tiles_of(sizes[m]) + 3u) & ~3u) * (m > 2u ? 1024u : 512u);
+    }
     return d;
 }
 
@@ -435,9 +479,11 @@ DeepLaunch deep_launch(uint32_t task, uint32_t n_layers, const uint32_t* sizes, 
 // Episodes per block; 0: not a policy for this kernel.
 uint32_t rollout_mlp_deep_eb(uint32_t n_layers, const uint32_t* sizes, uint32_t episodes)
 {
-    if (n_layers != 2u && n_layers != 4u && n_layers != 5u) return 0u;
-    for (uint32_t l = 1; l < n_layers; ++l)
-        if (tiles_of(sizes[l]) > 8u) return 0u;
+    if (n_layers < 2u || n_layers > 5u) return 0u;
+    uint32_t widest = 0;
+    for (uint32_t l = 1; l < n_layers; ++l) widest = tiles_of(sizes[l]) > widest ? tiles_of(sizes[l]) : widest;
+    if (widest > 12u || (n_layers == 3u && widest <= 8u)) return 0u;
+    if (deep_launch(EVO_TASK_CARTPOLE, n_layers, sizes, 4u).bytes > kMaxLowBytes) return 0u;
     return episodes > 4u ? 8u : 4u;
 }
 
@@ -446,15 +492,17 @@ uint32_t rollout_mlp_deep_eb(uint32_t n_layers, const uint32_t* sizes, uint32_t 
 int rollout_mlp_deep_pays(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t pop, uint32_t EB, uint32_t n_eb)
 {
     if (n_layers == 2u) return 1;
-    static std::atomic<uint64_t> known[2][2][2][2][2];
+    static std::atomic<uint64_t> known[2][2][3][3][2];
     const DeepLaunch d = deep_launch(task, n_layers, sizes, EB);
     uint32_t regs;
     size_t fixed;
-    if (!kernel_needs(d.kernel, known[EB == 8u][task == EVO_TASK_CARTPOLE][n_layers == 5u][d.wide][d.fine], &regs, &fixed)) return -1;
+    if (!kernel_needs(d.kernel, known[EB == 8u][task == EVO_TASK_CARTPOLE][n_layers - 3u][d.size][d.fine], &regs, &fixed)) return -1;
     const int mma = rollout_mlp_mma_resident(task, n_layers, sizes, EB);
     if (mma < 0) return -1;
-    return mlp_deep_pays(n_layers - 1u, d.wide, EB, static_cast<uint64_t>(pop) * n_eb, kSms, resident_blocks(regs, d.bytes + fixed, d.threads),
-                         static_cast<uint32_t>(mma));
+    const uint64_t blocks = static_cast<uint64_t>(pop) * n_eb;
+    const uint32_t deep = resident_blocks(regs, d.bytes + fixed, d.threads);
+    if (d.size == 2u) return mlp_widest_pays(blocks, kSms, deep, static_cast<uint32_t>(mma));
+    return mlp_deep_pays(n_layers - 1u, d.size == 1u, EB, blocks, kSms, deep, static_cast<uint32_t>(mma));
 }
 
 int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status)
@@ -462,7 +510,7 @@ int launch_rollout_mlp_deep(cudaStream_t st, const RolloutMlpArgs& a, DeviceStat
     const DeepLaunch d = deep_launch(a.task, a.n_layers, a.sizes, a.EB);
     const size_t bytes = spread_over_sms(d.kernel, d.bytes, static_cast<uint64_t>(a.P) * a.n_eb);
     if (!a.attr_done &&
-        cudaFuncSetAttribute(d.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) return -1;
+        cudaFuncSetAttribute(d.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamic) != cudaSuccess) return -1;
     return launch_dependent(d.kernel, dim3(a.P, a.n_eb), dim3(d.threads), bytes, st, a, status) == cudaSuccess ? 1 : -1;
 }
 

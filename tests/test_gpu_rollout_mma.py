@@ -122,6 +122,14 @@ def test_one_three_and_four_hidden_layers_with_the_weights_in_registers(sizes, e
     check(sizes, episodes, 40, scale=0.05 if sizes[0] == 28 else 0.25)
 
 
+@pytest.mark.parametrize("sizes", [(28, 129, 8), (28, 192, 8), (28, 192, 192, 8), (28, 192, 176, 180, 8), (28, 144, 145, 129, 8), (28, 20, 190, 5, 8),
+                                   (28, 129, 64, 65, 130, 8), (28, 192, 100, 64, 192, 8), (5, 130, 1), (5, 190, 180, 1), (5, 16, 17, 192, 1),
+                                   (5, 192, 192, 192, 1), (5, 160, 48, 49, 160, 1), (5, 3, 176, 128, 64, 1)])
+@pytest.mark.parametrize("episodes", [3, 11])
+def test_up_to_192_units_with_the_weights_in_registers(sizes, episodes):
+    check(sizes, episodes, 30, scale=0.04 if sizes[0] == 28 else 0.2)
+
+
 @pytest.mark.parametrize("sizes", [(28, 128, 8), (28, 64, 64, 64, 8), (28, 128, 100, 128, 8), (28, 64, 40, 64, 30, 8), (28, 128, 128, 128, 128, 8),
                                    (5, 60, 1), (5, 64, 64, 64, 1), (5, 128, 30, 100, 64, 1)])
 @pytest.mark.parametrize("episodes", [4, 5])

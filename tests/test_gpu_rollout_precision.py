@@ -70,6 +70,13 @@ def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, po
     _check_against_fp32(w, _population(w, sum(sizes) + pop))
 
 
+@pytest.mark.parametrize("sizes,episodes", [((28, 160, 8), 4), ((28, 192, 140, 8), 8), ((28, 150, 130, 190, 8), 4), ((28, 129, 60, 80, 180, 8), 8),
+                                            ((5, 192, 1), 4), ((5, 140, 150, 160, 1), 8)])
+def test_the_same_of_more_than_128_units(sizes, episodes):
+    w = _workload(sizes, 64, episodes)
+    _check_against_fp32(w, _population(w, sum(sizes)))
+
+
 @pytest.mark.parametrize("sizes,pop,episodes", [
     ((28, 64, 64, 8), 64, 4), ((28, 128, 128, 8), 300, 4), ((28, 64, 64, 64, 8), 64, 8), ((5, 16, 16, 1), 64, 4),
     ((5, 64, 64, 1), 64, 8), ((5, 128, 90, 1), 300, 4), ((5, 40, 40, 40, 1), 64, 4),

@@ -80,3 +80,23 @@ def test_waves(lib):
     (32, 57 * 1024 - 1024, 128, 4), (32, 57 * 1024 - 1023, 128, 3), (32, 227 * 1024, 128, 1)])
 def test_blocks_that_an_sm_holds(lib, regs, smem, threads, blocks):
     assert lib.resident(regs, smem, threads) == blocks
+
+
+# blocks, resident blocks of the kernel with the weights in registers and of that with them in shared memory, whether the former is faster
+@pytest.mark.parametrize("blocks,deep,mma,faster", [
+    (118, 1, 3, True),      # 5-15-189-54-1: 76 / 124 us
+    (676, 1, 3, False),     # 5-107-29-138-1: 430 / 325
+    (836, 1, 1, True),      # 28-145-157-59-8: 661 / 1,159
+    (424, 1, 3, False),     # 28-154-13-77-8: 259 / 158
+    (288, 1, 2, False),     # 28-168-47-11-8: 168 / 149
+    (354, 1, 1, True),      # 28-46-135-132-8: 245 / 486
+    (296, 1, 0, True),      # 28-180-180-180-8: 196 / 3,436 through the caches
+])
+def test_the_faster_kernel_is_taken_above_128_units(tmp_path, blocks, deep, mma, faster):
+    src, out = str(tmp_path / "widest.cc"), str(tmp_path / "libwidest.so")
+    with open(src, "w") as f:
+        f.write('#include "mlp_choice.h"\nextern "C" bool pays(uint64_t b, uint32_t rd, uint32_t rm) { return evo::mlp_widest_pays(b, 148, rd, rm); }\n')
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-o", out, src], check=True)
+    fn = C.CDLL(out).pays
+    fn.argtypes, fn.restype = [C.c_uint64, C.c_uint32, C.c_uint32], C.c_bool
+    assert fn(blocks, deep, mma) == faster
