@@ -55,11 +55,18 @@ __device__ __forceinline__ bool fetch_row(const RolloutMlpArgs& a, DeviceStatus*
 // registers and two members fill an SM.  RT = 2: four warps, the low parts of the second layer in shared memory,
 // three members per SM.  28-128-128-8, 4 episodes, per step of one / two / three resident members: RT = 1 0.76 / 0.97 us
 // (three do not fit), RT = 2 0.81 / 1.07 / 1.26 us; 28-96-40-8, 250 members: RT = 1 0.63 us, RT = 2 0.80 us.
-template <int EB, bool CART, int KT, int RT>
-__global__ void __launch_bounds__(RT == 1 && KT > 4 ? 256 : 128, RT == 2 ? 3 : KT > 4 ? 2 : 4)
+// RA, RB: row tiles per warp of the first and of the second layer, at least one of them RT.  A layer of at most half as many tiles as the other has
+// one per warp, and those of the other are dealt out in turn; four such members fit an SM.  (With two neighbouring tiles per warp in both, half
+// of the warps had nothing to do in the narrow layer: 28-90-40-8, 600 members x 4 episodes, 50 steps 171 -> 112 us; 28-40-90-8 164 -> 111;
+// 28-115-51-8, 3,470 x 4 923 -> 715; 5-120-60-1, 500 x 8 234 -> 143; 5-40-110-1, 372 x 8 114 -> 107.)  Where both layers have two a warp takes
+// neighbours: dealt out in turn, 28-128-128-8, 4,096 x 4 takes 1,426 instead of 1,331 us.  Cart-pole policies with RB = 2 have registers for
+// three members: with four 5-40-110-1, 372 x 8 takes 119.
+template <int EB, bool CART, int KT, int RA, int RB>
+__global__ void __launch_bounds__(RA + RB == 2 && KT > 4 ? 256 : 128, RA + RB == 4 || (CART && RB == 2) ? 3 : RA + RB == 3 ? 4 : KT > 4 ? 2 : 4)
 k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 {
     using U = Units<EB>;
+    constexpr int RT = RA > RB ? RA : RB;
     constexpr int NV = U::kValues, NH = NV / 2;                      // NH: values of one unit in a lane
     // The special-function unit is what several cart-pole members on an SM wait for (5-64-64-1, 256 members: 778 us with shared
     // reciprocals, 797 without), the issue slots what tanh-linear ones do (28-128-128-8, 4,096: 12.06 and 11.64 ms).
@@ -89,7 +96,8 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     const int n1 = static_cast<int>(a.sizes[1]), n2 = static_cast<int>(a.sizes[2]);
     const int nin = CART ? 5 : static_cast<int>(kTlNx), nout = CART ? 1 : static_cast<int>(kTlNa);
     const int mt1 = (n1 + 15) >> 4, mt2 = (n2 + 15) >> 4;
-    const int tile0 = warp * RT;                                     // the warp's first row tile
+    const int tile0 = RA + RB == 4 ? 2 * warp : warp, apart = RA + RB == 4 ? 1 : nw;                      // the warp's row tiles
+    auto tile_of = [&](int r) { return tile0 + r * apart; };
     const uint32_t traced = a.trace ? a.trace_T : 0u;
     const PhiloxKey key = philox_key(a.k0, a.k1);
     // The first warp (cart-pole) or two (tanh-linear) also step the task.  (Another warp in each of the blocks that share an SM was
@@ -130,49 +138,56 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
     const float* W3 = B2 + n2;
     const float* B3 = W3 + nout * n2;
     const bool pairs = ((n1 | w2_at) & 1) == 0;                      // the second layer's rows can be read two weights at a time
-    uint4 w2h[RT][KT], w2l[RT == 1 ? KT : 1];
-    uint4 w1h[CART ? 1 : RT][2], w1l[CART ? 1 : RT][2], w3[CART ? 1 : RT];           // w3: the action layer's own inputs (see Units::eight)
-    float w1c[CART ? RT : 1][10], w3c[RT][2], b1[RT][2], b2[RT][2], b3;
-    float* const ups1 = ups + 16 * tile0 + g, *const ups2 = ups1 + 16 * MW * RT, *const ups3 = ups + 2 * 16 * MW * RT + g;
-    uint4* const w2l_s = reinterpret_cast<uint4*>(stage) + warp * (RT * KT * 32) + lane;
+    uint4 w2h[RB][KT], w2l[RT == 1 ? KT : 1];
+    uint4 w1h[CART ? 1 : RA][2], w1l[CART ? 1 : RA][2], w3[CART ? 1 : RB];           // w3: the action layer's own inputs (see Units::eight)
+    float w1c[CART ? RA : 1][10], w3c[RB][2], b1[RA][2], b2[RB][2], b3;
+    float* const ups1 = ups + 16 * tile0 + g, *const ups2 = ups1 + 16 * MW * RT, *const ups3 = ups + 2 * 16 * MW * RT + g;       // + 16 apart per tile
+    uint4* const w2l_s = reinterpret_cast<uint4*>(stage) + warp * (RB * KT * 32) + lane;
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
-        const int tile = tile0 + r, u0 = 16 * tile + g, u1 = u0 + 8;              // this lane's two units
-        b2[r][0] = u0 < n2 ? times_f(B2[u0]) : 0.f; b2[r][1] = u1 < n2 ? times_f(B2[u1]) : 0.f;
-        b1[r][0] = u0 < n1 ? times_f(B1[u0]) : 0.f; b1[r][1] = u1 < n1 ? times_f(B1[u1]) : 0.f;
+        const int tile = tile_of(r), u0 = 16 * tile + g, u1 = u0 + 8;             // this lane's two units
+        if (r < RB) { b2[r < RB ? r : 0][0] = u0 < n2 ? times_f(B2[u0]) : 0.f; b2[r < RB ? r : 0][1] = u1 < n2 ? times_f(B2[u1]) : 0.f; }
+        if (r < RA) { b1[r < RA ? r : 0][0] = u0 < n1 ? times_f(B1[u0]) : 0.f; b1[r < RA ? r : 0][1] = u1 < n1 ? times_f(B1[u1]) : 0.f; }
         if constexpr (CART) {                                        // the observation is taken as it is, in fp32
+            if (r < RA) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) {
-                w1c[r][k] = u0 < n1 ? times_f(W1[u0 * 5 + k]) : 0.f;
-                w1c[r][5 + k] = u1 < n1 ? times_f(W1[u1 * 5 + k]) : 0.f;
+                for (int k = 0; k < 5; ++k) {
+                    w1c[r < RA ? r : 0][k] = u0 < n1 ? times_f(W1[u0 * 5 + k]) : 0.f;
+                    w1c[r < RA ? r : 0][5 + k] = u1 < n1 ? times_f(W1[u1 * 5 + k]) : 0.f;
+                }
             }
-            w3c[r][0] = u0 < n2 ? kF * kActInv * W3[u0] : 0.f; w3c[r][1] = u1 < n2 ? kF * kActInv * W3[u1] : 0.f;
+            if (r < RB) { w3c[r < RB ? r : 0][0] = u0 < n2 ? kF * kActInv * W3[u0] : 0.f; w3c[r < RB ? r : 0][1] = u1 < n2 ? kF * kActInv * W3[u1] : 0.f; }
         } else {
             int s0 = 0, s1 = 0, s3 = 0, none;
             if (scaled) {
                 row_exponents(W1, nin, n1, 16 * tile, 2, lane, s0, s1);
                 row_exponents(W3, n2, nout, 0, mt2, lane, s3, none);
-                ups1[16 * r] = scale_up(s0); ups1[16 * r + 8] = scale_up(s1); ups3[0] = scale_up(s3);
+                if (r < RA) { ups1[16 * r * apart] = scale_up(s0); ups1[16 * r * apart + 8] = scale_up(s1); }
+                ups3[0] = scale_up(s3);
             }
+            if (r < RA) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, s0, s1, w1h[r][k], w1l[r][k]);
-            uint4 lo3;
-            load_tile(W3, n2, nout, 0, 16 * tile, lane, s3, 0, w3[r], lo3);
-            w3[r].y = lo3.x; w3[r].w = lo3.z;
+                for (int k = 0; k < 2; ++k) load_tile(W1, nin, n1, 16 * tile, 16 * k, lane, s0, s1, w1h[r < RA ? r : 0][k], w1l[r < RA ? r : 0][k]);
+            }
+            if (r < RB) {
+                uint4 lo3;
+                load_tile(W3, n2, nout, 0, 16 * tile, lane, s3, 0, w3[r < RB ? r : 0], lo3);
+                w3[r < RB ? r : 0].y = lo3.x; w3[r < RB ? r : 0].w = lo3.z;
+            }
         }
     }
     if constexpr (RT > 1) __syncthreads();                           // every warp has read the first layer out of `stage`
 #pragma unroll
-    for (int r = 0; r < RT; ++r) {
+    for (int r = 0; r < RB; ++r) {
         int s0 = 0, s1 = 0;
         if (scaled) {
-            row_exponents(W2, n1, n2, 16 * (tile0 + r), KT, lane, s0, s1);
-            ups2[16 * r] = scale_up(s0); ups2[16 * r + 8] = scale_up(s1);
+            row_exponents(W2, n1, n2, 16 * tile_of(r), KT, lane, s0, s1);
+            ups2[16 * r * apart] = scale_up(s0); ups2[16 * r * apart + 8] = scale_up(s1);
         }
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             uint4 lo;
-            load_tile(W2, n1, n2, 16 * (tile0 + r), 16 * k, lane, s0, s1, w2h[r][k], lo, pairs);
+            load_tile(W2, n1, n2, 16 * tile_of(r), 16 * k, lane, s0, s1, w2h[r][k], lo, pairs);
             if constexpr (RT == 1) w2l[k] = lo;
             else w2l_s[32 * (r * KT + k)] = lo;
         }
@@ -238,7 +253,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
         constexpr bool kScaled = decltype(with_scales)::value;
         for (uint32_t step = 0; step < a.T; ++step) {
             if (tile0 < mt1) {
-                float v[RT][NV];
+                float v[RA][NV];
                 if constexpr (CART) {
                     float o[5][NH];
 #pragma unroll
@@ -247,7 +262,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                         else { const float2 q = *reinterpret_cast<const float2*>(&obs[k][2 * t]); o[k][0] = q.x; o[k][1] = q.y; }
                     }
 #pragma unroll
-                    for (int r = 0; r < RT; ++r)
+                    for (int r = 0; r < RA; ++r)
 #pragma unroll
                         for (int i = 0; i < NV; ++i) {
                             float s = b1[r][i / NH];
@@ -256,27 +271,27 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                             v[r][i] = s;
                         }
                 } else {
-                    U acc[RT];
+                    U acc[RA];
                     uint32_t b[2][4];
                     U::load(xin, b);
                     if (U::kLoadTiles == 1) U::load(xin + 32u, b + 1);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) acc[r].first(w1h[r][0], w1l[r][0], b[0]);
+                    for (int r = 0; r < RA; ++r) acc[r].first(w1h[r][0], w1l[r][0], b[0]);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) acc[r].add(w1h[r][1], w1l[r][1], b[1]);
+                    for (int r = 0; r < RA; ++r) acc[r].add(w1h[r][1], w1l[r][1], b[1]);
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) acc[r].sums(kScaled ? ups1[16 * r] : up, kScaled ? ups1[16 * r + 8] : up, b1[r][0], b1[r][1], v[r]);
+                    for (int r = 0; r < RA; ++r) acc[r].sums(kScaled ? ups1[16 * r * apart] : up, kScaled ? ups1[16 * r * apart + 8] : up, b1[r][0], b1[r][1], v[r]);
                 }
 #pragma unroll
-                for (int r = 0; r < RT; ++r) {
+                for (int r = 0; r < RA; ++r) {
                     tanh_units<EB, kTanh>(v[r]);
-                    if (RT == 1 || tile0 + r < KT) U::store(h1_row + 32u * (tile0 + r), v[r]);
+                    if (RA == 1 || tile_of(r) < KT) U::store(h1_row + 32u * tile_of(r), v[r]);
                 }
             }
             __syncthreads();
             CpAhead ahead;
             {
-                U acc[RT];
+                U acc[RB];
                 if (tile0 < mt2) {
                     uint32_t b[2][2][4];                                 // the operands of two tiles, those of the next two on their way
                     U::load(h1_row, b[0]);
@@ -289,7 +304,7 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                             if (U::kLoadTiles == 1 && k + 3 < KT) U::load(h1_row + 32u * k + 96u, next + 1);
                         }
 #pragma unroll
-                        for (int r = 0; r < RT; ++r) {
+                        for (int r = 0; r < RB; ++r) {
                             const uint4 lo = RT == 1 ? w2l[RT == 1 ? k : 0] : w2l_s[32 * (r * KT + k)];
                             if (k == 0) acc[r].first(w2h[r][k], lo, now[0]);
                             else acc[r].add(w2h[r][k], lo, now[k & 1]);
@@ -306,10 +321,10 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
                     if (step > 0u) ret = fmaf(csc, __expf(-cps.x * cps.x), ret);        // reward of the step before, on its post-step state
                 }
                 if (tile0 < mt2) {
-                    float v[RT][NV];
+                    float v[RB][NV];
 #pragma unroll
-                    for (int r = 0; r < RT; ++r) {
-                        acc[r].sums(kScaled ? ups2[16 * r] : up, kScaled ? ups2[16 * r + 8] : up, b2[r][0], b2[r][1], v[r]);
+                    for (int r = 0; r < RB; ++r) {
+                        acc[r].sums(kScaled ? ups2[16 * r * apart] : up, kScaled ? ups2[16 * r * apart + 8] : up, b2[r][0], b2[r][1], v[r]);
                         tanh_units<EB, kTanh>(v[r]);
                     }
                     if constexpr (CART) {
@@ -317,18 +332,18 @@ k_rollout_mlp2(const RolloutMlpArgs a, DeviceStatus* status)
 #pragma unroll
                         for (int i = 0; i < NH; ++i) {
                             p[i] = fmaf(w3c[0][1], v[0][NH + i], w3c[0][0] * v[0][i]);
-                            if constexpr (RT == 2) p[i] = fmaf(w3c[RT - 1][1], v[RT - 1][NH + i], fmaf(w3c[RT - 1][0], v[RT - 1][i], p[i]));
+                            if constexpr (RB == 2) p[i] = fmaf(w3c[RB - 1][1], v[RB - 1][NH + i], fmaf(w3c[RB - 1][0], v[RB - 1][i], p[i]));
                         }
                         if constexpr (EB == 4) part_c[warp][lane] = p[0];
                         else *reinterpret_cast<float2*>(&part_c[warp][2 * lane]) = make_float2(p[0], p[1]);
                     } else {                                             // the action layer's share of the warp's units
-                        uint32_t b[RT][4];
-                        float p[RT][2];
+                        uint32_t b[RB][4];
+                        float p[RB][2];
 #pragma unroll
-                        for (int r = 0; r < RT; ++r) U::transpose(v[r], b[r]);
+                        for (int r = 0; r < RB; ++r) U::transpose(v[r], b[r]);
 #pragma unroll
-                        for (int r = 0; r < RT; ++r) U::eight(w3[r], b[r], kScaled ? ups3[0] : up, 0.f, p[r]);
-                        if constexpr (RT == 2) { p[0][0] += p[RT - 1][0]; p[0][1] += p[RT - 1][1]; }
+                        for (int r = 0; r < RB; ++r) U::eight(w3[r], b[r], kScaled ? ups3[0] : up, 0.f, p[r]);
+                        if constexpr (RB == 2) { p[0][0] += p[RB - 1][0]; p[0][1] += p[RB - 1][1]; }
                         if constexpr (EB == 4) part_t[warp][lane] = p[0][0];
                         else *reinterpret_cast<float2*>(&part_t[warp][2 * lane]) = make_float2(p[0][0], p[0][1]);
                     }
@@ -527,17 +542,26 @@ k_rollout_cart_solo(const RolloutMlpArgs a, DeviceStatus* status)
     if (lane == 0) store_return(a, status, member, eb, v);
 }
 
-template <int EB, bool CART>
-auto pick_kernel(uint32_t kt, bool two_tiles)
+using Mlp2Kernel = void (*)(const RolloutMlpArgs, DeviceStatus*);
+
+// ra, rb: row tiles per warp of the two layers
+template <int EB, bool CART, int KT>
+Mlp2Kernel pick_tiles(uint32_t ra, uint32_t rb)
 {
-    if (two_tiles) return kt == 4u ? k_rollout_mlp2<EB, CART, 4, 2> : kt == 6u ? k_rollout_mlp2<EB, CART, 6, 2> : k_rollout_mlp2<EB, CART, 8, 2>;
+    if constexpr (KT == 4) { if (ra == 1u) return k_rollout_mlp2<EB, CART, KT, 1, 2>; }       // (the first layer has at most four tiles then)
+    return rb == 1u ? k_rollout_mlp2<EB, CART, KT, 2, 1> : k_rollout_mlp2<EB, CART, KT, 2, 2>;
+}
+template <int EB, bool CART>
+Mlp2Kernel pick_kernel(uint32_t kt, uint32_t ra, uint32_t rb)
+{
+    if (ra + rb > 2u) return kt == 4u ? pick_tiles<EB, CART, 4>(ra, rb) : kt == 6u ? pick_tiles<EB, CART, 6>(ra, rb) : pick_tiles<EB, CART, 8>(ra, rb);
     switch (kt) {
-        case 1: return k_rollout_mlp2<EB, CART, 1, 1>;
-        case 2: return k_rollout_mlp2<EB, CART, 2, 1>;
-        case 3: return k_rollout_mlp2<EB, CART, 3, 1>;
-        case 4: return k_rollout_mlp2<EB, CART, 4, 1>;
-        case 6: return k_rollout_mlp2<EB, CART, 6, 1>;
-        default: return k_rollout_mlp2<EB, CART, 8, 1>;
+        case 1: return k_rollout_mlp2<EB, CART, 1, 1, 1>;
+        case 2: return k_rollout_mlp2<EB, CART, 2, 1, 1>;
+        case 3: return k_rollout_mlp2<EB, CART, 3, 1, 1>;
+        case 4: return k_rollout_mlp2<EB, CART, 4, 1, 1>;
+        case 6: return k_rollout_mlp2<EB, CART, 6, 1, 1>;
+        default: return k_rollout_mlp2<EB, CART, 8, 1, 1>;
     }
 }
 
@@ -566,12 +590,13 @@ int launch_rollout_mlp2(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* 
     const bool wide = tiles > 4u, two_tiles = wide && blocks > 2u * kSms;
     uint32_t kt = (a.sizes[1] + 15u) / 16u;
     if (wide) kt = two_tiles && kt <= 4u ? 4u : kt <= 6u ? 6u : 8u;
-    auto kernel = a.EB == 4u ? (cart ? pick_kernel<4, true>(kt, two_tiles) : pick_kernel<4, false>(kt, two_tiles))
-                             : (cart ? pick_kernel<8, true>(kt, two_tiles) : pick_kernel<8, false>(kt, two_tiles));
     uint32_t warps = two_tiles ? (tiles + 1u) / 2u : tiles;
     if (!cart && warps < 2u) warps = 2u;
+    const uint32_t ra = two_tiles && (a.sizes[1] + 15u) / 16u > warps ? 2u : 1u, rb = two_tiles && (a.sizes[2] + 15u) / 16u > warps ? 2u : 1u;
+    auto kernel = a.EB == 4u ? (cart ? pick_kernel<4, true>(kt, ra, rb) : pick_kernel<4, false>(kt, ra, rb))
+                             : (cart ? pick_kernel<8, true>(kt, ra, rb) : pick_kernel<8, false>(kt, ra, rb));
     if (two_tiles) {                                                  // the first layer, then the low parts of the second
-        const size_t first = ((a.sizes[0] + 1u) * a.sizes[1] + 3u) * sizeof(float), low = warps * 2u * kt * 512u;
+        const size_t first = ((a.sizes[0] + 1u) * a.sizes[1] + 3u) * sizeof(float), low = warps * rb * kt * 512u;
         bytes = first > low ? first : low;
     }
     bytes = spread_over_sms(kernel, bytes, blocks);

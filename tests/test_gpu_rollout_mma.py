@@ -88,6 +88,14 @@ def test_two_row_tiles_per_warp(sizes, episodes):
     s.close()
 
 
+@pytest.mark.parametrize("sizes", [(28, 128, 64, 8), (28, 90, 33, 8), (28, 96, 5, 8), (28, 48, 81, 8), (28, 64, 113, 8), (28, 17, 65, 8),
+                                   (5, 128, 50, 1), (5, 70, 48, 1), (5, 64, 128, 1), (5, 3, 90, 1)])
+@pytest.mark.parametrize("episodes", [4, 5])
+def test_two_row_tiles_per_warp_in_one_layer(sizes, episodes):
+    """As above where the other layer has at most half as many tiles, one per warp."""
+    test_two_row_tiles_per_warp(sizes, episodes)
+
+
 @pytest.mark.parametrize("sizes,pop", [((28, 128, 128, 8), 4), ((28, 128, 128, 8), 300), ((5, 64, 64, 1), 4), ((5, 16, 16, 1), 4),
                                        ((28, 32, 32, 32, 8), 4)])
 def test_weights_far_beyond_the_fp16_range(sizes, pop):
