@@ -345,8 +345,8 @@ Plan make_plan(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t
 
 }  // namespace
 
-// Episodes per block: 4, or 8 if a member has more (three MMAs then serve twice the episodes that two do).  0: the
-// weights do not fit.
+// Episodes per block: 4, or 8 if a member has more (three MMAs then serve twice the episodes that two do; rollout_mlp_plan takes 4
+// all the same for small populations).  0: the weights do not fit.
 uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t episodes)
 {
     const uint32_t eb = episodes > 4u ? 8u : 4u;

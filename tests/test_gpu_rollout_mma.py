@@ -88,6 +88,34 @@ def test_two_row_tiles_per_warp(sizes, episodes):
     s.close()
 
 
+@pytest.mark.parametrize("sizes", [(28, 8), (28, 17, 8), (28, 130, 8), (28, 16, 15, 8), (28, 64, 64, 8), (28, 128, 127, 8), (28, 90, 33, 8), (28, 192, 140, 8),
+                                   (28, 64, 17, 49, 8), (28, 128, 65, 16, 8), (28, 129, 144, 60, 8), (28, 64, 33, 64, 49, 8), (28, 20, 60, 9, 100, 8),
+                                   (28, 250, 8), (5, 1), (5, 33, 1), (5, 128, 1), (5, 64, 64, 1), (5, 127, 65, 1), (5, 40, 110, 1), (5, 16, 16, 16, 1),
+                                   (5, 65, 128, 3, 1), (5, 16, 17, 150, 1), (5, 16, 65, 64, 128, 1), (5, 200, 12, 1)])
+@pytest.mark.parametrize("episodes", [5, 8, 11])
+def test_eight_episodes_per_block(sizes, episodes):
+    """What populations too large for blocks of four episodes take: states and fitness of a few of 150 members (300 and more blocks of four)."""
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    T, members = 20, [0, 1, 147, 149]
+    w = base.with_(pop_size=150, episodes=episodes, horizon=T, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes))
+    theta = W.random_parameters(sum(sizes), 150, w.param_dim, scale=0.05 if sizes[0] == 28 else 0.25)
+    s = Solver(w, trace_steps=T)
+    arg = s.padded_rows(150)
+    arg[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+    trace = torch.zeros(150, episodes, T, 4 if sizes[0] == 5 else 28, device="cuda")
+    fit = s.rollout(arg, trace=trace).cpu().numpy()
+    assert s.sync_status() == 0
+    fit_o, traces_o = oracle_fitness(w, theta[members], 0, T, want_trace=True)
+    assert rel_err(fit[members], fit_o, floor=1.0) < FIT_TOL
+    for m, want in zip(members, traces_o):
+        got = trace[m].cpu().numpy().astype(np.float64)
+        if sizes[0] == 5:
+            got, want = cartpole_features(got), cartpole_features(want)
+        for i in range(got.shape[-1]):
+            assert rel_err(got[..., i], want[..., i]) < STATE_TOL, (m, i)
+    s.close()
+
+
 @pytest.mark.parametrize("sizes", [(28, 128, 64, 8), (28, 90, 33, 8), (28, 96, 5, 8), (28, 48, 81, 8), (28, 64, 113, 8), (28, 17, 65, 8),
                                    (5, 128, 50, 1), (5, 70, 48, 1), (5, 64, 128, 1), (5, 3, 90, 1)])
 @pytest.mark.parametrize("episodes", [4, 5])

@@ -70,6 +70,13 @@ def test_states_are_as_close_to_the_oracle_as_those_of_the_fp32_kernel(sizes, po
     _check_against_fp32(w, _population(w, sum(sizes) + pop))
 
 
+@pytest.mark.parametrize("sizes", [(28, 64, 64, 8), (28, 20, 8), (28, 100, 90, 80, 8), (28, 52, 56, 60, 8), (28, 128, 128, 128, 128, 8), (28, 128, 90, 8),
+                                   (5, 64, 64, 1), (5, 100, 1), (5, 40, 40, 40, 1), (5, 64, 64, 64, 64, 1)])
+def test_the_same_of_eight_episodes_per_block(sizes):
+    w = _workload(sizes, 150, 8)                                  # (64 members have blocks of four)
+    _check_against_fp32(w, _population(w, sum(sizes)))
+
+
 @pytest.mark.parametrize("sizes,episodes", [((28, 160, 8), 4), ((28, 192, 140, 8), 8), ((28, 150, 130, 190, 8), 4), ((28, 129, 60, 80, 180, 8), 8),
                                             ((5, 192, 1), 4), ((5, 140, 150, 160, 1), 8)])
 def test_the_same_of_more_than_128_units(sizes, episodes):
