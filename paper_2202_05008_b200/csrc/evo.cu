@@ -197,8 +197,10 @@ evo_status evo_create(const evo_config* cfg_in, void* d_workspace, size_t worksp
     s->launches = 0;
     s->rollout_prepared = false;
     if (s->cfg.task_kind == EVO_TASK_SEQ2SEQ_ADD)
-        s->s2s = s2s_split(s->cfg.layer_sizes[0], s->local_pop, (s->cfg.batch + 7u) / 8u,
-                           static_cast<uint32_t>(s->cfg.task_param[EVO_S2S_DIGITS]), kSms);
+        s->s2s = s->cfg.layer_sizes[0] == 128u
+                     ? s2s_items(s->cfg.pop_size, s->cfg.batch, static_cast<uint32_t>(s->cfg.task_param[EVO_S2S_DIGITS]), kSms)
+                     : s2s_split(s->cfg.layer_sizes[0], s->local_pop, (s->cfg.batch + 7u) / 8u,
+                                 static_cast<uint32_t>(s->cfg.task_param[EVO_S2S_DIGITS]), kSms);
     s->deep = false;
     if (s->cfg.task_kind == EVO_TASK_CARTPOLE || s->cfg.task_kind == EVO_TASK_TANH_LINEAR) {
         const int deep = rollout_mlp_prepare(s->cfg, s->lay.EB, s->lay.n_eb);

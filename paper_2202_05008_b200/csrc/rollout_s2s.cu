@@ -85,6 +85,7 @@ struct S2sArgs {
     const DeviceStatus* status;  // holds the generation counter
     float* partial;              // [P][n_chunks] sums of token losses
     uint32_t n_chunks;
+    uint32_t per_chunk;          // k_s2s_tc: queries per item
     float* logits;               // nullable: [P][B][nd+1][12] (simple kernel only)
 };
 
@@ -590,18 +591,19 @@ __device__ __forceinline__ void half_barrier(uint32_t half)
     else      asm volatile("bar.sync 1, %0;" :: "n"(kTcHalfThreads) : "memory");
 }
 
-// FULL: every item has 128 queries, and the loops do not ask (1,036 members, 3 digits: 454 us; the other instance takes 465).
-template <bool FULL>
+// kPadded: items are worked off as 128 queries whatever they hold, and the loops do not ask (128 queries, 1,036 members, 3 digits: 456 us; kPartial
+// takes 465.  148 members: 66 us, kPartial with 120 queries 69, with 112 64).  kFull: they hold 128, and nothing asks (454 us).
+enum class Items { kPartial, kPadded, kFull };
+template <Items KIND>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_s2s_tc(const S2sArgs a, DeviceStatus* status)
 {
+    constexpr bool FULL = KIND != Items::kPartial;
     extern __shared__ __align__(128) unsigned char s2s_smem_raw[];
     S2sSmem& S = *reinterpret_cast<S2sSmem*>(s2s_smem_raw);
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
     const uint32_t Te = 2 * a.nd + 1, Td = a.nd + 1, T = Te + Td;
     const uint32_t n_items = a.P * a.n_chunks;
-    // chunks of equal size, so that blocks have equal work
-    const uint32_t per_chunk = FULL ? kTcQ : ((a.B + a.n_chunks - 1u) / a.n_chunks + 7u) & ~7u;
     const PhiloxKey key = philox_key(a.k0, a.k1);
 
     if (tid == 0) {
@@ -627,8 +629,8 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
 
     for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         const uint32_t member = item / a.n_chunks, chunk = item % a.n_chunks;
-        const uint32_t q0 = chunk * per_chunk;
-        const uint32_t nq = FULL ? kTcQ : min(per_chunk, a.B - q0);
+        const uint32_t q0 = chunk * (FULL ? kTcQ : a.per_chunk);
+        const uint32_t nq = FULL ? kTcQ : min(a.per_chunk, a.B - q0);
         // The halves share the queries evenly, to eights, and what holds none is left out: a half, eight queries of it, a warp's read-out.
         // Every item was worked off as 128 queries before.  1,036 members, 3 digits: 40 queries 456 -> 330 us, 64 456 -> 348, 100 457 -> 449,
         // 130 (two items of 65 instead of 128 and 2) 852 -> 672, 300 1,275 -> 1,217.
@@ -638,7 +640,7 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         // ---- per-item setup: queries, zero state, read-out weights, encoder weights ------------
         if (chunk != staged_chunk) {
             if (tid < kTcQ)
-                s2s_query(key, a.status->generation, q0 + min(tid < 64u ? tid : nq0 + tid - 64u, nq - 1u), a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
+                s2s_query(key, a.status->generation, KIND == Items::kPadded ? min(q0 + tid, a.B - 1u) : q0 + min(tid < 64u ? tid : nq0 + tid - 64u, nq - 1u), a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
             staged_chunk = chunk;
         }
         if (is_mma) {                                            // the decoder's weights will be wanted next
@@ -824,7 +826,7 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         for (uint32_t idx = tid; idx < Td * kTcQ; idx += kTcThreads) {
             const uint32_t pos = idx / kTcQ, q = idx % kTcQ;
             const uint32_t row = q < nq0 ? q : 64u + q - nq0;
-            if (q < nq) loss += token_loss(S.lg[pos][row], S.tgt[row][pos]);
+            if (q < nq && (KIND != Items::kPadded || q0 + q < a.B)) loss += token_loss(S.lg[pos][row], S.tgt[row][pos]);
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
@@ -856,8 +858,6 @@ bool s2s_supported(uint32_t h, uint32_t nd, uint32_t B)
     return h >= 32 && h <= 128 && h % 32 == 0 && nd >= 1 && nd <= kS2sMaxDigits && B >= 1;
 }
 
-static uint32_t s2s_chunks(uint32_t B, bool tc) { return tc ? (B + kTcQ - 1) / kTcQ : (B + kSimpleQ - 1) / kSimpleQ; }
-
 static cudaError_t launch_s2s_mma(cudaStream_t st, const S2sArgs& a, const S2sSplit& split)
 {
     if (split.chunk == 0u)
@@ -885,7 +885,8 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
     a.theta = theta; a.ldD = ldD; a.P = P; a.h = h; a.nd = nd; a.B = B;
     a.k0 = k0; a.k1 = k1; a.status = status;
     a.partial = static_cast<float*>(scratch);
-    a.n_chunks = mma ? (B + 7u) / 8u : s2s_chunks(B, tc);
+    a.n_chunks = mma ? (B + 7u) / 8u : (B + kSimpleQ - 1u) / kSimpleQ;
+    a.per_chunk = kSimpleQ;
     a.logits = logits;
     if (tc) {
         static int sm_count = 0;
@@ -894,7 +895,9 @@ int launch_rollout_s2s(cudaStream_t st, const float* theta, uint32_t ldD, uint32
             if (cudaGetDevice(&dev) != cudaSuccess) return -1;
             if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
         }
-        auto kernel = B % kTcQ == 0u ? k_s2s_tc<true> : k_s2s_tc<false>;
+        a.n_chunks = split.chunks;
+        a.per_chunk = split.chunk;
+        auto kernel = split.chunk != kTcQ ? k_s2s_tc<Items::kPartial> : B % kTcQ == 0u ? k_s2s_tc<Items::kFull> : k_s2s_tc<Items::kPadded>;
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(S2sSmem))) != cudaSuccess) return -1;
         const uint32_t items = P * a.n_chunks;
         const uint32_t grid = items < static_cast<uint32_t>(sm_count) ? items : static_cast<uint32_t>(sm_count);

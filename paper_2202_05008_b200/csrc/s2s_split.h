@@ -1,4 +1,4 @@
-// Host arithmetic of the narrow seq2seq kernels' launch (rollout_s2s.cu), without CUDA so that it can be tested anywhere.
+// Host arithmetic of the seq2seq kernels' launch (rollout_s2s.cu), without CUDA so that it can be tested anywhere.
 #pragma once
 #include <cstdint>
 
@@ -9,6 +9,27 @@ namespace evo {
 struct S2sSplit { uint32_t chunk, chunks, places; };
 
 constexpr uint32_t kS2sRunTiles64 = 14, kS2sRunTiles96 = 8;       // most n-tiles of a piece of a run
+
+// 128 units: items of `chunk` queries of a member, `chunks` of them, for a block per SM that takes them in turn.  An item of q queries takes about
+// 22 + T (1.36 + 0.0205 q) us for T steps (148 members, 3 digits: 32 queries 46 us, 64 51, 96 60, 128 66), so a population that leaves SMs idle
+// with items of 128 takes smaller ones, as far as the rounds of the blocks do not eat up what that saves; where it is less than 3 %
+// the items stay large.  `members`: of the whole population, so that shards sum up a member's loss alike.  Roll-outs, items of
+// at most 128 and as few as possible / as here, us: 22 x 314, 3 digits 61 / 48; 36 x 128, 3 62 / 45; 48 x 47, 1 32 / 29; 76 x 240, 4 129 / 125; 160 x 250, 3 191 / 192.
+inline S2sSplit s2s_items(uint32_t members, uint32_t queries, uint32_t digits, uint32_t sms)
+{
+    const uint64_t steps = 3u * digits + 2u;
+    const uint32_t least = (queries + 127u) / 128u, most = (queries + 15u) / 16u;
+    S2sSplit best = { 0u, 0u, sms };
+    uint64_t best_time = 0;
+    for (uint32_t n = least; n <= most && n <= least + sms; ++n) {
+        uint32_t chunk = ((queries + n - 1u) / n + 7u) / 8u * 8u;
+        if (chunk > 112u) chunk = 128u;                              // (the instance for these takes no longer for 128)
+        const uint32_t chunks = (queries + chunk - 1u) / chunk;
+        const uint64_t time = (static_cast<uint64_t>(members) * chunks + sms - 1u) / sms * (1100u + steps * (68u + chunk));       // units of 0.02 us
+        if (best.chunks == 0u || time * 100u < best_time * 97u) { best.chunk = chunk; best.chunks = chunks; best_time = time; }
+    }
+    return best;
+}
 
 // Pieces of the run of n-tiles [first, end), `tiles` of them to a member
 inline uint32_t s2s_pieces(uint32_t first, uint32_t end, uint32_t tiles, uint32_t most)

@@ -71,3 +71,23 @@ MEASURED = [(64, 1, 47, 52, True), (64, 2, 100, 300, True), (64, 2, 100, 600, Tr
 def test_the_faster_form_is_taken(lib, units, digits, queries, members, runs):
     """Sizes at which one of the two was measured at least 5 % faster."""
     assert (_split(lib, units, members, (queries + 7) // 8, digits)[0] == 0) == runs
+
+
+def test_items_of_128_units_cover_the_batch_and_fill_the_gpu(tmp_path):
+    src, out = str(tmp_path / "items.cc"), str(tmp_path / "libitems.so")
+    with open(src, "w") as f:
+        f.write('#include "s2s_split.h"\nextern "C" void items(uint32_t m, uint32_t q, uint32_t d, uint32_t* o)'
+                "{ const evo::S2sSplit s = evo::s2s_items(m, q, d, 148); o[0] = s.chunk; o[1] = s.chunks; }\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-o", out, src], check=True)
+    fn, o = C.CDLL(out).items, (C.c_uint32 * 2)()
+    rng = random.Random(3)
+    for members, queries, digits in [(2, 1, 1), (2, 16, 4), (1 << 20, 128, 3)] + [(rng.randint(2, 3000), rng.randint(1, 700), rng.randint(1, 4)) for _ in range(3000)]:
+        fn(members, queries, digits, o)
+        chunk, chunks = o
+        assert chunk % 8 == 0 and 0 < chunk <= 128 and (chunks - 1) * chunk < queries <= chunks * chunk
+        assert chunks <= (queries + 7) // 8                      # the scratch memory has a sum for every 8 queries
+        if members >= 148 * 20:
+            assert chunks == -(-queries // 128)                  # nothing to fill
+    for members, queries, chunk in [(1024, 128, 128), (37, 128, 32), (74, 128, 64), (148, 128, 128), (148, 130, 72), (82, 362, 128)]:
+        fn(members, queries, 3, o)
+        assert o[0] == chunk, (members, queries, o[0])
