@@ -22,7 +22,7 @@
 // Only the triangles that matter are then walked, in order, from the ballots, with the tests that cut the rectangle; the
 // covering ones without any.  Bound by instruction issue (84 %).  64 triangles on 128 x 128 pixels, 1,024 members in
 // mid-training: 357 us with tiles of 32 x 16 pixels, a list of the triangles whose bounding box meets the tile and
-// every test per pixel; 183 us with the classes; 151 us with the tests per edge.
+// every test per pixel; 183 us with the classes; 144 us with the tests per edge; 137 us with only the near triangles classified.
 #include "internal.h"
 
 namespace evo {
@@ -65,13 +65,18 @@ struct PaintArgs {
     uint32_t rects_x, rects, rects_per_block;
 };
 
+// NEAR (more than 32 triangles): a warp first lists the triangles whose box overlaps its rectangle, and classifies only these: of 64 triangles of a
+// painting on its way 15, one round instead of two.  64 triangles on 128 x 128, 1,024 members 144 -> 138 us; 37 on 170 x 123, 146 members 28.1 -> 27.0; 100 on
+// 200 x 200, 250 members 116 -> 100.  With 32 triangles and fewer there is one round in either case: 30 on 100 x 100, 400 members 29.0 us, with a list 30.3.
+template <bool NEAR>
 __global__ void __launch_bounds__(kPaintThreads)
 k_paint(const PaintArgs a)
 {
-    // sized by the launch: n_tri records, then n_tri kinds
+    // sized by the launch: n_tri records, NEAR: n_tri triangle numbers per warp, then n_tri kinds
     extern __shared__ __align__(16) unsigned char paint_smem[];
     PaintTri* tri = reinterpret_cast<PaintTri*>(paint_smem);
-    uint8_t* kind = paint_smem + sizeof(PaintTri) * a.n_tri;
+    uint16_t* near = reinterpret_cast<uint16_t*>(paint_smem + sizeof(PaintTri) * a.n_tri) + (threadIdx.x >> 5) * a.n_tri;
+    uint8_t* kind = paint_smem + (sizeof(PaintTri) + (NEAR ? kPaintThreads / 32 * sizeof(uint16_t) : 0u)) * a.n_tri;
     __shared__ float warp_sum[kPaintThreads / 32];
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
@@ -118,16 +123,32 @@ k_paint(const PaintArgs a)
             cr[q] = a.background; cg[q] = a.background; cb[q] = a.background;
         }
 
-        for (uint32_t base = 0; base < a.n_tri; base += 32u) {
+        // a pixel centre of the rectangle inside the closed box exists only if the ranges overlap
+        auto overlaps = [&](uint32_t k) {
+            const float4 box = *reinterpret_cast<const float4*>(&tri[k].xmin);
+            return kind[k] != kPaintsNothing && !(box.y < X0 || box.x > X1 || box.w < Y0 || box.z > Y1);
+        };
+        uint32_t n_tri = a.n_tri;
+        if constexpr (NEAR) {                                             // in order
+            n_tri = 0;
+            __syncwarp();                                                 // everyone is done with the rectangle before
+            for (uint32_t base = 0; base < a.n_tri; base += 32u) {
+                const uint32_t k = base + lane;
+                const bool here = k < a.n_tri && overlaps(k);
+                const uint32_t those = __ballot_sync(0xffffffffu, here);
+                if (here) near[n_tri + __popc(those & ((1u << lane) - 1u))] = static_cast<uint16_t>(k);
+                n_tri += __popc(those);
+            }
+            __syncwarp();
+        }
+        for (uint32_t base = 0; base < n_tri; base += 32u) {
             // what the walk has to look at per pixel: the box, each edge, or (thin triangles) the three edges with either sign
             bool walk = false, box_cuts = false, cuts[3] = { false, false, false }, thin = false;
-            const uint32_t k = base + lane;
-            if (k < a.n_tri) {
-                const uint8_t what = kind[k];
+            if (base + lane < n_tri) {
+                const uint32_t k = NEAR ? near[base + lane] : base + lane;
                 const PaintTri& t = tri[k];
-                // a pixel centre of the rectangle inside the closed box exists only if the ranges overlap
-                walk = what != kPaintsNothing && !(t.xmax < X0 || t.xmin > X1 || t.ymax < Y0 || t.ymin > Y1);
-                thin = what == kThinTriangle;
+                walk = NEAR || overlaps(k);
+                thin = kind[k] == kThinTriangle;
                 box_cuts = t.xmin > X0 || t.xmax < X1 || t.ymin > Y0 || t.ymax < Y1;
                 if (walk && !thin) {
                     float highest = 1.0f;                             // smallest of the edges' largest values
@@ -152,7 +173,7 @@ k_paint(const PaintArgs a)
             while (todo) {
                 const uint32_t n = __ffs(static_cast<int>(todo)) - 1u, bit = todo & (0u - todo);
                 todo ^= bit;
-                const PaintTri& t = tri[base + n];
+                const PaintTri& t = tri[NEAR ? near[base + n] : base + n];
                 const float4 c = *reinterpret_cast<const float4*>(&t.ar);
                 if (!(tested & bit)) {
 #pragma unroll
@@ -286,8 +307,9 @@ int launch_rollout_paint(cudaStream_t st, const float* theta, uint32_t ldD, uint
     a.theta = theta; a.ldD = ldD; a.P = P; a.n_tri = param_dim / 10u; a.W = W; a.H = H;
     a.background = background; a.target = target; a.partial = static_cast<float*>(scratch); a.canvas = canvas;
     a.rects_x = s.rects_x; a.rects = s.rects; a.rects_per_block = s.per_block;
-    const size_t smem = (sizeof(PaintTri) + sizeof(uint8_t)) * a.n_tri;        // at most 41 KB
-    if (launch_dependent(k_paint, dim3(P, s.blocks), dim3(kPaintThreads), smem, st, a) != cudaSuccess) return -1;
+    const bool near = a.n_tri > 32u;
+    const size_t smem = (sizeof(PaintTri) + (near ? kPaintThreads / 32 * sizeof(uint16_t) : 0u) + sizeof(uint8_t)) * a.n_tri;        // at most 45 KB
+    if (launch_dependent(near ? k_paint<true> : k_paint<false>, dim3(P, s.blocks), dim3(kPaintThreads), smem, st, a) != cudaSuccess) return -1;
     const float inv = 1.0f / (3.0f * static_cast<float>(W) * static_cast<float>(H));
     if (launch_dependent(k_paint_finalize, dim3((P + 255u) / 256u), dim3(256), 0, st, a.partial, P, s.blocks, inv, fitness) != cudaSuccess)
         return -1;

@@ -47,6 +47,21 @@ def test_canvas_and_fitness_match_oracle(n_tri, width, height, bg):
         assert abs(fit[m] - f) < 1e-6
 
 
+@pytest.mark.parametrize("n_tri", [32, 33, 64, 65])
+def test_needles_and_invisible_ones_among_many_triangles(n_tri):
+    """Either side of the number of triangles from which a rectangle lists those near it."""
+    rng = np.random.default_rng(n_tri)
+    P, width, height = 4, 53, 37
+    theta = rng.uniform(-1.2, 1.2, (P, n_tri, 10)).astype(np.float32)
+    theta[:, ::3, 4:6] = 0.5 * (theta[:, ::3, 0:2] + theta[:, ::3, 2:4]) + rng.normal(0, 1e-6, (P, len(range(0, n_tri, 3)), 2))
+    theta[:, 1::5, 9] = -3.0                                     # transparent
+    w = _workload(n_tri, width, height, P=P)
+    th, fit, canvas, _ = _render(w, theta=theta.reshape(P, -1))
+    for m in range(P):
+        want = oracle.paint_render(th[m].reshape(-1, 10), width, height, float(w.task_param[2]))
+        assert np.max(np.abs(canvas[m] - want)) < 2e-6 * (n_tri // 8)
+
+
 def test_coverage_is_bit_exact_for_opaque_single_triangles_needles_included():
     rng = np.random.default_rng(8)
     P, width, height = 96, 61, 47
