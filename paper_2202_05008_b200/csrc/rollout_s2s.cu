@@ -509,9 +509,11 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes)
 
 // One cell's weights -> A operand (all threads of the block).  The rows of the input, forget and
 // output gates are halved (exact in bf16) so that their sigma(x) = 0.5 tanh(x / 2) + 0.5 needs no
-// scaling of the accumulator.
-__device__ __forceinline__ void s2s_stage_weights(S2sSmem& S, const float* __restrict__ cellp, uint32_t tid)
+// scaling of the accumulator.  TIMES_ZERO: the sum of the thread's recurrent weights times zero (else 0), which is NaN where one is infinite.
+template <bool TIMES_ZERO>
+__device__ __forceinline__ float s2s_stage_weights(S2sSmem& S, const float* __restrict__ cellp, uint32_t tid)
 {
+    uint32_t zero = 0u;
     const float* Wx = cellp;
     const float* Wh = Wx + 4 * kTcH * kVocab;
     const float* bb = Wh + 4 * kTcH * kTcH;
@@ -544,6 +546,8 @@ __device__ __forceinline__ void s2s_stage_weights(S2sSmem& S, const float* __res
                 for (uint32_t r = 0; r < 8u; ++r) {
                     w0[r] = pack_bf16(sc * v[g][r].x, sc * v[g][r].y);
                     w1[r] = pack_bf16(sc * v[g][r].z, sc * v[g][r].w);
+                    if constexpr (TIMES_ZERO)
+                        asm("fma.rn.bf16x2 %0, %1, %3, %0;\n\tfma.rn.bf16x2 %0, %2, %3, %0;" : "+r"(zero) : "r"(w0[r]), "r"(w1[r]), "r"(0u));
                 }
                 unsigned char* dst = S.A + (lane >> 1) * kTcALbo + mg * 128u + (odd ? 64u : 0u);
 #pragma unroll
@@ -570,6 +574,7 @@ __device__ __forceinline__ void s2s_stage_weights(S2sSmem& S, const float* __res
         *reinterpret_cast<uint4*>(S.A + 17u * kTcALbo + (m >> 3) * 128u + (m & 7u) * 16u) =
             make_uint4(pack_bf16(sc * w2.x, sc * w2.y), pack_bf16(sc * w2.z, sc * w2.w), pack_bf16(bias, 0.f), 0u);
     }
+    return __uint_as_float(zero << 16) + __uint_as_float(zero & 0xFFFF0000u);
 }
 
 // one-hot (+ constant 1) rows of query n for the coming step
@@ -659,7 +664,8 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
             dst[4] = bf16_round(w1.x); dst[5] = bf16_round(w1.y); dst[6] = bf16_round(w1.z); dst[7] = bf16_round(w1.w);
         }
         if (tid < kVocab) S.ob[tid] = p[2u * kTcCellFloats + kVocab * kTcH + tid];
-        s2s_stage_weights(S, p, tid);
+        // kPartial: the first step leaves the zero state out, but an infinite weight times zero is NaN, and a step later so is every unit
+        float loss = s2s_stage_weights<!FULL>(S, p, tid);
         __syncthreads();                                        // tokens are there
         if (tid < kTcQ) s2s_write_onehot(S, tid, S.enc[tid][0]);
         fence_async_smem();
@@ -668,14 +674,13 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         float c[kTcCols];
 #pragma unroll
         for (int i = 0; i < kTcCols; ++i) c[i] = 0.f;
-        float loss = 0.f;
 
         for (uint32_t phase = 0; phase < 2u; ++phase) {
             const uint32_t t0 = phase ? Te : 0u, t1 = phase ? T : Te;
             if (phase) {
                 // every MMA of the encoder has been waited for by an epilogue warp: A may be replaced
                 __syncthreads();
-                s2s_stage_weights(S, p + kTcCellFloats, tid);
+                s2s_stage_weights<false>(S, p + kTcCellFloats, tid);
                 fence_async_smem();
                 __syncthreads();
                 if (is_mma && item + gridDim.x < n_items) {     // the next item's encoder cell

@@ -73,6 +73,25 @@ def test_batches_that_do_not_fill_an_item(B, P):
         assert abs(fit[m] - want[0]) < FIT_TOL, (m, fit[m], want[0])
 
 
+@pytest.mark.parametrize("kernel", [ROLLOUT_AUTO, ROLLOUT_GENERIC])
+@pytest.mark.parametrize("h,B", [(128, 9), (128, 40), (128, 100), (128, 128), (64, 40)])
+def test_an_infinite_recurrent_weight_meets_the_zero_state(h, B, kernel):
+    """Infinity times the start state is not a number, in the oracle and in every kernel, however many queries an item has."""
+    w = _workload(h, 2, B, P=4, sigma=0.1)
+    s = Solver(w, rollout_kernel=kernel)
+    rows = s.ask().cpu().numpy()
+    at = 4 * h * 12                                              # the encoder's recurrent weights
+    rows[0, at], rows[1, at + 2 * h * h + 5], rows[3, at + 4 * h * h - 1] = np.inf, -np.inf, np.inf
+    theta = s.padded_rows(4)
+    theta[:, :w.param_dim] = torch.tensor(rows, device="cuda")
+    fit = s.rollout(theta).cpu().numpy()
+    assert s.sync_status() == 0
+    want = np.array([f[0] for f in _oracle_fits(w, rows, 0)])
+    assert np.isnan(want).tolist() == [True, True, False, True]
+    assert np.isnan(fit).tolist() == np.isnan(want).tolist()
+    assert abs(fit[2] - want[2]) < FIT_TOL
+
+
 def _saturated_fitness(P, batch):
     """Gates and cells saturated by their biases: every hidden state is +-bf16(tanh 1) = +-195/256 exactly, whatever the query.  Only the
     logit of '=' (never an answer) has weights, all of its terms positive: the loss of every position is that logit (28 and
