@@ -45,7 +45,8 @@ inline bool mlp_deep_pays(uint32_t hidden, bool wide, uint32_t eb, uint64_t bloc
 // steps: 0.69 of the time of k_rollout_mlp_mma in the mean (geometric), 0.03 % more than with the faster kernel of the two, one takes
 // 0.5 % longer than there; with 1.5 and 1.9 for a limit 0.3 % more.  Examples, deep / mma in us: 5-15-189-54-1, 118 x 2 76 / 124; 28-145-157-59-8,
 // 836 blocks of 8 661 / 1,159; 5-107-29-138-1, 676 of 8 430 / 325; 28-154-13-77-8, 424 of 8 259 / 158; 28-180-180-180-8, 296 x 4 196, and
-// 3,436 with the weights read through the caches (they do not fit the shared memory).
+// 3,436 with the weights read through the caches.  (resident_mma = 0: they do not fit the shared memory.  The faster one then, but choose_kernel leaves such
+// policies to fp32 arithmetic.)
 inline bool mlp_widest_pays(uint64_t blocks, uint32_t sms, uint32_t resident_deep, uint32_t resident_mma)
 {
     if (resident_mma == 0u) return true;

@@ -203,8 +203,12 @@ uint32_t rollout_mlp_mma_eb(uint32_t task, uint32_t n_layers, const uint32_t* si
 int launch_rollout_mlp_mma(cudaStream_t st, const RolloutMlpArgs& a, DeviceStatus* status);
 
 // The kernel of a policy: AUTO takes a register-resident one where the policy has one to four hidden layers of up to 192
-// units (three and four, and any above 128 units, where that is the faster one, see mlp_choice.h), for other numbers of layers and wider ones the one with the weights in
-// shared memory as long as they fit it, and else the runtime-shape kernel, which reads them through the caches.
+// units (three and four, and two to four with one above 128 units, where that is the faster one, see mlp_choice.h), for other numbers of layers and
+// wider ones the one with the weights in shared memory as long as they fit it, and else the runtime-shape kernel, which reads them through the caches.
+// Policies with a layer above 128 units that don't fit the shared memory stay with the runtime-shape kernel, whose arithmetic is fp32: k_rollout_mlp_deep
+// holds many of them and is 17 to 34 times as fast (28-180-180-180-8, 100 members x 4 episodes 2.0 us a step instead of 67), but its error against 64 bits
+// is the larger one in part.  Over that of the runtime-shape kernel (geometric means of 70 such policies): tanh-linear states 0.76 to 0.87 after
+// 1 to 60 steps, their fitness 1.3 (4 episodes a block) and 1.5 (8); cart-pole states 0.90 after one step, 1.07 after 20, 1.03 after 60, their fitness 1.1.
 enum class MlpKernel { kNone, kGeneric, kTiled, kRegisters, kDeep, kSharedMemory };
 
 static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t* sizes, uint32_t choice, bool deep,
@@ -218,8 +222,11 @@ static MlpKernel choose_kernel(uint32_t task, uint32_t n_layers, const uint32_t*
     }
     if (choice == EVO_ROLLOUT_AUTO) {
         if ((*EB = rollout_mlp2_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kRegisters;
-        if (deep && (*EB = rollout_mlp_deep_eb(n_layers, sizes, episodes)) != 0u) return MlpKernel::kDeep;
-        if ((*EB = rollout_mlp_mma_eb(task, n_layers, sizes, episodes)) != 0u) return MlpKernel::kSharedMemory;
+        const uint32_t shared_eb = rollout_mlp_mma_eb(task, n_layers, sizes, episodes);
+        bool widest = false;
+        for (uint32_t l = 1; l < n_layers; ++l) widest = widest || sizes[l] > 128u;
+        if (deep && (shared_eb != 0u || !widest) && (*EB = rollout_mlp_deep_eb(n_layers, sizes, episodes)) != 0u) return MlpKernel::kDeep;
+        if ((*EB = shared_eb) != 0u) return MlpKernel::kSharedMemory;
     }
     return MlpKernel::kGeneric;
 }

@@ -12,8 +12,7 @@
 // registers too the compiler has none left to work with: 0.86 and 1.19 us, and 4.1 against 2.9 us for 16 episodes of 512 members.
 //
 // Above 128 units (KT = 12) a block has up to twelve warps and an SM to itself.  100 members, 4 episodes, us a step, with k_rollout_mlp_mma behind:
-// 28-160-8 0.47 / 1.34, 5-190-180-1 1.15 / 3.00, 5-145-52-48-1 1.31 / 2.22, 28-150-60-60-60-8 1.51 / 2.60; 28-180-180-180-8 1.97 / 66.7 (the runtime-shape
-// kernel: its weights do not fit the shared memory).
+// 28-160-8 0.47 / 1.34, 5-190-180-1 1.15 / 3.00, 5-145-52-48-1 1.31 / 2.22, 28-150-60-60-60-8 1.51 / 2.60.
 //
 // Paper: Section 2 (roll-out loop, central seeds), Section 4 (get_actions over the population with parameters as
 // data; stateless task step; identical initial observations).
