@@ -1,4 +1,4 @@
-// Which kernel a control policy of three or four hidden layers of up to 128 units runs on, without CUDA so that it can be tested anywhere.
+// Which kernel a control policy of up to 192 units runs on, and with how many episodes a block, without CUDA so that it can be tested anywhere.
 #pragma once
 #include <cstddef>
 #include <cstdint>
@@ -52,6 +52,23 @@ inline bool mlp_widest_pays(uint64_t blocks, uint32_t sms, uint32_t resident_dee
     if (resident_mma == 0u) return true;
     if (resident_deep == 0u) return false;
     return mlp_waves(blocks, sms, resident_deep) <= 1.7 * mlp_waves(blocks, sms, resident_mma);
+}
+
+// Whether blocks of four episodes are faster than blocks of eight for a member with more than four (registers: on k_rollout_mlp2).  Eight take three MMAs per tile
+// and twice the tanh of four: where blocks of four still find an SM each (two, for the wide policies of k_rollout_mlp2 on the tanh-linear task) the
+// step is shorter with them.  8 episodes, 50 steps, blocks of 8 / of 4 in us: 28-119-25-8, 70 members 97 / 77, 148 97 / 87; 28-64-64-8, 74 64 / 55;
+// 5-100-120-1, 74 101 / 90; 28-64-64-64-8, 74 86 / 77; 28-43-41-100-8, 74 143 / 105; 5-57-12-53-11-1, 74 138 / 98.  With more: 5-64-64-1, 148 59 / 61;
+// 28-28-38-8, 148 55 / 58; 28-64-64-64-8, 148 86 / 94.
+// Up to eight episodes, one block of eight writes the fitness itself, and two of four need k_fitness_finalize, 1.2 us, which takes the more steps to
+// make up for the less a step gains.  74 members x 8 after 20 / 50 / 80 / 128 steps: 5-64-64-1 15.1 / 16.1, 31.1 / 31.2, 47.1 / 46.2, 72.8 / 70.3;
+// 5-30-1 9.7 / 10.6, 20.3 / 21.0, 30.7 / 31.0, 47.5 / 47.1; 28-20-8 11.8 / 12.2, 23.2 / 22.4; 28-64-64-8 16.8 / 16.7, 33.8 / 30.9; 5-100-1 11.3 / 11.2,
+// 24.1 / 22.2; 28-119-25-8 23.9 / 21.6, 50.7 / 42.1; 28-64-64-64-8 22.6 / 21.7, 45.7 / 41.9; 28-8 18.2 / 17.7, 37.4 / 34.0.
+inline bool mlp_four_pay(uint32_t hidden, uint32_t widest, bool cart, bool registers, uint32_t members, uint32_t episodes, uint32_t horizon, uint32_t sms)
+{
+    const bool two = registers && !cart && widest > 64u;
+    if (static_cast<uint64_t>(members) * ((episodes + 3u) / 4u) > (two ? 2u : 1u) * sms) return false;
+    const bool long_step = hidden > 2u || widest > 64u || (!cart && (widest > 48u || hidden == 0u));
+    return episodes > 8u || horizon >= (long_step ? 20u : !cart ? 50u : hidden == 2u ? 80u : 120u);
 }
 
 }  // namespace evo

@@ -242,12 +242,10 @@ void rollout_mlp_plan(const evo_config& cfg, uint32_t* EB, uint32_t* n_eb)
         while (eb > 4u && static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + eb - 1u) / eb) < 4u * kSms)
             eb = (eb + 1u) / 2u;
     } else if (k != MlpKernel::kTiled && eb == 8u) {
-        // Eight episodes take three MMAs per tile and twice the tanh of four: where blocks of four still find an SM each (two, for the wide policies
-        // of k_rollout_mlp2 on the tanh-linear task) the step is shorter with them.  8 episodes, 50 steps, blocks of 8 / of 4 in us: 28-119-25-8, 70
-        // members 97 / 77, 148 97 / 87; 28-64-64-8, 74 64 / 55; 5-64-64-1, 74 59 / 57; 5-100-120-1, 74 101 / 90; 28-64-64-64-8, 74 86 / 77;
-        // 28-43-41-100-8, 74 143 / 105; 5-57-12-53-11-1, 74 138 / 98.  With more: 5-64-64-1, 148 59 / 61; 28-28-38-8, 148 55 / 58; 28-64-64-64-8, 148 86 / 94.
-        const bool wide = k == MlpKernel::kRegisters && cfg.task_kind == EVO_TASK_TANH_LINEAR && (cfg.layer_sizes[1] > 64u || cfg.layer_sizes[2] > 64u);
-        if (static_cast<uint64_t>(cfg.pop_size) * ((cfg.episodes + 3u) / 4u) <= (wide ? 2u : 1u) * kSms) eb = 4u;
+        uint32_t widest = 0;
+        for (uint32_t l = 1; l < cfg.n_layers; ++l) widest = cfg.layer_sizes[l] > widest ? cfg.layer_sizes[l] : widest;
+        if (mlp_four_pay(cfg.n_layers - 1u, widest, cfg.task_kind == EVO_TASK_CARTPOLE, k == MlpKernel::kRegisters, cfg.pop_size, cfg.episodes,
+                         cfg.horizon, kSms)) eb = 4u;
     }
     *EB = eb;
     *n_eb = (cfg.episodes + eb - 1u) / eb;

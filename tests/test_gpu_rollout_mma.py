@@ -116,6 +116,23 @@ def test_eight_episodes_per_block(sizes, episodes):
     s.close()
 
 
+@pytest.mark.parametrize("sizes,steps,launches", [((5, 64, 64, 1), 20, 1), ((5, 20, 30, 1), 79, 1), ((5, 20, 30, 1), 80, 2), ((28, 20, 8), 49, 1),
+                                                  ((28, 64, 64, 64, 8), 20, 2), ((5, 16, 16, 1), 20, 2)])
+def test_short_roll_outs_of_eight_episodes_are_one_launch(sizes, steps, launches):
+    """A block of eight episodes writes the fitness itself; the sums of blocks of four need a second launch.  (5-16-16-1 has a warp for four in any case.)"""
+    base = W.CFG2 if sizes[0] == 5 else W.CFG4
+    w = base.with_(pop_size=74, episodes=8, horizon=steps, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes), sigma=0.05)
+    s = Solver(w)
+    theta = s.ask().cpu().numpy()
+    before = s.launch_count()
+    fit = s.rollout().cpu().numpy()
+    assert s.launch_count() - before == launches
+    assert s.sync_status() == 0
+    fit_o, _ = oracle_fitness(w, theta[[0, 73]], 0, steps)
+    assert rel_err(fit[[0, 73]], fit_o, floor=1.0) < FIT_TOL
+    s.close()
+
+
 @pytest.mark.parametrize("sizes", [(28, 128, 64, 8), (28, 90, 33, 8), (28, 96, 5, 8), (28, 48, 81, 8), (28, 64, 113, 8), (28, 17, 65, 8),
                                    (5, 128, 50, 1), (5, 70, 48, 1), (5, 64, 128, 1), (5, 3, 90, 1)])
 @pytest.mark.parametrize("episodes", [4, 5])

@@ -100,3 +100,31 @@ def test_the_faster_kernel_is_taken_above_128_units(tmp_path, blocks, deep, mma,
     fn = C.CDLL(out).pays
     fn.argtypes, fn.restype = [C.c_uint64, C.c_uint32, C.c_uint32], C.c_bool
     assert fn(blocks, deep, mma) == faster
+
+
+# hidden layers, widest of them, cart-pole, on k_rollout_mlp2, members, episodes, steps, whether blocks of four episodes are the faster ones
+@pytest.mark.parametrize("hidden,widest,cart,registers,members,episodes,steps,faster", [
+    (2, 64, True, True, 74, 8, 20, False),       # 5-64-64-1: blocks of eight / of four 15.1 / 16.1 us
+    (2, 64, True, True, 74, 8, 200, True),       # 111.4 / 106.6
+    (2, 64, True, True, 37, 16, 20, True),       # 16.2 / 15.4 (36 members; both have the second launch)
+    (2, 40, True, True, 70, 5, 50, False),       # 5-17-40-1: 28.5 / 28.5
+    (1, 30, True, False, 74, 8, 80, False),      # 5-30-1: 30.7 / 31.0
+    (1, 20, False, False, 74, 8, 20, False),     # 28-20-8: 11.8 / 12.2
+    (1, 20, False, False, 74, 8, 50, True),      # 23.2 / 22.4
+    (2, 64, False, True, 16, 5, 20, True),       # 28-64-64-8: 16.8 / 16.1
+    (2, 119, False, True, 74, 8, 20, True),      # 28-119-25-8: 23.9 / 21.6
+    (2, 119, False, True, 148, 8, 50, True),     # 51.1 / 47.5
+    (2, 119, False, True, 149, 8, 50, False),    # more than two blocks an SM
+    (3, 64, False, False, 74, 8, 20, True),      # 28-64-64-64-8: 22.6 / 21.7
+    (3, 64, False, False, 75, 8, 200, False),
+    (0, 0, True, False, 74, 8, 32, False),       # 5-1: 17.3 / 17.6
+])
+def test_episodes_a_block(tmp_path, hidden, widest, cart, registers, members, episodes, steps, faster):
+    src, out = str(tmp_path / "four.cc"), str(tmp_path / "libfour.so")
+    with open(src, "w") as f:
+        f.write('#include "mlp_choice.h"\nextern "C" bool four(uint32_t h, uint32_t w, bool c, bool r, uint32_t m, uint32_t e, uint32_t t)'
+                "{ return evo::mlp_four_pay(h, w, c, r, m, e, t, 148); }\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-o", out, src], check=True)
+    fn = C.CDLL(out).four
+    fn.argtypes, fn.restype = [C.c_uint32, C.c_uint32, C.c_bool, C.c_bool, C.c_uint32, C.c_uint32, C.c_uint32], C.c_bool
+    assert fn(hidden, widest, cart, registers, members, episodes, steps) == faster
