@@ -10,8 +10,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libevo.so")
 LIB_DEBUG = os.path.join(HERE, "libevo_debug.so")     # checked build: -DEVO_DEBUG (bounds checks, guard words)
-SOURCES = ["evo.cu", "solver_kernels.cu", "rollout_mlp.cu", "rollout_mlp_tiled.cu", "rollout_mlp2.cu", "rollout_mlp_deep.cu", "rollout_mlp_mma.cu", "rollout_cnn.cu", "rollout_cnn_tc.cu", "gradient_static.cu", "rollout_s2s.cu", "rollout_paint.cu"]
-HEADERS = ["internal.h", "noise.cuh", "tasks.cuh", "async.cuh", "umma.cuh", "fp32x2.cuh", "mma_split.cuh", "spread.h", "s2s_split.h", "mlp_choice.h", os.path.join("..", "..", "include", "evo.h")]
+SOURCES = ["evo.cu", "solver_kernels.cu", "rollout_mlp.cu", "rollout_mlp_tiled.cu", "rollout_mlp2.cu", "rollout_mlp_deep.cu", "rollout_mlp_deep8.cu", "rollout_mlp_mma.cu", "rollout_cnn.cu", "rollout_cnn_tc.cu", "gradient_static.cu", "rollout_s2s.cu", "rollout_paint.cu"]
+HEADERS = ["internal.h", "noise.cuh", "tasks.cuh", "async.cuh", "umma.cuh", "fp32x2.cuh", "mma_split.cuh", "rollout_mlp_deep.cuh", "spread.h", "s2s_split.h", "mlp_choice.h", os.path.join("..", "..", "include", "evo.h")]
 
 
 def _nvcc() -> str:

@@ -548,8 +548,8 @@ using Mlp2Kernel = void (*)(const RolloutMlpArgs, DeviceStatus*);
 template <int EB, bool CART, int KT>
 Mlp2Kernel pick_tiles(uint32_t ra, uint32_t rb)
 {
-    if constexpr (KT == 4) { if (ra == 1u) return k_rollout_mlp2<EB, CART, KT, 1, 2>; }       // (the first layer has at most four tiles then)
-    return rb == 1u ? k_rollout_mlp2<EB, CART, KT, 2, 1> : k_rollout_mlp2<EB, CART, KT, 2, 2>;
+    if constexpr (KT == 4) return ra == 1u ? k_rollout_mlp2<EB, CART, KT, 1, 2> : k_rollout_mlp2<EB, CART, KT, 2, 2>;      // (the second layer is the wider one then)
+    else return rb == 1u ? k_rollout_mlp2<EB, CART, KT, 2, 1> : k_rollout_mlp2<EB, CART, KT, 2, 2>;
 }
 template <int EB, bool CART>
 Mlp2Kernel pick_kernel(uint32_t kt, uint32_t ra, uint32_t rb)
