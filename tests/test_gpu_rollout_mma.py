@@ -167,6 +167,22 @@ def test_policies_that_just_fit_the_shared_memory(sizes, episodes):
     check(sizes, episodes, 12, scale=0.02 if sizes[0] == 28 else 0.1)
 
 
+def test_eight_episodes_a_block_at_the_limit_of_the_shared_memory():
+    """222 KB with the operands of eight episodes; 76 members, so that blocks of four would not find an SM each."""
+    sizes = (5, 112, 384, 1)
+    w = W.CFG2.with_(pop_size=76, episodes=8, horizon=24, layer_sizes=sizes, param_dim=W.mlp_param_count(sizes), sigma=0.1)
+    s = Solver(w)
+    theta = s.ask().cpu().numpy()
+    before = s.launch_count()
+    fit = s.rollout().cpu().numpy()
+    assert s.launch_count() - before == 1
+    assert s.sync_status() == 0
+    members = [0, 1, 74, 75]
+    fit_o, _ = oracle_fitness(w, theta[members], 0, 24)
+    assert rel_err(fit[members], fit_o, floor=1.0) < FIT_TOL
+    s.close()
+
+
 @pytest.mark.parametrize("sizes", [(28, 128, 8), (28, 3, 8), (28, 64, 17, 49, 8), (28, 128, 128, 128, 8), (28, 65, 16, 100, 8), (28, 5, 128, 64, 8),
                                    (28, 64, 33, 64, 49, 8), (28, 128, 64, 65, 128, 8),
                                    (5, 128, 1), (5, 64, 64, 64, 1), (5, 65, 128, 3, 1), (5, 50, 64, 49, 64, 1), (5, 16, 65, 64, 128, 1)])

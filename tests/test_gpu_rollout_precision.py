@@ -114,6 +114,62 @@ def test_a_huge_weight_takes_nothing_from_the_others(sizes, pop, episodes):
     _check_against_fp32(w, theta)
 
 
+def _launches(w):
+    s = Solver(w)
+    s.ask()
+    before = s.launch_count()
+    s.rollout()
+    n = s.launch_count() - before
+    s.close()
+    return n
+
+
+def _huge_weights(w, theta, seed):
+    rng = np.random.default_rng(seed)
+    for m in range(w.pop_size):
+        theta[m, rng.integers(w.param_dim)] = rng.choice((-1.0, 1.0)) * rng.choice((2.0e4, 1.0e7, 1.0e12, 1.0e30))
+
+
+@pytest.mark.parametrize("huge", [False, True])
+@pytest.mark.parametrize("sizes,pop", [
+    # weights in registers, in one row tile a warp and (300 members) two, in both layers or one
+    ((28, 64, 64, 8), 150), ((28, 128, 128, 8), 150), ((5, 64, 64, 1), 150), ((28, 128, 128, 8), 300), ((5, 128, 90, 1), 300),
+    ((28, 90, 40, 8), 300), ((28, 40, 90, 8), 300), ((5, 120, 60, 1), 300), ((5, 40, 110, 1), 300),
+    # one, three and four hidden layers
+    ((28, 128, 8), 76), ((28, 64, 64, 64, 8), 76), ((28, 100, 128, 70, 128, 8), 76), ((5, 128, 100, 128, 1), 76), ((5, 50, 64, 49, 64, 1), 76),
+    # above 128 units
+    ((28, 160, 8), 76), ((28, 192, 140, 8), 76), ((28, 150, 130, 100, 8), 76), ((28, 192, 100, 64, 192, 8), 76), ((28, 129, 64, 65, 130, 8), 76),
+    ((5, 160, 1), 76), ((5, 190, 180, 1), 76), ((5, 140, 90, 120, 1), 76), ((5, 160, 48, 49, 160, 1), 76),
+    # weights in shared memory
+    ((28, 200, 8), 76), ((28, 32, 32, 32, 32, 32, 8), 76), ((5, 200, 12, 1), 76)])
+def test_blocks_of_eight_episodes(sizes, pop, huge):
+    """Every kernel with blocks of eight episodes, with weights in the fp16 range and beyond."""
+    w = _workload(sizes, pop, 8)
+    assert _launches(w) == 1                                      # (blocks of four, or the runtime-shape kernel, need a second one)
+    theta = _population(w, 2 + sum(sizes))
+    if huge:
+        _huge_weights(w, theta, pop)
+    _check_against_fp32(w, theta)
+
+
+@pytest.mark.parametrize("huge", [False, True])
+@pytest.mark.parametrize("sizes", [(28, 90, 40, 8), (28, 40, 90, 8), (28, 115, 51, 8), (5, 120, 60, 1), (5, 40, 110, 1)])
+def test_two_row_tiles_a_warp_in_one_layer(sizes, huge):
+    w = _workload(sizes, 300, 4)
+    theta = _population(w, 3 + sum(sizes))
+    if huge:
+        _huge_weights(w, theta, 300)
+    _check_against_fp32(w, theta)
+
+
+@pytest.mark.parametrize("sizes", [(28, 160, 8), (28, 150, 130, 100, 8), (28, 192, 100, 64, 192, 8), (5, 160, 1), (5, 140, 90, 120, 1), (5, 160, 48, 49, 160, 1)])
+def test_a_huge_weight_above_128_units(sizes):
+    w = _workload(sizes, 64, 4)
+    theta = _population(w, 4 + sum(sizes))
+    _huge_weights(w, theta, 64)
+    _check_against_fp32(w, theta)
+
+
 @pytest.mark.parametrize("sizes", [(28, 24, 40, 8), (28, 24, 24, 24, 8), (5, 16, 16, 1), (5, 30, 40, 1), (5, 16, 16, 16, 1)])
 def test_infinite_weights_saturate(sizes):
     w = _workload(sizes, 64, 4).with_(pop_size=8, horizon=3)
@@ -130,6 +186,27 @@ def test_infinite_weights_saturate(sizes):
         s.close()
     np.testing.assert_allclose(fit[ROLLOUT_AUTO], fit[ROLLOUT_GENERIC], rtol=1e-5)
     assert np.isnan(fit[ROLLOUT_AUTO]).tolist() == [False] * 3 + [True] + [False] * 4
+
+
+@pytest.mark.parametrize("sizes,pop,episodes", [
+    ((28, 150, 60, 8), 8, 4), ((28, 150, 60, 8), 8, 8), ((28, 129, 64, 65, 130, 8), 8, 4), ((28, 129, 64, 65, 130, 8), 8, 8), ((5, 160, 48, 49, 160, 1), 8, 4),
+    ((5, 160, 48, 49, 160, 1), 8, 8), ((28, 90, 40, 8), 300, 4), ((5, 40, 110, 1), 300, 4), ((28, 90, 40, 8), 300, 8), ((28, 24, 40, 8), 8, 8), ((5, 16, 16, 16, 1), 8, 8)])
+def test_infinite_weights_saturate_in_every_kernel(sizes, pop, episodes):
+    """As above: above 128 units, with one row tile a warp in one layer and two in the other, with blocks of eight episodes."""
+    w = _workload(sizes, pop, episodes).with_(horizon=3)
+    theta = _population(w, 9)
+    second = sizes[0] * sizes[1] + sizes[1]
+    theta[0, 3], theta[1, second + 1], theta[2, second + sizes[1] * sizes[2]] = np.inf, -np.inf, np.inf
+    theta[3, second + 1], theta[3, second + 2] = np.inf, np.nan
+    fit = {}
+    for kernel in (ROLLOUT_AUTO, ROLLOUT_GENERIC):
+        s = Solver(w, rollout_kernel=kernel)
+        rows = s.padded_rows(pop)
+        rows[:, :w.param_dim] = torch.tensor(theta, device="cuda")
+        fit[kernel] = s.rollout(rows).cpu().numpy()
+        s.close()
+    np.testing.assert_allclose(fit[ROLLOUT_AUTO], fit[ROLLOUT_GENERIC], rtol=1e-5)
+    assert np.flatnonzero(np.isnan(fit[ROLLOUT_AUTO])).tolist() == [3]
 
 
 @pytest.mark.parametrize("sizes,pop", [((28, 24, 40, 8), 64), ((28, 128, 100, 8), 300), ((28, 24, 24, 24, 8), 64)])
