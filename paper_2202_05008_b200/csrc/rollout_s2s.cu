@@ -637,15 +637,19 @@ k_s2s_tc(const S2sArgs a, DeviceStatus* status)
         const uint32_t q0 = chunk * (FULL ? kTcQ : a.per_chunk);
         const uint32_t nq = FULL ? kTcQ : min(a.per_chunk, a.B - q0);
         // The halves share the queries evenly, to eights, and what holds none is left out: a half, eight queries of it, a warp's read-out.
-        // Every item was worked off as 128 queries before.  1,036 members, 3 digits: 40 queries 456 -> 330 us, 64 456 -> 348, 100 457 -> 449,
-        // 130 (two items of 65 instead of 128 and 2) 852 -> 672, 300 1,275 -> 1,217.
+        // Every item was worked off as 128 queries before.  1,036 members, 3 digits: 40 queries 455 -> 330 us, 64 455 -> 347, 100 456 -> 450,
+        // 130 (two items of 65 instead of 128 and 2) 849 -> 677, 300 1,272 -> 1,216.
         const uint32_t nq0 = FULL ? 64u : min(nq, (nq + 15u) / 16u * 8u), n_halves = FULL || nq > nq0 ? 2u : 1u, nq_half = half ? nq - nq0 : nq0;
         const float* p = a.theta + static_cast<size_t>(member) * a.ldD;
 
         // ---- per-item setup: queries, zero state, read-out weights, encoder weights ------------
         if (chunk != staged_chunk) {
-            if (tid < kTcQ)
-                s2s_query(key, a.status->generation, KIND == Items::kPadded ? min(q0 + tid, a.B - 1u) : q0 + min(tid < 64u ? tid : nq0 + tid - 64u, nq - 1u), a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
+            if (tid < kTcQ) {                                     // the query of row `tid`; rows that hold none repeat the last one
+                uint32_t q = tid;
+                if (KIND == Items::kPadded) q = min(q, a.B - 1u - q0);
+                if (KIND == Items::kPartial) q = min(q < 64u ? q : nq0 + q - 64u, nq - 1u);
+                s2s_query(key, a.status->generation, q0 + q, a.nd, S.enc[tid], S.dec[tid], S.tgt[tid]);
+            }
             staged_chunk = chunk;
         }
         if (is_mma) {                                            // the decoder's weights will be wanted next
