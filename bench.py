@@ -88,12 +88,12 @@ def stage_work(w, stored):
 # that digest; once a kernel's source changes its entry reads null until it is captured again.
 CSRC = os.path.join(ROOT, "paper_2202_05008_b200", "csrc")
 NCU_TRAFFIC = {
-    ("cfg4", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 3.535300e+08,
+    ("cfg4", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 3.536300e+08,
                          "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
-                         "digest": "c9171f29d050486e", "capture": "T = 200 (the parameters are read once, whatever the horizon)"},
+                         "digest": "57f64970386150f7", "capture": "T = 200 (the parameters are read once, whatever the horizon)"},
     ("cfg2", "stored"): {"kernel": "k_rollout_mlp2", "bytes": 4.793000e+06,
                          "files": ['rollout_mlp2.cu', 'mma_split.cuh', 'async.cuh', 'tasks.cuh', 'noise.cuh', 'internal.h'],
-                         "digest": "c9171f29d050486e", "capture": "full size"},
+                         "digest": "57f64970386150f7", "capture": "full size"},
     ("cfg3", "stored"): {"kernel": "k_cnn_conv2_tc", "bytes": 1.565100e+08,
                          "files": ['rollout_cnn_tc.cu', 'umma.cuh', 'async.cuh', 'fp32x2.cuh', 'internal.h'],
                          "digest": "92dd5c5bb53fc0c1", "capture": "full size"},

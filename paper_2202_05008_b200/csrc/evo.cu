@@ -25,7 +25,7 @@ struct evo_solver {
     const float*   d_target;
     uint64_t     launches;
     uint32_t     k0, k1;
-    S2sSplit     s2s;              // how a roll-out of narrow seq2seq cells is split
+    S2sSplit     s2s;              // how the queries of a seq2seq roll-out are split
     bool         deep;             // the control policy runs on k_rollout_mlp_deep
     bool         rollout_prepared;  // per-kernel attributes are set by the solver's first roll-out only
 };

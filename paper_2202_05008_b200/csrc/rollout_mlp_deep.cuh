@@ -11,7 +11,8 @@
 // reads the operands of every layer from shared memory in runtime loops, takes 1.69 and 2.21 us.  With the low parts in
 // registers too the compiler has none left to work with: 0.86 and 1.19 us, and 4.1 against 2.9 us for 16 episodes of 512 members.
 //
-// Above 128 units (KT = 12) a block has up to twelve warps and an SM to itself.  100 members, 4 episodes, us a step, with k_rollout_mlp_mma behind:
+// Above 128 units (KT = 12) a block has up to twelve warps, and an SM to itself unless it has one hidden layer (72 to 92 registers a thread: two blocks
+// of up to ten warps fit, of twelve for cart-pole and four episodes).  100 members, 4 episodes, us a step, with k_rollout_mlp_mma behind:
 // 28-160-8 0.47 / 1.34, 5-190-180-1 1.15 / 3.00, 5-145-52-48-1 1.31 / 2.22, 28-150-60-60-60-8 1.51 / 2.60.
 //
 // The instances are compiled in two files, by the episodes of a block: 72 kernels, and the longest of all the sources in one (the library in 134 s, now 59).

@@ -22,7 +22,7 @@
 // Only the triangles that matter are then walked, in order, from the ballots, with the tests that cut the rectangle; the
 // covering ones without any.  Bound by instruction issue (84 %).  64 triangles on 128 x 128 pixels, 1,024 members in
 // mid-training: 357 us with tiles of 32 x 16 pixels, a list of the triangles whose bounding box meets the tile and
-// every test per pixel; 183 us with the classes; 144 us with the tests per edge; 137 us with only the near triangles classified.
+// every test per pixel; 183 us with the classes; 142 us with the tests per edge; 135 us with only the near triangles classified.
 #include "internal.h"
 
 namespace evo {
@@ -66,8 +66,11 @@ struct PaintArgs {
 };
 
 // NEAR (more than 32 triangles): a warp first lists the triangles whose box overlaps its rectangle, and classifies only these: of 64 triangles of a
-// painting on its way 15, one round instead of two.  64 triangles on 128 x 128, 1,024 members 144 -> 138 us; 37 on 170 x 123, 146 members 28.1 -> 27.0; 100 on
-// 200 x 200, 250 members 116 -> 100.  With 32 triangles and fewer there is one round in either case: 30 on 100 x 100, 400 members 29.0 us, with a list 30.3.
+// painting on its way 15, one round instead of two.  64 triangles on 128 x 128, 1,024 members 142 -> 135 us; 158 on 61 x 131, 788 members 176 -> 162; 40 on
+// 128 x 128, 256 members 35.4 -> 33.4, gathered at the centre 26.0 -> 24.5, uniform over 1.2 times the canvas 37.7 -> 36.3.  Only where nearly every box covers
+// the canvas does the list save no round: 40 on 128 x 128 52.3 -> 53.8, 200 196 -> 199.  (Listing only where the boxes' mean share pays, by the last rectangle
+// or for the block, takes 6 to 8 registers more and costs every painting 3 to 13 %.)  With 32 triangles and fewer there is one round in either case: 30 on
+// 100 x 100, 400 members 29.0 us, with a list 30.3.
 template <bool NEAR>
 __global__ void __launch_bounds__(kPaintThreads)
 k_paint(const PaintArgs a)

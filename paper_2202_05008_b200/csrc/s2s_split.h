@@ -4,7 +4,8 @@
 
 namespace evo {
 
-// How the n-tiles (8 queries) of all members come to blocks: chunks of `chunk` n-tiles of a member, `chunks` of them per member, or
+// How the queries of all members come to blocks.  128 units (s2s_items): items of `chunk` queries of a member, `chunks` of them per member, which `places`
+// blocks take in turn.  Narrower cells (s2s_split), in n-tiles of 8 queries: chunks of `chunk` n-tiles of a member, `chunks` of them per member, or
 // (chunk = 0) a run of the tiles of all members for each of `places` blocks, worked off in pieces of one member.
 struct S2sSplit { uint32_t chunk, chunks, places; };
 
